@@ -1101,13 +1101,14 @@ extern "C" PIC_API int pic_collide(pic_t *h, const pic_collisions *p, int64_t *n
             return PIC_ERR_ARG;
         }
     if (int rc = settle(h)) return rc;
-    unsigned long long *d = nullptr;
-    if (cudaMallocAsync((void **)&d, sizeof(unsigned long long), h->st) != cudaSuccess) {
+    unsigned long long *d = nullptr;   // the pair count, then a work-queue counter per entry
+    const size_t db = sizeof(unsigned long long) + PIC_MAX_COLLISION_PAIRS * sizeof(int);
+    if (cudaMallocAsync((void **)&d, db, h->st) != cudaSuccess) {
         cudaGetLastError();
         set_error("pic_collide: allocation failed");
         return PIC_ERR_OOM;
     }
-    cudaMemsetAsync(d, 0, sizeof(unsigned long long), h->st);
+    cudaMemsetAsync(d, 0, db, h->st);
     int rc = collide(h, p, d);
     unsigned long long total = 0;
     if (!rc && (cudaMemcpyAsync(&total, d, sizeof(total), cudaMemcpyDeviceToHost, h->st) != cudaSuccess ||
