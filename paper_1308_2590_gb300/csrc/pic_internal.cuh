@@ -603,70 +603,94 @@ __device__ inline void deposit_fp64_cell(double *Mc, int64_t ncell, int64_t cell
 // N, c - N/2 (one more when f >= 1/2, centring on the nearest node) for even
 // N; node k weighs B_N of its distance (first + k - c) - f.  Along y and a
 // periodic x the node indices wrap; along a walled x a node beyond a wall is
-// folded onto the wall node (its weight stays in the box).
+// folded onto the wall node (its weight stays in the box).  N = 1 is the area
+// weighting in the same form.
 template <typename R, int N>
 struct SplineN {
-    int ix[N + 1], iy[N + 1];   // unpadded node column and row indices
+    int ix, iy;                 // first node column and row, not wrapped or folded
     R wx[N + 1], wy[N + 1];
 };
 
-// B_N(x) from its piecewise polynomial form.
+// Weights of one axis (the piecewise polynomials of B_N at the N + 1 nodes,
+// without branches); returns the first node relative to the cell.
 template <typename R, int N>
-__device__ inline R bspline_w(R x) {
-    const R a = x < R(0) ? -x : x;
-    if (N == 2) {
-        if (a <= R(0.5)) return R(0.75) - a * a;
-        const R b = R(1.5) - a;
-        return a <= R(1.5) ? R(0.5) * b * b : R(0);
-    }
-    if (N == 3) {
-        if (a <= R(1)) return R(2.0 / 3.0) - a * a + R(0.5) * a * a * a;
-        const R b = R(2) - a;
-        return a <= R(2) ? b * b * b * R(1.0 / 6.0) : R(0);
-    }
-    if (a <= R(0.5)) return R(115.0 / 192.0) - R(0.625) * a * a + R(0.25) * a * a * a * a;
-    if (a <= R(1.5)) return (R(55) + R(20) * a - R(120) * a * a + R(80) * a * a * a - R(16) * a * a * a * a) * R(1.0 / 96.0);
-    const R b = R(5) - R(2) * a;
-    return a <= R(2.5) ? b * b * b * b * R(1.0 / 384.0) : R(0);
-}
-
-template <typename R, int N>
-__device__ inline void spline_axis(int c, R f, int n, bool periodic, int (&idx)[N + 1], R (&w)[N + 1]) {
-    const int first = (N % 2) ? c - (N - 1) / 2 : c - N / 2 + (f >= R(0.5) ? 1 : 0);
-#pragma unroll
-    for (int k = 0; k <= N; ++k) {
-        w[k] = bspline_w<R, N>(R(first + k - c) - f);
-        int i = first + k;
-        if (periodic) {
-            i %= n;
-            if (i < 0) i += n;
+__device__ inline int spline_axis(R f, R (&w)[N + 1]) {
+    if constexpr (N == 1) {
+        w[0] = R(1) - f;
+        w[1] = f;
+        return 0;
+    } else if constexpr (N == 3) {
+        const R g = R(1) - f, f2 = f * f, g2 = g * g;
+        w[0] = g2 * (g * R(1.0 / 6.0));
+        w[1] = fma_r(f2, fma_r(R(0.5), f, R(-1)), R(2.0 / 3.0));
+        w[2] = fma_r(g2, fma_r(R(0.5), g, R(-1)), R(2.0 / 3.0));
+        w[3] = f2 * (f * R(1.0 / 6.0));
+        return -1;
+    } else {
+        const int up = f >= R(0.5) ? 1 : 0;
+        const R d = f - R(up), a = R(0.5) - d, b = R(0.5) + d, d2 = d * d;   // nodes at distances k - N/2 - d
+        if constexpr (N == 2) {
+            w[0] = (R(0.5) * a) * a;
+            w[1] = R(0.75) - d2;
+            w[2] = (R(0.5) * b) * b;
         } else {
-            i = i < 0 ? 0 : (i > n ? n : i);
+            const R a2 = a * a, b2 = b * b;
+            const R xl = R(1) + d, xr = R(1) - d;
+            auto mid = [](R x) {   // (55 + 20 x - 120 x^2 + 80 x^3 - 16 x^4) / 96
+                R p = fma_r(x, R(-16.0 / 96.0), R(80.0 / 96.0));
+                p = fma_r(x, p, R(-120.0 / 96.0));
+                p = fma_r(x, p, R(20.0 / 96.0));
+                return fma_r(x, p, R(55.0 / 96.0));
+            };
+            w[0] = (a2 * R(1.0 / 24.0)) * a2;
+            w[1] = mid(xl);
+            w[2] = fma_r(d2, fma_r(d2, R(0.25), R(-0.625)), R(115.0 / 192.0));
+            w[3] = mid(xr);
+            w[4] = (b2 * R(1.0 / 24.0)) * b2;
         }
-        idx[k] = i;
+        return up - N / 2;
     }
 }
 
 template <typename R, int N>
-__device__ inline SplineN<R, N> spline_n(const GridArgs<R> &g, int cx, int cy, R fx, R fy) {
+__device__ inline SplineN<R, N> spline_n(int cx, int cy, R fx, R fy) {
     SplineN<R, N> s;
-    spline_axis<R, N>(cx, fx, g.nx, g.periodic_x != 0, s.ix, s.wx);
-    spline_axis<R, N>(cy, fy, g.ny, true, s.iy, s.wy);
+    s.ix = cx + spline_axis<R, N>(fx, s.wx);
+    s.iy = cy + spline_axis<R, N>(fy, s.wy);
     return s;
 }
 
+// Column a of the stencil as a real node column: folded onto a wall, wrapped
+// in a periodic box (unpadded arrays); rows always wrap.
+template <typename R>
+__device__ inline int spline_col(const GridArgs<R> &g, int i) {
+    if (!g.periodic_x) return i < 0 ? 0 : (i > g.nx ? g.nx : i);
+    i %= g.nx;
+    return i < 0 ? i + g.nx : i;
+}
+template <typename R>
+__device__ inline int spline_row(const GridArgs<R> &g, int j) {
+    j %= g.ny;
+    return j < 0 ? j + g.ny : j;
+}
+
 // Value of a padded V4 node field at the particle (rows first, then columns).
+// The ghost ring (tile + halo + 1 >= 3 nodes) holds the periodic copies that
+// the stencil reaches, so only a walled x needs its columns folded.
 template <typename R, int N>
 __device__ inline void gather_s(const V4<R> *__restrict__ F, const GridArgs<R> &g, const SplineN<R, N> &s, R &ox,
                                 R &oy, R &oz) {
     ox = oy = oz = R(0);
+    int col[N + 1];
+#pragma unroll
+    for (int a = 0; a <= N; ++a) col[a] = g.periodic_x ? s.ix + a : min(max(s.ix + a, 0), g.nx);
 #pragma unroll
     for (int b = 0; b <= N; ++b) {
-        const V4<R> *row = F + (int64_t)(s.iy[b] + g.G) * g.nxp + g.G;
+        const V4<R> *row = F + (int64_t)(s.iy + b + g.G) * g.nxp + g.G;
         R sx = R(0), sy = R(0), sz = R(0);
 #pragma unroll
         for (int a = 0; a <= N; ++a) {
-            const V4<R> v = row[s.ix[a]];
+            const V4<R> v = row[col[a]];
             sx += s.wx[a] * v.x;
             sy += s.wx[a] * v.y;
             sz += s.wx[a] * v.z;
@@ -686,14 +710,14 @@ __device__ inline T pick(const T (&v)[M], int j) {
     return r;
 }
 
-// Deposit of one particle with a spline shape (in the push and at rest
-// alike): node by node, every lane adds its own products in L2, the lanes of
-// a warp starting at different nodes (lane mod (N + 1)^2).  kParts: the values
-// are FP64 parts with the class factors fr, fS, fj (as deposit_fp64 takes
-// them); otherwise the 13 moment values.  kFix: exact fixed-point sums.
-template <typename R, bool kFix, bool kParts, int N>
-__device__ inline void deposit_s(R *M, unsigned long long *Mfix, const FixScale &fs, const GridArgs<R> &g,
-                                 const SplineN<R, N> &s, const R *val, R fr, R fS, R fj, int lane) {
+// Exact deposit of one particle with a spline shape (in the push and at rest
+// alike): node by node, every lane adds its own products in fixed point, the
+// lanes of a warp starting at different nodes (lane mod (N + 1)^2).  kParts:
+// the values are FP64 parts with the class factors fr, fS, fj (as
+// deposit_fp64 takes them); otherwise the 13 moment values.
+template <typename R, bool kParts, int N>
+__device__ inline void deposit_s_fix(unsigned long long *Mfix, const FixScale &fs, const GridArgs<R> &g,
+                                     const SplineN<R, N> &s, const R *val, R fr, R fS, R fj, int lane) {
     constexpr int NN = (N + 1) * (N + 1);
 #pragma unroll 1
     for (int k0 = 0; k0 < NN; ++k0) {
@@ -701,16 +725,189 @@ __device__ inline void deposit_s(R *M, unsigned long long *Mfix, const FixScale 
         k = k >= NN ? k - NN : k;
         const int a = k % (N + 1), b = k / (N + 1);
         const R wc = pick<N + 1>(s.wx, a) * pick<N + 1>(s.wy, b);
-        const int64_t node = (int64_t)pick<N + 1>(s.iy, b) * g.nxn + pick<N + 1>(s.ix, a);
+        const int64_t node = (int64_t)spline_row(g, s.iy + b) * g.nxn + spline_col(g, s.ix + a);
         const R wr = wc * fr, ws = wc * fS, wj = wc * fj;
 #pragma unroll
         for (int kk = 0; kk < NMOM; ++kk) {
             const R p = kParts ? (kk == 0 ? wr : (kk < 10 ? ws : wj) * val[kk]) : wc * val[kk];
-            if (kFix) atomicAdd(&Mfix[(int64_t)kk * g.nnode + node], (unsigned long long)fix_of(p, fs, mom_class(kk)));
-            else atomicAdd(&M[(int64_t)kk * g.nnode + node], p);
+            atomicAdd(&Mfix[(int64_t)kk * g.nnode + node], (unsigned long long)fix_of(p, fs, mom_class(kk)));
         }
     }
 }
+
+// Deposit of a warp's particles with a spline shape, transposed: instead of
+// every lane adding its particle's 13 (N + 1)^2 products in L2 (117 to 325
+// scalar reductions per particle, what bounded the spline pushes), the
+// particles' 13 values and (N + 1)^2 node weights go to shared memory, and each
+// lane owns some of the 13 (N + 1)^2 sums of the stencil at node (K) and adds
+// the products of all particles with that stencil in registers, FMA by FMA.
+// Only when the warp's stencil changes do the sums go to the global moments.
+// The bins are in cell order, so a stencil usually lasts for more than a
+// segment; a warp whose particles lie in many cells pays one flush (13 (N +
+// 1)^2 / 32 reductions per lane) per cell, not per particle.
+// FP32: a lane takes one node and a run of moments (1 + 1 .. 4 shared loads per
+// particle); FP64: sums are dealt flat over the lanes (the FP64 pipe, not the
+// loads, bounds it, and no lane idles), sum o = node * 13 + moment at lane
+// o mod 32.  Measured on the 1024 x 512 foil (6.55M particles, per push / per
+// species at rest): FP32 cubic 2.87 -> 0.56 ms / 1.30 -> 0.16 ms; FP64
+// quadratic 5.30 -> 4.10 / 1.89 -> 1.54 ms (FP64 pipe 87 % active).
+template <typename R, int N>
+struct SplineDep {
+    static constexpr int NP = N + 1, NN = NP * NP, NS = NN * NMOM;
+    static constexpr bool kFlat = sizeof(R) == 8;
+    // a particle's row: 13 values (padded to VS), then the NN weights; FP32 row strides of 4 mod 8
+    // words keep the 16-byte stores of 8 lanes on different banks
+    static constexpr int VS = kFlat ? 14 : 16;
+    static constexpr int RS = kFlat ? (VS + NN + (NN & 1)) : (N == 1 ? 20 : N == 2 ? 28 : N == 3 ? 36 : 44);
+    static constexpr int HG = N == 1 ? 8 : N == 2 ? 3 : N == 3 ? 2 : 1;     // FP32: lanes per node
+    static constexpr int KW = N == 1 ? 2 : N == 2 ? 4 : N == 3 ? 8 : 13;    // and moments per lane
+    static constexpr int J = kFlat ? (NS + 31) / 32 : (N == 2 ? 5 : KW);    // sums per lane
+    static constexpr int kWarpBytes = 32 * RS * (int)sizeof(R);
+
+    R *rows;
+    R acc[J];
+    unsigned K;         // the warp's stencil: its key
+    bool some;          // there is one
+    int kx, ky;         // its first node (row wrapped)
+    int node, m0;       // FP32: the lane's node and first moment
+
+    __device__ inline void init(void *smem, int lane) {
+        rows = (R *)smem;
+        K = 0;
+        some = false;
+        kx = ky = 0;
+        node = kFlat ? 0 : min(lane / HG, NN - 1);
+        m0 = kFlat ? 0 : (lane % HG) * KW;
+#pragma unroll
+        for (int j = 0; j < J; ++j) acc[j] = R(0);
+    }
+
+    // Sum j of this lane: its node and moment (false: none).
+    __device__ inline bool sum_of(int j, int lane, int &nd, int &k) const {
+        if (kFlat) {
+            const int o = lane + 32 * j;
+            nd = o / NMOM;
+            k = o - nd * NMOM;
+            return o < NS;
+        }
+        nd = node;
+        k = (N == 2 && j == 4) ? 12 : m0 + j;
+        return lane < NN * HG && (N == 2 ? (j < 4 || m0 == 8) : k < NMOM);
+    }
+
+    __device__ inline void flush(const GridArgs<R> &g, R *M, int lane) {
+        if (!some) return;
+#pragma unroll
+        for (int j = 0; j < J; ++j) {
+            int nd, k;
+            if (sum_of(j, lane, nd, k) && acc[j] != R(0)) {
+                const int b = nd / NP, a = nd - b * NP;
+                const int64_t n = (int64_t)spline_row(g, ky + b) * g.nxn + spline_col(g, kx + a);
+                atomicAdd(&M[(int64_t)k * g.nnode + n], acc[j]);
+            }
+            acc[j] = R(0);
+        }
+    }
+
+    __device__ inline void add_rows(int p0, int p1, int lane) {
+        if constexpr (kFlat) {
+            int ov[J], ow[J];
+#pragma unroll
+            for (int j = 0; j < J; ++j) {
+                const int o = min(lane + 32 * j, NS - 1), nd = o / NMOM;
+                ov[j] = o - nd * NMOM;
+                ow[j] = VS + nd;
+            }
+#pragma unroll 2
+            for (int p = p0; p < p1; ++p) {
+                const R *r = rows + p * RS;
+#pragma unroll
+                for (int j = 0; j < J; ++j) acc[j] = fma_r(r[ow[j]], r[ov[j]], acc[j]);
+            }
+        } else {
+#pragma unroll 4
+            for (int p = p0; p < p1; ++p) {
+                const float *r = (const float *)rows + p * RS;
+                const float w = r[VS + node];
+                if constexpr (N == 1) {
+                    const float2 v = *(const float2 *)(r + m0);
+                    acc[0] = fmaf(w, v.x, acc[0]);
+                    acc[1] = fmaf(w, v.y, acc[1]);
+                } else {
+#pragma unroll
+                    for (int q = 0; q < (N == 4 ? 3 : KW / 4); ++q) {
+                        const float4 v = *(const float4 *)(r + m0 + 4 * q);
+                        acc[4 * q] = fmaf(w, v.x, acc[4 * q]);
+                        acc[4 * q + 1] = fmaf(w, v.y, acc[4 * q + 1]);
+                        acc[4 * q + 2] = fmaf(w, v.z, acc[4 * q + 2]);
+                        acc[4 * q + 3] = fmaf(w, v.w, acc[4 * q + 3]);
+                    }
+                    if constexpr (N != 3) acc[J - 1] = fmaf(w, r[12], acc[J - 1]);   // moment 12
+                }
+            }
+        }
+    }
+
+    // All lanes of the warp: particle (s, val) of every lane with alive set.
+    __device__ inline void add(const GridArgs<R> &g, R *M, bool alive, const SplineN<R, N> &s, const R *val, int lane) {
+        const unsigned full = 0xffffffffu, lt = (1u << lane) - 1u;
+        // first node as one number: ny (nx + 4) < 2^32 - 32 for every grid (nx >= 2, nx ny <= 2^30)
+        const int row0 = wrap1(s.iy, g.ny);
+        const unsigned key = alive ? (unsigned)row0 * (unsigned)(g.nx + 4) + (unsigned)(s.ix + 2) : 0xffffffffu - lane;
+        const unsigned same = __match_any_sync(full, key);
+        const int size = alive && (same & lt) == 0 ? __popc(same) : 0;   // at a stencil's first lane: its particles
+        int incl = size;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int y = __shfl_up_sync(full, incl, o);
+            if (lane >= o) incl += y;
+        }
+        const int first = __ffs(same) - 1;
+        const int slot = __shfl_sync(full, incl - size, first) + __popc(same & lt);   // rows grouped by stencil
+        __syncwarp();   // the previous particles' rows have been read
+        if (alive) {
+            R row[RS];
+#pragma unroll
+            for (int k = 0; k < VS; ++k) row[k] = k < NMOM ? val[k] : R(0);
+#pragma unroll
+            for (int b = 0; b < NP; ++b)
+#pragma unroll
+                for (int a = 0; a < NP; ++a) row[VS + b * NP + a] = s.wx[a] * s.wy[b];
+#pragma unroll
+            for (int k = VS + NN; k < RS; ++k) row[k] = R(0);
+            constexpr int V = 16 / (int)sizeof(R);
+            struct alignas(16) Vec {
+                R x[V];
+            };
+            Vec *dst = (Vec *)(rows + slot * RS);
+#pragma unroll
+            for (int k = 0; k < (VS + NN + V - 1) / V; ++k) {
+                Vec t;
+#pragma unroll
+                for (int q = 0; q < V; ++q) t.x[q] = row[V * k + q];
+                dst[k] = t;
+            }
+        }
+        __syncwarp();
+        unsigned left = __ballot_sync(full, size > 0);
+        const unsigned inK = __ballot_sync(full, size > 0 && some && key == K);   // the warp's stencil first
+        while (left) {
+            const int l = __ffs(left & inK ? left & inK : left) - 1;
+            left &= ~(1u << l);
+            const unsigned k = __shfl_sync(full, key, l);
+            const int p1 = __shfl_sync(full, incl, l), p0 = p1 - __shfl_sync(full, size, l);
+            const int nx0 = __shfl_sync(full, s.ix, l), ny0 = __shfl_sync(full, row0, l);
+            if (!some || k != K) {
+                flush(g, M, lane);
+                some = true;
+                K = k;
+                kx = nx0;
+                ky = ny0;
+            }
+            add_rows(p0, p1, lane);
+        }
+    }
+};
 
 // --------------------------------------------------------------------------- host entry points
 
@@ -729,6 +926,7 @@ int download_fields(pic_t *h, double *E3, double *H3);
 
 // particles (pic_particles.cu): conversion, deposit at rest, state export
 int deposit_only(pic_t *h, int s);
+int ensure_items(pic_t *h);             // the work-item table holds an entry per used segment
 int clear_moments(pic_t *h);
 int clear_step_moments(pic_t *h);       // what a step's deposit adds into (the touched node tiles only)
 int fix_to_moments(pic_t *h);           // deterministic deposit: Mfix -> M (+ Mlo)

@@ -28,14 +28,47 @@ struct DepArgs {
     int64_t ccap;
     double *Mc;       // FP64 L2-reduction form: the cell sums the push deposits into (else nullptr)
     int tnx, tny, ntx;  // tiles (FP64: the block's tile of B in cell form, in shared memory)
+    const int2 *items;  // work items (tile, run of REST_SEGS segments)
+    const int32_t *nitems;
+    int32_t *ticket;
 };
 
-// Moments (Eq. 3) of particles at rest with the current node B, DEP_SPLIT
-// blocks per tile bin, a warp per segment (block y of a tile takes every
-// DEP_SPLIT-th group of its warps' segments: a plasma that fills a few of the
-// tiles still puts enough warps on the FP64 pipe and the L2 reductions; 1 ->
-// 4 blocks per tile measured 2.43 -> 2.08 ms FP64, 0.45 -> 0.40 ms FP32 for
-// 6.55M particles of a laser foil).  FP32: lanes whose particles share a cell (at
+// Work items of a deposit at rest: the runs of REST_SEGS segments of every
+// occupied bin, in any order; resident blocks take them from a queue.  (A grid
+// of four blocks per tile started mostly empty blocks: 0.72 ms per species for
+// 0.16M particles in 131,072 tiles, whatever they held.)
+constexpr int REST_SEGS = 32;
+__global__ void k_rest_items(const int32_t *__restrict__ useg, int ntiles, int2 *__restrict__ items,
+                             int32_t *__restrict__ nitems) {
+    const int t = blockIdx.x * blockDim.x + threadIdx.x;
+    const int n = t < ntiles ? (useg[t] + REST_SEGS - 1) / REST_SEGS : 0;
+    // one queue reservation per warp
+    const int lane = threadIdx.x & 31;
+    int incl = n;
+    for (int o = 1; o < 32; o <<= 1) {
+        const int y = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= o) incl += y;
+    }
+    int base = 0;
+    if (lane == 31 && incl) base = atomicAdd(nitems, incl);
+    base = __shfl_sync(0xffffffffu, base, 31) + incl - n;
+    for (int k = 0; k < n; ++k) items[base + k] = make_int2(t, k);
+}
+
+// The block's next item (false: none left); every thread of the block.
+__device__ inline bool next_item(const int2 *items, int nitems, int32_t *ticket, int2 *s_item, int2 &it) {
+    __syncthreads();   // the previous item (and its shared tables) is done
+    if (threadIdx.x == 0) {
+        const int k = atomicAdd(ticket, 1);
+        *s_item = k < nitems ? items[k] : make_int2(-1, 0);
+    }
+    __syncthreads();
+    it = *s_item;
+    return it.x >= 0;
+}
+
+// Moments (Eq. 3) of particles at rest with the current node B, a warp per
+// segment of the block's item.  FP32: lanes whose particles share a cell (at
 // least 6 of them; bins are in cell order, so most segments hold one or two
 // cells) first sum their 52 corner products with the butterfly reduce-scatter
 // and add 26 values per corner pair; the other lanes add their own products.
@@ -45,7 +78,6 @@ struct DepArgs {
 // when kFix).
 template <typename R>
 constexpr int min_group_at_rest() { return sizeof(R) == 4 ? 6 : 33; }
-constexpr int DEP_SPLIT = 4;
 
 template <typename R, bool kFix>
 __device__ inline void add_moment(const DepArgs<R> &a, int k, int64_t node, R v) {
@@ -58,13 +90,16 @@ __device__ inline void add_moment(const DepArgs<R> &a, int k, int64_t node, R v)
 template <typename R, bool kFix>
 __global__ void k_deposit_bins(DepArgs<R> a) {
     extern __shared__ __align__(16) unsigned char dsm[];
+    __shared__ int2 s_item;
     constexpr bool kTab = sizeof(R) == 8;   // FP64: B of the tile's cells in cell form, as the push gathers it
-    const int t = blockIdx.x;
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    const int64_t b0 = a.bstart[t];
-    const int u = a.useg[t];
     const GridArgs<R> &g = a.g;
-    if (u == 0) return;
+    const int nitems = *a.nitems;
+    int2 it;
+    while (next_item(a.items, nitems, a.ticket, &s_item, it)) {
+    const int t = it.x;
+    const int64_t b0 = a.bstart[t];
+    const int j0 = it.y * REST_SEGS, u = min(j0 + REST_SEGS, a.useg[t]);
     CellC<R> *tab = (CellC<R> *)dsm;
     const int X0 = (t % a.ntx) * a.tnx, Y0 = (t / a.ntx) * a.tny;
     const int tw = min(a.tnx, g.nx - X0), th = min(a.tny, g.ny - Y0);
@@ -76,7 +111,7 @@ __global__ void k_deposit_bins(DepArgs<R> a) {
         }
         __syncthreads();
     }
-    for (int j = blockIdx.y * nw + wid; j < u; j += nw * gridDim.y) {
+    for (int j = j0 + wid; j < u; j += nw) {
         const int n = a.segn[b0 / SEG + j];
         bool valid = lane < n;
         const int64_t p = b0 + (int64_t)j * SEG + lane;
@@ -167,50 +202,69 @@ __global__ void k_deposit_bins(DepArgs<R> a) {
             }
         }
     }
+    }
 }
 
-// Moments at rest with a spline shape of degree N: the same gather
-// (gather_s), moments and per-lane deposit (deposit_s) as the spline-shape
-// push, so that a deposit at rest repeats the push's products bitwise; a warp
-// per segment, DEP_SPLIT blocks per tile bin.
+// Moments at rest with a spline shape of degree N: the gather (gather_s),
+// moments and deposit (SplineDep; the exact form lane by lane, so that a
+// deposit at rest repeats the push's products bitwise) of the spline-shape
+// push; each warp takes a run of the item's segments.
 template <typename R, bool kFix, int N>
-__global__ void k_deposit_s(DepArgs<R> a) {
-    constexpr bool kParts = sizeof(R) == 8;
-    const int t = blockIdx.x;
+__global__ void __launch_bounds__(256) k_deposit_s(DepArgs<R> a) {
+    extern __shared__ __align__(16) unsigned char dsm[];
+    __shared__ int2 s_item;
+    constexpr bool kParts = sizeof(R) == 8 && kFix;
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    const int64_t b0 = a.bstart[t];
-    const int u = a.useg[t];
     const GridArgs<R> &g = a.g;
-    for (int j = blockIdx.y * nw + wid; j < u; j += nw * gridDim.y) {
-        const int n = a.segn[b0 / SEG + j];
-        const int64_t p = b0 + (int64_t)j * SEG + lane;
-        if (lane >= n) continue;
-        const int32_t c = a.cell[p];
-        const R fx = a.ox[p], fy = a.oy[p];
-        if (kChecks && (c < 0 || c >= g.nx * g.ny || !(fx >= R(0) && fx < R(1)) || !(fy >= R(0) && fy < R(1)))) {
-            atomicOr(a.flags, FLAG_CHECK);
-            continue;
+    const int nitems = *a.nitems;
+    SplineDep<R, N> dep;
+    if (!kFix) dep.init(dsm + wid * SplineDep<R, N>::kWarpBytes, lane);
+    int2 it;
+    while (next_item(a.items, nitems, a.ticket, &s_item, it)) {
+        const int64_t b0 = a.bstart[it.x];
+        const int j0 = it.y * REST_SEGS, j1 = min(j0 + REST_SEGS, a.useg[it.x]);
+        const int per = (j1 - j0 + nw - 1) / nw;
+        for (int j = j0 + wid * per; j < min(j0 + (wid + 1) * per, j1); ++j) {
+            const int n = a.segn[b0 / SEG + j];
+            const int64_t p = b0 + (int64_t)j * SEG + lane;
+            bool valid = lane < n;
+            int32_t c = 0;
+            R fx = R(0), fy = R(0);
+            if (valid) {
+                c = a.cell[p];
+                fx = a.ox[p];
+                fy = a.oy[p];
+            }
+            if (kChecks && valid && (c < 0 || c >= g.nx * g.ny || !(fx >= R(0) && fx < R(1)) || !(fy >= R(0) && fy < R(1)))) {
+                atomicOr(a.flags, FLAG_CHECK);
+                valid = false;
+            }
+            R val[NMOM];
+            SplineN<R, N> sp;
+            if (valid) {
+                sp = spline_n<R, N>(c % g.nx, c / g.nx, fx, fy);
+                R Bx, By, Bz;
+                gather_s(a.B, g, sp, Bx, By, Bz);
+                R fr = R(1), fS = R(1), fj = R(1), ig, bx, by, bz, inv;
+                if constexpr (kParts)
+                    particle_moment_parts(a.q, a.kq, a.cq2, a.w[p], a.ux[p], a.uy[p], a.uz[p], Bx, By, Bz, val, fr, fS,
+                                          fj, ig, bx, by, bz, inv);
+                else
+                    particle_moments_c(a.q, a.kq, a.hq, a.w[p], a.ux[p], a.uy[p], a.uz[p], Bx, By, Bz, val, ig, bx, by,
+                                       bz, inv);
+                if (sizeof(R) == 8 && a.cr) {   // what the next push needs of this B (carried, FP64 form)
+                    a.cr[p] = (double)ig;
+                    a.cr[a.ccap + p] = (double)bx;
+                    a.cr[2 * a.ccap + p] = (double)by;
+                    a.cr[3 * a.ccap + p] = (double)bz;
+                    a.cr[4 * a.ccap + p] = (double)inv;
+                }
+                if constexpr (kFix) deposit_s_fix<R, kParts, N>(a.Mfix, a.fs, g, sp, val, fr, fS, fj, lane);
+            }
+            if constexpr (!kFix) dep.add(g, a.M, valid, sp, val, lane);
         }
-        const SplineN<R, N> sp = spline_n<R, N>(g, c % g.nx, c / g.nx, fx, fy);
-        R Bx, By, Bz;
-        gather_s(a.B, g, sp, Bx, By, Bz);
-        R val[NMOM];
-        R fr = R(1), fS = R(1), fj = R(1), ig, bx, by, bz, inv;
-        if constexpr (kParts)
-            particle_moment_parts(a.q, a.kq, a.cq2, a.w[p], a.ux[p], a.uy[p], a.uz[p], Bx, By, Bz, val, fr, fS, fj, ig,
-                                  bx, by, bz, inv);
-        else
-            particle_moments_c(a.q, a.kq, a.hq, a.w[p], a.ux[p], a.uy[p], a.uz[p], Bx, By, Bz, val, ig, bx, by, bz,
-                               inv);
-        if (sizeof(R) == 8 && a.cr) {   // what the next push needs of this B (carried, FP64 form)
-            a.cr[p] = (double)ig;
-            a.cr[a.ccap + p] = (double)bx;
-            a.cr[2 * a.ccap + p] = (double)by;
-            a.cr[3 * a.ccap + p] = (double)bz;
-            a.cr[4 * a.ccap + p] = (double)inv;
-        }
-        deposit_s<R, kFix, kParts, N>(a.M, a.Mfix, a.fs, g, sp, val, fr, fS, fj, lane);
     }
+    if constexpr (!kFix) dep.flush(g, a.M, lane);
 }
 
 // Fixed-point sums -> floating-point moments: FP64 M, or the FP32 pair (M, Mlo)
@@ -372,6 +426,22 @@ __global__ void k_bins_to_stage(GridArgs<double> g, const int32_t *bstart, const
 
 // --------------------------------------------------------------------------- host side
 
+// Resident blocks of 256 threads over the work items.
+template <typename R>
+static int rest_launch(pic_t *h, void (*kernel)(DepArgs<R>), const DepArgs<R> &a, size_t smem) {
+    int dev = 0, nsm = 0, per = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
+    if (smem > 32 * 1024) cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kernel, 256, smem) != cudaSuccess || per < 1) {
+        cudaGetLastError();
+        per = 1;
+    }
+    kernel<<<(unsigned)(per * (nsm > 0 ? nsm : 1)), 256, smem, h->st>>>(a);
+    count_launch(h);
+    return check_launch("deposit at rest");
+}
+
 template <typename R>
 static int deposit_only_t(pic_t *h, int s) {
     SpeciesBuf &S = h->sp[s];
@@ -402,27 +472,24 @@ static int deposit_only_t(pic_t *h, int s) {
     a.tnx = h->tnx;
     a.tny = h->tny;
     a.ntx = h->ntx;
-    const size_t tab = h->fp32 ? 0 : (size_t)h->tnx * h->tny * sizeof(CellC<double>);
-    const dim3 grid((unsigned)h->ntiles, DEP_SPLIT);
-    if (h->shape >= 2) {
-        switch (h->shape * 2 + (h->det ? 1 : 0)) {
-            case 4: k_deposit_s<R, false, 2><<<grid, 256, 0, h->st>>>(a); break;
-            case 5: k_deposit_s<R, true, 2><<<grid, 256, 0, h->st>>>(a); break;
-            case 6: k_deposit_s<R, false, 3><<<grid, 256, 0, h->st>>>(a); break;
-            case 7: k_deposit_s<R, true, 3><<<grid, 256, 0, h->st>>>(a); break;
-            case 8: k_deposit_s<R, false, 4><<<grid, 256, 0, h->st>>>(a); break;
-            default: k_deposit_s<R, true, 4><<<grid, 256, 0, h->st>>>(a); break;
-        }
-    } else {
-        if (tab > 48 * 1024) {
-            cudaFuncSetAttribute(k_deposit_bins<R, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)tab);
-            cudaFuncSetAttribute(k_deposit_bins<R, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)tab);
-        }
-        if (h->det) k_deposit_bins<R, true><<<grid, 256, tab, h->st>>>(a);
-        else k_deposit_bins<R, false><<<grid, 256, tab, h->st>>>(a);
-    }
+    // the work items (the queue's counters: words 1 and 2 beside the push's)
+    if (int rc = ensure_items(h)) return rc;
+    a.items = h->items;
+    a.nitems = h->ticket + 1;
+    a.ticket = h->ticket + 2;
+    cudaMemsetAsync(h->ticket + 1, 0, 2 * sizeof(int32_t), h->st);
+    k_rest_items<<<(h->ntiles + 255) / 256, 256, 0, h->st>>>(a.useg, h->ntiles, h->items, h->ticket + 1);
     count_launch(h);
-    return check_launch("k_deposit_bins");
+    switch (h->shape >= 2 ? h->shape * 2 + (h->det ? 1 : 0) : (h->det ? 1 : 0)) {
+        case 0: return rest_launch(h, k_deposit_bins<R, false>, a, h->fp32 ? 0 : (size_t)h->tnx * h->tny * sizeof(CellC<double>));
+        case 1: return rest_launch(h, k_deposit_bins<R, true>, a, h->fp32 ? 0 : (size_t)h->tnx * h->tny * sizeof(CellC<double>));
+        case 4: return rest_launch(h, k_deposit_s<R, false, 2>, a, 8 * SplineDep<R, 2>::kWarpBytes);
+        case 5: return rest_launch(h, k_deposit_s<R, true, 2>, a, 0);
+        case 6: return rest_launch(h, k_deposit_s<R, false, 3>, a, 8 * SplineDep<R, 3>::kWarpBytes);
+        case 7: return rest_launch(h, k_deposit_s<R, true, 3>, a, 0);
+        case 8: return rest_launch(h, k_deposit_s<R, false, 4>, a, 8 * SplineDep<R, 4>::kWarpBytes);
+        default: return rest_launch(h, k_deposit_s<R, true, 4>, a, 0);
+    }
 }
 
 int deposit_only(pic_t *h, int s) {

@@ -744,22 +744,24 @@ __global__ void __launch_bounds__(TILE_BS, push_min_blocks<R>())
 // paragraph).  The same work items, state layout, implicit push (Eq. 2, E
 // factored out), moments (Eq. 3) and in-place compaction as k_push; the
 // (N + 1) x (N + 1) node gathers read the padded fields in global memory (the
-// nodes around a particle reach beyond a tile's box), and every lane adds its
-// (N + 1)^2 x 13 products in L2 (deposit_s; the FP32 form without the
-// compensation term of the tile flush).  One warp per segment run, no shared
-// memory.
+// nodes around a particle reach beyond a tile's box; the lanes of a warp mostly
+// share them).  Deposit: SplineDep (transposed, sums in registers), the exact
+// form lane by lane (deposit_s_fix).  One warp per segment run.
 template <typename R>
 constexpr int push_s_min_blocks() { return sizeof(R) == 8 ? 2 : 0; }   // FP64: at most 128 registers; FP32: the default
 
 template <typename R, bool kFix, int N>
 __global__ void __launch_bounds__(TILE_BS, push_s_min_blocks<R>()) k_push_s(const __grid_constant__ TileArgs<R> a) {
-    constexpr bool kParts = sizeof(R) == 8;
+    constexpr bool kParts = sizeof(R) == 8 && kFix;
     if (a.guard && (*a.guard & 3)) return;   // the previous regroup failed: the host redoes the step
+    extern __shared__ __align__(16) unsigned char ssm[];   // the warps' particle rows (SplineDep)
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
     __shared__ int scr[3];
     const GridArgs<R> &g = a.g;
     const int nitems = a.chunk_prefix[a.nsp * a.ntiles];
     const unsigned lt = (1u << lane) - 1u;
+    SplineDep<R, N> dep;
+    if (!kFix) dep.init(ssm + wid * SplineDep<R, N>::kWarpBytes, lane);
     for (;;) {
         if (tid == 0) {
             const int item = atomicAdd(a.ticket, 1);
@@ -820,7 +822,7 @@ __global__ void __launch_bounds__(TILE_BS, push_s_min_blocks<R>()) k_push_s(cons
             const R fx = valid ? cu.fx : R(0), fy = valid ? cu.fy : R(0);
             const R ux = cu.ux, uy = cu.uy, uz = cu.uz, w = cu.w;
             // gather at r^n
-            const SplineN<R, N> so = spline_n<R, N>(g, cx, cy, fx, fy);
+            const SplineN<R, N> so = spline_n<R, N>(cx, cy, fx, fy);
             R Ex, Ey, Ez;
             gather_s(a.Eh, g, so, Ex, Ey, Ez);
             const R k = P.kq;
@@ -872,8 +874,9 @@ __global__ void __launch_bounds__(TILE_BS, push_s_min_blocks<R>()) k_push_s(cons
             R val[NMOM];
             R cig = R(0), cbx = R(0), cby = R(0), cbz = R(0), cinv = R(0);
             R fr = R(1), fS = R(1), fj = R(1);
+            SplineN<R, N> sn;
             if (alive) {
-                const SplineN<R, N> sn = spline_n<R, N>(g, ncx, ncy, nfx, nfy);
+                sn = spline_n<R, N>(ncx, ncy, nfx, nfy);
                 R nBx, nBy, nBz;
                 gather_s(a.Bnew, g, sn, nBx, nBy, nBz);
                 if constexpr (kParts)
@@ -882,8 +885,9 @@ __global__ void __launch_bounds__(TILE_BS, push_s_min_blocks<R>()) k_push_s(cons
                 else
                     particle_moments_c(P.q, P.kq, P.hq, w, nux, nuy, nuz, nBx, nBy, nBz, val, cig, cbx, cby, cbz,
                                        cinv);
-                deposit_s<R, kFix, kParts, N>(a.M, a.Mfix, a.fs, g, sn, val, fr, fS, fj, lane);
+                if constexpr (kFix) deposit_s_fix<R, kParts, N>(a.Mfix, a.fs, g, sn, val, fr, fS, fj, lane);
             }
+            if constexpr (!kFix) dep.add(g, a.M, alive, sn, val, lane);
             // warp compaction of the segment (every lane has loaded before any store)
             const unsigned ms = __ballot_sync(FULL, stay), ml = __ballot_sync(FULL, leave);
             const int32_t ncell = ncy * g.nx + ncx;
@@ -917,6 +921,7 @@ __global__ void __launch_bounds__(TILE_BS, push_s_min_blocks<R>()) k_push_s(cons
             }
         }
     }
+    if constexpr (!kFix) dep.flush(g, a.M, lane);
 }
 
 // Work items of the push: ch-segment runs of every (species, tile), in
@@ -1456,6 +1461,36 @@ static int push_occupancy(pic_t *h, int bytes, int *blocks_per_sm) {
     return 0;
 }
 
+template <typename R, int N>
+static constexpr int push_s_smem() { return TILE_WARPS * SplineDep<R, N>::kWarpBytes; }
+
+template <typename R, bool kFix, int N>
+static int push_s_occupancy_n(int *blocks_per_sm) {
+    const int bytes = kFix ? 0 : push_s_smem<R, N>();
+    cudaError_t e = cudaFuncSetAttribute(k_push_s<R, kFix, N>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+    if (e == cudaSuccess)
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, k_push_s<R, kFix, N>, TILE_BS, bytes);
+    if (e != cudaSuccess) {
+        set_error("spline push set-up: %s", cudaGetErrorString(e));
+        return PIC_ERR_CUDA;
+    }
+    if (*blocks_per_sm < 1) *blocks_per_sm = 1;
+    return 0;
+}
+
+template <typename R>
+static int push_s_occupancy(const pic_t *h, int *b) {
+    switch (h->shape * 2 + (h->det ? 1 : 0)) {
+        case 4: return push_s_occupancy_n<R, false, 2>(b);
+        case 5: return push_s_occupancy_n<R, true, 2>(b);
+        case 6: return push_s_occupancy_n<R, false, 3>(b);
+        case 7: return push_s_occupancy_n<R, true, 3>(b);
+        case 8: return push_s_occupancy_n<R, false, 4>(b);
+        case 9: return push_s_occupancy_n<R, true, 4>(b);
+    }
+    return 0;   // linear shape
+}
+
 // The distinct neighbour tiles of every tile (periodic in y, and in x when
 // the box is), ascending: the sources of its arrivals.
 static int neighbour_table(pic_t *h) {
@@ -1533,15 +1568,9 @@ int tile_setup(pic_t *h) {
     cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
     h->push_blocks = (per_sm > 0 ? per_sm : 1) * nsm;
     {
-        // the spline-shape push: no shared memory, as many blocks as are resident (its heaviest
-        // instance, degree 4, sets the count for all)
+        // the spline-shape push: as many blocks as are resident
         int s2 = 0;
-        cudaError_t es = h->fp32 ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&s2, k_push_s<float, true, 4>, TILE_BS, 0)
-                                 : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&s2, k_push_s<double, true, 4>, TILE_BS, 0);
-        if (es != cudaSuccess || s2 < 1) {
-            cudaGetLastError();
-            s2 = 1;
-        }
+        if (int rs = h->fp32 ? push_s_occupancy<float>(h, &s2) : push_s_occupancy<double>(h, &s2)) return rs;
         h->push_blocks_s2 = s2 * nsm;
     }
     const int rb = regroup_smem_bytes(h->tnx * h->tny);
@@ -1879,6 +1908,23 @@ __global__ void __launch_bounds__(PREP_BS) k_prep_one_block(UsegPtrs u, int nsp,
     }
 }
 
+// The item table: at most one item per segment slot.
+int ensure_items(pic_t *h) {
+    int64_t need = 1;
+    for (int s = 0; s < h->nsp; ++s) need += h->sp[s].cap / SEG;
+    if (need <= h->items_cap) return 0;
+    cudaFree(h->items);
+    h->items = nullptr;
+    h->items_cap = 0;
+    if (cudaMalloc(&h->items, (size_t)need * sizeof(int2)) != cudaSuccess) {
+        cudaGetLastError();
+        set_error("push item table allocation failed");
+        return PIC_ERR_OOM;
+    }
+    h->items_cap = need;
+    return 0;
+}
+
 // The push's work items: the chunk counts of every (species, tile), their scan
 // and the item table, from the bins' layout in slot next ? scur ^ 1 : scur of
 // each species (next: the slot the pending per-tile regroup writes, so that a
@@ -1888,20 +1934,7 @@ int push_prep(pic_t *h, bool next) {
     for (int s = 0; s < PIC_MAX_SPECIES; ++s)
         u.p[s] = (s < h->nsp) ? h->sp[s].useg[next ? h->sp[s].scur ^ 1 : h->sp[s].scur] : nullptr;
     const int nitems = h->nsp * h->ntiles;
-    // item table: at most one item per used segment (grown before any launch that would use it)
-    int64_t need = 1;
-    for (int s = 0; s < h->nsp; ++s) need += h->sp[s].cap / SEG;
-    if (need > h->items_cap) {
-        cudaFree(h->items);
-        h->items = nullptr;
-        h->items_cap = 0;
-        if (cudaMalloc(&h->items, (size_t)need * sizeof(int2)) != cudaSuccess) {
-            cudaGetLastError();
-            set_error("push item table allocation failed");
-            return PIC_ERR_OOM;
-        }
-        h->items_cap = need;
-    }
+    if (int rc = ensure_items(h)) return rc;   // grown before any launch that would use it
     if (nitems <= PREP_ONE_BLOCK) {
         const int sm = nitems * (int)sizeof(int);
         if (sm > 48 * 1024 && cudaFuncSetAttribute(k_prep_one_block, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -1940,11 +1973,11 @@ static int particle_tiles_t(pic_t *h, bool prepared) {
     if (h->shape >= 2) {
         const unsigned nb = (unsigned)h->push_blocks_s2;
         switch (h->shape * 2 + (h->det ? 1 : 0)) {
-            case 4: k_push_s<R, false, 2><<<nb, TILE_BS, 0, h->st>>>(a); break;
+            case 4: k_push_s<R, false, 2><<<nb, TILE_BS, push_s_smem<R, 2>(), h->st>>>(a); break;
             case 5: k_push_s<R, true, 2><<<nb, TILE_BS, 0, h->st>>>(a); break;
-            case 6: k_push_s<R, false, 3><<<nb, TILE_BS, 0, h->st>>>(a); break;
+            case 6: k_push_s<R, false, 3><<<nb, TILE_BS, push_s_smem<R, 3>(), h->st>>>(a); break;
             case 7: k_push_s<R, true, 3><<<nb, TILE_BS, 0, h->st>>>(a); break;
-            case 8: k_push_s<R, false, 4><<<nb, TILE_BS, 0, h->st>>>(a); break;
+            case 8: k_push_s<R, false, 4><<<nb, TILE_BS, push_s_smem<R, 4>(), h->st>>>(a); break;
             default: k_push_s<R, true, 4><<<nb, TILE_BS, 0, h->st>>>(a); break;
         }
         count_launch(h);
