@@ -326,6 +326,7 @@ static int resolve_pending(pic_t *h, bool *rebuilt = nullptr) {
     if (f & 3) {
         commit_regroup(h);   // back to the layout the push left
         if (int rc = rebuild_from_step(h)) return rc;
+        if (h->post) h->moments_stale = true;   // that step's deposit, after its regroup, did nothing
         if (rebuilt) *rebuilt = true;
     }
     return 0;
@@ -460,6 +461,7 @@ static void setup_geometry(pic_t *h, const pic_config &c) {
     h->rs = h->fp32 ? 4 : 8;
     h->det = (c.deposit == PIC_DEPOSIT_DETERMINISTIC);
     h->shape = c.shape > 1 ? c.shape : 1;
+    h->post = post_deposit(h);
     h->periodic_x = (c.bc_x == PIC_BC_PERIODIC);
     h->nx = c.nx;
     h->ny = c.ny;
@@ -1298,6 +1300,26 @@ static int particle_step(pic_t *h, int p, const int32_t *guard, cudaStream_t mai
     return 0;
 }
 
+// After a step's regroup is committed, where its moments are deposited from the
+// regrouped bins: the next push's work items, which that deposit shares, and
+// the deposit (nothing if this step's regroup, or the guarding one, failed).
+static int step_deposit(pic_t *h, int p, const int32_t *guard) {
+    timing_begin(h);
+    const int64_t l0 = h->timing.launches[4];
+    if (int rc = push_prep(h, false)) return rc;
+    if (int rc = deposit_step(h, h->d_step_flags + p, guard)) return rc;
+    timing_end(h, 0, (int)(h->timing.launches[4] - l0));
+    return 0;
+}
+
+// Field solve of the time-centred mode, node B of the new H, ghost rings.
+static int field_cn_step(pic_t *h) {
+    int rc = field_cn(h);
+    if (!rc) rc = node_average(h, 1 - h->hcur, 1 - h->bcur);
+    if (!rc) rc = fill_ghosts(h, h->Ehalf);
+    return rc;
+}
+
 extern "C" PIC_API int pic_step(pic_t *h, int nsteps) {
     if (!h || nsteps < 0) {
         set_error("pic_step: bad handle or step count");
@@ -1347,8 +1369,13 @@ extern "C" PIC_API int pic_step(pic_t *h, int nsteps) {
         // 3. push, deposit, regroup -- queued at once: they do nothing if the previous step's regroup
         //    (still in flight) fails, and the host redoes them after the full sort below
         const bool prev = h->flags_pending;
-        if ((rc = particle_step(h, p, prev ? h->d_step_flags + (1 - p) : nullptr, main_st, overlap))) return rc;
+        const int32_t *guard = prev ? h->d_step_flags + (1 - p) : nullptr;
+        if ((rc = particle_step(h, p, guard, main_st, overlap))) return rc;
         commit_regroup(h);
+        if (h->post) {
+            if ((rc = step_deposit(h, p, guard))) return rc;
+            prepped = true;
+        }
         if (prev) {
             // the previous step's regroup decision (the host waits for its flags while the GPU works)
             int32_t f = 0;
@@ -1358,9 +1385,17 @@ extern "C" PIC_API int pic_step(pic_t *h, int nsteps) {
                 // layout is the one the previous push left
                 cudaMemsetAsync(h->d_step_flags + (1 - p), 0, sizeof(int32_t), h->st);
                 if ((rc = rebuild_from_step(h))) return rc;
+                if (h->post) {
+                    // nor were that step's moments deposited: this step's field solve again from them
+                    if ((rc = redeposit(h))) return rc;
+                    if ((rc = field_cn_step(h))) return rc;
+                    if ((rc = clear_step_moments(h))) return rc;
+                }
                 if ((rc = step_reset(h, p, true))) return rc;
                 if ((rc = particle_step(h, p, nullptr, main_st, overlap))) return rc;
                 commit_regroup(h);
+                if (h->post)
+                    if ((rc = step_deposit(h, p, nullptr))) return rc;
             }
         }
         h->flags_pending = true;
@@ -1372,7 +1407,7 @@ extern "C" PIC_API int pic_step(pic_t *h, int nsteps) {
         for (int s = 0; s < h->nsp; ++s) h->sp[s].n_exact = false;
         // the next step's work items right behind this regroup, beside the next field solve (only
         // within this call: between calls a load or a rebuild may change the layout)
-        if (k + 1 < nsteps) {
+        if (k + 1 < nsteps && !h->post) {
             timing_begin(h);
             l0 = h->timing.launches[4];
             if ((rc = push_prep(h, false))) return rc;
@@ -1459,7 +1494,7 @@ extern "C" PIC_API int pic_batch_step(pic_batch *p, pic_t **hs, int n, int nstep
     }
     BatchScratch &b = p->b;
     for (int r = 0; r < n; ++r)
-        if (hs[r]->moments_stale)
+        if (hs[r]->moments_stale || hs[r]->post)   // (post: a pending step's moments exist once its regroup succeeded)
             if (int rc = settle(hs[r])) return rc;
     std::vector<char> prev(n);
     struct Reset {
@@ -1528,6 +1563,8 @@ extern "C" PIC_API int pic_batch_step(pic_batch *p, pic_t **hs, int n, int nstep
                 if (int rc = step_reset(h, ph, true)) return rc;
                 if (int rc = particle_step(h, ph, nullptr, h->st, false)) return rc;
                 commit_regroup(h);
+                if (h->post)
+                    if (int rc = step_deposit(h, ph, nullptr)) return rc;
             }
         }
         for (int r = 0; r < n; ++r) {

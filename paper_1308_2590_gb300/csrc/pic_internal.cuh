@@ -150,6 +150,7 @@ struct pic_t {
     unsigned long long *d_bad = nullptr;  // per species: first invalid particle index of a load
     uint32_t *scan_sums = nullptr;      // per-block totals of the multi-block scans
     bool moments_stale = false;         // particles or B changed since the last deposit at rest
+    bool post = false;                  // steps deposit after the regroup (post_deposit)
     cudaEvent_t ev_batch = nullptr;     // a batched step: this run's prologue is queued
     cudaStream_t st2 = nullptr;         // loads: regroups of converted species, beside the next conversion
     cudaEvent_t ev_load = nullptr;      // loads: st2's work joined back to st
@@ -751,6 +752,23 @@ __device__ inline void deposit_s_fix(unsigned long long *Mfix, const FixScale &f
 // o mod 32.  Measured on the 1024 x 512 foil (6.55M particles, per push / per
 // species at rest): FP32 cubic 2.87 -> 0.56 ms / 1.30 -> 0.16 ms; FP64
 // quadratic 5.30 -> 4.10 / 1.89 -> 1.54 ms (FP64 pipe 87 % active).
+// Where a stencil's sums go.  GlobalSink: the moments, columns folded or wrapped.
+template <typename R>
+struct GlobalSink {
+    const GridArgs<R> &g;
+    R *M;
+    __device__ inline void operator()(int i, int j, int k, R v) const {
+        atomicAdd(&M[(int64_t)k * g.nnode + (int64_t)spline_row(g, j) * g.nxn + spline_col(g, i)], v);
+    }
+};
+// TileSink: a block's accumulator of W nodes per row, RN per moment, in shared memory.
+template <typename R>
+struct TileSink {
+    R *acc;
+    int W, RN;
+    __device__ inline void operator()(int i, int j, int k, R v) const { atomicAdd(&acc[k * RN + j * W + i], v); }
+};
+
 template <typename R, int N>
 struct SplineDep {
     static constexpr int NP = N + 1, NN = NP * NP, NS = NN * NMOM;
@@ -795,15 +813,15 @@ struct SplineDep {
         return lane < NN * HG && (N == 2 ? (j < 4 || m0 == 8) : k < NMOM);
     }
 
-    __device__ inline void flush(const GridArgs<R> &g, R *M, int lane) {
+    template <typename Sink>
+    __device__ inline void flush(const Sink &sink, int lane) {
         if (!some) return;
 #pragma unroll
         for (int j = 0; j < J; ++j) {
             int nd, k;
             if (sum_of(j, lane, nd, k) && acc[j] != R(0)) {
                 const int b = nd / NP, a = nd - b * NP;
-                const int64_t n = (int64_t)spline_row(g, ky + b) * g.nxn + spline_col(g, kx + a);
-                atomicAdd(&M[(int64_t)k * g.nnode + n], acc[j]);
+                sink(kx + a, ky + b, k, acc[j]);
             }
             acc[j] = R(0);
         }
@@ -848,12 +866,15 @@ struct SplineDep {
         }
     }
 
-    // All lanes of the warp: particle (s, val) of every lane with alive set.
-    __device__ inline void add(const GridArgs<R> &g, R *M, bool alive, const SplineN<R, N> &s, const R *val, int lane) {
+    // All lanes of the warp: particle (s, val) of every lane with alive set; nx, ny: the grid's (or the
+    // block's tile's) cells, in whose numbering s's first node lies within -2 .. n + 1.
+    template <typename Sink>
+    __device__ inline void add(const Sink &sink, int nx, int ny, bool alive, const SplineN<R, N> &s, const R *val,
+                               int lane) {
         const unsigned full = 0xffffffffu, lt = (1u << lane) - 1u;
         // first node as one number: ny (nx + 4) < 2^32 - 32 for every grid (nx >= 2, nx ny <= 2^30)
-        const int row0 = wrap1(s.iy, g.ny);
-        const unsigned key = alive ? (unsigned)row0 * (unsigned)(g.nx + 4) + (unsigned)(s.ix + 2) : 0xffffffffu - lane;
+        const int row0 = wrap1(s.iy, ny);
+        const unsigned key = alive ? (unsigned)row0 * (unsigned)(nx + 4) + (unsigned)(s.ix + 2) : 0xffffffffu - lane;
         const unsigned same = __match_any_sync(full, key);
         const int size = alive && (same & lt) == 0 ? __popc(same) : 0;   // at a stencil's first lane: its particles
         int incl = size;
@@ -898,7 +919,7 @@ struct SplineDep {
             const int p1 = __shfl_sync(full, incl, l), p0 = p1 - __shfl_sync(full, size, l);
             const int nx0 = __shfl_sync(full, s.ix, l), ny0 = __shfl_sync(full, row0, l);
             if (!some || k != K) {
-                flush(g, M, lane);
+                flush(sink, lane);
                 some = true;
                 K = k;
                 kx = nx0;
@@ -926,6 +947,9 @@ int download_fields(pic_t *h, double *E3, double *H3);
 
 // particles (pic_particles.cu): conversion, deposit at rest, state export
 int deposit_only(pic_t *h, int s);
+bool post_deposit(const pic_t *h);      // the form whose steps deposit after the regroup
+int deposit_step(pic_t *h, const int32_t *guard0, const int32_t *guard1);   // that deposit, over the push's next work items
+int push_item_segs(const pic_t *h);     // segments per work item of the push
 int ensure_items(pic_t *h);             // the work-item table holds an entry per used segment
 int clear_moments(pic_t *h);
 int clear_step_moments(pic_t *h);       // what a step's deposit adds into (the touched node tiles only)

@@ -327,18 +327,21 @@ __device__ inline void load_state(const SpPtr<R> &P, int64_t slot, bool valid, P
 template <typename R>
 constexpr int push_min_blocks() { return 2; }
 
+// kDep = false: the push moves the particles only; their moments are deposited
+// after the regroup, cell by cell (deposit_step).
+
 // kBatch: the launch serves several independent runs.  Their argument
 // blocks are in device memory (runs[r]), run_items[r] is the exclusive prefix
 // of their work-item counts (run_items[nrun] the total), the queue counter is
 // a0.ticket, and each item's fields are loaded into shared memory with plain
 // loads (the runs' TMA descriptors stay on the host side).
-template <typename R, bool kFix, bool kBatch>
-__global__ void __launch_bounds__(TILE_BS, push_min_blocks<R>())
+template <typename R, bool kFix, bool kBatch, bool kDep = true>
+__global__ void __launch_bounds__(TILE_BS, kDep ? push_min_blocks<R>() : 3)
     k_push(const __grid_constant__ TileArgs<R> a0, const TileArgs<R> *__restrict__ runs,
            const int32_t *__restrict__ run_items, int nrun, const __grid_constant__ CUtensorMap tmE,
            const __grid_constant__ CUtensorMap tmBo, const __grid_constant__ CUtensorMap tmBn) {
     extern __shared__ __align__(128) unsigned char smem[];
-    constexpr bool kShared = sizeof(R) == 4;  // FP32: shared accumulator; FP64: L2 reductions
+    constexpr bool kShared = sizeof(R) == 4 && kDep;  // FP32: shared accumulator; FP64: L2 reductions
     constexpr bool kCellG = sizeof(R) == 8;   // FP64: gathers from per-cell coefficient tables
     constexpr bool kCellDep = sizeof(R) == 8 && !kFix && !kBatch;   // FP64 L2 reductions into cell sums
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
@@ -352,7 +355,7 @@ __global__ void __launch_bounds__(TILE_BS, push_min_blocks<R>())
     if (!kBatch && tid == 0) {
         mbar_init(bar, 1);
         fence_mbar_init();
-        if (kChecks)
+        if (kChecks && kDep)
             for (int k = 0; k < 4; ++k) ((volatile uint32_t *)(smem + a0.offCanary))[k] = CANARY + k;
     }
     __syncthreads();
@@ -417,10 +420,10 @@ __global__ void __launch_bounds__(TILE_BS, push_min_blocks<R>())
         const int X0 = tx * a.tnx, Y0 = ty * a.tny;
         const int tw = min(a.tnx, g.nx - X0), th = min(a.tny, g.ny - Y0);   // actual extent (ragged last tiles)
         if (!kBatch && tid == 0) {
-            mbar_arrive_expect_tx(bar, a.tma_bytes);
+            mbar_arrive_expect_tx(bar, kDep ? a.tma_bytes : a.tma_bytes - (uint32_t)(RN * sizeof(V4<R>)));
             tma_load_3d(sE, &tmE, 0, X0 + g.G, Y0 + g.G, bar);
             if (!kCarry<R>) tma_load_3d(sBo, &tmBo, 0, X0 + g.G, Y0 + g.G, bar);   // FP64: b is carried
-            tma_load_3d(sBn, &tmBn, 0, X0 + g.G - H, Y0 + g.G - H, bar);
+            if (kDep) tma_load_3d(sBn, &tmBn, 0, X0 + g.G - H, Y0 + g.G - H, bar);
         }
         if (kBatch) {
             // the padded arrays hold every node a tile box addresses (ghost ring >= tile + halo + 1)
@@ -573,7 +576,8 @@ __global__ void __launch_bounds__(TILE_BS, push_min_blocks<R>())
             R val[NMOM];   // FP32: the 13 moment values; FP64: their parts (the class factors go to the weights)
             R cig, cbx, cby, cbz, cinv;   // carried to the next push (FP64 form)
             R fr, fS, fj;                 // FP64: the class factors of the moments
-            if (inreg) {
+            if (!kDep) {
+            } else if (inreg) {
                 if constexpr (kCellG) {
                     const CellC<R> &cb = sBc[ry * RWc + rx];
                     const R fxy = nfx * nfy;
@@ -584,7 +588,8 @@ __global__ void __launch_bounds__(TILE_BS, push_min_blocks<R>())
                     sm_gather(sBn, a.RW, rx, ry, nfx, nfy, nBx, nBy, nBz);
                 }
             } else if (alive) gather4(a.Bnew, g, ncx, ncy, nfx, nfy, nBx, nBy, nBz);
-            if constexpr (kShared || kCellDep)   // the 13 moment values
+            if constexpr (!kDep) {
+            } else if constexpr (kShared || kCellDep)   // the 13 moment values
                 particle_moments_c(P.q, P.kq, P.hq, w, nux, nuy, nuz, nBx, nBy, nBz, val, cig, cbx, cby, cbz, cinv);
             else   // class factors and parts (the corner-form FP64 deposit)
                 particle_moment_parts(P.q, P.kq, P.cq2, w, nux, nuy, nuz, nBx, nBy, nBz, val, fr, fS, fj, cig, cbx, cby,
@@ -651,9 +656,10 @@ __global__ void __launch_bounds__(TILE_BS, push_min_blocks<R>())
                     }
                     qn += np;
                 }
-            } else if (alive) {
+            } else if constexpr (kDep) {
                 // FP64: every lane adds its own products in L2 (the single-run push: cell sums)
-                if constexpr (kCellDep)
+                if (!alive) {
+                } else if constexpr (kCellDep)
                     deposit_fp64_cell(a.Mc, (int64_t)g.nx * g.ny, (int64_t)ncy * g.nx + ncx, nfx, nfy, val, lane);
                 else
                     deposit_fp64<kFix>(a.M, a.Mfix, a.fs, g, ncx, ncy, nfx, nfy, val, fr, fS, fj, lane);
@@ -734,7 +740,7 @@ __global__ void __launch_bounds__(TILE_BS, push_min_blocks<R>())
             }
             __syncthreads();
         }
-        if (kChecks && !kBatch && tid == 0)
+        if (kChecks && kDep && !kBatch && tid == 0)
             for (int k = 0; k < 4; ++k)
                 if (((volatile uint32_t *)(smem + a0.offCanary))[k] != CANARY + k) atomicOr(a.flags, FLAG_CHECK);
     }
@@ -887,7 +893,7 @@ __global__ void __launch_bounds__(TILE_BS, push_s_min_blocks<R>()) k_push_s(cons
                                        cinv);
                 if constexpr (kFix) deposit_s_fix<R, kParts, N>(a.Mfix, a.fs, g, sn, val, fr, fS, fj, lane);
             }
-            if constexpr (!kFix) dep.add(g, a.M, alive, sn, val, lane);
+            if constexpr (!kFix) dep.add(GlobalSink<R>{g, a.M}, g.nx, g.ny, alive, sn, val, lane);
             // warp compaction of the segment (every lane has loaded before any store)
             const unsigned ms = __ballot_sync(FULL, stay), ml = __ballot_sync(FULL, leave);
             const int32_t ncell = ncy * g.nx + ncx;
@@ -921,7 +927,7 @@ __global__ void __launch_bounds__(TILE_BS, push_s_min_blocks<R>()) k_push_s(cons
             }
         }
     }
-    if constexpr (!kFix) dep.flush(g, a.M, lane);
+    if constexpr (!kFix) dep.flush(GlobalSink<R>{g, a.M}, lane);
 }
 
 // Work items of the push: ch-segment runs of every (species, tile), in
@@ -1416,6 +1422,7 @@ static size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 
 struct Carve {
     int offBo, offBn, offAcc, offBar, offScr, offCanary, offQ, offEc, offBc, bytes;
+    int bytes_post;     // of the push without a deposit (FP32): the E and B tiles of the gather
     uint32_t tma_bytes;
 };
 
@@ -1429,6 +1436,7 @@ static Carve carve(const pic_t *h) {
     c.offBo = (int)o;
     if (h->fp32) o += align_up(EW * EH * v4, 128);   // the FP64 form carries b: no push B tile
     c.offBn = (int)o;
+    c.bytes_post = (int)o;
     o += align_up(RW * RH * v4, 128);
     c.offAcc = (int)o;
     // shared moment accumulator of the FP32 form (fixed point when deterministic)
@@ -1449,11 +1457,11 @@ static Carve carve(const pic_t *h) {
     return c;
 }
 
-template <typename R, bool kFix, bool kBatch = false>
+template <typename R, bool kFix, bool kBatch = false, bool kDep = true>
 static int push_occupancy(pic_t *h, int bytes, int *blocks_per_sm) {
-    cudaError_t e = cudaFuncSetAttribute(k_push<R, kFix, kBatch>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+    cudaError_t e = cudaFuncSetAttribute(k_push<R, kFix, kBatch, kDep>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
     if (e == cudaSuccess)
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, k_push<R, kFix, kBatch>, TILE_BS, bytes);
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, k_push<R, kFix, kBatch, kDep>, TILE_BS, bytes);
     if (e != cudaSuccess) {
         set_error("push kernel set-up: %s", cudaGetErrorString(e));
         return PIC_ERR_CUDA;
@@ -1557,7 +1565,9 @@ int tile_setup(pic_t *h) {
     };
     h->tmaps = new Both{tm, dep};
     int per_sm = 0;
-    if (h->det)
+    if (h->post)
+        rc = push_occupancy<float, false, false, false>(h, c.bytes_post, &per_sm);
+    else if (h->det)
         rc = h->fp32 ? push_occupancy<float, true>(h, c.bytes, &per_sm) : push_occupancy<double, true>(h, c.bytes, &per_sm);
     else
         rc = h->fp32 ? push_occupancy<float, false>(h, c.bytes, &per_sm)
@@ -1683,6 +1693,8 @@ int push_work_list(pic_t *h) {
     count_launch(h);
     return scan_i32_inplace(h, h->chunk_prefix, nitems + 1);
 }
+
+int push_item_segs(const pic_t *h) { return item_segs(h); }
 
 // The touch and regroup lists and the regroup queues, emptied for the next
 // push (after whatever read the previous push's lists: the clear of its tiles).
@@ -1982,6 +1994,13 @@ static int particle_tiles_t(pic_t *h, bool prepared) {
         }
         count_launch(h);
         return check_launch("k_push_s");
+    }
+    if constexpr (sizeof(R) == 4) {
+        if (h->post) {
+            k_push<R, false, false, false><<<h->push_blocks, TILE_BS, c.bytes_post, h->st>>>(a, nullptr, nullptr, 0, mE, mBo, mBn);
+            count_launch(h);
+            return check_launch("k_push");
+        }
     }
     if (h->det) k_push<R, true, false><<<h->push_blocks, TILE_BS, c.bytes, h->st>>>(a, nullptr, nullptr, 0, mE, mBo, mBn);
     else k_push<R, false, false><<<h->push_blocks, TILE_BS, c.bytes, h->st>>>(a, nullptr, nullptr, 0, mE, mBo, mBn);
