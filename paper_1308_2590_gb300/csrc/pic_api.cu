@@ -179,11 +179,11 @@ static void free_particle_buffers(SpeciesBuf &S) {
         S.cell[b] = nullptr; S.ox[b] = S.oy[b] = S.ux[b] = S.uy[b] = S.uz[b] = S.w[b] = nullptr;
         S.carry[b] = nullptr;
     }
-    cudaFree(S.mkey);
+    cudaFree(S.segd);
     cudaFree(S.segn[0]);
     cudaFree(S.segn[1]);
     cudaFree(S.segml);
-    S.mkey = nullptr;
+    S.segd = nullptr;
     S.segn[0] = S.segn[1] = S.segml = nullptr;
     S.cap = 0;
 }
@@ -218,7 +218,7 @@ static int ensure_species_capacity(pic_t *h, int s, int64_t slots) {
         if (!rc) rc = dalloc(&N.w[b], rb, "particles");
         if (!rc && !h->fp32) rc = dalloc((void **)&N.carry[b], (size_t)NCARRY * cap * sizeof(double), "particles");
     }
-    if (!rc) rc = dalloc((void **)&N.mkey, cap * sizeof(uint32_t), "mirror keys");
+    if (!rc) rc = dalloc((void **)&N.segd, (cap / SEG) * sizeof(unsigned long long), "segment counts");
     if (!rc) rc = dalloc((void **)&N.segn[0], (cap / SEG) * sizeof(int32_t), "segment counts");
     if (!rc) rc = dalloc((void **)&N.segn[1], (cap / SEG) * sizeof(int32_t), "segment counts");
     if (!rc) rc = dalloc((void **)&N.segml, (cap / SEG) * sizeof(int32_t), "segment counts");
@@ -246,7 +246,7 @@ static int ensure_species_capacity(pic_t *h, int s, int64_t slots) {
         S.ux[b] = N.ux[b]; S.uy[b] = N.uy[b]; S.uz[b] = N.uz[b]; S.w[b] = N.w[b];
         S.carry[b] = N.carry[b];
     }
-    S.mkey = N.mkey;
+    S.segd = N.segd;
     S.segn[0] = N.segn[0];
     S.segn[1] = N.segn[1];
     S.segml = N.segml;
@@ -516,7 +516,7 @@ static uint64_t estimate_bytes(const pic_t *h, const int64_t *n) {
         const int64_t ns = n ? n[s] : 0;
         if (ns <= 0) continue;
         const int64_t cap = slots_needed(h, ns);
-        b += 3ull * cap * (4 + 6 * h->rs + (h->fp32 ? 0 : NCARRY * 8)) + (uint64_t)cap * 4 + 3ull * (cap / SEG) * 4;
+        b += 3ull * cap * (4 + 6 * h->rs + (h->fp32 ? 0 : NCARRY * 8)) + 5ull * (cap / SEG) * 4;
         if (cap > maxcap) maxcap = cap;
         if (7 * ns > stage) stage = 7 * ns;
     }

@@ -67,7 +67,7 @@ struct SpeciesBuf {
     void *ux[3] = {nullptr, nullptr, nullptr}, *uy[3] = {nullptr, nullptr, nullptr};
     void *uz[3] = {nullptr, nullptr, nullptr}, *w[3] = {nullptr, nullptr, nullptr};
     double *carry[3] = {nullptr, nullptr, nullptr};   // FP64 form: [NCARRY][cap] carried quantities per set
-    uint32_t *mkey = nullptr;   // [cap] destination tile of each mirror entry
+    unsigned long long *segd = nullptr;   // [cap/SEG] leavers per mirror segment and neighbour (8 bits each)
     int32_t *segn[2] = {nullptr, nullptr};  // [cap/SEG] valid particles per bin segment
     int32_t *useg[2] = {nullptr, nullptr};  // [ntiles] segments in use per bin
     int scur = 0;               // segn[scur], useg[scur] describe the bins; the regroup writes the other pair

@@ -420,6 +420,55 @@ constexpr int LOAD_BS = 256;
 constexpr int LOAD_SM_PERMILLE = 500;   // conversion blocks per 1000 SMs (measured: 76 x 256 on GB300
                                         // reads the link at full rate beside a regroup at nearly full speed)
 
+// x / d from the correctly rounded reciprocal rd of d: with q = x rd and the
+// remainder r = x - q d (one FMA), q + r rd is the correctly rounded quotient
+// (P. Markstein, "Computation of elementary functions on the IBM RISC
+// System/6000 processor", 1990) but for quotients within a few 2^-53 of an ulp
+// of a rounding boundary or in the denormal range.  Three operations of the FP64
+// pipe, which bounds the conversion, instead of a division's dozen.
+__device__ inline double div_by(double x, double d, double rd) {
+    const double q = x * rd;
+    return fma(fma(-q, d, x), rd, q);
+}
+
+// The FP32 value nearest to v (ties to even) from its bits: a conversion
+// instruction issues on the FP64 pipe.
+__device__ inline float narrow(double v) {
+    const unsigned long long u = (unsigned long long)__double_as_longlong(v), m = u & 0x7fffffffffffffffull;
+    const unsigned e = (unsigned)(m >> 52);
+    if (e < 897 || e > 1150) return (float)v;   // zero, FP32 denormals, overflow
+    const unsigned long long t = m - (896ull << 52) + 0x0fffffffull + ((m >> 29) & 1);
+    return __uint_as_float((unsigned)(t >> 29) | ((unsigned)(u >> 32) & 0x80000000u));
+}
+template <typename R>
+__device__ inline R stored(double v) {
+    if constexpr (sizeof(R) == 4) return narrow(v);
+    else return v;
+}
+
+// floor(x) of 0 <= x < 2^31 as a double and an integer, from the bits.
+__device__ inline double floor_cell(double x, int &c) {
+    const long long b = __double_as_longlong(x);
+    const int e = (int)(b >> 52) - 1023;
+    if (e < 0) {
+        c = 0;
+        return 0.0;
+    }
+    const int sh = 52 - e;
+    c = (int)(((b & 0xFFFFFFFFFFFFFll) | 0x10000000000000ll) >> sh);
+    return __longlong_as_double((b >> sh) << sh);
+}
+
+// 0 <= x < L of a position: false for NaN, infinities and negative values but
+// -0, by integer compares (FP64 compares issue on the FP64 pipe).
+__device__ inline bool in_box(double x, double L) {
+    const long long b = __double_as_longlong(x);
+    return (b >= 0 && b < __double_as_longlong(L)) || b == (long long)0x8000000000000000ull;
+}
+__device__ inline bool finite_bits(double x) {
+    return (__double_as_longlong(x) & 0x7FF0000000000000ll) != 0x7FF0000000000000ll;
+}
+
 template <typename R>
 __global__ void __launch_bounds__(LOAD_BS) k_load_convert(GridArgs<double> g, double Lx, double Ly, LoadSrc src, int64_t n,
                                int32_t *cell, R *ox, R *oy, R *ux, R *uy, R *uz, R *w,
@@ -432,25 +481,23 @@ __global__ void __launch_bounds__(LOAD_BS) k_load_convert(GridArgs<double> g, do
     for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < n; t += (int64_t)gridDim.x * blockDim.x) {
         const double x = src.a[0][t], y = src.a[1][t];
         const double vx = src.a[2][t], vy = src.a[3][t], vz = src.a[4][t], vw = src.a[5][t];
-        if (!(x >= 0.0 && x < Lx && y >= 0.0 && y < Ly) || !isfinite(vx) || !isfinite(vy) || !isfinite(vz) ||
-            !isfinite(vw)) {
+        if (!in_box(x, Lx) || !in_box(y, Ly) || !finite_bits(vx) || !finite_bits(vy) || !finite_bits(vz) ||
+            !finite_bits(vw)) {
             atomicMin(bad, (unsigned long long)t);
             // an in-range placeholder, so that a regroup queued before the check stays in bounds
             cell[t] = 0;
             ox[t] = oy[t] = ux[t] = uy[t] = uz[t] = w[t] = R(0);
             continue;
         }
-        double sxx = x / g.dx, syy = y / g.dy;
-        double flx = floor(sxx), fly = floor(syy);
-        int cx = (int)flx, cy = (int)fly;
+        const double sxx = div_by(x, g.dx, g.inv_dx), syy = div_by(y, g.dy, g.inv_dy);
+        int cx, cy;
+        const double flx = floor_cell(sxx, cx), fly = floor_cell(syy, cy);
         double fx = sxx - flx, fy = syy - fly;
         // x < Lx whose x/dx rounds to nx (walls): the last cell, at the largest offset below 1 of the
         // form's precision, so that every stored offset lies in [0, 1)
         if (cx >= g.nx) { if (g.periodic_x) cx -= g.nx; else { cx = g.nx - 1; fx = 0x1.fffffffffffffp-1; } }
-        if (cx < 0) { if (g.periodic_x) cx += g.nx; else { cx = 0; fx = 0.0; } }
         if (cy >= g.ny) cy -= g.ny;
-        if (cy < 0) cy += g.ny;
-        R rfx = (R)fx, rfy = (R)fy;
+        R rfx = stored<R>(fx), rfy = stored<R>(fy);
         if (sizeof(R) == 4) {
             if (rfx >= R(1)) {
                 if (g.periodic_x || cx + 1 < g.nx) { rfx = R(0); cx = (cx + 1 == g.nx) ? 0 : cx + 1; }
@@ -461,10 +508,10 @@ __global__ void __launch_bounds__(LOAD_BS) k_load_convert(GridArgs<double> g, do
         cell[t] = cy * g.nx + cx;
         ox[t] = rfx;
         oy[t] = rfy;
-        ux[t] = (R)vx;
-        uy[t] = (R)vy;
-        uz[t] = (R)vz;
-        w[t] = (R)vw;
+        ux[t] = stored<R>(vx);
+        uy[t] = stored<R>(vy);
+        uz[t] = stored<R>(vz);
+        w[t] = stored<R>(vw);
     }
 }
 

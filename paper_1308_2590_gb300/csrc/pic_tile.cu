@@ -99,7 +99,7 @@ struct SpPtr {
     int32_t *cell, *mcell;
     R *ox, *oy, *ux, *uy, *uz, *w;
     R *mox, *moy, *mux, *muy, *muz, *mw;
-    uint32_t *mkey;
+    unsigned long long *segd;
     const int32_t *bstart;
     int32_t *useg, *segn, *segml;   // current counts (push reads/writes, the regroup reads)
     int32_t *useg2, *segn2;         // next counts (the regroup writes)
@@ -319,6 +319,28 @@ __device__ inline void load_state(const SpPtr<R> &P, int64_t slot, bool valid, P
         s.fx = s.fy = s.ux = s.uy = s.uz = s.w = R(0);
         s.ig = s.bx = s.by = s.bz = s.inv = R(0);
     }
+}
+
+// Places of a segment's leavers in its mirror segment (a warp): grouped by the
+// neighbour tile they are bound for (in the order of the source tile's
+// neighbour table nb; a farther tile last), in lane order inside a group, so
+// that a tile's regroup finds its arrivals of a segment as one run without
+// looking at the others.  Returns the counts per neighbour, 8 bits each.
+__device__ inline unsigned long long mirror_places(const int32_t *__restrict__ nb, int tn, bool leave, unsigned lt, int &pos) {
+    const int n = nb[0];
+    int b = leave ? 8 : 9;
+    for (int q = 0; q < n; ++q)
+        if (leave && nb[1 + q] == tn) b = q;
+    unsigned long long counts = 0;
+    int off = 0;
+#pragma unroll
+    for (int q = 0; q <= 8; ++q) {
+        const unsigned m = __ballot_sync(FULL, b == q);
+        if (b == q) pos = off + __popc(m & lt);
+        off += __popc(m);
+        if (q < 8) counts |= (unsigned long long)__popc(m) << (8 * q);
+    }
+    return counts;
 }
 
 // Resident blocks per SM the push is compiled for (128 registers a thread):
@@ -667,6 +689,8 @@ __global__ void __launch_bounds__(TILE_BS, kDep ? push_min_blocks<R>() : 3)
             // warp compaction of the segment (every lane has loaded before any store)
             const unsigned ms = __ballot_sync(FULL, stay), ml = __ballot_sync(FULL, leave);
             const int32_t ncell = ncy * g.nx + ncx;
+            int mpos = 0;   // place among the segment's leavers
+            const unsigned long long md = ml ? mirror_places(a.nbr + t * 9, tn, leave, lt, mpos) : 0ull;
             if (stay) {
                 const int64_t d = slot0 + __popc(ms & lt);
                 P.cell[d] = ncell;
@@ -678,7 +702,7 @@ __global__ void __launch_bounds__(TILE_BS, kDep ? push_min_blocks<R>() : 3)
                 P.w[d] = w;
                 if constexpr (kCarry<R>) store_carry(P.cr, P.ccap, d, cig, cbx, cby, cbz, cinv);
             } else if (leave) {
-                const int64_t d = slot0 + __popc(ml & lt);
+                const int64_t d = slot0 + mpos;
                 P.mcell[d] = ncell;
                 P.mox[d] = nfx;
                 P.moy[d] = nfy;
@@ -686,7 +710,6 @@ __global__ void __launch_bounds__(TILE_BS, kDep ? push_min_blocks<R>() : 3)
                 P.muy[d] = nuy;
                 P.muz[d] = nuz;
                 P.mw[d] = w;
-                P.mkey[d] = (uint32_t)tn;
                 if constexpr (kCarry<R>) store_carry(P.mcr, P.ccap, d, cig, cbx, cby, cbz, cinv);
             } else if (valid && dead) {
                 atomicAdd(P.removed, 1ull);
@@ -694,6 +717,7 @@ __global__ void __launch_bounds__(TILE_BS, kDep ? push_min_blocks<R>() : 3)
             if (lane == 0) {
                 P.segn[sbase + sg] = __popc(ms);
                 P.segml[sbase + sg] = __popc(ml);
+                P.segd[sbase + sg] = md;
             }
         }
         if constexpr (kShared) {
@@ -897,6 +921,8 @@ __global__ void __launch_bounds__(TILE_BS, push_s_min_blocks<R>()) k_push_s(cons
             // warp compaction of the segment (every lane has loaded before any store)
             const unsigned ms = __ballot_sync(FULL, stay), ml = __ballot_sync(FULL, leave);
             const int32_t ncell = ncy * g.nx + ncx;
+            int mpos = 0;   // place among the segment's leavers
+            const unsigned long long md = ml ? mirror_places(a.nbr + t * 9, tn, leave, lt, mpos) : 0ull;
             if (stay) {
                 const int64_t d = slot0 + __popc(ms & lt);
                 P.cell[d] = ncell;
@@ -908,7 +934,7 @@ __global__ void __launch_bounds__(TILE_BS, push_s_min_blocks<R>()) k_push_s(cons
                 P.w[d] = w;
                 if constexpr (kCarry<R>) store_carry(P.cr, P.ccap, d, cig, cbx, cby, cbz, cinv);
             } else if (leave) {
-                const int64_t d = slot0 + __popc(ml & lt);
+                const int64_t d = slot0 + mpos;
                 P.mcell[d] = ncell;
                 P.mox[d] = nfx;
                 P.moy[d] = nfy;
@@ -916,7 +942,6 @@ __global__ void __launch_bounds__(TILE_BS, push_s_min_blocks<R>()) k_push_s(cons
                 P.muy[d] = nuy;
                 P.muz[d] = nuz;
                 P.mw[d] = w;
-                P.mkey[d] = (uint32_t)tn;
                 if constexpr (kCarry<R>) store_carry(P.mcr, P.ccap, d, cig, cbx, cby, cbz, cinv);
             } else if (valid && dead) {
                 atomicAdd(P.removed, 1ull);
@@ -924,6 +949,7 @@ __global__ void __launch_bounds__(TILE_BS, push_s_min_blocks<R>()) k_push_s(cons
             if (lane == 0) {
                 P.segn[sbase + sg] = __popc(ms);
                 P.segml[sbase + sg] = __popc(ml);
+                P.segd[sbase + sg] = md;
             }
         }
     }
@@ -1064,11 +1090,15 @@ __device__ inline int block_excl_scan_int(int v, int *wsum, int *total) {
 // order).  A stable counting sort of that sequence by cell inside the tile
 // (row-major) writes the tile densely into the spare buffer set, and the
 // tile's new counts to segn2 / useg2.  Ranges of the sort: the warps' stayer
-// segment ranges, then the arrivals (sorted by the last warp).  If the bin
-// cannot hold the result, or the arrivals overflow their list, the step flag
+// segment ranges, then the arrivals -- as one range that the last warp sorts,
+// or, from ARR_SPLIT on, as one per warp (a hot plasma: a tenth of a tile
+// arrives every step, and one warp's copies kept the others waiting).  If the
+// bin cannot hold the result, or the arrivals overflow their list, the step flag
 // asks for the full regroup, which rebuilds from the bins and the mirror.
-constexpr int REGROUP_RANGES = TILE_WARPS + 1;
+// Bound by the latency of its dependent loads.
+constexpr int REGROUP_RANGES = 2 * TILE_WARPS;
 constexpr int ARR_MAX = 8192;
+constexpr int ARR_SPLIT = 128;
 
 __host__ __device__ inline int regroup_smem_bytes(int tile_cells) {
     return (REGROUP_RANGES * tile_cells + ARR_MAX) * (int)sizeof(int);
@@ -1131,7 +1161,13 @@ __device__ __forceinline__ void regroup_one(const TileArgs<R> &a, int t, int s, 
         return;
     }
     for (int i = tid; i < REGROUP_RANGES * nc; i += TILE_BS) hist[i] = 0;
-    // 1. the arrivals: warp q scans neighbour q's mirror (neighbours ascending), counts, then lists
+    // 1. the arrivals: warp q takes neighbour q's mirror (neighbours ascending), counts, then lists: of
+    // each segment the run bound for this tile (mirror_places)
+    int qi = 0;   // this tile's place in neighbour wid's table
+    if (wid < nnb) {
+        const int32_t *nb = a.nbr + s_nb[wid] * 9;
+        while (qi < 7 && nb[1 + qi] != t) ++qi;
+    }
     auto scan_mirror = [&](bool write, int pos) {
         const int src = s_nb[wid];
         const int64_t sb = P.bstart[src] / SEG, so = P.bstart[src];
@@ -1139,22 +1175,19 @@ __device__ __forceinline__ void regroup_one(const TileArgs<R> &a, int t, int s, 
         int tot = 0;
         for (int j0 = 0; j0 < us; j0 += SEG) {
             const int j = j0 + lane;
-            const int ml = (j < us) ? P.segml[sb + j] : 0;
-            int c = 0;
-            for (int r = 0; r < ml; ++r) c += (P.mkey[so + (int64_t)j * SEG + r] == (uint32_t)t);
+            const unsigned long long d = (j < us) ? P.segd[sb + j] : 0ull;
+            const int c = (int)(d >> (8 * qi)) & 255;
             int incl = c;
             for (int o = 1; o < 32; o <<= 1) {
                 const int y = __shfl_up_sync(FULL, incl, o);
                 if (lane >= o) incl += y;
             }
             if (write && c) {
-                int k = pos + tot + incl - c;
-                for (int r = 0; r < ml; ++r) {
-                    const int64_t si = so + (int64_t)j * SEG + r;
-                    if (P.mkey[si] != (uint32_t)t) continue;
-                    if (k < ARR_MAX) arr[k] = (int)si;
-                    ++k;
-                }
+                // the run starts after the lower neighbours' (a sum of bytes)
+                const int off = (int)(((d & ((1ull << (8 * qi)) - 1)) * 0x0101010101010101ull) >> 56);
+                const int k = pos + tot + incl - c;
+                const int si = (int)(so + (int64_t)j * SEG) + off;
+                for (int r = 0; r < c && k + r < ARR_MAX; ++r) arr[k + r] = si + r;
             }
             tot += __shfl_sync(FULL, incl, 31);
         }
@@ -1180,6 +1213,10 @@ __device__ __forceinline__ void regroup_one(const TileArgs<R> &a, int t, int s, 
         return;
     }
     if (wid < nnb && s_cnt[wid] > 0) scan_mirror(true, s_base[wid]);
+    // the arrivals' ranges: arrival i is in range TILE_WARPS + i / pera
+    const int nra = narr >= ARR_SPLIT ? TILE_WARPS : 1;
+    const int pera = nra == 1 ? max(narr, 1) : ((narr + SEG * TILE_WARPS - 1) / (SEG * TILE_WARPS)) * SEG;
+    const int nrange = TILE_WARPS + nra;
     // 2. counts per (range, cell); a warp's next segment is loaded while it works on this one
     const int per = (ut + TILE_WARPS - 1) / TILE_WARPS;
     const int j0w = min(wid * per, ut), j1w = min(j0w + per, ut);
@@ -1210,7 +1247,7 @@ __device__ __forceinline__ void regroup_one(const TileArgs<R> &a, int t, int s, 
     __syncthreads();   // the arrival list and the stayer counts are complete
     for (int i = tid; i < narr; i += TILE_BS) {
         const int loc = local_of(P.mcell[arr[i]]);
-        if (loc >= 0) atomicAdd(&hist[TILE_WARPS * nc + loc], 1);
+        if (loc >= 0) atomicAdd(&hist[(TILE_WARPS + i / pera) * nc + loc], 1);
         else atomicOr(a.flags, 16);
     }
     __syncthreads();
@@ -1220,11 +1257,11 @@ __device__ __forceinline__ void regroup_one(const TileArgs<R> &a, int t, int s, 
         const int c = c0 + tid;
         int col = 0;
         if (c < nc)
-            for (int r = 0; r < REGROUP_RANGES; ++r) col += hist[r * nc + c];
+            for (int r = 0; r < nrange; ++r) col += hist[r * nc + c];
         int blk = 0;
         int run = carry + block_excl_scan_int(col, wsum, &blk);
         if (c < nc)
-            for (int r = 0; r < REGROUP_RANGES; ++r) {
+            for (int r = 0; r < nrange; ++r) {
                 const int hcount = hist[r * nc + c];
                 hist[r * nc + c] = run;
                 run += hcount;
@@ -1274,26 +1311,30 @@ __device__ __forceinline__ void regroup_one(const TileArgs<R> &a, int t, int s, 
             __syncwarp();
         }
     }
-    if (wid == TILE_WARPS - 1)
-        for (int i0 = 0; i0 < narr; i0 += SEG) {
+    {
+        const int q = nra == 1 ? 0 : wid;   // this warp's range of the arrivals
+        const int i1 = nra > 1 ? min((q + 1) * pera, narr) : (wid == TILE_WARPS - 1 ? narr : 0);
+        int *ha = hist + (TILE_WARPS + q) * nc;
+        for (int i0 = q * pera; i0 < i1; i0 += SEG) {
             const int i = i0 + lane;
             PState<R> v;
             int loc = -1;
-            if (i < narr) {
+            if (i < i1) {
                 load_particle(P, true, arr[i], v);
                 loc = local_of(v.c);
             }
             const unsigned m = __match_any_sync(FULL, loc >= 0 ? loc : -1 - lane);
-            const int base = (loc >= 0) ? hist[TILE_WARPS * nc + loc] : 0;
+            const int base = (loc >= 0) ? ha[loc] : 0;
             __syncwarp();
             if (loc >= 0) {
-                if (lane == __ffs(m) - 1) hist[TILE_WARPS * nc + loc] = base + __popc(m);
+                if (lane == __ffs(m) - 1) ha[loc] = base + __popc(m);
                 const int64_t dst = to + base + __popc(m & lt);
                 if (kChecks && (dst < to || dst >= P.bstart[t + 1])) atomicOr(a.flags, FLAG_CHECK);
                 else store_particle(P, dst, v);
             }
             __syncwarp();
         }
+    }
     // 5. dense counts of the new bin
     for (int j = tid; j < need; j += TILE_BS) P.segn2[tb + j] = min(SEG, total - j * SEG);
     if (tid == 0) P.useg2[t] = need;
@@ -1645,7 +1686,7 @@ static TileArgs<R> tile_args(pic_t *h) {
         p.ux = (R *)S.ux[b]; p.uy = (R *)S.uy[b]; p.uz = (R *)S.uz[b]; p.w = (R *)S.w[b];
         p.mcell = S.cell[m]; p.mox = (R *)S.ox[m]; p.moy = (R *)S.oy[m];
         p.mux = (R *)S.ux[m]; p.muy = (R *)S.uy[m]; p.muz = (R *)S.uz[m]; p.mw = (R *)S.w[m];
-        p.mkey = S.mkey;
+        p.segd = S.segd;
         p.bstart = S.bstart;
         p.useg = S.useg[S.scur]; p.segn = S.segn[S.scur];
         p.useg2 = S.useg[1 - S.scur]; p.segn2 = S.segn[1 - S.scur];
