@@ -162,6 +162,7 @@ struct pic_t {
     cudaEvent_t ev_field = nullptr;     // steps: the field solve is done (st2 -> st)
     cudaEvent_t ev_cellm = nullptr;     // steps: the push's cell sums are in the node moments (st2 -> st)
     int push_blocks = 0;                // persistent grid size of the push
+    int items_ch = 0;                   // segments per work item of the current item table
 
     // sort scratch
     uint32_t *keys[2] = {nullptr, nullptr};   // sort scratch, 2*cap entries

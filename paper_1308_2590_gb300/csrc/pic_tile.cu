@@ -151,9 +151,19 @@ struct TileArgs {
 constexpr int CH_SEGS_FP32 = 256;
 constexpr int CH_SEGS_FP64 = 48;
 constexpr int CH_SEGS_SPLINE = 32;
+// A small FP64 run takes shorter items still, so that every block gets two or
+// so, down to 16 segments (64 x 64 plasma, 131,072 particles in 16 x 16 tiles:
+// 96 items of 48 segments for 304 blocks kept most of the GPU's FP64 pipes idle,
+// 148 us per push; 256 items of 16: 66 us.  An item's coefficient tables cost
+// about as much as 5 segments there).
+constexpr int CH_SEGS_MIN = 16;
 inline int item_segs(const pic_t *h) {
     if (h->fp32 && h->shape != 2) return CH_SEGS_FP32;
-    return h->shape == 1 ? CH_SEGS_FP64 : CH_SEGS_SPLINE;
+    if (h->shape != 1) return CH_SEGS_SPLINE;
+    int64_t segs = 0;
+    for (int s = 0; s < h->nsp; ++s) segs += (h->sp[s].n + SEG - 1) / SEG;   // (as last counted)
+    const int64_t ch = (segs / (2 * (h->push_blocks > 0 ? h->push_blocks : 1)) + 7) / 8 * 8;
+    return ch < CH_SEGS_MIN ? CH_SEGS_MIN : ch > CH_SEGS_FP64 ? CH_SEGS_FP64 : (int)ch;
 }
 
 // Shared memory of the push: a fixed header (mbarrier, then the block's
@@ -1100,8 +1110,58 @@ constexpr int REGROUP_RANGES = 2 * TILE_WARPS;
 constexpr int ARR_MAX = 8192;
 constexpr int ARR_SPLIT = 128;
 
-__host__ __device__ inline int regroup_smem_bytes(int tile_cells) {
-    return (REGROUP_RANGES * tile_cells + ARR_MAX) * (int)sizeof(int);
+// Staged copy of a tile whose segments scatter over many cells (more than
+// STAGE_GROUPS of them per segment on average): stored particle by particle,
+// such a segment writes some twenty partial sectors per array.  The tile's
+// destinations are kept (16 bits each) and the arrays go one after another
+// through a buffer in shared memory, from which they are written in order.
+// Where it can pay: steps in which particles may cross several cells (the
+// deposit halo is wider than a cell); elsewhere the buffer would only cost
+// resident blocks.  FP32: 67M particles at c dt / dx = 25, 2.38 -> 1.63 ms.  The
+// FP64 form (twelve arrays, fewer blocks) was slower staged: 41 -> 100 us on the
+// 64 x 64 plasma.
+constexpr int STAGE_GROUPS = 5;
+constexpr int STAGE_BYTES = 36 * 1024;      // a tile's values of one array
+constexpr int STAGE_DST = 10 * 1024;        // source places (segment slots, then arrivals)
+constexpr int STAGE_ARR = 2048;             // arrivals of a staged tile
+inline bool regroup_stages(const pic_t *h) {
+    return h->fp32 && h->halo > 1 && REGROUP_RANGES * h->tnx * h->tny * (int)sizeof(int) <= STAGE_BYTES;
+}
+
+inline int regroup_smem_bytes(const pic_t *h) {
+    const int plain = (REGROUP_RANGES * h->tnx * h->tny + ARR_MAX) * (int)sizeof(int);
+    const int staged = STAGE_BYTES + STAGE_ARR * (int)sizeof(int) + STAGE_DST * (int)sizeof(uint16_t);
+    return regroup_stages(h) && staged > plain ? staged : plain;
+}
+
+// One array of a staged tile: every source place's value to its destination in
+// the buffer (hist's place: the ranks have been taken), then out in order.
+template <typename T>
+__device__ inline void stage_array(const T *__restrict__ bins, const T *__restrict__ mirror, T *__restrict__ out,
+                                   const uint16_t *sdst, const int *arr, T *buf, int nslot, int narr, int total) {
+    const int tid = threadIdx.x;
+    constexpr int D = 16;   // loads in flight per thread
+    for (int e0 = tid; e0 < nslot; e0 += D * TILE_BS) {
+        T v[D];
+#pragma unroll
+        for (int u = 0; u < D; ++u) {
+            const int e = e0 + u * TILE_BS;
+            v[u] = bins[min(e, nslot - 1)];   // (an unused slot's value goes nowhere)
+        }
+#pragma unroll
+        for (int u = 0; u < D; ++u) {
+            const int e = e0 + u * TILE_BS;
+            const int d = e < nslot ? sdst[e] : 0xFFFF;
+            if (d != 0xFFFF) buf[d] = v[u];
+        }
+    }
+    for (int i = tid; i < narr; i += TILE_BS) {
+        const int d = sdst[nslot + i];
+        if (d != 0xFFFF) buf[d] = mirror[arr[i]];
+    }
+    __syncthreads();
+    for (int i = tid; i < total; i += TILE_BS) out[i] = buf[i];
+    __syncthreads();
 }
 
 template <typename R>
@@ -1126,10 +1186,10 @@ __device__ inline void store_particle(const SpPtr<R> &P, int64_t d, const PState
 // kBatch: blocks of several runs; run_tiles[r] is the exclusive prefix of the
 // runs' tile counts (blockIdx.x indexes the concatenation), runs[r] their
 // argument blocks.
-template <typename R, bool kBatch>
+template <typename R, bool kBatch, bool kStage>
 __device__ __forceinline__ void regroup_one(const TileArgs<R> &a, int t, int s, int *rsm) {
     __shared__ int s_nb[8], s_cnt[TILE_WARPS], s_base[TILE_WARPS + 1];
-    __shared__ int wsum[33];
+    __shared__ int wsum[33], s_groups;
     if (s >= a.nsp) return;
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
     const SpPtr<R> &P = a.sp[s];
@@ -1140,6 +1200,7 @@ __device__ __forceinline__ void regroup_one(const TileArgs<R> &a, int t, int s, 
     const int nc = tw * th;
     int *hist = rsm;                          // [REGROUP_RANGES][nc]
     int *arr = rsm + REGROUP_RANGES * nc;     // mirror slots of the arrivals, in sequence order
+    if (tid == 0) s_groups = 0;
     const int64_t tb = P.bstart[t] / SEG, to = P.bstart[t];
     const int ut = P.useg[t];
     const unsigned lt = (1u << lane) - 1u;
@@ -1173,9 +1234,11 @@ __device__ __forceinline__ void regroup_one(const TileArgs<R> &a, int t, int s, 
         const int64_t sb = P.bstart[src] / SEG, so = P.bstart[src];
         const int us = P.useg[src];
         int tot = 0;
+        unsigned long long dn = lane < us ? P.segd[sb + lane] : 0ull;
         for (int j0 = 0; j0 < us; j0 += SEG) {
             const int j = j0 + lane;
-            const unsigned long long d = (j < us) ? P.segd[sb + j] : 0ull;
+            const unsigned long long d = dn;
+            dn = (j + SEG < us) ? P.segd[sb + j + SEG] : 0ull;   // the next words in flight meanwhile
             const int c = (int)(d >> (8 * qi)) & 255;
             int incl = c;
             for (int o = 1; o < 32; o <<= 1) {
@@ -1217,12 +1280,18 @@ __device__ __forceinline__ void regroup_one(const TileArgs<R> &a, int t, int s, 
     const int nra = narr >= ARR_SPLIT ? TILE_WARPS : 1;
     const int pera = nra == 1 ? max(narr, 1) : ((narr + SEG * TILE_WARPS - 1) / (SEG * TILE_WARPS)) * SEG;
     const int nrange = TILE_WARPS + nra;
+    // staged copy (kStage): [arrivals | hist, then the buffer | destinations]
+    int *sarr = rsm + STAGE_BYTES / (int)sizeof(int);
+    uint16_t *sdst = (uint16_t *)(sarr + STAGE_ARR);
+    const int nslot = ut * SEG;
+    const bool fits = kStage && narr <= STAGE_ARR && nslot + narr <= STAGE_DST;
     // 2. counts per (range, cell); a warp's next segment is loaded while it works on this one
     const int per = (ut + TILE_WARPS - 1) / TILE_WARPS;
     const int j0w = min(wid * per, ut), j1w = min(j0w + per, ut);
     {
         // four segments' counts and cells are loaded before any is used
-        constexpr int D = 4;
+        constexpr int D = kStage ? 8 : 4;
+        int groups = 0;   // cells per segment, added up
         for (int j0 = j0w; j0 < j1w; j0 += D) {
             int n[D];
             int32_t c[D];
@@ -1240,9 +1309,13 @@ __device__ __forceinline__ void regroup_one(const TileArgs<R> &a, int t, int s, 
                     if (loc < 0) atomicOr(a.flags, 16);
                 }
                 const unsigned m = __match_any_sync(FULL, loc >= 0 ? loc : -1 - lane);
-                if (loc >= 0 && lane == __ffs(m) - 1) atomicAdd(&hist[wid * nc + loc], __popc(m));
+                if (fits && j0 + u < j1w) sdst[(j0 + u) * SEG + lane] = (uint16_t)loc;   // for the ranks (-1: 0xFFFF)
+                const bool first = loc >= 0 && lane == __ffs(m) - 1;
+                if (first) atomicAdd(&hist[wid * nc + loc], __popc(m));
+                if (kStage) groups += __popc(__ballot_sync(FULL, first));
             }
         }
+        if (kStage && lane == 0 && groups) atomicAdd(&s_groups, groups);
     }
     __syncthreads();   // the arrival list and the stayer counts are complete
     for (int i = tid; i < narr; i += TILE_BS) {
@@ -1277,6 +1350,50 @@ __device__ __forceinline__ void regroup_one(const TileArgs<R> &a, int t, int s, 
     }
     __syncthreads();
     // 4. stable ranks inside each range, then the copy into the spare set
+    if (fits && s_groups > STAGE_GROUPS * ut && total * (int)sizeof(R) <= STAGE_BYTES) {
+        // the arrivals move from beside hist to behind the buffer's place
+        int keep[STAGE_ARR / TILE_BS];
+#pragma unroll
+        for (int u = 0; u < STAGE_ARR / TILE_BS; ++u) {
+            const int i = tid + u * TILE_BS;
+            keep[u] = i < narr ? arr[i] : 0;
+        }
+        __syncthreads();
+#pragma unroll
+        for (int u = 0; u < STAGE_ARR / TILE_BS; ++u) {
+            const int i = tid + u * TILE_BS;
+            if (i < narr) sarr[i] = keep[u];
+        }
+        __syncthreads();
+        auto place = [&](int loc, int *hr, int at) {
+            const unsigned m = __match_any_sync(FULL, loc >= 0 ? loc : -1 - lane);
+            const int base = (loc >= 0) ? hr[loc] : 0;
+            __syncwarp();
+            if (loc >= 0 && lane == __ffs(m) - 1) hr[loc] = base + __popc(m);
+            if (at >= 0) sdst[at] = loc >= 0 ? (uint16_t)(base + __popc(m & lt)) : (uint16_t)0xFFFF;
+            __syncwarp();
+        };
+        for (int j = j0w; j < j1w; ++j) {
+            const int l16 = sdst[j * SEG + lane];
+            place(l16 == 0xFFFF ? -1 : l16, hist + wid * nc, j * SEG + lane);
+        }
+        {
+            const int q = nra == 1 ? 0 : wid;
+            const int i1 = nra > 1 ? min((q + 1) * pera, narr) : (wid == TILE_WARPS - 1 ? narr : 0);
+            for (int i0 = q * pera; i0 < i1; i0 += SEG) {
+                const int i = i0 + lane;
+                place(i < i1 ? local_of(P.mcell[sarr[i]]) : -1, hist + (TILE_WARPS + q) * nc, i < i1 ? nslot + i : -1);
+            }
+        }
+        __syncthreads();
+        stage_array(P.cell + to, P.mcell, P.ocell + to, sdst, sarr, (int32_t *)rsm, nslot, narr, total);
+        stage_array(P.ox + to, P.mox, P.oox + to, sdst, sarr, (R *)rsm, nslot, narr, total);
+        stage_array(P.oy + to, P.moy, P.ooy + to, sdst, sarr, (R *)rsm, nslot, narr, total);
+        stage_array(P.ux + to, P.mux, P.oux + to, sdst, sarr, (R *)rsm, nslot, narr, total);
+        stage_array(P.uy + to, P.muy, P.ouy + to, sdst, sarr, (R *)rsm, nslot, narr, total);
+        stage_array(P.uz + to, P.muz, P.ouz + to, sdst, sarr, (R *)rsm, nslot, narr, total);
+        stage_array(P.w + to, P.mw, P.ow + to, sdst, sarr, (R *)rsm, nslot, narr, total);
+    } else {
     {
         // two segments ahead: the next two are in flight while one is ranked and stored
         int n_a = 0, n_b = 0;
@@ -1335,6 +1452,7 @@ __device__ __forceinline__ void regroup_one(const TileArgs<R> &a, int t, int s, 
             __syncwarp();
         }
     }
+    }
     // 5. dense counts of the new bin
     for (int j = tid; j < need; j += TILE_BS) P.segn2[tb + j] = min(SEG, total - j * SEG);
     if (tid == 0) P.useg2[t] = need;
@@ -1343,8 +1461,8 @@ __device__ __forceinline__ void regroup_one(const TileArgs<R> &a, int t, int s, 
 // One block per (tile, species) in a batched launch (every tile of every run);
 // a single run's launch visits only the tiles of its regroup list, a fixed
 // grid striding over the list.
-template <typename R, bool kBatch>
-__global__ void __launch_bounds__(TILE_BS) k_regroup(const __grid_constant__ TileArgs<R> a0,
+template <typename R, bool kBatch, bool kStage>
+__global__ void __launch_bounds__(TILE_BS, kStage ? 3 : 0) k_regroup(const __grid_constant__ TileArgs<R> a0,
                                                      const TileArgs<R> *__restrict__ runs,
                                                      const int32_t *__restrict__ run_tiles, int nrun) {
     extern __shared__ int rsm[];
@@ -1360,7 +1478,7 @@ __global__ void __launch_bounds__(TILE_BS) k_regroup(const __grid_constant__ Til
         t -= run_tiles[lo];
         const int32_t *guard = runs[lo].guard;
         if (guard && (*guard & 3)) return;   // the run's previous regroup failed: the host redoes its step
-        regroup_one<R, kBatch>(runs[lo], t, s, rsm);
+        regroup_one<R, kBatch, kStage>(runs[lo], t, s, rsm);
     } else {
         // tiles from the list in turn (a queue per species: bins differ widely in size)
         if (a0.guard && (*a0.guard & 3)) return;
@@ -1371,7 +1489,7 @@ __global__ void __launch_bounds__(TILE_BS) k_regroup(const __grid_constant__ Til
             __syncthreads();
             const int li = s_li;
             if (li >= n) break;
-            regroup_one<R, kBatch>(a0, a0.rg_list[li], s, rsm);
+            regroup_one<R, kBatch, kStage>(a0, a0.rg_list[li], s, rsm);
             __syncthreads();   // the shared arrays (and s_li) are reused by the next tile
         }
     }
@@ -1576,6 +1694,12 @@ static int neighbour_table(pic_t *h) {
     return 0;
 }
 
+// A single run's regroup kernel.
+static const void *regroup_kernel(const pic_t *h) {
+    if (regroup_stages(h)) return (const void *)k_regroup<float, false, true>;
+    return h->fp32 ? (const void *)k_regroup<float, false, false> : (const void *)k_regroup<double, false, false>;
+}
+
 int tile_setup(pic_t *h) {
     int RW = h->tnx + 2 * h->halo + 1, RH = h->tny + 2 * h->halo + 1;
     if (RW > 256 || RH > 256) {
@@ -1624,18 +1748,16 @@ int tile_setup(pic_t *h) {
         if (int rs = h->fp32 ? push_s_occupancy<float>(h, &s2) : push_s_occupancy<double>(h, &s2)) return rs;
         h->push_blocks_s2 = s2 * nsm;
     }
-    const int rb = regroup_smem_bytes(h->tnx * h->tny);
-    cudaError_t e = h->fp32
-                        ? cudaFuncSetAttribute(k_regroup<float, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, rb)
-                        : cudaFuncSetAttribute(k_regroup<double, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, rb);
+    const int rb = regroup_smem_bytes(h);
+    const void *rk = regroup_kernel(h);
+    cudaError_t e = cudaFuncSetAttribute(rk, cudaFuncAttributeMaxDynamicSharedMemorySize, rb);
     if (e != cudaSuccess) {
         set_error("regroup kernel set-up: %s", cudaGetErrorString(e));
         return PIC_ERR_CUDA;
     }
     // the list-driven regroup: as many blocks per species as fit on the GPU at once (at most one per tile)
     int rper = 0;
-    e = h->fp32 ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&rper, k_regroup<float, false>, TILE_BS, rb)
-                : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&rper, k_regroup<double, false>, TILE_BS, rb);
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&rper, rk, TILE_BS, rb);
     if (e != cudaSuccess || rper < 1) rper = 1;
     int64_t rb_total = (int64_t)rper * nsm / (h->nsp > 0 ? h->nsp : 1);
     if (rb_total < 1) rb_total = 1;
@@ -1719,7 +1841,7 @@ static TileArgs<R> tile_args(pic_t *h) {
     a.items = h->items;
     a.nbr = h->nbr;
     a.ticket = h->ticket;
-    a.ch = item_segs(h);
+    a.ch = h->items_ch > 0 ? h->items_ch : item_segs(h);
     a.rg_list = h->rg_list;
     a.list_n = h->list_n;
     return a;
@@ -1729,13 +1851,14 @@ int push_work_list(pic_t *h) {
     UsegPtrs u;
     for (int s = 0; s < PIC_MAX_SPECIES; ++s) u.p[s] = (s < h->nsp) ? h->sp[s].useg[h->sp[s].scur] : nullptr;
     const int nitems = h->nsp * h->ntiles;
-    k_chunk_counts<<<(nitems + 256) / 256, 256, 0, h->st>>>(u, h->nsp, h->ntiles, item_segs(h), h->chunk_prefix,
+    h->items_ch = item_segs(h);
+    k_chunk_counts<<<(nitems + 256) / 256, 256, 0, h->st>>>(u, h->nsp, h->ntiles, h->items_ch, h->chunk_prefix,
                                                             h->ticket, h->occ);
     count_launch(h);
     return scan_i32_inplace(h, h->chunk_prefix, nitems + 1);
 }
 
-int push_item_segs(const pic_t *h) { return item_segs(h); }
+int push_item_segs(const pic_t *h) { return h->items_ch; }
 
 // The touch and regroup lists and the regroup queues, emptied for the next
 // push (after whatever read the previous push's lists: the clear of its tiles).
@@ -1819,17 +1942,17 @@ template <typename R>
 static int batch_regroup_t(BatchScratch &b, pic_t **hs, int n) {
     int smem = 0, nsp = 0;
     for (int r = 0; r < n; ++r) {
-        const int bytes = regroup_smem_bytes(hs[r]->tnx * hs[r]->tny);
+        const int bytes = regroup_smem_bytes(hs[r]);
         if (bytes > smem) smem = bytes;
         if (hs[r]->nsp > nsp) nsp = hs[r]->nsp;
     }
-    if (cudaFuncSetAttribute(k_regroup<R, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess)
+    if (cudaFuncSetAttribute(k_regroup<R, true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess)
         return check_launch("regroup (batched) set-up");
     const TileArgs<R> *dargs = (const TileArgs<R> *)b.args_dev;
     const int32_t *tiles_dev = b.idx + (b.cap + 1);
     const int total = b.idx_host[b.slot][n];
     TileArgs<R> a0 = ((const TileArgs<R> *)b.args_host[b.slot])[0];
-    k_regroup<R, true><<<dim3(total, nsp), TILE_BS, smem, b.st>>>(a0, dargs, tiles_dev, n);
+    k_regroup<R, true, false><<<dim3(total, nsp), TILE_BS, smem, b.st>>>(a0, dargs, tiles_dev, n);
     for (int r = 0; r < n; ++r) count_launch(hs[r]);
     return check_launch("k_regroup (batched)");
 }
@@ -1988,17 +2111,18 @@ int push_prep(pic_t *h, bool next) {
         u.p[s] = (s < h->nsp) ? h->sp[s].useg[next ? h->sp[s].scur ^ 1 : h->sp[s].scur] : nullptr;
     const int nitems = h->nsp * h->ntiles;
     if (int rc = ensure_items(h)) return rc;   // grown before any launch that would use it
+    h->items_ch = item_segs(h);
     if (nitems <= PREP_ONE_BLOCK) {
         const int sm = nitems * (int)sizeof(int);
         if (sm > 48 * 1024 && cudaFuncSetAttribute(k_prep_one_block, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                                    PREP_ONE_BLOCK * (int)sizeof(int)) != cudaSuccess)
             return check_launch("push work items set-up");
-        k_prep_one_block<<<1, PREP_BS, sm, h->st>>>(u, h->nsp, h->ntiles, item_segs(h), h->chunk_prefix, h->ticket,
+        k_prep_one_block<<<1, PREP_BS, sm, h->st>>>(u, h->nsp, h->ntiles, h->items_ch, h->chunk_prefix, h->ticket,
                                                     h->occ, h->items);
         count_launch(h);
         return check_launch("push work items");
     }
-    k_chunk_counts<<<(nitems + 256) / 256, 256, 0, h->st>>>(u, h->nsp, h->ntiles, item_segs(h), h->chunk_prefix,
+    k_chunk_counts<<<(nitems + 256) / 256, 256, 0, h->st>>>(u, h->nsp, h->ntiles, h->items_ch, h->chunk_prefix,
                                                             h->ticket, h->occ);
     count_launch(h);
     if (int rc = scan_i32_inplace(h, h->chunk_prefix, nitems + 1)) return rc;
@@ -2056,8 +2180,15 @@ int particle_tiles(pic_t *h, bool prepared) {
 template <typename R>
 static int regroup_t(pic_t *h) {
     TileArgs<R> a = tile_args<R>(h);
-    k_regroup<R, false><<<dim3(h->regroup_blocks, h->nsp), TILE_BS, regroup_smem_bytes(h->tnx * h->tny), h->st>>>(a, nullptr,
-                                                                                                       nullptr, 0);
+    const dim3 grid(h->regroup_blocks, h->nsp);
+    if constexpr (sizeof(R) == 4) {
+        if (regroup_stages(h)) {
+            k_regroup<R, false, true><<<grid, TILE_BS, regroup_smem_bytes(h), h->st>>>(a, nullptr, nullptr, 0);
+            count_launch(h);
+            return check_launch("k_regroup");
+        }
+    }
+    k_regroup<R, false, false><<<grid, TILE_BS, regroup_smem_bytes(h), h->st>>>(a, nullptr, nullptr, 0);
     count_launch(h);
     return check_launch("k_regroup");
 }
