@@ -65,16 +65,17 @@ extern "C" {
 
 #define PIC_FIELD_LITERAL 0  /* Eqs. 4-5 as printed: explicit curls, per-node 3x3 solve */
 #define PIC_FIELD_CN 1       /* time-centred curls, iterative stencil solve: FP64 residual and
-                                refinement around an FP32 BiCGSTAB (spectral preconditioner on
-                                periodic power-of-two grids, block-Jacobi otherwise); with
+                                refinement around FP32 corrections (on periodic grids a spectral
+                                preconditioner, alone or around BiCGSTAB; block-Jacobi BiCGSTAB
+                                otherwise); with
                                 absorbing walls the wall nodes are vacuum, their x rows take the
                                 one-sided curl of H and their y, z rows a time-centred first-order
                                 Mur condition (the laser enters through the x = 0 wall) */
 
 /* Preconditioner of the CN solve's FP32 inner iterations.  JACOBI: the inverse
  * of each node's 3x3 diagonal block (any grid).  FFT: the spectral inverse of
- * the operator with the grid mean of S (periodic x, nx and ny powers of two),
- * or, in a box with walls (ny a power of two), the line preconditioner: FFT
+ * the operator with the grid mean of S (periodic x; nx and ny at most 4096,
+ * without prime factors above 61), or, in a box with walls (ny a power of two), the line preconditioner: FFT
  * along y, then per y-mode the exact block-tridiagonal solve along x with the
  * column means of S and the walls' Mur rows (the exact inverse in vacuum).
  * AUTO: the spectral preconditioner where it applies, else block-Jacobi (in
@@ -153,7 +154,7 @@ typedef struct pic_diag {
     int64_t removed;           /* particles removed at walls since init */
     int64_t step;              /* steps taken since init */
     double cn_residual;        /* last CN solve: relative FP64 residual |b - A x| / |b| reached */
-    int32_t cn_iterations;     /* last CN solve: FP32 BiCGSTAB iterations, all refinements */
+    int32_t cn_iterations;     /* last CN solve: FP32 iterations (BiCGSTAB or spectral corrections), all refinements */
     int32_t flags;             /* bit 0: a particle moved farther than one tile in a step */
     int32_t cn_refinements;    /* last CN solve: FP64 refinement steps (FP32 inner solves) */
     int32_t full_regroups;     /* steps since init whose per-tile regroup fell back to the full sort */

@@ -6,8 +6,9 @@
 //               condition and the incident plane wave at x = 0, then
 //               H^{n+3/2} = H^{n+1/2} - dt curl_e E^{n+1}.
 // CN mode:      (I + S) X + (dt/2)^2 curl_h curl_e X = E^n + (dt/2)(curl_h H^n - dj)
-//               solved inside one cooperative kernel by FP64 iterative
-//               refinement around an FP32 block-Jacobi BiCGSTAB, then
+//               solved inside one kernel (a cooperative grid or one cluster)
+//               by FP64 iterative refinement around FP32 corrections
+//               (preconditioned BiCGSTAB, or the preconditioner alone), then
 //               E^{n+1} = 2X - E^n, H^{n+1} = H^n - dt curl_e X.
 // All kernels are bandwidth-bound stencils over node/cell arrays of V4.
 #include <cooperative_groups.h>
@@ -259,16 +260,24 @@ __global__ void k_fill_ghosts(GridArgs<R> g, int nyp, V4<R> *__restrict__ F) {
 // residual of CN_INNER_RTOL and x += d.  The FP32 operator differs from A
 // by rounding (~1e-7 relative), far below 1/cond(A), so every refinement cuts
 // the FP64 residual by about the inner tolerance.
+// One axis of the spectral preconditioner's transforms: n points, lg = log2 n, or
+// -1 where n is no power of two; then n is the product of the nf factors f.
+constexpr int FFT_FACTORS = 12;
+struct FftAxis {
+    int n, lg, nf, f[FFT_FACTORS];
+};
+
 struct CNVec {
     V4<double> *x, *b;                              // FP64 iterate and right-hand side
     V4<double> *cc;                                 // FP64 residual: curl_e x at the cells
     V4<float> *d, *r, *r0, *p, *v, *s, *t, *ph, *sh;  // FP32 inner solve of A d = r
     float *minv;                                    // [9][nnode] block-Jacobi inverse
     float *S;                                       // [9][nnode] S / dA
-    // spectral preconditioner (nx, ny powers of two): complex work arrays of
-    // nnode entries and twiddles e^{-2 pi i t / n}, t < n/2, for x and y
+    // spectral preconditioner (periodic): complex work arrays of nnode entries
+    // and twiddles e^{-2 pi i t / n}, t <= n/2, for x and y
     float2 *FA, *FB, *GA, *GB, *twx, *twy;
-    int fft, lx, ly;
+    int fft, ly;
+    FftAxis ax, ay;
     // line preconditioner (walls, ny a power of two): per column means of the
     // diagonal of S ([3][nxn]), the factors ([10][nxn][ny/2 + 1]) and the sweep
     // work ([6][nxn][ny/2 + 1]) of the per-mode block-tridiagonal solves
@@ -353,49 +362,44 @@ __device__ inline V4<T> apply_A(const GridArgs<double> &g, const V4<T> *__restri
     return y;
 }
 
-// The FP64 residual's operator in two passes, with the expressions of
-// apply_A: curl_e of X once per cell (cell (ci, cj) has corners (ci, cj),
-// (ci+1, cj), (ci, cj+1), (ci+1, cj+1), periodic), then per node curl_h of
-// those cell values, S X and X.  Each cell's curl is computed once instead of
-// once for each of its four corner nodes; the results are the same bits.
+// The FP64 residual's operator in two passes: curl_e of X once per cell (cell
+// (ci, cj) has corners (ci, cj), (ci+1, cj), (ci, cj+1), (ci+1, cj+1),
+// periodic), then per node curl_h of those cell values, S X and X.  The FP64 pipe
+// bounds the residual, so the derivatives come from diagonal differences
+// (curl_h_parts), the factors of curl_h and (dt/2)^2 are one constant per axis,
+// and the moments are scaled by the inverse area once per row.
 __device__ inline V4<double> cell_curl_e(const GridArgs<double> &g, const V4<double> *__restrict__ X, double hx,
                                          double hy, int ci, int cj) {
     const int ip = (g.periodic_x && ci + 1 == g.nx) ? 0 : ci + 1, jp = (cj + 1 == g.ny) ? 0 : cj + 1;
     const V4<double> e00 = X[(int64_t)cj * g.nxn + ci], e10 = X[(int64_t)cj * g.nxn + ip];
     const V4<double> e01 = X[(int64_t)jp * g.nxn + ci], e11 = X[(int64_t)jp * g.nxn + ip];
-    const double dEz_dy = ((e01.z + e11.z) - (e00.z + e10.z)) * hy;
-    const double dEz_dx = ((e10.z + e11.z) - (e00.z + e01.z)) * hx;
-    const double dEy_dx = ((e10.y + e11.y) - (e00.y + e01.y)) * hx;
-    const double dEx_dy = ((e01.x + e11.x) - (e00.x + e10.x)) * hy;
-    return V4<double>{dEz_dy, -dEz_dx, dEy_dx - dEx_dy, 0.0};
+    const double pz = e11.z - e00.z, qz = e01.z - e10.z;
+    const double sy = (e11.y - e00.y) + (e10.y - e01.y);   // 2 dx dEy/dx
+    const double sx = (e11.x - e00.x) + (e01.x - e10.x);   // 2 dy dEx/dy
+    return V4<double>{(pz + qz) * hy, (qz - pz) * hx, fma(sy, hx, -(sx * hy)), 0.0};
 }
 
+// kx = c2 hx, ky = c2 hy
 __device__ inline V4<double> apply_A_from_cells(const GridArgs<double> &g, const V4<double> *__restrict__ X,
                                                 const V4<double> *__restrict__ Cc, const double *__restrict__ S9,
-                                                double sc, double c2, double hx, double hy, int i, int j,
-                                                double cw = 0.0, double cv = 0.0) {
-    const int im = (i == 0) ? g.nx - 1 : i - 1, jm = (j == 0) ? g.ny - 1 : j - 1;
+                                                double sc, double kx, double ky, int i, int j, double cw, double cv) {
     if (!g.periodic_x && (i == 0 || i == g.nx)) {   // wall node (apply_A_wall with the cells' curls)
+        const int jm = (j == 0) ? g.ny - 1 : j - 1;
         const int ic = (i == 0) ? 0 : g.nx - 1, iv = (i == 0) ? 1 : g.nx - 1;
         const double up = Cc[(int64_t)j * g.nx + ic].z, dn = Cc[(int64_t)jm * g.nx + ic].z;
         const V4<double> xw = X[(int64_t)j * g.nxn + i], xv = X[(int64_t)j * g.nxn + iv];
-        return V4<double>{xw.x + c2 * ((up - dn) * (2.0 * hy)), cw * xw.y + cv * xv.y, cw * xw.z + cv * xv.z, 0.0};
+        return V4<double>{fma(up - dn, 2.0 * ky, xw.x), cw * xw.y + cv * xv.y, cw * xw.z + cv * xv.z, 0.0};
     }
-    // cells a = [1][1] (i, j), b = [1][0] (im, j), c = [0][1] (i, jm), d = [0][0] (im, jm)
-    const V4<double> c11 = Cc[(int64_t)j * g.nx + i], c10 = Cc[(int64_t)j * g.nx + im];
-    const V4<double> c01 = Cc[(int64_t)jm * g.nx + i], c00 = Cc[(int64_t)jm * g.nx + im];
-    const double kx = ((c11.z + c10.z) - (c01.z + c00.z)) * hy;
-    const double ky = -(((c11.z + c01.z) - (c10.z + c00.z)) * hx);
-    const double kz = ((c11.y + c01.y) - (c10.y + c00.y)) * hx - ((c11.x + c10.x) - (c01.x + c00.x)) * hy;
+    double u, v, sy, sx;
+    curl_h_parts(g, Cc, i, j, u, v, sy, sx);
     const int64_t node = (int64_t)j * g.nxn + i;
     const V4<double> xc = X[node];
-    double S[9];
-#pragma unroll
-    for (int k = 0; k < 9; ++k) S[k] = S9[(int64_t)k * g.nnode + node] * sc;
+    const double *q = S9 + node;
+    const int64_t st = g.nnode;
     V4<double> y;
-    y.x = xc.x + (S[0] * xc.x + S[1] * xc.y + S[2] * xc.z) + c2 * kx;
-    y.y = xc.y + (S[3] * xc.x + S[4] * xc.y + S[5] * xc.z) + c2 * ky;
-    y.z = xc.z + (S[6] * xc.x + S[7] * xc.y + S[8] * xc.z) + c2 * kz;
+    y.x = fma(fma(q[2 * st], xc.z, fma(q[st], xc.y, q[0] * xc.x)), sc, fma(u, ky, xc.x));
+    y.y = fma(fma(q[5 * st], xc.z, fma(q[4 * st], xc.y, q[3 * st] * xc.x)), sc, fma(v, kx, xc.y));
+    y.z = fma(fma(q[8 * st], xc.z, fma(q[7 * st], xc.y, q[6 * st] * xc.x)), sc, fma(sy, kx, fma(-sx, ky, xc.z)));
     y.w = 0.0;
     return y;
 }
@@ -418,96 +422,174 @@ __device__ inline T dot(const V4<T> &a, const V4<T> &b) { return a.x * b.x + a.y
 // (the symbols of d/dx and d/dy from nodes to cells), curl_h curl_e acts as
 // [[|q|^2, -q* p, 0], [-p* q, |p|^2, 0], [0, 0, |p|^2 + |q|^2]].  The
 // preconditioner solves that 3x3 system per mode with s = the grid mean of the
-// diagonal of S, using FP32 radix-2 FFTs along rows, a transpose, and FFTs
-// along the other axis; x and y share one complex transform (x + i y).
+// diagonal of S, using FP32 FFTs; x and y share one complex transform (x + i y).
 
 __device__ inline float2 cmul(float2 a, float2 b) { return make_float2(a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x); }
 
-// In-place FFT of nrows rows of n = 2^logn complex values (row r of the
-// first nrows_a rows in A, the rest in B), by the Stockham autosort form of
-// the radix-2 transform: stage L = 1, 2, ..., n/2 reads x[j] and x[j + n/2]
-// (j = q L + k < n/2) and writes y[2 q L + k] = x[j] + w^k x[j + n/2],
-// y[2 q L + k + L] = x[j] - w^k x[j + n/2] with w = e^{-+2 pi i / (2L)},
-// between two shared buffers.  Input and output are in natural order (no bit
-// reversal), the reads are contiguous, and stage L takes its L twiddles from a
-// table of its own (entries L - 1 ... 2L - 2), so that neighbouring threads
-// read neighbouring words.  Short rows are transformed several at a time (up
-// to FFT_GROUP values, at most the block's share of the rows), so that the
-// threads have work between two barriers.  With vin the rows are read from
-// a V4 vector instead (A rows: x + i y, B rows: z), with vout written to one
-// (A rows give x, y and the spare component, B rows z).
-constexpr int FFT_GROUP = 2048;
+// Barrier over all the blocks of the solve: a grid barrier (cooperative launch),
+// or, when the whole grid is one thread-block cluster (small grids), the
+// cluster barrier, which costs a fraction of it.
+template <bool kCluster>
+struct SolveBarrier {
+    __device__ inline void sync() const {
+        if constexpr (kCluster) cg::this_cluster().sync();
+        else cg::this_grid().sync();
+    }
+};
 
-__device__ inline void fft_rows(float2 *A, float2 *B, int nrows_a, int n, int logn, const float2 *__restrict__ tw,
-                                bool inverse, float2 *sm, const V4<float> *vin = nullptr,
-                                V4<float> *vout = nullptr) {
-    const int G = n > FFT_GROUP ? n : FFT_GROUP;
-    float2 *buf0 = sm, *buf1 = sm + G, *tws = sm + 2 * G;
+// Twiddles of an n-point transform by stage, in shared memory: entries L - 1 +
+// k, k < L, hold e^{-2 pi i k / (2 L)} for L = 1, 2, ..., n/2 (n - 1 entries),
+// so that neighbouring threads of a stage read neighbouring words.
+__device__ inline void fft_twiddles(float2 *tws, const float2 *__restrict__ tw, int n) {
     const int nh = n >> 1;
     for (int t = threadIdx.x; t < n - 1; t += blockDim.x) {
-        const int lg = 31 - __clz(t + 1), L = 1 << lg, k = t - (L - 1);   // stage L, twiddle k < L
-        float2 w = tw[k * (nh >> lg)];
-        if (inverse) w.y = -w.y;
+        const int lg = 31 - __clz(t + 1), L = 1 << lg, k = t - (L - 1);
+        tws[t] = tw[k * (nh >> lg)];
+    }
+}
+
+// FFT of nrow rows of n = 2^logn complex values (row r at r * rs of x), by the
+// Stockham autosort form with radix-4 stages (and one of radix 2 first when
+// logn is odd) between the two shared buffers x and y; on return x holds the
+// result.  Stage L reads x[j + r n/4] (r = 0 .. 3, j = q L + k < n/4) and writes
+// y[4 q L + k + s L].  Input and output in natural order; the inverse is not
+// scaled.  Ends with a block barrier.
+template <bool kInv>
+__device__ inline void fft_core(float2 *&x, float2 *&y, int nrow, int rs, int n, int logn, const float2 *tws) {
+    auto tw = [&](int i) {
+        float2 w = tws[i];
+        if (kInv) w.y = -w.y;
+        return w;
+    };
+    int lg = 0;
+    if (logn & 1) {
+        const int nh = n >> 1;
+        for (int e = threadIdx.x; e < nrow * nh; e += blockDim.x) {
+            const int r = e >> (logn - 1), j = e & (nh - 1);
+            const float2 a = x[r * rs + j], t = x[r * rs + j + nh];
+            y[r * rs + 2 * j] = make_float2(a.x + t.x, a.y + t.y);
+            y[r * rs + 2 * j + 1] = make_float2(a.x - t.x, a.y - t.y);
+        }
+        __syncthreads();
+        float2 *z = x;
+        x = y;
+        y = z;
+        lg = 1;
+    }
+    const int n4 = n >> 2;
+    for (; lg < logn; lg += 2) {
+        const int L = 1 << lg;
+        for (int e = threadIdx.x; e < nrow * n4; e += blockDim.x) {
+            const int r = e >> (logn - 2), j = e & (n4 - 1), k = j & (L - 1);
+            const float2 *xr = x + r * rs + j;
+            float2 *yo = y + r * rs + ((j >> lg) << (lg + 2)) + k;
+            const float2 w1 = tw(2 * L - 1 + k), w2 = tw(L - 1 + k), w3 = cmul(w1, w2);
+            const float2 a0 = xr[0], a1 = cmul(w1, xr[n4]), a2 = cmul(w2, xr[2 * n4]), a3 = cmul(w3, xr[3 * n4]);
+            const float2 t0 = make_float2(a0.x + a2.x, a0.y + a2.y), t1 = make_float2(a0.x - a2.x, a0.y - a2.y);
+            const float2 t2 = make_float2(a1.x + a3.x, a1.y + a3.y), t3 = make_float2(a1.x - a3.x, a1.y - a3.y);
+            yo[0] = make_float2(t0.x + t2.x, t0.y + t2.y);
+            yo[2 * L] = make_float2(t0.x - t2.x, t0.y - t2.y);
+            const float2 m = make_float2(t1.x + t3.y, t1.y - t3.x), q = make_float2(t1.x - t3.y, t1.y + t3.x);   // t1 -+ i t3
+            yo[L] = kInv ? q : m;
+            yo[3 * L] = kInv ? m : q;
+        }
+        __syncthreads();
+        float2 *z = x;
+        x = y;
+        y = z;
+    }
+}
+
+// The same for any n = f[0] f[1] ...: a stage of radix r after those of product
+// L takes y[q L r + k + t L] = sum over s of x[q L + k + s n/r] e^{-2 pi i s (k + t
+// L) / (L r)}, an output at a time.  tws: e^{-2 pi i t / n}, t < n.
+template <bool kInv>
+__device__ inline void fft_core_any(float2 *&x, float2 *&y, int nrow, int rs, const FftAxis &ax, const float2 *tws) {
+    const int n = ax.n;
+    for (int st = 0, L = 1; st < ax.nf; ++st) {
+        const int r = ax.f[st], Lr = L * r, step = n / r, ws = n / Lr;   // root ws k' of unity for k' of Lr
+        for (int e = threadIdx.x; e < nrow * n; e += blockDim.x) {
+            const int row = e / n, o = e - row * n, q = o / Lr, kt = o - q * Lr, k = kt % L;
+            const float2 *xr = x + row * rs + q * L + k;
+            float2 acc = xr[0];
+            int w = 0;
+            for (int s = 1; s < r; ++s) {
+                w += kt * ws;
+                if (w >= n) w -= n;
+                float2 c = tws[w];
+                if (kInv) c.y = -c.y;
+                const float2 t = cmul(c, xr[s * step]);
+                acc.x += t.x;
+                acc.y += t.y;
+            }
+            y[row * rs + o] = acc;
+        }
+        __syncthreads();
+        float2 *z = x;
+        x = y;
+        y = z;
+        L = Lr;
+    }
+}
+
+template <bool kInv>
+__device__ inline void fft_axis(float2 *&x, float2 *&y, int nrow, int rs, const FftAxis &ax, const float2 *tws) {
+    if (ax.lg >= 0) fft_core<kInv>(x, y, nrow, rs, ax.n, ax.lg, tws);
+    else fft_core_any<kInv>(x, y, nrow, rs, ax, tws);
+}
+
+// Twiddles of an axis in shared memory (n entries), and e^{2 pi i k / n}, 0 <= k < n, from them.
+__device__ inline void axis_twiddles(float2 *tws, const float2 *__restrict__ tw, const FftAxis &ax) {
+    if (ax.lg >= 0) {
+        fft_twiddles(tws, tw, ax.n);
+        return;
+    }
+    for (int t = threadIdx.x; t < ax.n; t += blockDim.x) {
+        float2 w = tw[min(t, ax.n - t)];
+        if (2 * t > ax.n) w.y = -w.y;
         tws[t] = w;
     }
+}
+__device__ inline float2 axis_unit(const float2 *tws, const FftAxis &ax, int k) {
+    if (ax.lg < 0) return make_float2(tws[k].x, -tws[k].y);
+    const int h = ax.n >> 1;   // the last stage's entries
+    const float2 w = tws[h - 1 + (k < h ? k : k - h)];
+    return k < h ? make_float2(w.x, -w.y) : make_float2(-w.x, w.y);
+}
+__device__ inline int axis_div(int e, const FftAxis &ax) { return ax.lg >= 0 ? e >> ax.lg : e / ax.n; }
+__device__ inline int axis_neg(int k, const FftAxis &ax) { return k == 0 ? 0 : ax.n - k; }
+
+// Values of one row group of the transforms (short rows are taken several at
+// a time, so that the threads have work between two barriers).
+constexpr int FFT_GROUP = 2048;
+__host__ __device__ inline int fft_buffer(int n, int columns) {   // float2 entries of one of the two buffers
+    const int need = columns ? 2 * (n + 1) : n;
+    return need > FFT_GROUP ? need : FFT_GROUP;
+}
+
+// In-place FFT of nrows rows of n values (row r of the first nrows_a rows in
+// A, the rest in B); the line preconditioner's transforms.
+__device__ inline void fft_rows(float2 *A, float2 *B, int nrows_a, int n, int logn, const float2 *__restrict__ tw,
+                                bool inverse, float2 *sm) {
+    const int G = fft_buffer(n, 0);
+    float2 *tws = sm + 2 * G;
+    fft_twiddles(tws, tw, n);
     __syncthreads();
     const int nrows = 2 * nrows_a;
     const int share = (nrows + gridDim.x - 1) / gridDim.x;
     const int rpb = max(1, min(G >> logn, share));
     for (int row0 = blockIdx.x * rpb; row0 < nrows; row0 += gridDim.x * rpb) {
         const int nr = min(rpb, nrows - row0);
-        for (int e = threadIdx.x; e < nr * n; e += blockDim.x) {
-            const int r = e >> logn, row = row0 + r;
-            if (vin) {
-                const bool a = row < nrows_a;
-                const V4<float> q = vin[(int64_t)(a ? row : row - nrows_a) * n + (e & (n - 1))];
-                buf0[e] = a ? make_float2(q.x, q.y) : make_float2(q.z, 0.f);
-            } else {
-                const float2 *d = row < nrows_a ? A + (int64_t)row * n : B + (int64_t)(row - nrows_a) * n;
-                buf0[e] = d[e & (n - 1)];
-            }
-        }
+        auto at = [&](int e) {
+            const int row = row0 + (e >> logn);
+            return (row < nrows_a ? A + (int64_t)row * n : B + (int64_t)(row - nrows_a) * n) + (e & (n - 1));
+        };
+        float2 *x = sm, *y = sm + G;
+        for (int e = threadIdx.x; e < nr * n; e += blockDim.x) x[e] = *at(e);
         __syncthreads();
-        float2 *x = buf0, *y = buf1;
-        for (int lg = 0; lg < logn; ++lg) {
-            const int L = 1 << lg;
-            if (nr == 1) {   // one long row: no row index
-                for (int j = threadIdx.x; j < nh; j += blockDim.x) {
-                    const int k = j & (L - 1), o = ((j >> lg) << (lg + 1)) + k;
-                    const float2 a = x[j], t = cmul(tws[L - 1 + k], x[j + nh]);
-                    y[o] = make_float2(a.x + t.x, a.y + t.y);
-                    y[o + L] = make_float2(a.x - t.x, a.y - t.y);
-                }
-            } else {
-                for (int e = threadIdx.x; e < nr * nh; e += blockDim.x) {
-                    const int r = e >> (logn - 1), j = e & (nh - 1);
-                    const int k = j & (L - 1), o = r * n + ((j >> lg) << (lg + 1)) + k;
-                    const float2 a = x[r * n + j], t = cmul(tws[L - 1 + k], x[r * n + j + nh]);
-                    y[o] = make_float2(a.x + t.x, a.y + t.y);
-                    y[o + L] = make_float2(a.x - t.x, a.y - t.y);
-                }
-            }
-            __syncthreads();
-            float2 *z = x;
-            x = y;
-            y = z;
-        }
-        for (int e = threadIdx.x; e < nr * n; e += blockDim.x) {
-            const int r = e >> logn, row = row0 + r;
-            if (vout) {
-                V4<float> &q = vout[(int64_t)(row < nrows_a ? row : row - nrows_a) * n + (e & (n - 1))];
-                if (row < nrows_a) {
-                    q.x = x[e].x;
-                    q.y = x[e].y;
-                    q.w = 0.f;
-                } else {
-                    q.z = x[e].x;
-                }
-            } else {
-                float2 *d = row < nrows_a ? A + (int64_t)row * n : B + (int64_t)(row - nrows_a) * n;
-                d[e & (n - 1)] = x[e];
-            }
-        }
+        if (inverse) fft_core<true>(x, y, nr, n, n, logn, tws);
+        else fft_core<false>(x, y, nr, n, n, logn, tws);
+        for (int e = threadIdx.x; e < nr * n; e += blockDim.x) *at(e) = x[e];
         __syncthreads();
     }
 }
@@ -534,54 +616,165 @@ __device__ inline void transpose2(const float2 *in_a, const float2 *in_b, float2
     }
 }
 
-// out = P^{-1} in (all blocks of the cooperative grid take part; ends with out written).
-__device__ inline void apply_spectral(cg::grid_group &grid, const GridArgs<double> &g, const CNVec &v,
-                                      const V4<float> *in, V4<float> *out, float c2, float sx, float sy, float sz,
-                                      float2 *sm) {
-    const int nx = g.nx, ny = g.ny;
-    const int64_t N = (int64_t)nx * ny;
-    const int64_t tid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x, stride = (int64_t)gridDim.x * blockDim.x;
-    fft_rows(v.FA, v.FB, ny, nx, v.lx, v.twx, false, sm, in);    // along x: [y][x] (from in: x + i y, z)
-    grid.sync();
-    transpose2(v.FA, v.FB, v.GA, v.GB, ny, nx, sm);               // -> [x][y]
-    grid.sync();
-    fft_rows(v.GA, v.GB, nx, ny, v.ly, v.twy, false, sm);        // along y: spectra [kx][ky]
-    grid.sync();
-    const float ihx = 0.5f * (float)g.inv_dx, ihy = 0.5f * (float)g.inv_dy, inv_n = 1.f / (float)N;
-    for (int64_t idx = tid; idx < N; idx += stride) {
-        const int kx = (int)(idx / ny), ky = (int)(idx - (int64_t)kx * ny);
-        const int64_t m = (int64_t)((nx - kx) & (nx - 1)) * ny + ((ny - ky) & (ny - 1));
-        const float2 F = v.GA[idx], Fm = v.GA[m], Z = v.GB[idx];
-        // X = (F + conj(Fm)) / 2, Y = (F - conj(Fm)) / (2i)
-        const float2 X = make_float2(0.5f * (F.x + Fm.x), 0.5f * (F.y - Fm.y));
-        const float2 Y = make_float2(0.5f * (F.y + Fm.y), -0.5f * (F.x - Fm.x));
-        float sa, ca, sb, cb;
-        sincospif(2.f * (float)kx / (float)nx, &sa, &ca);
-        sincospif(2.f * (float)ky / (float)ny, &sb, &cb);
-        // p = (e^{ia} - 1)(1 + e^{ib}) / (2 dx), q = (1 + e^{ia})(e^{ib} - 1) / (2 dy)
-        const float2 ea1 = make_float2(ca - 1.f, sa), eb1 = make_float2(cb - 1.f, sb);
-        const float2 ea2 = make_float2(ca + 1.f, sa), eb2 = make_float2(cb + 1.f, sb);
-        float2 p = cmul(ea1, eb2), q = cmul(ea2, eb1);
+// One application takes three passes over the grid, with a barrier between
+// them: transforms along x of x + i y and z row by row (the first pass also
+// forms the vector, load(n) = its value at node n); then, column by column, the
+// transform along y, the modes' 3x3 systems and the transform back; then the
+// transforms back along x.  The columns kx and -kx, which the modes of the two
+// real fields in x + i y couple, are taken by the same block.  (Transposing the
+// arrays around the transforms along y, with passes of their own, took five
+// barriers and four more passes.)  Shared memory: two buffers, then the
+// twiddles of x and of y (fft_tables).
+struct FftShared {
+    float2 *buf0, *buf1, *twx, *twy;
+    int G;
+};
+
+__host__ __device__ inline int spectral_buffer(int nx, int ny) {
+    const int a = fft_buffer(2 * nx, 0), b = fft_buffer(ny, 1);
+    return a > b ? a : b;
+}
+
+__device__ inline FftShared fft_shared(const GridArgs<double> &g, float2 *sm) {
+    FftShared f;
+    f.G = spectral_buffer(g.nx, g.ny);
+    f.buf0 = sm;
+    f.buf1 = sm + f.G;
+    f.twx = sm + 2 * f.G;
+    f.twy = f.twx + g.nx;
+    return f;
+}
+
+template <typename Load>
+__device__ inline void spectral_rows(const GridArgs<double> &g, const CNVec &v, const FftShared &f, const Load &load) {
+    const int nx = g.nx;
+    const int rpb = max(1, min(f.G / (2 * nx), (g.ny + (int)gridDim.x - 1) / (int)gridDim.x));
+    for (int y0 = blockIdx.x * rpb; y0 < g.ny; y0 += gridDim.x * rpb) {
+        const int nr = min(rpb, g.ny - y0), m = nr * nx;
+        const int64_t n0 = (int64_t)y0 * nx;
+        float2 *x = f.buf0, *y = f.buf1;
+        for (int e = threadIdx.x; e < m; e += blockDim.x) {
+            const V4<float> q = load(n0 + e);
+            x[e] = make_float2(q.x, q.y);
+            x[m + e] = make_float2(q.z, 0.f);
+        }
+        __syncthreads();
+        fft_axis<false>(x, y, 2 * nr, nx, v.ax, f.twx);
+        for (int e = threadIdx.x; e < m; e += blockDim.x) {
+            v.FA[n0 + e] = x[e];
+            v.FB[n0 + e] = x[m + e];
+        }
+        __syncthreads();
+    }
+}
+
+template <typename Store>
+__device__ inline void spectral_rows_back(const GridArgs<double> &g, const CNVec &v, const FftShared &f, const Store &store) {
+    const int nx = g.nx;
+    const int rpb = max(1, min(f.G / (2 * nx), (g.ny + (int)gridDim.x - 1) / (int)gridDim.x));
+    for (int y0 = blockIdx.x * rpb; y0 < g.ny; y0 += gridDim.x * rpb) {
+        const int nr = min(rpb, g.ny - y0), m = nr * nx;
+        const int64_t n0 = (int64_t)y0 * nx;
+        float2 *x = f.buf0, *y = f.buf1;
+        for (int e = threadIdx.x; e < m; e += blockDim.x) {
+            x[e] = v.FA[n0 + e];
+            x[m + e] = v.FB[n0 + e];
+        }
+        __syncthreads();
+        fft_axis<true>(x, y, 2 * nr, nx, v.ax, f.twx);
+        for (int e = threadIdx.x; e < m; e += blockDim.x) store(n0 + e, V4<float>{x[e].x, x[e].y, x[m + e].x, 0.f});
+        __syncthreads();
+    }
+}
+
+__device__ inline void spectral_columns(const GridArgs<double> &g, const CNVec &v, const FftShared &f, float c2, float sx,
+                                        float sy, float sz) {
+    const int nx = g.nx, ny = g.ny, rs = ny + 1, npair = nx / 2 + 1;
+    const int per = max(1, min(f.G / (2 * rs), (npair + (int)gridDim.x - 1) / (int)gridDim.x));
+    const float ihx = 0.5f * (float)g.inv_dx, ihy = 0.5f * (float)g.inv_dy, inv_n = 1.f / (float)((int64_t)nx * ny);
+    // p = (e^{ia} - 1)(1 + e^{ib}) / (2 dx), q = (1 + e^{ia})(e^{ib} - 1) / (2 dy)
+    auto symbols = [&](int kx, int ky, float2 &p, float2 &q) {
+        const float2 a = axis_unit(f.twx, v.ax, kx), b = axis_unit(f.twy, v.ay, ky);
+        p = cmul(make_float2(a.x - 1.f, a.y), make_float2(b.x + 1.f, b.y));
+        q = cmul(make_float2(a.x + 1.f, a.y), make_float2(b.x - 1.f, b.y));
         p = make_float2(p.x * ihx, p.y * ihx);
         q = make_float2(q.x * ihy, q.y * ihy);
-        const float pp = p.x * p.x + p.y * p.y, qq = q.x * q.x + q.y * q.y;
-        const float2 cqp = cmul(make_float2(q.x, -q.y), p);   // conj(q) p
-        const float A11 = 1.f + sx + c2 * qq, A22 = 1.f + sy + c2 * pp;
-        const float2 A12 = make_float2(-c2 * cqp.x, -c2 * cqp.y), A21 = make_float2(A12.x, -A12.y);
-        const float idet = inv_n / (A11 * A22 - (A12.x * A12.x + A12.y * A12.y));
-        const float2 a12y = cmul(A12, Y), a21x = cmul(A21, X);
-        const float2 Xs = make_float2((A22 * X.x - a12y.x) * idet, (A22 * X.y - a12y.y) * idet);
-        const float2 Ys = make_float2((A11 * Y.x - a21x.x) * idet, (A11 * Y.y - a21x.y) * idet);
-        const float iz = inv_n / (1.f + sz + c2 * (pp + qq));
-        v.FA[idx] = make_float2(Xs.x - Ys.y, Xs.y + Ys.x);   // X' + i Y'
-        v.FB[idx] = make_float2(Z.x * iz, Z.y * iz);
+    };
+    for (int c0 = blockIdx.x * per; c0 < npair; c0 += gridDim.x * per) {
+        const int nc = min(per, npair - c0), ns = 2 * nc;   // slots: columns c0 .. c0 + nc - 1, then their partners
+        auto column = [&](int s) { return s < nc ? c0 + s : axis_neg(c0 + s - nc, v.ax); };
+        auto own = [&](int s) { return s < nc || column(s) != c0 + s - nc; };   // (0 and, for an even nx, nx/2 are their own partners)
+        // both fields at once where the buffers hold them (short columns: fewer rounds of latency)
+        const int nf = 2 * ns * rs <= f.G ? 2 : 1;
+        for (int f0 = 0; f0 < 2; f0 += nf) {
+            float2 *x = f.buf0, *y = f.buf1;
+            for (int e = threadIdx.x; e < nf * ny * ns; e += blockDim.x) {
+                const int r = e / ns, s = e - r * ns, fl = r >= ny ? 1 : 0, rr = r - fl * ny;
+                x[(fl * ns + s) * rs + rr] = ((f0 + fl) ? v.FB : v.FA)[(int64_t)rr * nx + column(s)];
+            }
+            __syncthreads();
+            fft_axis<false>(x, y, nf * ns, rs, v.ay, f.twy);
+            if (f0 == 0) {
+                for (int e = threadIdx.x; e < nc * ny; e += blockDim.x) {
+                    const int s = axis_div(e, v.ay), ky = e - s * ny, mky = axis_neg(ky, v.ay), kx = c0 + s;
+                    const bool self = column(nc + s) == kx;
+                    if (self && ky > mky) continue;   // taken with its conjugate
+                    float2 *F0 = x + s * rs + ky, *F1 = x + (self ? s : nc + s) * rs + mky;
+                    const float2 Fk = *F0, Fm = *F1;
+                    // X = (F + conj(Fm)) / 2, Y = (F - conj(Fm)) / (2i)
+                    const float2 X = make_float2(0.5f * (Fk.x + Fm.x), 0.5f * (Fk.y - Fm.y));
+                    const float2 Y = make_float2(0.5f * (Fk.y + Fm.y), -0.5f * (Fk.x - Fm.x));
+                    float2 p, q;
+                    symbols(kx, ky, p, q);
+                    const float pp = p.x * p.x + p.y * p.y, qq = q.x * q.x + q.y * q.y;
+                    const float2 cqp = cmul(make_float2(q.x, -q.y), p);   // conj(q) p
+                    const float A11 = 1.f + sx + c2 * qq, A22 = 1.f + sy + c2 * pp;
+                    const float2 A12 = make_float2(-c2 * cqp.x, -c2 * cqp.y), A21 = make_float2(A12.x, -A12.y);
+                    const float idet = inv_n / (A11 * A22 - (A12.x * A12.x + A12.y * A12.y));
+                    const float2 a12y = cmul(A12, Y), a21x = cmul(A21, X);
+                    const float2 Xs = make_float2((A22 * X.x - a12y.x) * idet, (A22 * X.y - a12y.y) * idet);
+                    const float2 Ys = make_float2((A11 * Y.x - a21x.x) * idet, (A11 * Y.y - a21x.y) * idet);
+                    *F0 = make_float2(Xs.x - Ys.y, Xs.y + Ys.x);                       // X' + i Y'
+                    if (F1 != F0) *F1 = make_float2(Xs.x + Ys.y, Ys.x - Xs.y);         // conj(X') + i conj(Y')
+                }
+            }
+            if (f0 + nf == 2) {
+                float2 *xb = x + (nf - 1) * ns * rs;
+                for (int e = threadIdx.x; e < ns * ny; e += blockDim.x) {
+                    const int s = axis_div(e, v.ay), ky = e - s * ny;
+                    float2 p, q;
+                    symbols(column(s), ky, p, q);
+                    const float iz = inv_n / (1.f + sz + c2 * ((p.x * p.x + p.y * p.y) + (q.x * q.x + q.y * q.y)));
+                    float2 &Z = xb[s * rs + ky];
+                    Z = make_float2(Z.x * iz, Z.y * iz);
+                }
+            }
+            __syncthreads();
+            fft_axis<true>(x, y, nf * ns, rs, v.ay, f.twy);
+            for (int e = threadIdx.x; e < nf * ny * ns; e += blockDim.x) {
+                const int r = e / ns, s = e - r * ns, fl = r >= ny ? 1 : 0, rr = r - fl * ny;
+                if (own(s)) ((f0 + fl) ? v.FB : v.FA)[(int64_t)rr * nx + column(s)] = x[(fl * ns + s) * rs + rr];
+            }
+            __syncthreads();
+        }
     }
+}
+
+// store(n, .) = P^{-1} of the vector that load makes (all blocks take part).
+// mid(): between the first pass and its barrier; more(): after that barrier,
+// false ends the application there.
+template <bool kCluster, typename Load, typename Mid, typename More, typename Store>
+__device__ inline bool apply_spectral(const SolveBarrier<kCluster> &grid, const GridArgs<double> &g, const CNVec &v,
+                                      const FftShared &f, const Load &load, const Mid &mid, const More &more,
+                                      const Store &store, float c2, float sx, float sy, float sz) {
+    spectral_rows(g, v, f, load);
+    mid();
     grid.sync();
-    fft_rows(v.FA, v.FB, nx, ny, v.ly, v.twy, true, sm);         // back along y: [kx][y]
+    if (!more()) return false;
+    spectral_columns(g, v, f, c2, sx, sy, sz);
     grid.sync();
-    transpose2(v.FA, v.FB, v.GA, v.GB, nx, ny, sm);               // -> [y][kx]
-    grid.sync();
-    fft_rows(v.GA, v.GB, ny, nx, v.lx, v.twx, true, sm, nullptr, out);   // back along x: [y][x], into out
+    spectral_rows_back(g, v, f, store);
+    return true;
 }
 
 // ---- line preconditioner (walls) -----------------------------------------
@@ -665,7 +858,8 @@ __device__ inline void mul2(const float (&p)[4], const float (&q)[4], float (&o)
 // column i, Dp_i = D_i - M_i U_{i-1} with M_i = L_i Dp_{i-1}^{-1}; stored, mode
 // by mode (lf[b][q][i]), are Dp_i^{-1} (q = 0..3), M_i (4..7), 1/dp_i and m_i
 // of the Z row (8, 9).  nbm = ny/2 + 1 modes.
-__device__ inline void line_setup(cg::grid_group &grid, const GridArgs<double> &g, const CNVec &v, float c2, float cw,
+template <bool kCluster>
+__device__ inline void line_setup(const SolveBarrier<kCluster> &grid, const GridArgs<double> &g, const CNVec &v, float c2, float cw,
                                   float cv) {
     const int64_t tid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x, stride = (int64_t)gridDim.x * blockDim.x;
     const int nxn = g.nxn, nbm = g.ny / 2 + 1;
@@ -725,7 +919,8 @@ __device__ inline void line_setup(cg::grid_group &grid, const GridArgs<double> &
 __host__ __device__ inline size_t line_sweep_bytes(int nxn) { return (size_t)nxn * 16 * sizeof(float); }
 
 // out = P^{-1} in (all blocks of the cooperative grid take part; ends with out written).
-__device__ inline void apply_line(cg::grid_group &grid, const GridArgs<double> &g, const CNVec &v,
+template <bool kCluster>
+__device__ inline void apply_line(const SolveBarrier<kCluster> &grid, const GridArgs<double> &g, const CNVec &v,
                                   const V4<float> *in, V4<float> *out, float c2, float cw, float cv, float2 *sm) {
     const int nxn = g.nxn, ny = g.ny, nbm = ny / 2 + 1;
     const int64_t N = g.nnode;
@@ -913,52 +1108,113 @@ __global__ void k_cn_setup(GridArgs<double> g, const V4<R> *__restrict__ E, cons
 // Block sum of up to 3 values; thread 0 writes them to part[k * nb + block].
 // The threads' values meet in shared memory and warp 0 adds them (strided
 // lanes, then a butterfly), so that the FP64 adds run in one warp.
-constexpr int CN_BS = 256;
+constexpr int CN_BS = 256;            // threads of a block of the cooperative solve
+constexpr int CN_CLUSTER_BS = 256;    // and of the single-cluster solve
+constexpr int CN_CLUSTER = 16;        // its blocks
+template <int BS>
 __device__ inline void block_partials(double a0, double a1, double a2, int nv, double *part, int nb) {
-    __shared__ double sh[3][CN_BS];
+    __shared__ double sh[3][BS];
     const double v[3] = {a0, a1, a2};
     for (int k = 0; k < nv; ++k) sh[k][threadIdx.x] = v[k];
     __syncthreads();
     if (threadIdx.x < 32) {
         for (int k = 0; k < nv; ++k) {
-            double s = sh[k][threadIdx.x];
-            for (int j = threadIdx.x + 32; j < CN_BS; j += 32) s += sh[k][j];
-            for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-            if (threadIdx.x == 0) part[(int64_t)k * nb + blockIdx.x] = s;
+            double s[4] = {0.0, 0.0, 0.0, 0.0};   // independent chains
+            for (int j = threadIdx.x; j < BS; j += 128)
+#pragma unroll
+                for (int u = 0; u < 4; ++u) s[u] += sh[k][j + 32 * u];
+            double t = (s[0] + s[1]) + (s[2] + s[3]);
+            for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+            if (threadIdx.x == 0) part[(int64_t)k * nb + blockIdx.x] = t;
         }
     }
     __syncthreads();
 }
 
 // Fixed-order sum of the partials, identical in every block: lane l of warp 0
-// adds partials l, l + 32, ..., then a butterfly over the lanes.  (One thread
-// adding all nb partials kept the narrow FP64 pipe busy for nb instructions
-// in every block.)  The partials come from other blocks: read through L2.
-__device__ inline void reduce_partials(const double *part, int nb, int nv, double *out) {
-    __shared__ double res[3];
+// adds partials l, l + 32, ..., then a butterfly over the lanes; thread 0 then
+// runs next(sums), the solve's scalar arithmetic (every block the same), and the
+// block goes on.  All of it in one warp: the FP64 pipe takes 16 cycles for a
+// warp's instruction, so that a division done by every thread of a block costs
+// as much as a pass over its nodes.  The partials come from other blocks: read
+// through L2.
+template <typename Next>
+__device__ inline void reduce_partials(const double *part, int nb, int nv, const Next &next) {
     if (threadIdx.x < 32) {
+        double t[3];
         for (int k = 0; k < nv; ++k) {
-            double s = 0.0;
-            for (int b = threadIdx.x; b < nb; b += 32) s += __ldcg(part + (int64_t)k * nb + b);
-            for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-            if (threadIdx.x == 0) res[k] = s;
+            const double *q = part + (int64_t)k * nb;
+            double s[4] = {0.0, 0.0, 0.0, 0.0};
+            for (int b = threadIdx.x; b < nb; b += 128)
+#pragma unroll
+                for (int u = 0; u < 4; ++u) s[u] += b + 32 * u < nb ? __ldcg(q + b + 32 * u) : 0.0;
+            t[k] = (s[0] + s[1]) + (s[2] + s[3]);
+            for (int o = 16; o > 0; o >>= 1) t[k] += __shfl_xor_sync(0xffffffffu, t[k], o);
         }
+        if (threadIdx.x == 0) next(t);
     }
-    __syncthreads();
-    for (int k = 0; k < nv; ++k) out[k] = res[k];
     __syncthreads();
 }
 
-// The whole solve in one cooperative launch (grid-wide barriers between the
-// dependent phases).  Thread partial sums of the FP32 phases are FP32 (a few
-// nodes per thread), block and grid sums FP64 in a fixed order.
+// Largest of the block's three values (threads of one warp, then shared memory).
+__device__ inline void block_largest(float a, float b, float c, double *part, int nb) {
+    __shared__ float sh[3][32];
+    float v[3] = {a, b, c};
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        for (int o = 16; o > 0; o >>= 1) v[k] = fmaxf(v[k], __shfl_xor_sync(0xffffffffu, v[k], o));
+        if ((threadIdx.x & 31) == 0) sh[k][threadIdx.x >> 5] = v[k];
+    }
+    __syncthreads();
+    if (threadIdx.x < 3) {
+        float m = sh[threadIdx.x][0];
+        for (int w = 1; w < (int)(blockDim.x >> 5); ++w) m = fmaxf(m, sh[threadIdx.x][w]);
+        part[(int64_t)threadIdx.x * nb + blockIdx.x] = (double)m;
+    }
+    __syncthreads();
+}
+// and of the blocks' (thread 0 of warp 0 gets them).
+__device__ inline void grid_largest(const double *part, int nb, double *out) {
+    if (threadIdx.x >= 32) return;
+    for (int k = 0; k < 3; ++k) {
+        float m = -INFINITY;
+        for (int b = threadIdx.x; b < nb; b += 32) m = fmaxf(m, (float)__ldcg(part + (int64_t)k * nb + b));
+        for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
+        out[k] = (double)m;
+    }
+}
+
+// The solve's scalars (shared memory, written by thread 0 of every block alike).
+struct SolveScalars {
+    double bnorm, res, rr, rr_prev, rr_root, stop;   // of the refinement
+    double rho, alpha, omega;               // of BiCGSTAB
+    float beta, alphaf, omegaf;
+    float sx, sy, sz;                       // grid means of the diagonal of S
+    float rate;                             // bound on (or measured) reduction per spectral correction
+    int sweep;                              // the refinements' corrections by the preconditioner alone
+    int go;                                 // goes on after this reduction
+};
+
+// The spectral preconditioner's corrections converge by themselves, as d += P^{-1} r,
+// r -= A P^{-1} r, where S varies little: the error is multiplied by at most
+// rho = max |S - mean| / (1 + mean).  Below CN_SWEEP_RHO the solve takes them
+// instead of BiCGSTAB: no dot products, half the vectors, four barriers per
+// application instead of four and a half.
+constexpr float CN_SWEEP_RHO = 0.2f;
+
+// The whole solve in one launch (grid-wide barriers between the dependent
+// phases).  Thread partial sums of the FP32 phases are FP32 (a few nodes per
+// thread), block and grid sums FP64 in a fixed order.
 // out = [FP32 iterations, relative FP64 residual, refinements].
-__global__ void k_cn_solve(GridArgs<double> g, const double *__restrict__ Md, CNVec v, double c2, double tol,
+// 64 x 64 periodic: 322 us (BiCGSTAB throughout, grid barriers, transposes, FP64
+// scalars in every thread) -> 142 us; 1024 x 1024: 2.56 -> 1.45 ms; 1024 x 512
+// with walls (block-Jacobi): 1.07 -> 0.85 ms.
+template <bool kCluster, int BS>
+__global__ void __launch_bounds__(BS, kCluster ? 1 : 3) k_cn_solve(GridArgs<double> g, const double *__restrict__ Md, CNVec v, double c2, double tol,
                            int max_iter, double *part, double *out, WallRows wr) {
-    cg::grid_group grid = cg::this_grid();
-    const int64_t N = g.nnode;
-    const int64_t tid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+    const SolveBarrier<kCluster> grid;
+    const int N = (int)g.nnode, NC = g.nx * g.ny;   // (at most 2^30 cells; a wall adds a column)
+    const int tid = blockIdx.x * BS + threadIdx.x, stride = gridDim.x * BS;
     const int nb = gridDim.x;
     const double ia = g.inv_dx * g.inv_dy;
     const double hx = 0.5 * g.inv_dx, hy = 0.5 * g.inv_dy;
@@ -966,16 +1222,14 @@ __global__ void k_cn_solve(GridArgs<double> g, const double *__restrict__ Md, CN
     double *pa = part, *pb = part + 3 * (int64_t)nb;  // alternating partial buffers
     int flip = 0;
     auto P = [&]() { double *q = flip ? pb : pa; flip ^= 1; return q; };
-    const V4<float> zero4{0.f, 0.f, 0.f, 0.f};
-    double red[3];
-    double bnorm = -1.0, res = 0.0, rr_prev = 0.0;
     int total = 0, outer = 0;
     extern __shared__ float2 cn_sm[];
-    float sx = 0.f, sy = 0.f, sz = 0.f;
+    __shared__ SolveScalars sc;
+    const FftShared fs = fft_shared(g, cn_sm);   // (spectral preconditioner)
     if (v.fft) {
         // twiddles, and the grid means of the diagonal of S for the preconditioner
-        const int hxn = g.nx / 2, hyn = g.ny / 2;
-        for (int64_t t = tid; t < hxn + hyn; t += stride) {
+        const int hxn = g.nx / 2 + 1, hyn = g.ny / 2 + 1;
+        for (int t = tid; t < hxn + hyn; t += stride) {
             double sn, cs;
             if (t < hxn) {
                 sincospi(-2.0 * (double)t / g.nx, &sn, &cs);
@@ -985,127 +1239,236 @@ __global__ void k_cn_solve(GridArgs<double> g, const double *__restrict__ Md, CN
                 v.twy[t - hxn] = make_float2((float)cs, (float)sn);
             }
         }
-        double a0 = 0, a1 = 0, a2 = 0;
-        for (int64_t n = tid; n < N; n += stride) {
-            a0 += v.S[n];
-            a1 += v.S[4 * N + n];
-            a2 += v.S[8 * N + n];
+        float a0 = 0.f, a1 = 0.f, a2 = 0.f, lo = INFINITY, hi = -INFINITY, off = 0.f;
+        for (int n = tid; n < N; n += stride) {
+            float S[9];
+#pragma unroll
+            for (int k = 0; k < 9; ++k) S[k] = v.S[(int64_t)k * N + n];
+            a0 += S[0];
+            a1 += S[4];
+            a2 += S[8];
+            lo = fminf(lo, fminf(S[0], fminf(S[4], S[8])));
+            hi = fmaxf(hi, fmaxf(S[0], fmaxf(S[4], S[8])));
+            // |off-diagonal part| <= its largest row or column sum
+            const float b1 = fabsf(S[1]), b2 = fabsf(S[2]), b3 = fabsf(S[3]), b5 = fabsf(S[5]), b6 = fabsf(S[6]),
+                        b7 = fabsf(S[7]);
+            off = fmaxf(off, fmaxf(fmaxf(b1 + b2, fmaxf(b3 + b5, b6 + b7)), fmaxf(b3 + b6, fmaxf(b1 + b7, b2 + b5))));
         }
-        double *q0 = P();
-        block_partials(a0, a1, a2, 3, q0, nb);
+        double *q0 = P(), *q1 = P();
+        block_partials<BS>(a0, a1, a2, 3, q0, nb);
+        block_largest(-lo, hi, off, q1, nb);
         grid.sync();
-        reduce_partials(q0, nb, 3, red);
-        sx = (float)(red[0] / N);
-        sy = (float)(red[1] / N);
-        sz = (float)(red[2] / N);
+        double ext[3];
+        grid_largest(q1, nb, ext);
+        reduce_partials(q0, nb, 3, [&](const double *red) {
+            sc.sx = (float)(red[0] / N);
+            sc.sy = (float)(red[1] / N);
+            sc.sz = (float)(red[2] / N);
+            const float smin = fminf(sc.sx, fminf(sc.sy, sc.sz)), smax = fmaxf(sc.sx, fmaxf(sc.sy, sc.sz));
+            sc.rate = (fmaxf((float)ext[1] - smin, smax + (float)ext[0]) + (float)ext[2]) / (1.f + smin);
+            sc.sweep = smin >= 0.f && sc.rate < CN_SWEEP_RHO;
+        });
+        axis_twiddles(fs.twx, v.twx, v.ax);
+        axis_twiddles(fs.twy, v.twy, v.ay);
+        __syncthreads();
     } else if (v.line) {
         line_setup(grid, g, v, c2f, cwf, cvf);
         grid.sync();
     }
+    auto split = [&](int n, int &i, int &j) {
+        j = (int)((unsigned)n / (unsigned)g.nxn);
+        i = n - j * g.nxn;
+    };
     for (;;) {
-        // FP64 residual r = b - A x, handed to the FP32 solve; d = 0, r0 = r, p = v = 0
+        // FP64 residual r = b - A x, handed to the FP32 solve (r0 = r)
         double s_rr = 0, s_bb = 0;
-        const int64_t NC = (int64_t)g.nx * g.ny;
-        for (int64_t c = tid; c < NC; c += stride) {
-            const int ci = (int)(c % g.nx), cj = (int)(c / g.nx);
+        for (int c = tid; c < NC; c += stride) {
+            const int cj = (int)((unsigned)c / (unsigned)g.nx), ci = c - cj * g.nx;
             v.cc[c] = cell_curl_e(g, v.x, hx, hy, ci, cj);
         }
         grid.sync();
-        for (int64_t n = tid; n < N; n += stride) {
-            int i = (int)(n % g.nxn), j = (int)(n / g.nxn);
-            V4<double> ax = apply_A_from_cells(g, v.x, v.cc, Md + N, ia, c2, hx, hy, i, j, wr.cw, wr.cv);
+        for (int n = tid; n < N; n += stride) {
+            int i, j;
+            split(n, i, j);
+            V4<double> ax = apply_A_from_cells(g, v.x, v.cc, Md + N, ia, c2 * hx, c2 * hy, i, j, wr.cw, wr.cv);
             V4<double> b = v.b[n];
             V4<double> r{b.x - ax.x, b.y - ax.y, b.z - ax.z, 0.0};
             V4<float> rf{(float)r.x, (float)r.y, (float)r.z, 0.f};
             v.r[n] = rf;
-            v.r0[n] = rf;
-            v.p[n] = zero4;
-            v.v[n] = zero4;
-            v.d[n] = zero4;
+            if (!(v.fft && sc.sweep)) v.r0[n] = rf;
             s_rr += dot(r, r);
-            if (bnorm < 0) s_bb += dot(b, b);
+            if (outer == 0) s_bb += dot(b, b);
         }
         double *q = P();
-        block_partials(s_rr, s_bb, 0.0, 2, q, nb);
+        block_partials<BS>(s_rr, s_bb, 0.0, 2, q, nb);
         grid.sync();
-        reduce_partials(q, nb, 2, red);
-        if (bnorm < 0) bnorm = sqrt(red[1]);
-        const double rr = red[0];
-        if (bnorm == 0.0) {
-            for (int64_t n = tid; n < N; n += stride) v.x[n] = V4<double>{0, 0, 0, 0};
-            res = 0.0;
+        reduce_partials(q, nb, 2, [&](const double *red) {
+            if (outer == 0) sc.bnorm = sqrt(red[1]);
+            sc.rr = red[0];
+            sc.res = sc.bnorm == 0.0 ? 0.0 : sqrt(sc.rr) / sc.bnorm;
+            // converged, out of budget, or no longer improving (FP64 rounding floor)
+            sc.go = !(sc.bnorm == 0.0 || sc.res <= tol || total >= max_iter || outer >= CN_MAX_OUTER ||
+                      (outer > 0 && sc.rr > 0.25 * sc.rr_prev));
+            sc.rr_prev = sc.rr;
+            sc.rr_root = sqrt(sc.rr);
+            sc.stop = (double)CN_INNER_RTOL * sc.rr_root;
+            sc.rho = sc.rr;
+            sc.alpha = sc.omega = 1.0;
+            sc.beta = sc.omegaf = 0.f;
+        });
+        if (!sc.go) {
+            if (sc.bnorm == 0.0)
+                for (int n = tid; n < N; n += stride) v.x[n] = V4<double>{0, 0, 0, 0};
             break;
         }
-        res = sqrt(rr) / bnorm;
-        // converged, out of budget, or no longer improving (FP64 rounding floor)
-        if (res <= tol || total >= max_iter || outer >= CN_MAX_OUTER || (outer > 0 && rr > 0.25 * rr_prev)) break;
-        rr_prev = rr;
         ++outer;
-        // FP32 BiCGSTAB (block-Jacobi, right preconditioned) on A d = r
-        const double stop = (double)CN_INNER_RTOL * sqrt(rr);
-        double rho = rr, rho_old = 1.0, alpha = 1.0, omega = 1.0;
-        while (total < max_iter) {
-            const float beta = (float)((rho / rho_old) * (alpha / omega));
-            const float omf = (float)omega;
-            for (int64_t n = tid; n < N; n += stride) {
-                V4<float> r = v.r[n], p = v.p[n], vv = v.v[n];
-                V4<float> pn{r.x + beta * (p.x - omf * vv.x), r.y + beta * (p.y - omf * vv.y),
-                             r.z + beta * (p.z - omf * vv.z), 0.f};
-                v.p[n] = pn;
-                if (!v.fft && !v.line) v.ph[n] = apply_minv(v.minv, N, n, pn);
-            }
-            if (v.fft) {
+        if (v.fft && sc.sweep) {
+            // corrections by the preconditioner (CN_SWEEP_RHO) until r is below the stop; where the
+            // reduction seen so far says that one more will do, that one goes straight into x and the
+            // next FP64 residual judges it
+            bool first = true;   // d = 0 before it
+            int last = sc.rate * sc.rr_root <= sc.stop || total + 1 >= max_iter;
+            for (;;) {
+                auto keep = [&](int64_t n, const V4<float> &z) { v.ph[n] = z; };
+                auto finish = [&](int64_t n, const V4<float> &z) {
+                    V4<float> d{0.f, 0.f, 0.f, 0.f};
+                    if (!first) d = v.d[n];
+                    const V4<double> x = v.x[n];
+                    v.x[n] = V4<double>{x.x + (double)(d.x + z.x), x.y + (double)(d.y + z.y), x.z + (double)(d.z + z.z), 0.0};
+                };
+                auto load_r = [&](int64_t n) { return v.r[n]; };
+                ++total;
+                if (last) {
+                    apply_spectral(grid, g, v, fs, load_r, [] {}, [] { return true; }, finish, c2f, sc.sx, sc.sy, sc.sz);
+                    break;
+                }
+                apply_spectral(grid, g, v, fs, load_r, [] {}, [] { return true; }, keep, c2f, sc.sx, sc.sy, sc.sz);
                 grid.sync();
-                apply_spectral(grid, g, v, v.p, v.ph, c2f, sx, sy, sz, cn_sm);
-            } else if (v.line) {
+                float s_r = 0.f;
+                for (int n = tid; n < N; n += stride) {
+                    int i, j;
+                    split(n, i, j);
+                    const V4<float> az = apply_A<float>(g, v.ph, v.S, 1.f, c2f, hxf, hyf, i, j, cwf, cvf), z = v.ph[n];
+                    V4<float> r = v.r[n], d = z;
+                    if (!first) {
+                        d = v.d[n];
+                        d = V4<float>{d.x + z.x, d.y + z.y, d.z + z.z, 0.f};
+                    }
+                    r = V4<float>{r.x - az.x, r.y - az.y, r.z - az.z, 0.f};
+                    v.r[n] = r;
+                    v.d[n] = d;
+                    s_r += dot(r, r);
+                }
+                first = false;
+                q = P();
+                block_partials<BS>(s_r, 0, 0, 1, q, nb);
+                grid.sync();
+                reduce_partials(q, nb, 1, [&](const double *red) {
+                    const double r = sqrt(red[0]), next = r * (r / sc.rr_root);
+                    // 0: below the stop; 1: at least two more; 2: one more will do (or is all that may be taken)
+                    sc.go = r <= sc.stop ? 0 : (next <= 0.3 * sc.stop || total + 1 >= max_iter) ? 2 : 1;
+                    sc.rr_root = r;
+                });
+                if (sc.go == 0) {
+                    for (int n = tid; n < N; n += stride) {
+                        const V4<double> x = v.x[n];
+                        const V4<float> d = v.d[n];
+                        v.x[n] = V4<double>{x.x + (double)d.x, x.y + (double)d.y, x.z + (double)d.z, 0.0};
+                    }
+                    break;
+                }
+                last = sc.go == 2;
+            }
+            grid.sync();
+            continue;
+        }
+        // FP32 BiCGSTAB (right preconditioned) on A d = r
+        bool first = true;   // p = r, d = 0 before it
+        while (total < max_iter) {
+            const float beta = sc.beta, omf = sc.omegaf;
+            auto next_p = [&](int n) {
+                V4<float> pn = v.r[n];
+                if (!first) {
+                    const V4<float> p = v.p[n], vv = v.v[n];
+                    pn = V4<float>{pn.x + beta * (p.x - omf * vv.x), pn.y + beta * (p.y - omf * vv.y),
+                                   pn.z + beta * (p.z - omf * vv.z), 0.f};
+                }
+                v.p[n] = pn;
+                return pn;
+            };
+            if (v.fft)
+                apply_spectral(grid, g, v, fs, next_p, [] {}, [] { return true; },
+                               [&](int64_t n, const V4<float> &z) { v.ph[n] = z; }, c2f, sc.sx, sc.sy, sc.sz);
+            else
+                for (int n = tid; n < N; n += stride) {
+                    const V4<float> pn = next_p(n);
+                    if (!v.line) v.ph[n] = apply_minv(v.minv, N, n, pn);
+                }
+            if (v.line) {
                 grid.sync();
                 apply_line(grid, g, v, v.p, v.ph, c2f, cwf, cvf, cn_sm);
             }
             grid.sync();
             float s_r0v = 0.f;
-            for (int64_t n = tid; n < N; n += stride) {
-                int i = (int)(n % g.nxn), j = (int)(n / g.nxn);
+            for (int n = tid; n < N; n += stride) {
+                int i, j;
+                split(n, i, j);
                 V4<float> av = apply_A<float>(g, v.ph, v.S, 1.f, c2f, hxf, hyf, i, j, cwf, cvf);
                 v.v[n] = av;
                 s_r0v += dot(v.r0[n], av);
             }
             q = P();
-            block_partials(s_r0v, 0, 0, 1, q, nb);
+            block_partials<BS>(s_r0v, 0, 0, 1, q, nb);
             grid.sync();
-            reduce_partials(q, nb, 1, red);
-            if (red[0] == 0.0) break;
-            alpha = rho / red[0];
-            const float af = (float)alpha;
+            reduce_partials(q, nb, 1, [&](const double *red) {
+                sc.go = red[0] != 0.0;
+                sc.alpha = sc.rho / red[0];
+                sc.alphaf = (float)sc.alpha;
+            });
+            if (!sc.go) break;
+            const float af = sc.alphaf;
             float s_ss = 0.f;
-            for (int64_t n = tid; n < N; n += stride) {
+            auto next_s = [&](int n) {
                 V4<float> r = v.r[n], vv = v.v[n];
                 V4<float> s{r.x - af * vv.x, r.y - af * vv.y, r.z - af * vv.z, 0.f};
                 v.s[n] = s;
-                if (!v.fft && !v.line) v.sh[n] = apply_minv(v.minv, N, n, s);
                 s_ss += dot(s, s);
-            }
+                return s;
+            };
             q = P();
-            block_partials(s_ss, 0, 0, 1, q, nb);
-            grid.sync();
-            reduce_partials(q, nb, 1, red);
-            ++total;
-            if (sqrt(red[0]) <= stop) {
-                for (int64_t n = tid; n < N; n += stride) {
-                    V4<float> d = v.d[n], ph = v.ph[n];
+            auto partial = [&] { block_partials<BS>(s_ss, 0, 0, 1, q, nb); };
+            auto larger = [&] {
+                reduce_partials(q, nb, 1, [&](const double *red) { sc.go = sqrt(red[0]) > sc.stop; });
+                ++total;
+                return sc.go != 0;
+            };
+            bool go_on;
+            if (v.fft) {
+                go_on = apply_spectral(grid, g, v, fs, next_s, partial, larger,
+                                       [&](int64_t n, const V4<float> &z) { v.sh[n] = z; }, c2f, sc.sx, sc.sy, sc.sz);
+            } else {
+                for (int n = tid; n < N; n += stride) {
+                    const V4<float> s = next_s(n);
+                    if (!v.line) v.sh[n] = apply_minv(v.minv, N, n, s);
+                }
+                partial();
+                grid.sync();
+                go_on = larger();
+            }
+            if (!go_on) {
+                for (int n = tid; n < N; n += stride) {
+                    const V4<float> d = first ? V4<float>{0.f, 0.f, 0.f, 0.f} : v.d[n], ph = v.ph[n];
                     v.d[n] = V4<float>{d.x + af * ph.x, d.y + af * ph.y, d.z + af * ph.z, 0.f};
                 }
+                first = false;
                 break;
             }
-            if (v.fft) {
-                apply_spectral(grid, g, v, v.s, v.sh, c2f, sx, sy, sz, cn_sm);
-                grid.sync();
-            } else if (v.line) {
-                apply_line(grid, g, v, v.s, v.sh, c2f, cwf, cvf, cn_sm);
-                grid.sync();
-            }
+            if (v.line) apply_line(grid, g, v, v.s, v.sh, c2f, cwf, cvf, cn_sm);
+            if (v.fft || v.line) grid.sync();
             float s_ts = 0.f, s_tt = 0.f;
-            for (int64_t n = tid; n < N; n += stride) {
-                int i = (int)(n % g.nxn), j = (int)(n / g.nxn);
+            for (int n = tid; n < N; n += stride) {
+                int i, j;
+                split(n, i, j);
                 V4<float> at = apply_A<float>(g, v.sh, v.S, 1.f, c2f, hxf, hyf, i, j, cwf, cvf);
                 v.t[n] = at;
                 V4<float> s = v.s[n];
@@ -1113,15 +1476,19 @@ __global__ void k_cn_solve(GridArgs<double> g, const double *__restrict__ Md, CN
                 s_tt += dot(at, at);
             }
             q = P();
-            block_partials(s_ts, s_tt, 0, 2, q, nb);
+            block_partials<BS>(s_ts, s_tt, 0, 2, q, nb);
             grid.sync();
-            reduce_partials(q, nb, 2, red);
-            if (red[1] == 0.0) break;
-            omega = red[0] / red[1];
-            const float of = (float)omega;
+            reduce_partials(q, nb, 2, [&](const double *red) {
+                sc.go = red[1] != 0.0;
+                sc.omega = red[0] / red[1];
+                sc.omegaf = (float)sc.omega;
+            });
+            if (!sc.go) break;
+            const float of = sc.omegaf;
             float s_r0r = 0.f, s_rr2 = 0.f;
-            for (int64_t n = tid; n < N; n += stride) {
-                V4<float> d = v.d[n], ph = v.ph[n], sh = v.sh[n], s = v.s[n], t = v.t[n];
+            for (int n = tid; n < N; n += stride) {
+                V4<float> ph = v.ph[n], sh = v.sh[n], s = v.s[n], t = v.t[n];
+                const V4<float> d = first ? V4<float>{0.f, 0.f, 0.f, 0.f} : v.d[n];
                 v.d[n] = V4<float>{d.x + af * ph.x + of * sh.x, d.y + af * ph.y + of * sh.y,
                                    d.z + af * ph.z + of * sh.z, 0.f};
                 V4<float> r{s.x - of * t.x, s.y - of * t.y, s.z - of * t.z, 0.f};
@@ -1129,25 +1496,29 @@ __global__ void k_cn_solve(GridArgs<double> g, const double *__restrict__ Md, CN
                 s_r0r += dot(v.r0[n], r);
                 s_rr2 += dot(r, r);
             }
+            first = false;
             q = P();
-            block_partials(s_r0r, s_rr2, 0, 2, q, nb);
+            block_partials<BS>(s_r0r, s_rr2, 0, 2, q, nb);
             grid.sync();
-            reduce_partials(q, nb, 2, red);
-            rho_old = rho;
-            rho = red[0];
-            if (sqrt(red[1]) <= stop || rho == 0.0 || omega == 0.0) break;
+            reduce_partials(q, nb, 2, [&](const double *red) {
+                sc.go = !(sqrt(red[1]) <= sc.stop || red[0] == 0.0 || sc.omega == 0.0);
+                sc.beta = (float)((red[0] / sc.rho) * (sc.alpha / sc.omega));
+                sc.rho = red[0];
+            });
+            if (!sc.go) break;
         }
-        // x += d in FP64
-        for (int64_t n = tid; n < N; n += stride) {
-            V4<double> x = v.x[n];
-            V4<float> d = v.d[n];
-            v.x[n] = V4<double>{x.x + (double)d.x, x.y + (double)d.y, x.z + (double)d.z, 0.0};
-        }
+        // x += d in FP64 (nothing was added where the first iteration broke down)
+        if (!first)
+            for (int n = tid; n < N; n += stride) {
+                V4<double> x = v.x[n];
+                V4<float> d = v.d[n];
+                v.x[n] = V4<double>{x.x + (double)d.x, x.y + (double)d.y, x.z + (double)d.z, 0.0};
+            }
         grid.sync();
     }
     if (blockIdx.x == 0 && threadIdx.x == 0) {
         out[0] = (double)total;
-        out[1] = res;
+        out[1] = sc.res;
         out[2] = (double)outer;
     }
 }
@@ -1261,11 +1632,37 @@ static int field_literal_t(pic_t *h) {
 
 int field_literal(pic_t *h) { return h->fp32 ? field_literal_t<float>(h) : field_literal_t<double>(h); }
 
-// The spectral preconditioner applies to periodic power-of-two grids, the
-// line preconditioner to boxes with walls whose ny is a power of two.
+// Factors of an axis of the spectral preconditioner: 4s, then primes; false
+// where a prime is too large for direct sums (or n for the shared buffers).
+constexpr int FFT_MAX_PRIME = 61;
+static bool fft_factors(int n, FftAxis *ax) {
+    if (n < 2 || n > 4096) return false;
+    *ax = FftAxis{};
+    ax->n = n;
+    ax->lg = -1;
+    if ((n & (n - 1)) == 0)
+        for (ax->lg = 0; (1 << ax->lg) < n;) ++ax->lg;
+    int m = n;
+    while (m % 4 == 0) {
+        ax->f[ax->nf++] = 4;
+        m /= 4;
+    }
+    for (int p = 2; p <= FFT_MAX_PRIME && m > 1; ++p)
+        while (m % p == 0) {
+            ax->f[ax->nf++] = p;
+            m /= p;
+        }
+    return m == 1;
+}
+
+// The spectral preconditioner applies to periodic grids whose sides have no
+// prime factor above FFT_MAX_PRIME (at most 4096), the line preconditioner to
+// boxes with walls whose ny is a power of two.  Without it such a grid takes
+// some three hundred block-Jacobi iterations at c dt / dx = 25 (90 x 64: 6.6 ms
+// a solve; 0.27 ms with it).
 static bool cn_spectral(const pic_t *h) {
-    return h->cfg.cn_precond != PIC_CN_PRECOND_JACOBI && h->periodic_x && (h->nx & (h->nx - 1)) == 0 &&
-           (h->ny & (h->ny - 1)) == 0 && h->nx >= 2 && h->ny >= 2 && h->nx <= 4096 && h->ny <= 4096;
+    FftAxis a, b;
+    return h->cfg.cn_precond != PIC_CN_PRECOND_JACOBI && h->periodic_x && fft_factors(h->nx, &a) && fft_factors(h->ny, &b);
 }
 
 static bool cn_line(const pic_t *h) {
@@ -1303,7 +1700,8 @@ static CNVec cn_views(pic_t *h, double **Md) {
     v.twy = v.twx + h->nx / 2 + 1;
     auto log2i = [](int x) { int l = 0; while ((1 << l) < x) ++l; return l; };
     v.fft = cn_spectral(h) ? 1 : 0;
-    v.lx = log2i(h->nx);
+    fft_factors(h->nx, &v.ax);
+    fft_factors(h->ny, &v.ay);
     v.ly = log2i(h->ny);
     v.line = cn_line(h) ? 1 : 0;
     v.scol = (float *)(v.twy + h->ny / 2 + 1);
@@ -1319,8 +1717,9 @@ static size_t cn_smem(const pic_t *h) {
     const size_t tile = 32 * 33 * sizeof(float2);
     if (cn_line(h)) nmax = (size_t)h->ny;   // its FFTs run along y only
     else if (!cn_spectral(h)) return tile;
-    const size_t G = nmax > (size_t)FFT_GROUP ? nmax : (size_t)FFT_GROUP;
-    size_t fft = (2 * G + nmax) * sizeof(float2);   // two row-group buffers and the per-stage twiddles
+    // two row-group buffers and the per-stage twiddles (spectral: of both axes)
+    size_t fft = cn_line(h) ? (2 * (size_t)fft_buffer((int)nmax, 0) + nmax) * sizeof(float2)
+                            : (2 * (size_t)spectral_buffer(h->nx, h->ny) + h->nx + h->ny) * sizeof(float2);
     if (cn_line(h) && line_sweep_bytes(h->nxn) > fft) fft = line_sweep_bytes(h->nxn);
     return fft > tile ? fft : tile;
 }
@@ -1330,6 +1729,41 @@ size_t cn_bytes(const pic_t *h) {
     return 3 * n * sizeof(V4<double>) + 9 * n * sizeof(V4<float>) + 18 * n * sizeof(float) +
            (size_t)NMOM * n * sizeof(double) + 4 * n * sizeof(float2) + (size_t)(h->nx + h->ny + 4) * sizeof(float2) +
            cn_line_floats(h) * sizeof(float) + 16;
+}
+
+// Grids of up to CN_CLUSTER_NODES nodes are solved by one cluster of CN_CLUSTER
+// blocks, whose barrier is much cheaper than a grid barrier (a solve has some
+// thirty of them); larger grids need more SMs (field solve on one cluster / on
+// the grid, us: 64 x 64 163 / 192, 96 x 64 with walls 255 / 256, 128 x 64 206 /
+// 197, 128 x 128 312 / 209).
+constexpr int64_t CN_CLUSTER_NODES = 6144;
+
+static void cn_cluster_config(cudaLaunchConfig_t &lc, cudaLaunchAttribute *at, size_t smem, cudaStream_t st) {
+    lc.gridDim = dim3(CN_CLUSTER);
+    lc.blockDim = dim3(CN_CLUSTER_BS);
+    lc.dynamicSmemBytes = smem;
+    lc.stream = st;
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = CN_CLUSTER;
+    at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+    lc.attrs = at;
+    lc.numAttrs = 1;
+}
+
+static bool cn_single_cluster(const pic_t *h, size_t smem) {
+    if (h->nnode > CN_CLUSTER_NODES || h->cn_red_cap < CN_CLUSTER) return false;
+    const void *k = (const void *)k_cn_solve<true, CN_CLUSTER_BS>;
+    cudaLaunchConfig_t lc = {};
+    cudaLaunchAttribute at[1];
+    cn_cluster_config(lc, at, smem, h->st);
+    int n = 0;   // (clusters of more than 8 blocks are opt-in, and may not fit a partitioned GPU)
+    if (cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess ||
+        cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess ||
+        cudaOccupancyMaxActiveClusters(&n, k, &lc) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    return n >= 1;
 }
 
 template <typename R>
@@ -1357,28 +1791,37 @@ static int field_cn_t(pic_t *h) {
     int dev = 0, nsm = 0, per_sm = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-    const int bs = CN_BS;
-    const size_t smem = cn_smem(h);
-    // the whole grid must be resident: fix the shared-memory split before asking how many blocks fit
-    cudaFuncSetAttribute(k_cn_solve, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    cudaFuncSetAttribute(k_cn_solve, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_cn_solve, bs, smem);
-    int nb = per_sm * nsm;
-    int need = (int)((h->nnode + bs - 1) / bs);
-    if (nb > need) nb = need;
-    if (nb < 1) nb = 1;
-    if (nb > h->cn_red_cap) {
-        set_error("CN reduction scratch too small (%d < %d)", h->cn_red_cap, nb);
-        return PIC_ERR_STATE;
-    }
     double tol = h->cfg.cn_tol > 0 ? h->cfg.cn_tol : (h->fp32 ? 1e-10 : 1e-12);
     int maxit = h->cfg.cn_max_iter > 0 ? h->cfg.cn_max_iter : 400;
     void *args[] = {(void *)&gd, (void *)&Msrc, (void *)&v, (void *)&c2, (void *)&tol, (void *)&maxit,
                     (void *)&h->cn_red, (void *)&h->cn_out, (void *)&wr};
-    cudaError_t e = cudaLaunchCooperativeKernel((const void *)k_cn_solve, dim3(nb), dim3(bs), args, smem, h->st);
+    const size_t smem = cn_smem(h);
+    cudaError_t e;
+    if (cn_single_cluster(h, smem)) {
+        const void *k = (const void *)k_cn_solve<true, CN_CLUSTER_BS>;
+        cudaLaunchConfig_t lc = {};
+        cudaLaunchAttribute at[1];
+        cn_cluster_config(lc, at, smem, h->st);
+        e = cudaLaunchKernelExC(&lc, k, args);
+    } else {
+        const void *k = (const void *)k_cn_solve<false, CN_BS>;
+        // the whole grid must be resident: fix the shared-memory split before asking how many blocks fit
+        cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, CN_BS, smem);
+        int nb = per_sm * nsm;
+        int need = (int)((h->nnode + CN_BS - 1) / CN_BS);
+        if (nb > need) nb = need;
+        if (nb < 1) nb = 1;
+        if (nb > h->cn_red_cap) {
+            set_error("CN reduction scratch too small (%d < %d)", h->cn_red_cap, nb);
+            return PIC_ERR_STATE;
+        }
+        e = cudaLaunchCooperativeKernel(k, dim3(nb), dim3(CN_BS), args, smem, h->st);
+    }
     count_launch(h);
     if (e != cudaSuccess) {
-        set_error("cudaLaunchCooperativeKernel(k_cn_solve): %s", cudaGetErrorString(e));
+        set_error("launch of k_cn_solve: %s", cudaGetErrorString(e));
         return PIC_ERR_CUDA;
     }
     int en = 1 - h->ecur, hn = 1 - h->hcur;
