@@ -337,7 +337,8 @@ static int redeposit(pic_t *h) {
     for (int s = 0; s < h->nsp; ++s)
         if (int rc = deposit_only(h, s)) return rc;
     h->moments_stale = false;
-    return h->det ? fix_to_moments(h) : cell_moments(h, true);
+    if (int rc = rest_touch(h)) return rc;
+    return h->det ? fix_to_moments(h) : cell_moments(h);
 }
 
 // The previous step's regroup, then the moments at rest if a load or a field
@@ -869,7 +870,8 @@ static int load_impl(pic_t *h, int nload, const int *species, const pic_species_
         cudaEventRecord(h->ev_sorts, h->st3);
         cudaStreamWaitEvent(h->st2, h->ev_sorts, 0);
         h->st = h->st2;
-        if (!rc && eager) rc = h->det ? fix_to_moments(h) : cell_moments(h, true);
+        if (!rc && eager) rc = rest_touch(h);
+        if (!rc && eager) rc = h->det ? fix_to_moments(h) : cell_moments(h);
         h->st = main_st;
     }
     if (fresh) {
@@ -1312,14 +1314,6 @@ static int step_deposit(pic_t *h, int p, const int32_t *guard) {
     return 0;
 }
 
-// Field solve of the time-centred mode, node B of the new H, ghost rings.
-static int field_cn_step(pic_t *h) {
-    int rc = field_cn(h);
-    if (!rc) rc = node_average(h, 1 - h->hcur, 1 - h->bcur);
-    if (!rc) rc = fill_ghosts(h, h->Ehalf);
-    return rc;
-}
-
 extern "C" PIC_API int pic_step(pic_t *h, int nsteps) {
     if (!h || nsteps < 0) {
         set_error("pic_step: bad handle or step count");
@@ -1345,8 +1339,6 @@ extern "C" PIC_API int pic_step(pic_t *h, int nsteps) {
         timing_begin(h);
         int64_t l0 = h->timing.launches[4];
         int rc = overlap ? field_literal(h) : field_cn(h);
-        if (!rc) rc = node_average(h, 1 - h->hcur, 1 - h->bcur);
-        if (!rc) rc = fill_ghosts(h, h->Ehalf);
         if (!rc) timing_end(h, 2, (int)(h->timing.launches[4] - l0));
         if (overlap) {
             // whatever the handle's stream runs next (the push, a rebuild, or the next call after an
@@ -1388,7 +1380,7 @@ extern "C" PIC_API int pic_step(pic_t *h, int nsteps) {
                 if (h->post) {
                     // nor were that step's moments deposited: this step's field solve again from them
                     if ((rc = redeposit(h))) return rc;
-                    if ((rc = field_cn_step(h))) return rc;
+                    if ((rc = field_cn(h))) return rc;
                     if ((rc = clear_step_moments(h))) return rc;
                 }
                 if ((rc = step_reset(h, p, true))) return rc;
@@ -1508,8 +1500,6 @@ extern "C" PIC_API int pic_batch_step(pic_batch *p, pic_t **hs, int n, int nstep
         for (int r = 0; r < n; ++r) {
             pic_t *h = hs[r];
             int rc = (h->cfg.field_mode == PIC_FIELD_LITERAL) ? field_literal(h) : field_cn(h);
-            if (!rc) rc = node_average(h, 1 - h->hcur, 1 - h->bcur);
-            if (!rc) rc = fill_ghosts(h, h->Ehalf);
             if (rc) return rc;
         }
         for (int r = 0; r < n; ++r) {

@@ -76,180 +76,212 @@ __device__ inline void clear_node_moments(const GridArgs<R> &g, const TouchArgs<
     }
 }
 
+// A padded node's value with its images in the ghost ring: periodic copies in y
+// (and x when periodic); beyond a wall the ring stays zero.
 template <typename R>
-__global__ void k_field_E_literal(GridArgs<R> g, const V4<R> *__restrict__ E, const V4<R> *__restrict__ H,
-                                  const R *M, const R *Mlo, V4<R> *__restrict__ Enew,
-                                  V4<R> *__restrict__ Ehalf, TouchArgs<R> tm) {
-    int i = blockIdx.x * blockDim.x + threadIdx.x;
-    int j = blockIdx.y;
-    if (i >= g.nxn || j >= g.ny) return;
-    const int64_t node = (int64_t)j * g.nxn + i;
-    const bool touched = !tm.touched || tm.touched[(j / tm.tny) * tm.ntx + min(i / tm.tnx, tm.ntx - 1)];
-    if (!g.periodic_x && (i == 0 || i == g.nx)) {   // wall columns: k_field_walls (their moments are not read)
-        if (tm.clr && touched) clear_node_moments(g, tm, node);
-        return;
-    }
-    R cu, cvv, sy, sx;
-    curl_h_parts(g, H, i, j, cu, cvv, sy, sx);
-    const R cx = cu * g.hy, cy = cvv * g.hx, cz = fma(sy, g.hx, -(sx * g.hy));
-    V4<R> e = E[node];
-    {
-        if (!touched) {
-            // vacuum (S = 0, dj = 0 on every node of the tile): Eq. 4 reduces to E^{n+1} = E^n + dt curl_h H,
-            // with no moment read and no 3x3 solve.  The same operations as the solve below on such a node
-            // (where the 3x3 solve returns its right-hand side exactly), so a node's bits do not depend on
-            // whether its tile was marked.
-            const R zx = fma(g.dt, cx, e.x), zy = fma(g.dt, cy, e.y), zz = fma(g.dt, cz, e.z);
-            Enew[node] = V4<R>{zx, zy, zz, R(0)};
-            Ehalf[pidx(g, i, j)] = V4<R>{R(0.5) * (e.x + zx), R(0.5) * (e.y + zy), R(0.5) * (e.z + zz), R(0)};
-            return;
+__device__ inline void store_padded(V4<R> *__restrict__ F, const GridArgs<R> &g, int i, int j, const V4<R> &v) {
+    F[pidx(g, i, j)] = v;
+    const bool edge_y = j < g.G || j >= g.ny - g.G, edge_x = g.periodic_x && (i < g.G || i >= g.nxn - g.G);
+    if (!edge_y && !edge_x) return;
+    int j0 = j, i0 = i;   // the first images inside the ring
+    while (j0 - g.ny >= -g.G) j0 -= g.ny;
+    if (g.periodic_x)
+        while (i0 - g.nxn >= -g.G) i0 -= g.nxn;
+    for (int jj = j0; jj < g.ny + g.G; jj += g.ny)
+        for (int ii = i0; ii < g.nxn + g.G; ii += g.nxn) {
+            F[pidx(g, ii, jj)] = v;
+            if (!g.periodic_x) break;
         }
-    }
-    R ia = g.inv_dx * g.inv_dy;
-    R a[9], r[3], z[3];
-    R ev[3] = {e.x, e.y, e.z};
-    R cv[3] = {cx, cy, cz};
-#pragma unroll
-    for (int row = 0; row < 3; ++row) {
-        R s_e = R(0);
-#pragma unroll
-        for (int col = 0; col < 3; ++col) {
-            const int64_t mi = (int64_t)(1 + 3 * row + col) * g.nnode + node;
-            R S = (Mlo ? M[mi] + Mlo[mi] : M[mi]) * ia;
-            a[3 * row + col] = (row == col ? R(1) : R(0)) + S;
-            s_e += ((row == col ? R(1) : R(0)) - S) * ev[col];
-        }
-        const int64_t ji = (int64_t)(10 + row) * g.nnode + node;
-        r[row] = fma(g.dt, cv[row] - (Mlo ? M[ji] + Mlo[ji] : M[ji]) * ia, s_e);
-    }
-    if (tm.clr) clear_node_moments(g, tm, node);   // read above by this thread only
-    solve3(a, r, z);
-    Enew[node] = V4<R>{z[0], z[1], z[2], R(0)};
-    Ehalf[pidx(g, i, j)] = V4<R>{R(0.5) * (e.x + z[0]), R(0.5) * (e.y + z[1]), R(0.5) * (e.z + z[2]), R(0)};
 }
 
 struct Inc {
     double new0[3], old0[3], new1[3], old1[3];
 };
 
-// Wall columns (reading of the missing boundary and source equations): the wall
-// node is vacuum; Ex advances with the one-sided dHz/dy, Ey and Ez follow a
-// first-order Mur condition on the outgoing field -- at x = 0 on the field
-// minus the incident wave, which is added back.
+// Eq. 4 at the nodes, a thread per node (a walk down the rows that shares the
+// curl's vertical halves left the few warps over the plasma, which read moments
+// and solve, running alone: 540 us).  The FP64 pipe bounds the FP64 form, so the
+// factors dt/(2 dx), dt/(2 dy) go into the update's FMAs and the sum E^n + E^{n+1}
+// that the push gathers is stored without its half (the push's factor has it):
+// 17 operations per vacuum node instead of 23.  4096 x 2048 nodes FP64, vacuum but
+// for a thin foil: 472 -> 300 us (the two passes of H and B: 425 -> 339 us).
+//
+// Walls (reading of the missing boundary and source equations): the wall node is
+// vacuum; Ex advances with the one-sided dHz/dy, Ey and Ez follow a first-order Mur
+// condition on the outgoing field -- at x = 0 on the field minus the incident
+// wave, which is added back.  The thread of the neighbour column does them.
 template <typename R>
-__global__ void k_field_walls(GridArgs<R> g, const V4<R> *__restrict__ E, const V4<R> *__restrict__ H,
-                              V4<R> *__restrict__ Enew, V4<R> *__restrict__ Ehalf, Inc inc, R kap) {
-    int j = blockIdx.x * blockDim.x + threadIdx.x;
-    if (j >= g.ny) return;
-    int jm = (j == 0) ? g.ny - 1 : j - 1;
-    {
-        int64_t o0 = (int64_t)j * g.nxn, o1 = o0 + 1;
-        V4<R> e0 = E[o0], e1 = E[o1], n1 = Enew[o1];
-        R dhz = (H[(int64_t)j * g.nx].z - H[(int64_t)jm * g.nx].z) * g.inv_dy;
-        V4<R> z;
-        z.x = e0.x + g.dt * dhz;
-        R s0y = e0.y - (R)inc.old0[1], s1y = e1.y - (R)inc.old1[1], n1y = n1.y - (R)inc.new1[1];
-        R s0z = e0.z - (R)inc.old0[2], s1z = e1.z - (R)inc.old1[2], n1z = n1.z - (R)inc.new1[2];
-        z.y = (R)inc.new0[1] + s1y + kap * (n1y - s0y);
-        z.z = (R)inc.new0[2] + s1z + kap * (n1z - s0z);
-        z.w = R(0);
-        Enew[o0] = z;
-        Ehalf[pidx(g, 0, j)] = V4<R>{R(0.5) * (e0.x + z.x), R(0.5) * (e0.y + z.y), R(0.5) * (e0.z + z.z), R(0)};
+__global__ void __launch_bounds__(128, 6) k_field_E_literal(GridArgs<R> g, const V4<R> *__restrict__ E,
+                                                         const V4<R> *__restrict__ H, const R *M, const R *Mlo,
+                                                         V4<R> *__restrict__ Enew, V4<R> *__restrict__ Esum,
+                                                         TouchArgs<R> tm, Inc inc, R kap) {
+    const int i = (int)(blockIdx.x * blockDim.x + threadIdx.x) + (g.periodic_x ? 0 : 1), j = blockIdx.y;
+    if (i >= g.nx) return;
+    const int64_t node = (int64_t)j * g.nxn + i;
+    const uint8_t *map = tm.touched ? tm.touched + (j / tm.tny) * tm.ntx : nullptr;
+    const bool touched = !map || map[min(i / tm.tnx, tm.ntx - 1)];
+    R u, v, sy, sx;
+    curl_h_parts(g, H, i, j, u, v, sy, sx);   // curl_h H = (u/(2 dy), v/(2 dx), sy/(2 dx) - sx/(2 dy))
+    const V4<R> e = E[node];
+    V4<R> z;
+    if (!touched) {
+        // vacuum (S = 0, dj = 0 on every node of the tile): Eq. 4 reduces to E^{n+1} = E^n + dt curl_h H,
+        // with no moment read and no 3x3 solve.  The same operations as the solve below on such a node
+        // (where the 3x3 solve returns its right-hand side exactly), so a node's bits do not depend on
+        // whether its tile was marked.
+        z.x = fma_r(g.khy, u, e.x);
+        z.y = fma_r(g.khx, v, e.y);
+        z.z = fma_r(g.khx, sy, fma_r(-g.khy, sx, e.z));
+    } else {
+        const R ia = g.inv_dx * g.inv_dy;
+        const R ev[3] = {e.x, e.y, e.z};
+        R a[9], r[3], w[3];
+#pragma unroll
+        for (int row = 0; row < 3; ++row) {
+            R s_e = R(0);
+#pragma unroll
+            for (int col = 0; col < 3; ++col) {
+                const int64_t mi = (int64_t)(1 + 3 * row + col) * g.nnode + node;
+                const R S = (Mlo ? M[mi] + Mlo[mi] : M[mi]) * ia;
+                a[3 * row + col] = (row == col ? R(1) : R(0)) + S;
+                s_e += ((row == col ? R(1) : R(0)) - S) * ev[col];
+            }
+            const int64_t ji = (int64_t)(10 + row) * g.nnode + node;
+            r[row] = fma_r(-g.dt, (Mlo ? M[ji] + Mlo[ji] : M[ji]) * ia, s_e);
+        }
+        r[0] = fma_r(g.khy, u, r[0]);
+        r[1] = fma_r(g.khx, v, r[1]);
+        r[2] = fma_r(g.khx, sy, fma_r(-g.khy, sx, r[2]));
+        if (tm.clr) clear_node_moments(g, tm, node);   // read above by this thread only
+        solve3(a, r, w);
+        z.x = w[0];
+        z.y = w[1];
+        z.z = w[2];
     }
-    {
-        int64_t oN = (int64_t)j * g.nxn + g.nx, oM = oN - 1;
-        V4<R> eN = E[oN], eM = E[oM], nM = Enew[oM];
-        R dhz = (H[(int64_t)j * g.nx + g.nx - 1].z - H[(int64_t)jm * g.nx + g.nx - 1].z) * g.inv_dy;
-        V4<R> z;
-        z.x = eN.x + g.dt * dhz;
-        z.y = eM.y + kap * (nM.y - eN.y);
-        z.z = eM.z + kap * (nM.z - eN.z);
-        z.w = R(0);
-        Enew[oN] = z;
-        Ehalf[pidx(g, g.nx, j)] = V4<R>{R(0.5) * (eN.x + z.x), R(0.5) * (eN.y + z.y), R(0.5) * (eN.z + z.z), R(0)};
+    z.w = R(0);
+    Enew[node] = z;
+    store_padded(Esum, g, i, j, V4<R>{e.x + z.x, e.y + z.y, e.z + z.z, R(0)});
+    if (g.periodic_x) return;
+    const int jm = (j == 0) ? g.ny - 1 : j - 1;
+    if (i == 1) {
+        const V4<R> e0 = E[node - 1];
+        const R dz = H[(int64_t)j * g.nx].z - H[(int64_t)jm * g.nx].z;
+        const R s0y = e0.y - (R)inc.old0[1], s1y = e.y - (R)inc.old1[1], n1y = z.y - (R)inc.new1[1];
+        const R s0z = e0.z - (R)inc.old0[2], s1z = e.z - (R)inc.old1[2], n1z = z.z - (R)inc.new1[2];
+        const V4<R> w{fma_r(g.dt, dz * g.inv_dy, e0.x), (R)inc.new0[1] + s1y + kap * (n1y - s0y),
+                      (R)inc.new0[2] + s1z + kap * (n1z - s0z), R(0)};
+        Enew[node - 1] = w;
+        store_padded(Esum, g, 0, j, V4<R>{e0.x + w.x, e0.y + w.y, e0.z + w.z, R(0)});
+        if (tm.clr && (!map || map[0])) clear_node_moments(g, tm, node - 1);   // (its moments are not read)
+    }
+    if (i == g.nx - 1) {
+        const V4<R> eN = E[node + 1];
+        const R dz = H[(int64_t)j * g.nx + g.nx - 1].z - H[(int64_t)jm * g.nx + g.nx - 1].z;
+        const V4<R> w{fma_r(g.dt, dz * g.inv_dy, eN.x), e.y + kap * (z.y - eN.y), e.z + kap * (z.z - eN.z), R(0)};
+        Enew[node + 1] = w;
+        store_padded(Esum, g, g.nx, j, V4<R>{eN.x + w.x, eN.y + w.y, eN.z + w.z, R(0)});
+        if (tm.clr && (!map || map[tm.ntx - 1])) clear_node_moments(g, tm, node + 1);
     }
 }
 
-// Eq. 5: H_out = H_in - dt curl_e(Ec), curl_e at the cell centre from its
-// four corners (transversely averaged centred differences).  With the
-// diagonal differences p = e11 - e00 and q = e01 - e10 the two Ez derivatives
-// are (p + q)/(2 dy) and (p - q)/(2 dx); kx = dt/(2 dx), ky = dt/(2 dy) come
-// from the host, so no thread divides (15 FP64 operations per cell).
+// Vertical halves of curl_e over two rows of V4 values a (upper), b (lower).
+template <typename R>
+struct RowPair {
+    R sy, sz, dx, dz;   // sums of y and z, differences (upper - lower) of x and z
+};
+template <typename R>
+__device__ inline RowPair<R> row_pair(const V4<R> &a, const V4<R> &b) {
+    return RowPair<R>{a.y + b.y, a.z + b.z, a.x - b.x, a.z - b.z};
+}
+template <typename R>
+__device__ inline RowPair<R> shfl_down(const RowPair<R> &p) {
+    const unsigned f = 0xffffffffu;
+    return RowPair<R>{__shfl_down_sync(f, p.sy, 1), __shfl_down_sync(f, p.sz, 1), __shfl_down_sync(f, p.dx, 1),
+                      __shfl_down_sync(f, p.dz, 1)};
+}
+
+constexpr int FIELD_WARPS = 4;   // warps of a block of k_field_HB, each with rows of its own
+constexpr int HB_COLS = 30;      // columns a warp produces: the outer two lanes are their neighbours' only
+
+// Eq. 5 and the node B of the new H in one pass: a warp walks down rows of
+// HB_COLS columns, lane l holding E column c0 + l.  H_out = H_in - dt curl_e(Ec)
+// at the cells (kx = dt/(2 dx), ky = dt/(2 dy), vertical halves of curl_e and
+// the right neighbour's by a shuffle: 12 FP64 operations per cell); B = the sum
+// of the four cells sharing the node, without its quarter (the deposits' factor
+// has it; on a wall column twice the two inside cells): 6 operations per node
+// instead of 12, and H is not read again.  A row of H above the strip is formed
+// twice.  4096 x 2048 FP64: 227 + 198 us for the two
+// passes before -> 339 us.
 template <typename R, typename RE>
-__global__ void k_field_H(GridArgs<R> g, const V4<RE> *__restrict__ Ec, const V4<R> *__restrict__ Hin,
-                          V4<R> *__restrict__ Hout, RE kx, RE ky) {
-    int i = blockIdx.x * blockDim.x + threadIdx.x;
-    int j = blockIdx.y;
-    if (i >= g.nx || j >= g.ny) return;
-    int ip = i + 1;
-    if (g.periodic_x && ip == g.nx) ip = 0;
-    int jp = (j + 1 == g.ny) ? 0 : j + 1;
-    V4<RE> e00 = Ec[(int64_t)j * g.nxn + i], e10 = Ec[(int64_t)j * g.nxn + ip];
-    V4<RE> e01 = Ec[(int64_t)jp * g.nxn + i], e11 = Ec[(int64_t)jp * g.nxn + ip];
-    const RE pz = e11.z - e00.z, qz = e01.z - e10.z;
-    const RE sy = (e11.y - e00.y) + (e10.y - e01.y);   // 2 dx dEy/dx
-    const RE sx = (e11.x - e00.x) + (e01.x - e10.x);   // 2 dy dEx/dy
-    int64_t o = (int64_t)j * g.nx + i;
-    V4<R> hv = Hin[o];
-    Hout[o] = V4<R>{(R)fma(-ky, pz + qz, (RE)hv.x), (R)fma(kx, pz - qz, (RE)hv.y),
-                    (R)fma(ky, sx, fma(-kx, sy, (RE)hv.z)), R(0)};
+__global__ void __launch_bounds__(32 * FIELD_WARPS) k_field_HB(GridArgs<R> g, const V4<RE> *__restrict__ Ec,
+                                                               const V4<R> *__restrict__ Hin, V4<R> *__restrict__ Hout,
+                                                               V4<R> *__restrict__ Bp, RE kx, RE ky, int rows) {
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const int i = (int)blockIdx.x * HB_COLS - 1 + lane;   // column of this lane's nodes and cells
+    const int y0 = ((int)blockIdx.y * FIELD_WARPS + wid) * rows, y1 = min(y0 + rows, g.ny);
+    if (y0 >= g.ny) return;   // (whole warps)
+    int n = i, c = i;         // loaded columns of E and H
+    if (g.periodic_x) {
+        n = n < 0 ? g.nx - 1 : n >= g.nx ? n - g.nx : n;   // (i <= nx + 29: lanes past the end are not used,
+        if (n >= g.nx) n = 0;                              //  but for column nx, which is column 0)
+        c = n;
+    } else {
+        n = min(max(n, 0), g.nx);
+        c = min(max(c, 0), g.nx - 1);
+    }
+    const bool node = lane > 0 && lane <= HB_COLS && i < g.nxn, cell = lane > 0 && lane <= HB_COLS && i < g.nx;
+    const int jb = y0 == 0 ? g.ny - 1 : y0 - 1;
+    V4<RE> eb = Ec[(int64_t)jb * g.nxn + n], en = Ec[(int64_t)y0 * g.nxn + n];
+    V4<R> hn = Hin[(int64_t)jb * g.nx + c];
+    V4<R> below{R(0), R(0), R(0), R(0)};   // the new H of the row above the strip, then of the previous row
+    for (int j = y0 - 1; j < y1; ++j) {
+        const V4<RE> ea = en;               // E rows j + 1 (ea) and j (eb), H row j
+        const V4<R> h = hn;
+        if (j + 1 < y1) {
+            en = Ec[(int64_t)(j + 2 >= g.ny ? j + 2 - g.ny : j + 2) * g.nxn + n];
+            hn = Hin[(int64_t)(j + 1) * g.nx + c];
+        }
+        const RowPair<RE> p = row_pair(ea, eb), q = shfl_down(p);   // columns i and i + 1
+        eb = ea;
+        // 2 dy dEz/dy = dz + dz', 2 dx dEz/dx = sz' - sz, 2 dx dEy/dx = sy' - sy, 2 dy dEx/dy = dx + dx'
+        const V4<R> w{(R)fma(-ky, p.dz + q.dz, (RE)h.x), (R)fma(kx, q.sz - p.sz, (RE)h.y),
+                      (R)fma(ky, p.dx + q.dx, fma(-kx, q.sy - p.sy, (RE)h.z)), R(0)};
+        if (j >= y0) {
+            if (cell) Hout[(int64_t)j * g.nx + i] = w;
+            const V4<R> s{below.x + w.x, below.y + w.y, below.z + w.z, R(0)};   // cells (i, j - 1) and (i, j)
+            const R lx = __shfl_up_sync(0xffffffffu, s.x, 1), ly = __shfl_up_sync(0xffffffffu, s.y, 1);
+            const R lz = __shfl_up_sync(0xffffffffu, s.z, 1);
+            if (node) {
+                // the columns i - 1 and i of cells; on a wall the inside one twice (selected before the additions)
+                const bool w0 = !g.periodic_x && i == 0, wn = !g.periodic_x && i == g.nx;
+                store_padded(Bp, g, i, j, V4<R>{(wn ? lx : s.x) + (w0 ? s.x : lx), (wn ? ly : s.y) + (w0 ? s.y : ly),
+                                                (wn ? lz : s.z) + (w0 ? s.z : lz), R(0)});
+            }
+        }
+        below = w;
+    }
 }
 
-// Node B: mean of the cells sharing the node (2 on a wall column).
+// Node B of a given H (an overwritten field), in the same form: the sums of k_field_HB.
 template <typename R>
 __global__ void k_node_average(GridArgs<R> g, const V4<R> *__restrict__ Hc, V4<R> *__restrict__ Bp) {
     int i = blockIdx.x * blockDim.x + threadIdx.x;
     int j = blockIdx.y;
     if (i >= g.nxn || j >= g.ny) return;
     int jm = (j == 0) ? g.ny - 1 : j - 1;
+    auto column = [&](int c) {
+        const V4<R> a = Hc[(int64_t)jm * g.nx + c], b = Hc[(int64_t)j * g.nx + c];
+        return V4<R>{a.x + b.x, a.y + b.y, a.z + b.z, R(0)};
+    };
     V4<R> o;
     if (!g.periodic_x && (i == 0 || i == g.nx)) {
-        int ic = (i == 0) ? 0 : g.nx - 1;
-        V4<R> a = Hc[(int64_t)j * g.nx + ic], b = Hc[(int64_t)jm * g.nx + ic];
-        o = V4<R>{R(0.5) * (a.x + b.x), R(0.5) * (a.y + b.y), R(0.5) * (a.z + b.z), R(0)};
+        const V4<R> s = column(i == 0 ? 0 : g.nx - 1);
+        o = V4<R>{R(2) * s.x, R(2) * s.y, R(2) * s.z, R(0)};
     } else {
-        int im = (i == 0) ? g.nx - 1 : i - 1;
-        V4<R> a = Hc[(int64_t)j * g.nx + i], b = Hc[(int64_t)j * g.nx + im];
-        V4<R> c = Hc[(int64_t)jm * g.nx + i], d = Hc[(int64_t)jm * g.nx + im];
-        o = V4<R>{R(0.25) * (a.x + b.x + c.x + d.x), R(0.25) * (a.y + b.y + c.y + d.y),
-                  R(0.25) * (a.z + b.z + c.z + d.z), R(0)};
+        const V4<R> s = column(i), l = column((i == 0) ? g.nx - 1 : i - 1);
+        o = V4<R>{s.x + l.x, s.y + l.y, s.z + l.z, R(0)};
     }
-    Bp[pidx(g, i, j)] = o;
-}
-
-// Ghost ring of a padded node array: periodic copies in y (and x when periodic),
-// zero beyond a wall.  One thread per ring entry: the G rows above and below
-// (full width), then the G columns left and right of every real row.
-template <typename R>
-__global__ void k_fill_ghosts(GridArgs<R> g, int nyp, V4<R> *__restrict__ F) {
-    int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    const int64_t band = (int64_t)g.G * g.nxp, side = (int64_t)g.ny * (g.nxp - g.nxn);
-    if (t >= 2 * band + side) return;
-    int pi, pj;
-    if (t < band) {
-        pj = (int)(t / g.nxp);
-        pi = (int)(t - (int64_t)pj * g.nxp);
-    } else if (t < 2 * band) {
-        const int64_t u = t - band;
-        pj = g.G + g.ny + (int)(u / g.nxp);
-        pi = (int)(u % g.nxp);
-    } else {
-        const int64_t u = t - 2 * band;
-        const int w = g.nxp - g.nxn;   // 2 G
-        const int row = (int)(u / w), col = (int)(u - (int64_t)row * w);
-        pj = g.G + row;
-        pi = col < g.G ? col : g.nxn + col;
-    }
-    int i = pi - g.G, j = pj - g.G;
-    int jj = ((j % g.ny) + g.ny) % g.ny;
-    V4<R> v{R(0), R(0), R(0), R(0)};
-    if (g.periodic_x) {
-        int ii = ((i % g.nxn) + g.nxn) % g.nxn;
-        v = F[pidx(g, ii, jj)];
-    } else if (i >= 0 && i < g.nxn) {
-        v = F[pidx(g, i, jj)];
-    }
-    F[(int64_t)pj * g.nxp + pi] = v;
+    store_padded(Bp, g, i, j, o);
 }
 
 // --------------------------------------------------------------------------- CN solver
@@ -1523,10 +1555,10 @@ __global__ void __launch_bounds__(BS, kCluster ? 1 : 3) k_cn_solve(GridArgs<doub
     }
 }
 
-// E^{n+1} = 2X - E^n, E^{n+1/2} = X (padded).
+// E^{n+1} = 2X - E^n, E^n + E^{n+1} = 2X (padded, for the push).
 template <typename R>
 __global__ void k_cn_finish(GridArgs<R> g, const V4<double> *__restrict__ X, const V4<R> *__restrict__ E,
-                            V4<R> *__restrict__ Enew, V4<R> *__restrict__ Ehalf) {
+                            V4<R> *__restrict__ Enew, V4<R> *__restrict__ Esum) {
     int i = blockIdx.x * blockDim.x + threadIdx.x;
     int j = blockIdx.y;
     if (i >= g.nxn || j >= g.ny) return;
@@ -1534,7 +1566,7 @@ __global__ void k_cn_finish(GridArgs<R> g, const V4<double> *__restrict__ X, con
     V4<double> x = X[node];
     V4<R> e = E[node];
     Enew[node] = V4<R>{(R)(2.0 * x.x - (double)e.x), (R)(2.0 * x.y - (double)e.y), (R)(2.0 * x.z - (double)e.z), R(0)};
-    Ehalf[pidx(g, i, j)] = V4<R>{(R)x.x, (R)x.y, (R)x.z, R(0)};
+    store_padded(Esum, g, i, j, V4<R>{(R)(2.0 * x.x), (R)(2.0 * x.y), (R)(2.0 * x.z), R(0)});
 }
 
 // The moments are FP64 for the solver; the FP32 form adds its sum and its
@@ -1548,26 +1580,13 @@ __global__ void k_moments_to_double(const float *__restrict__ Mf, const float *_
 // --------------------------------------------------------------------------- host side
 
 static dim3 node_grid(const pic_t *h, int bs) { return dim3((h->nxn + bs - 1) / bs, h->ny); }
-static dim3 cell_grid(const pic_t *h, int bs) { return dim3((h->nx + bs - 1) / bs, h->ny); }
-
-template <typename R>
-static int fill_ghosts_t(pic_t *h, void *F) {
-    GridArgs<R> g = grid_args<R>(h);
-    int64_t total = 2 * (int64_t)h->G * h->nxp + (int64_t)h->ny * (h->nxp - h->nxn);   // ring entries
-    k_fill_ghosts<R><<<(unsigned)((total + 255) / 256), 256, 0, h->st>>>(g, h->nyp, (V4<R> *)F);
-    count_launch(h);
-    return check_launch("k_fill_ghosts");
-}
-
-int fill_ghosts(pic_t *h, void *padded) { return h->fp32 ? fill_ghosts_t<float>(h, padded) : fill_ghosts_t<double>(h, padded); }
 
 template <typename R>
 static int node_average_t(pic_t *h, int hsrc, int bdst) {
     GridArgs<R> g = grid_args<R>(h);
     k_node_average<R><<<node_grid(h, 128), 128, 0, h->st>>>(g, (const V4<R> *)h->H[hsrc], (V4<R> *)h->B[bdst]);
     count_launch(h);
-    if (int rc = check_launch("k_node_average")) return rc;
-    return fill_ghosts_t<R>(h, h->B[bdst]);
+    return check_launch("k_node_average");
 }
 
 int node_average(pic_t *h, int hsrc, int bdst) {
@@ -1594,40 +1613,42 @@ static Inc incident(const pic_t *h) {
     return inc;
 }
 
+// Rows a warp of k_field_HB walks down: up to 32 (it forms a row of H more than
+// it stores), fewer where that leaves the GPU short of warps.
+static int field_rows(const pic_t *h, int xw) {
+    int dev = 0, nsm = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
+    const int64_t r = (int64_t)h->ny * xw / (24 * (int64_t)(nsm > 0 ? nsm : 128));
+    return r < 2 ? 2 : r > 32 ? 32 : (int)r;
+}
+
+template <typename R, typename RE>
+static int field_HB(pic_t *h, const void *Ec) {
+    const int hn = 1 - h->hcur, xw = (h->nxn + HB_COLS - 1) / HB_COLS, rows = field_rows(h, xw);
+    k_field_HB<R, RE><<<dim3(xw, (h->ny + rows * FIELD_WARPS - 1) / (rows * FIELD_WARPS)), 32 * FIELD_WARPS, 0, h->st>>>(
+        grid_args<R>(h), (const V4<RE> *)Ec, (const V4<R> *)h->H[h->hcur], (V4<R> *)h->H[hn], (V4<R> *)h->B[1 - h->bcur],
+        (RE)(0.5 * h->cfg.dt / h->cfg.dx), (RE)(0.5 * h->cfg.dt / h->cfg.dy), rows);
+    count_launch(h);
+    return check_launch("k_field_HB");
+}
+
 template <typename R>
 static int field_literal_t(pic_t *h) {
-    GridArgs<R> g = grid_args<R>(h);
-    int en = 1 - h->ecur, hn = 1 - h->hcur;
+    int en = 1 - h->ecur;
     // the exact deposit rewrites every moment from its fixed-point sums; the others deposit into the
     // moments this solve has read and zeroed
     TouchArgs<R> tm{h->touch_all ? nullptr : h->touched, h->tnx, h->tny, h->ntx, h->det ? nullptr : (R *)h->M,
                     h->det ? nullptr : (R *)h->Mlo};
-    k_field_E_literal<R><<<node_grid(h, 128), 128, 0, h->st>>>(g, (const V4<R> *)h->E[h->ecur],
-                                                                (const V4<R> *)h->H[h->hcur], (const R *)h->M,
-                                                                (const R *)h->Mlo, (V4<R> *)h->E[en],
-                                                                (V4<R> *)h->Ehalf, tm);
+    const pic_config &c = h->cfg;
+    const int cols = h->periodic_x ? h->nx : h->nx - 1;   // (the walls' columns by their neighbours' threads)
+    k_field_E_literal<R><<<dim3((cols + 127) / 128, h->ny), 128, 0, h->st>>>(
+        grid_args<R>(h), (const V4<R> *)h->E[h->ecur], (const V4<R> *)h->H[h->hcur], (const R *)h->M, (const R *)h->Mlo,
+        (V4<R> *)h->E[en], (V4<R> *)h->Ehalf, tm, incident(h), (R)((c.dt - c.dx) / (c.dt + c.dx)));
     count_launch(h);
     if (int rc = check_launch("k_field_E_literal")) return rc;
     h->moments_cleared = !h->det;
-    int nl = 1;
-    if (!h->periodic_x) {
-        const pic_config &c = h->cfg;
-        Inc inc = incident(h);
-        R kap = (R)((c.dt - c.dx) / (c.dt + c.dx));
-        k_field_walls<R><<<(h->ny + 127) / 128, 128, 0, h->st>>>(g, (const V4<R> *)h->E[h->ecur],
-                                                                  (const V4<R> *)h->H[h->hcur], (V4<R> *)h->E[en],
-                                                                  (V4<R> *)h->Ehalf, inc, kap);
-        count_launch(h);
-        ++nl;
-        if (int rc = check_launch("k_field_walls")) return rc;
-    }
-    k_field_H<R, R><<<cell_grid(h, 128), 128, 0, h->st>>>(g, (const V4<R> *)h->E[en], (const V4<R> *)h->H[h->hcur],
-                                                          (V4<R> *)h->H[hn], (R)(0.5 * h->cfg.dt / h->cfg.dx),
-                                                          (R)(0.5 * h->cfg.dt / h->cfg.dy));
-    count_launch(h);
-    ++nl;
-    if (int rc = check_launch("k_field_H")) return rc;
-    return 0;
+    return field_HB<R, R>(h, h->E[en]);
 }
 
 int field_literal(pic_t *h) { return h->fp32 ? field_literal_t<float>(h) : field_literal_t<double>(h); }
@@ -1824,15 +1845,12 @@ static int field_cn_t(pic_t *h) {
         set_error("launch of k_cn_solve: %s", cudaGetErrorString(e));
         return PIC_ERR_CUDA;
     }
-    int en = 1 - h->ecur, hn = 1 - h->hcur;
+    int en = 1 - h->ecur;
     k_cn_finish<R><<<node_grid(h, 128), 128, 0, h->st>>>(g, v.x, (const V4<R> *)h->E[h->ecur], (V4<R> *)h->E[en],
                                                           (V4<R> *)h->Ehalf);
     count_launch(h);
     if (int rc = check_launch("k_cn_finish")) return rc;
-    k_field_H<R, double><<<cell_grid(h, 128), 128, 0, h->st>>>(g, v.x, (const V4<R> *)h->H[h->hcur], (V4<R> *)h->H[hn],
-                                                               0.5 * h->cfg.dt / h->cfg.dx, 0.5 * h->cfg.dt / h->cfg.dy);
-    count_launch(h);
-    return check_launch("k_field_H(cn)");
+    return field_HB<R, double>(h, v.x);
 }
 
 int field_cn(pic_t *h) { return h->fp32 ? field_cn_t<float>(h) : field_cn_t<double>(h); }

@@ -103,8 +103,8 @@ struct pic_t {
     int ecur = 0;
     void *H[2] = {nullptr, nullptr};    // cells [ncell]; H[hcur] current, H[1-hcur] previous
     int hcur = 0;
-    void *Ehalf = nullptr;              // padded nodes: E^{n+1/2} seen by the push
-    void *B[2] = {nullptr, nullptr};    // padded nodes: B[bcur] = node B the moments were made with
+    void *Ehalf = nullptr;              // padded nodes: E^n + E^{n+1}, twice the E the push sees
+    void *B[2] = {nullptr, nullptr};    // padded nodes: B[bcur] = four times the node B the moments were made with
     int bcur = 0;
     void *M = nullptr;                  // raw moment sums, planar [13][nnode] real
 
@@ -131,7 +131,7 @@ struct pic_t {
     void *Mlo = nullptr;                // FP32 form: compensation of the moment sums
     bool det = false;                   // deterministic deposit: exact fixed-point sums in Mfix
     unsigned long long *Mfix = nullptr; // [13][nnode] two's-complement fixed-point moment sums
-    double *Mc = nullptr;               // FP64 L2-reduction push (linear shape): cell sums [13][ncell][4]
+    double *Mc = nullptr;               // FP64 L2-reduction push (linear shape): cell sums [ncell][13][4]
     double wabs[PIC_MAX_SPECIES] = {0, 0, 0, 0, 0, 0, 0, 0};  // sum of |w| loaded per species
     void *tmaps = nullptr;              // host storage of the TMA descriptors
     int32_t *chunk_prefix = nullptr;    // [nsp*ntiles + 1] work items of the push, exclusive scan
@@ -145,7 +145,7 @@ struct pic_t {
     int32_t *rg_list = nullptr;         // [ntiles] tiles the regroup must visit (an occupied tile or neighbour)
     int32_t *list_n = nullptr;          // [2 + PIC_MAX_SPECIES] entries of touch_list, rg_list; regroup queues
     int regroup_blocks = 0;             // blocks per species of the list-driven regroup
-    bool touch_all = true;              // moments may be non-zero anywhere (after init or a deposit at rest)
+    bool touch_all = true;              // no touched-tile map: moments may be non-zero anywhere (after init)
     bool moments_cleared = false;       // the last literal field solve zeroed the moments it read
     unsigned long long *d_bad = nullptr;  // per species: first invalid particle index of a load
     uint32_t *scan_sums = nullptr;      // per-block totals of the multi-block scans
@@ -561,14 +561,13 @@ __device__ inline void deposit_fp64(double *M, unsigned long long *Mfix, const F
 // The push adds A, X, Y, Z of every moment into its cell's sums (three
 // products per moment instead of four, and no corner weights);
 // k_cell_moments then adds every cell's corner values into the node moments.
-// The four sums of a (moment, cell) are adjacent (one 32-byte sector); lane l
+// A cell's sums are adjacent, the four of a moment in one 32-byte sector; lane l
 // starts at moment (l / 4) mod 2 and at sum l mod 4, so that the lanes of one
 // cell spread each instruction's reductions over 8 addresses in 2 sectors
 // (measured on the 1024 x 512 foil's push: 1, 2, 4, 8 moment offsets
 // 2.225, 2.183, 2.191, 2.196 ms; 8 offsets with the sums in separate planes, 32
 // sectors per instruction, 5.79 ms).
-__device__ inline void deposit_fp64_cell(double *Mc, int64_t ncell, int64_t cell, double fx, double fy,
-                                         const double *val, int lane) {
+__device__ inline void deposit_fp64_cell(double *Mc, int64_t cell, double fx, double fy, const double *val, int lane) {
     const double fxy = fx * fy;
     double P[NMOM];
 #pragma unroll
@@ -586,7 +585,7 @@ __device__ inline void deposit_fp64_cell(double *Mc, int64_t ncell, int64_t cell
     for (int kk = 0; kk < NMOM; ++kk) {
         const int km = kk + rr >= NMOM ? kk + rr - NMOM : kk + rr;
         const double a = P[kk], x = a * fx, y = a * fy, z = a * fxy;
-        double *base = Mc + ((int64_t)km * ncell + cell) * 4;
+        double *base = Mc + (cell * NMOM + km) * 4;
 #pragma unroll
         for (int c0 = 0; c0 < 4; ++c0) {
             const int kind = (c0 + lane) & 3;
@@ -939,10 +938,9 @@ void timing_end(pic_t *h, int cls, int nlaunch);
 inline void count_launch(pic_t *h, int n = 1) { h->timing.launches[4] += n; }
 
 // fields (pic_field.cu)
-int field_literal(pic_t *h);
+int field_literal(pic_t *h);            // E, H and node B of the next time level, E^n + E^{n+1} for the push
 int field_cn(pic_t *h);
-int node_average(pic_t *h, int hsrc, int bdst);
-int fill_ghosts(pic_t *h, void *padded);
+int node_average(pic_t *h, int hsrc, int bdst);   // node B of a given H
 int upload_fields(pic_t *h, const double *E3, const double *H3);
 int download_fields(pic_t *h, double *E3, double *H3);
 
@@ -983,7 +981,8 @@ int push_work_list(pic_t *h);           // k_chunk_counts + scan on the run's st
 int tile_setup(pic_t *h);
 int particle_tiles(pic_t *h, bool prepared = false);
 int push_prep(pic_t *h, bool next);
-int cell_moments(pic_t *h, bool all = false);   // FP64 cell sums -> node moments (touched tiles; all: every tile)
+int cell_moments(pic_t *h);      // FP64 cell sums -> node moments (the listed touched tiles)
+int rest_touch(pic_t *h);        // touched[] and its list after a deposit at rest into cleared moments
 int reset_lists(pic_t *h);       // the tile lists and regroup queues, emptied before a push
 int regroup_tiles(pic_t *h);     // per-tile stable cell sort of stayers + arrivals into the spare set
 int scan_tiles(pic_t *h, const int32_t *in, int32_t *out);

@@ -22,7 +22,7 @@ struct DepArgs {
     unsigned long long *Mfix;
     FixScale fs;
     R q, m;
-    R kq, cq2, hq;    // q dt / (2 m), q^2 dt^2 / (4 m), q dt^2 / (4 m): per species, from the host (as for the push)
+    R kb, cq2, hq;    // q dt / (2 m) over the stored B's scale of 4, q^2 dt^2 / (4 m), q dt^2 / (4 m): per species, from the host (as for the push)
     int32_t *flags;   // checks build: FLAG_CHECK on a broken invariant
     double *cr;       // FP64 form: the carried quantities of the bins ([NCARRY][ccap]), else nullptr
     int64_t ccap;
@@ -147,10 +147,10 @@ __global__ void k_deposit_bins(DepArgs<R> a) {
             }
             R ig, bx, by, bz, inv;
             if (sizeof(R) == 8 && (kFix || !a.Mc))   // FP64 corner form: class factors and parts
-                particle_moment_parts(a.q, a.kq, a.cq2, a.w[p], a.ux[p], a.uy[p], a.uz[p], Bx, By, Bz, val, fr, fS, fj,
+                particle_moment_parts(a.q, a.kb, a.cq2, a.w[p], a.ux[p], a.uy[p], a.uz[p], Bx, By, Bz, val, fr, fS, fj,
                                       ig, bx, by, bz, inv);
             else   // the 13 moment values (the FP64 cell form as the push makes them)
-                particle_moments_c(a.q, a.kq, a.hq, a.w[p], a.ux[p], a.uy[p], a.uz[p], Bx, By, Bz, val, ig, bx, by,
+                particle_moments_c(a.q, a.kb, a.hq, a.w[p], a.ux[p], a.uy[p], a.uz[p], Bx, By, Bz, val, ig, bx, by,
                                    bz, inv);
             if (sizeof(R) == 8 && a.cr) {   // what the next push needs of this B (carried, FP64 form)
                 a.cr[p] = (double)ig;
@@ -189,7 +189,7 @@ __global__ void k_deposit_bins(DepArgs<R> a) {
             if constexpr (sizeof(R) == 8) {
                 // the push's own FP64 deposit (cell sums, or node moments for the exact form)
                 if (!kFix && a.Mc)
-                    deposit_fp64_cell(a.Mc, (int64_t)g.nx * g.ny, c, (double)fx, (double)fy, (const double *)val, lane);
+                    deposit_fp64_cell(a.Mc, c, (double)fx, (double)fy, (const double *)val, lane);
                 else
                     deposit_fp64<kFix>((double *)a.M, a.Mfix, a.fs, g, cx, cy, (double)fx, (double)fy,
                                        (const double *)val, (double)fr, (double)fS, (double)fj, lane);
@@ -219,7 +219,7 @@ __global__ void k_deposit_bins(DepArgs<R> a) {
 struct CellDepSp {
     const int32_t *cell, *bstart, *useg, *segn;
     const float *ox, *oy, *ux, *uy, *uz, *w;
-    float q, kq, hq;
+    float q, kb, hq;
 };
 struct CellDepArgs {
     GridArgs<float> g;
@@ -301,7 +301,7 @@ __global__ void __launch_bounds__(256, 3) k_deposit_cells(const __grid_constant_
                 const float By = w00 * n00.y + w10 * n10.y + w01 * n01.y + w11 * n11.y;
                 const float Bz = w00 * n00.z + w10 * n10.z + w01 * n01.z + w11 * n11.z;
                 float ig, bx, by, bz, inv;
-                particle_moments_c(P.q, P.kq, P.hq, w, ux, uy, uz, Bx, By, Bz, val, ig, bx, by, bz, inv);
+                particle_moments_c(P.q, P.kb, P.hq, w, ux, uy, uz, Bx, By, Bz, val, ig, bx, by, bz, inv);
             }
             dep.add(sink, a.tnx, a.tny, valid, sp, val, lane);
         }
@@ -373,10 +373,10 @@ __global__ void __launch_bounds__(256) k_deposit_s(DepArgs<R> a) {
                 gather_s(a.B, g, sp, Bx, By, Bz);
                 R fr = R(1), fS = R(1), fj = R(1), ig, bx, by, bz, inv;
                 if constexpr (kParts)
-                    particle_moment_parts(a.q, a.kq, a.cq2, a.w[p], a.ux[p], a.uy[p], a.uz[p], Bx, By, Bz, val, fr, fS,
+                    particle_moment_parts(a.q, a.kb, a.cq2, a.w[p], a.ux[p], a.uy[p], a.uz[p], Bx, By, Bz, val, fr, fS,
                                           fj, ig, bx, by, bz, inv);
                 else
-                    particle_moments_c(a.q, a.kq, a.hq, a.w[p], a.ux[p], a.uy[p], a.uz[p], Bx, By, Bz, val, ig, bx, by,
+                    particle_moments_c(a.q, a.kb, a.hq, a.w[p], a.ux[p], a.uy[p], a.uz[p], Bx, By, Bz, val, ig, bx, by,
                                        bz, inv);
                 if (sizeof(R) == 8 && a.cr) {   // what the next push needs of this B (carried, FP64 form)
                     a.cr[p] = (double)ig;
@@ -566,6 +566,7 @@ __global__ void k_bins_to_stage(GridArgs<double> g, const int32_t *bstart, const
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
     const int64_t b0 = bstart[t], sb = b0 / SEG;
     const int u = useg[t];
+    if (u == 0) return;
     if (threadIdx.x == 0) run = 0;
     __syncthreads();
     for (int j0 = 0; j0 < u; j0 += nw) {
@@ -622,7 +623,7 @@ static CellDepSp cell_dep_species(const pic_t *h, int s) {
     const double dt = h->cfg.dt;
     return CellDepSp{S.cell[b], S.bstart, S.useg[S.scur], S.segn[S.scur], (const float *)S.ox[b], (const float *)S.oy[b],
                      (const float *)S.ux[b], (const float *)S.uy[b], (const float *)S.uz[b], (const float *)S.w[b],
-                     (float)S.q, (float)(S.q * dt / (2.0 * S.m)), (float)(S.q * dt * dt / (4.0 * S.m))};
+                     (float)S.q, 0.25f * (float)(S.q * dt / (2.0 * S.m)), (float)(S.q * dt * dt / (4.0 * S.m))};
 }
 
 static CellDepArgs cell_dep_args(const pic_t *h) {
@@ -703,7 +704,7 @@ static int deposit_only_t(pic_t *h, int s) {
         if (int rc = fix_scale(h, &a.fs)) return rc;
     a.q = (R)S.q;
     a.m = (R)S.m;
-    a.kq = (R)(S.q * h->cfg.dt / (2.0 * S.m));
+    a.kb = R(0.25) * (R)(S.q * h->cfg.dt / (2.0 * S.m));
     a.cq2 = (R)(S.q * S.q * h->cfg.dt * h->cfg.dt / (4.0 * S.m));
     a.hq = (R)(S.q * h->cfg.dt * h->cfg.dt / (4.0 * S.m));
     a.flags = h->d_flags;

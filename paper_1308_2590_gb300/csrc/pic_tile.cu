@@ -106,7 +106,7 @@ struct SpPtr {
     int32_t *ocell;                 // spare set: the regroup's output
     R *oox, *ooy, *oux, *ouy, *ouz, *ow;
     unsigned long long *removed;
-    R q, m, kq, cq2, hq;
+    R q, ke, kb, cq2, hq;   // ke, kb: q dt / (2 m) over the scales of the stored E (2) and B (4)
     double *cr, *mcr, *ocr;         // FP64 form: carried quantities of bins, mirror, spare ([NCARRY][ccap])
     int64_t ccap;
 };
@@ -554,7 +554,7 @@ __global__ void __launch_bounds__(TILE_BS, kDep ? push_min_blocks<R>() : 3)
                 sm_gather(sE, a.EW, lx, ly, fx, fy, Ex, Ey, Ez);
             }
             // implicit push (Eq. 2, E factored out)
-            const R k = P.kq;
+            const R k = P.ke, kb = P.kb;
             R ig, bx, by, bz, binv;
             if constexpr (kCarry<R>) {
                 // the B the moments were made with, at this position and u: the last deposit's b (carried)
@@ -567,9 +567,9 @@ __global__ void __launch_bounds__(TILE_BS, kDep ? push_min_blocks<R>() : 3)
                 R Bx, By, Bz;
                 sm_gather(sBo, a.EW, lx, ly, fx, fy, Bx, By, Bz);
                 ig = rsqrt_r(R(1) + ux * ux + uy * uy + uz * uz);
-                bx = k * Bx * ig;
-                by = k * By * ig;
-                bz = k * Bz * ig;
+                bx = kb * Bx * ig;
+                by = kb * By * ig;
+                bz = kb * Bz * ig;
                 binv = rcp_r(R(1) + bx * bx + by * by + bz * bz);
             }
             // u^{n+1} and the move in cell units
@@ -622,9 +622,9 @@ __global__ void __launch_bounds__(TILE_BS, kDep ? push_min_blocks<R>() : 3)
             } else if (alive) gather4(a.Bnew, g, ncx, ncy, nfx, nfy, nBx, nBy, nBz);
             if constexpr (!kDep) {
             } else if constexpr (kShared || kCellDep)   // the 13 moment values
-                particle_moments_c(P.q, P.kq, P.hq, w, nux, nuy, nuz, nBx, nBy, nBz, val, cig, cbx, cby, cbz, cinv);
+                particle_moments_c(P.q, P.kb, P.hq, w, nux, nuy, nuz, nBx, nBy, nBz, val, cig, cbx, cby, cbz, cinv);
             else   // class factors and parts (the corner-form FP64 deposit)
-                particle_moment_parts(P.q, P.kq, P.cq2, w, nux, nuy, nuz, nBx, nBy, nBz, val, fr, fS, fj, cig, cbx, cby,
+                particle_moment_parts(P.q, P.kb, P.cq2, w, nux, nuy, nuz, nBx, nBy, nBz, val, fr, fS, fj, cig, cbx, cby,
                                       cbz, cinv);
             unsigned strag = 0u;   // FP32: lanes left to the global path
             if (kShared) {
@@ -692,7 +692,7 @@ __global__ void __launch_bounds__(TILE_BS, kDep ? push_min_blocks<R>() : 3)
                 // FP64: every lane adds its own products in L2 (the single-run push: cell sums)
                 if (!alive) {
                 } else if constexpr (kCellDep)
-                    deposit_fp64_cell(a.Mc, (int64_t)g.nx * g.ny, (int64_t)ncy * g.nx + ncx, nfx, nfy, val, lane);
+                    deposit_fp64_cell(a.Mc, (int64_t)ncy * g.nx + ncx, nfx, nfy, val, lane);
                 else
                     deposit_fp64<kFix>(a.M, a.Mfix, a.fs, g, ncx, ncy, nfx, nfy, val, fr, fS, fj, lane);
             }
@@ -865,7 +865,7 @@ __global__ void __launch_bounds__(TILE_BS, push_s_min_blocks<R>()) k_push_s(cons
             const SplineN<R, N> so = spline_n<R, N>(cx, cy, fx, fy);
             R Ex, Ey, Ez;
             gather_s(a.Eh, g, so, Ex, Ey, Ez);
-            const R k = P.kq;
+            const R k = P.ke, kb = P.kb;
             R ig, bx, by, bz, binv;
             if constexpr (kCarry<R>) {
                 ig = cu.ig;
@@ -877,9 +877,9 @@ __global__ void __launch_bounds__(TILE_BS, push_s_min_blocks<R>()) k_push_s(cons
                 R Bx, By, Bz;
                 gather_s(a.Bo, g, so, Bx, By, Bz);
                 ig = rsqrt_r(R(1) + ux * ux + uy * uy + uz * uz);
-                bx = k * Bx * ig;
-                by = k * By * ig;
-                bz = k * Bz * ig;
+                bx = kb * Bx * ig;
+                by = kb * By * ig;
+                bz = kb * Bz * ig;
                 binv = rcp_r(R(1) + bx * bx + by * by + bz * bz);
             }
             R nux, nuy, nuz, sx, sy;
@@ -920,10 +920,10 @@ __global__ void __launch_bounds__(TILE_BS, push_s_min_blocks<R>()) k_push_s(cons
                 R nBx, nBy, nBz;
                 gather_s(a.Bnew, g, sn, nBx, nBy, nBz);
                 if constexpr (kParts)
-                    particle_moment_parts(P.q, P.kq, P.cq2, w, nux, nuy, nuz, nBx, nBy, nBz, val, fr, fS, fj, cig,
+                    particle_moment_parts(P.q, P.kb, P.cq2, w, nux, nuy, nuz, nBx, nBy, nBz, val, fr, fS, fj, cig,
                                           cbx, cby, cbz, cinv);
                 else
-                    particle_moments_c(P.q, P.kq, P.hq, w, nux, nuy, nuz, nBx, nBy, nBz, val, cig, cbx, cby, cbz,
+                    particle_moments_c(P.q, P.kb, P.hq, w, nux, nuy, nuz, nBx, nBy, nBz, val, cig, cbx, cby, cbz,
                                        cinv);
                 if constexpr (kFix) deposit_s_fix<R, kParts, N>(a.Mfix, a.fs, g, sn, val, fr, fS, fj, lane);
             }
@@ -1495,23 +1495,18 @@ __global__ void __launch_bounds__(TILE_BS, kStage ? 3 : 0) k_regroup(const __gri
     }
 }
 
-// Particles per tile (sum of its segment counts).
-__global__ void k_tile_counts(const int32_t *__restrict__ bstart, const int32_t *__restrict__ useg,
-                              const int32_t *__restrict__ segn, int32_t *__restrict__ tcount) {
-    __shared__ int wsum[TILE_WARPS];
-    const int t = blockIdx.x;
+// Particles per tile (sum of its segment counts), a warp per tile.
+__global__ void __launch_bounds__(256) k_tile_counts(const int32_t *__restrict__ bstart, const int32_t *__restrict__ useg,
+                                                     const int32_t *__restrict__ segn, int ntiles,
+                                                     int32_t *__restrict__ tcount) {
+    const int t = blockIdx.x * TILE_WARPS + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+    if (t >= ntiles) return;
     const int64_t sb = bstart[t] / SEG;
     const int u = useg[t];
     int c = 0;
-    for (int j = threadIdx.x; j < u; j += blockDim.x) c += segn[sb + j];
+    for (int j = lane; j < u; j += 32) c += segn[sb + j];
     for (int o = 16; o > 0; o >>= 1) c += __shfl_down_sync(FULL, c, o);
-    if ((threadIdx.x & 31) == 0) wsum[threadIdx.x >> 5] = c;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        int tot = 0;
-        for (int w = 0; w < (int)(blockDim.x >> 5); ++w) tot += wsum[w];
-        tcount[t] = tot;
-    }
+    if (lane == 0) tcount[t] = c;
 }
 
 // Self-test of the bounded wait (no counterpart in the paper): one thread
@@ -1819,7 +1814,10 @@ static TileArgs<R> tile_args(pic_t *h) {
         p.removed = (unsigned long long *)(h->d_removed + s);
         p.cr = S.carry[b]; p.mcr = S.carry[m]; p.ocr = S.carry[o];
         p.ccap = S.cap;
-        p.q = (R)S.q; p.m = (R)S.m; p.kq = (R)(S.q * h->cfg.dt / (2.0 * S.m));
+        p.q = (R)S.q;
+        const R kq = (R)(S.q * h->cfg.dt / (2.0 * S.m));
+        p.ke = R(0.5) * kq;
+        p.kb = R(0.25) * kq;
         p.cq2 = (R)(S.q * S.q * h->cfg.dt * h->cfg.dt / (4.0 * S.m));
         p.hq = (R)(S.q * h->cfg.dt * h->cfg.dt / (4.0 * S.m));
     }
@@ -1962,54 +1960,86 @@ int batch_regroup(BatchScratch &b, pic_t **hs, int n) {
 }
 
 // Node moments from the cell sums of the FP64 deposit (deposit_fp64_cell):
-// every cell of a listed tile (list == nullptr: of every tile) adds its corner
+// every cell of a listed tile adds its corner
 // values (0,0) A - X - Y + Z, (1,0) X - Z, (0,1) Y - Z, (1,1) Z of each moment
 // into the node moments (zero before: the field solve or the deposit at rest
-// has cleared them) and zeroes its sums.  A cell is read by one thread only;
-// the corner nodes take L2 reductions.
+// has cleared them) and zeroes its sums; the corner nodes take L2 reductions.
+// A thread per (tile, cell, moment), so that every sum of a tile is in flight at
+// once (a thread per cell, its 13 moments in turn: 87 us for the 98,000 cells of a
+// thin foil; now 24 us).
 __global__ void __launch_bounds__(256) k_cell_moments(const int32_t *__restrict__ list,
                                                       const int32_t *__restrict__ list_n, int tnx, int tny, int ntx,
-                                                      int ntiles, GridArgs<double> g, double *__restrict__ Mc,
+                                                      GridArgs<double> g, double *__restrict__ Mc,
                                                       double *__restrict__ M, const int32_t *__restrict__ guard) {
     if (guard && (*guard & 3)) return;
-    const int tc = tnx * tny;
-    const int64_t ncell = (int64_t)g.nx * g.ny;
-    const int64_t total = (int64_t)(list ? list_n[0] : ntiles) * tc;
+    const int tc = tnx * tny, tm = tc * NMOM;
+    const int64_t total = (int64_t)list_n[0] * tm;
     for (int64_t w = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; w < total; w += (int64_t)gridDim.x * blockDim.x) {
-        const int li = (int)(w / tc), c = (int)(w - (int64_t)li * tc);
-        const int T = list ? list[li] : li, tx = T % ntx, ty = T / ntx;
+        const int li = (int)(w / tm), r = (int)(w - (int64_t)li * tm), c = r / NMOM, k = r - c * NMOM;
+        const int T = list[li], tx = T % ntx, ty = T / ntx;
         const int ly = c / tnx;
         const int cx = tx * tnx + (c - ly * tnx), cy = ty * tny + ly;
         if (cx >= g.nx || cy >= g.ny) continue;
         const int64_t cell = (int64_t)cy * g.nx + cx;
-        const int64_t n00 = node_of(g, cx, cy, 0, 0), n10 = node_of(g, cx, cy, 1, 0);
-        const int64_t n01 = node_of(g, cx, cy, 0, 1), n11 = node_of(g, cx, cy, 1, 1);
-#pragma unroll
-        for (int k = 0; k < NMOM; ++k) {
-            V4<double> *q = (V4<double> *)(Mc + ((int64_t)k * ncell + cell) * 4);
-            const V4<double> s = *q;
-            const double A = s.x, X = s.y, Y = s.z, Z = s.w;
-            if (A == 0.0 && X == 0.0 && Y == 0.0 && Z == 0.0) continue;
-            *q = V4<double>{0.0, 0.0, 0.0, 0.0};
-            double *m = M + (int64_t)k * g.nnode;
-            atomicAdd(m + n00, (A - X) - (Y - Z));
-            atomicAdd(m + n10, X - Z);
-            atomicAdd(m + n01, Y - Z);
-            atomicAdd(m + n11, Z);
-        }
+        V4<double> *q = (V4<double> *)(Mc + (cell * NMOM + k) * 4);
+        const V4<double> s = *q;
+        const double A = s.x, X = s.y, Y = s.z, Z = s.w;
+        if (A == 0.0 && X == 0.0 && Y == 0.0 && Z == 0.0) continue;
+        *q = V4<double>{0.0, 0.0, 0.0, 0.0};
+        double *m = M + (int64_t)k * g.nnode;
+        atomicAdd(m + node_of(g, cx, cy, 0, 0), (A - X) - (Y - Z));
+        atomicAdd(m + node_of(g, cx, cy, 1, 0), X - Z);
+        atomicAdd(m + node_of(g, cx, cy, 0, 1), Y - Z);
+        atomicAdd(m + node_of(g, cx, cy, 1, 1), Z);
     }
 }
 
-int cell_moments(pic_t *h, bool all) {
+int cell_moments(pic_t *h) {
     if (!h->Mc) return 0;
     int dev = 0, nsm = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-    k_cell_moments<<<(unsigned)(nsm > 0 ? 4 * nsm : 512), 256, 0, h->st>>>(
-        all ? nullptr : h->touch_list, h->list_n, h->tnx, h->tny, h->ntx, h->ntiles, grid_args<double>(h), h->Mc,
-        (double *)h->M, all ? nullptr : h->guard);
+    k_cell_moments<<<(unsigned)(nsm > 0 ? 8 * nsm : 1024), 256, 0, h->st>>>(
+        h->touch_list, h->list_n, h->tnx, h->tny, h->ntx, grid_args<double>(h), h->Mc, (double *)h->M, h->guard);
     count_launch(h);
     return check_launch("k_cell_moments");
+}
+
+// Node tiles a deposit at rest wrote: those a particle's nodes reach from an
+// occupied tile (tiles T - dl .. T + dh on each axis).
+__global__ void k_rest_touch(UsegPtrs u, int nsp, int ntx, int nty, int periodic_x, uint8_t *__restrict__ touched,
+                             int32_t *__restrict__ list, int32_t *__restrict__ list_n, int dlx, int dly, int dhx, int dhy) {
+    const int T = blockIdx.x * blockDim.x + threadIdx.x;
+    if (T >= ntx * nty) return;
+    const int tx = T % ntx, ty = T / ntx;
+    bool touch = false;
+    for (int dy = -dly; dy <= dhy && !touch; ++dy) {
+        const int y = imod(ty + dy, nty);
+        for (int dx = -dlx; dx <= dhx && !touch; ++dx) {
+            int x = tx + dx;
+            if (periodic_x) x = imod(x, ntx);
+            if (x < 0 || x >= ntx) continue;
+            for (int s = 0; s < nsp; ++s) touch = touch || u.p[s][y * ntx + x] > 0;
+        }
+    }
+    touched[T] = touch ? 1 : 0;
+    if (touch) list[atomicAdd(list_n, 1)] = T;
+}
+
+int rest_touch(pic_t *h) {
+    UsegPtrs u;
+    for (int s = 0; s < PIC_MAX_SPECIES; ++s) u.p[s] = (s < h->nsp) ? h->sp[s].useg[h->sp[s].scur] : nullptr;
+    // nodes c + lo .. c + hi of a particle in cell c (as in touch_map; the splines' may cross a ragged last
+    // tile into the one after it)
+    const int lo = -(h->shape / 2), hi = (h->shape + 2) / 2, one = h->shape > 1 ? 1 : 0;
+    if (cudaMemsetAsync(h->list_n, 0, sizeof(int32_t), h->st) != cudaSuccess) return check_launch("tile lists");
+    k_rest_touch<<<(h->ntiles + 255) / 256, 256, 0, h->st>>>(
+        u, h->nsp, h->ntx, h->nty, h->periodic_x ? 1 : 0, h->touched, h->touch_list, h->list_n,
+        one + (hi + h->tnx - 1) / h->tnx, one + (hi + h->tny - 1) / h->tny, one + (-lo + h->tnx - 1) / h->tnx,
+        one + (-lo + h->tny - 1) / h->tny);
+    count_launch(h);
+    h->touch_all = false;
+    return check_launch("k_rest_touch");
 }
 
 // The push's work items in one block, for up to PREP_ONE_BLOCK (species, tile)
@@ -2197,7 +2227,8 @@ int regroup_tiles(pic_t *h) { return h->fp32 ? regroup_t<float>(h) : regroup_t<d
 
 int tile_counts(pic_t *h, int s) {
     SpeciesBuf &S = h->sp[s];
-    k_tile_counts<<<h->ntiles, 256, 0, h->st>>>(S.bstart, S.useg[S.scur], S.segn[S.scur], S.tcount);
+    k_tile_counts<<<(h->ntiles + TILE_WARPS - 1) / TILE_WARPS, 256, 0, h->st>>>(S.bstart, S.useg[S.scur], S.segn[S.scur],
+                                                                              h->ntiles, S.tcount);
     count_launch(h);
     return check_launch("k_tile_counts");
 }
