@@ -34,12 +34,50 @@ __global__ void k_ion_seg_counts(const int32_t *__restrict__ bstart, const int32
     for (int64_t j = s0 + threadIdx.x; j < s1; j += blockDim.x) cnt[j] = (j - s0 < u) ? segn[j] : 0;
 }
 
+struct IonChain32 {
+    float lead, expo, K, fmax, field_au;   // lead = log2(|C|^2 Ip dt)
+};
+
+// u < P in FP64, u = r 2^-53.
+__device__ inline bool ion_decide(double F2, const IonChain &c, uint64_t r) {
+    const double F = sqrt(F2) * c.field_au;
+    double prob = 0.0;
+    if (F > 0.0) {
+        const double Fp = F < c.fmax ? F : c.fmax;
+        const double w = c.c2ip * pow(c.K / Fp, c.expo) * exp(-c.K / (3.0 * Fp));
+        prob = -expm1(-w * c.dt_au);
+    }
+    return (double)r * 0x1.0p-53 < prob;
+}
+
+// The same decision from FP32 bounds of P where they decide it: +1 yes, 0 no, -1
+// undecided.  log2 of w dt is a sum of three terms, each off by a few 1e-7 of its
+// size (the rounding of r = K / F', under 4e-7, changes expo log2 r by expo
+// 6e-7); the margin is 4e-6 of their sizes' sum.  Whatever is outside FP32's range
+// or not a number fails every comparison and stays undecided.
+__device__ inline int ion_bounds(double F2, const IonChain32 &c, uint64_t r) {
+    if (F2 == 0.0) return 0;
+    const float f2 = (float)F2;
+    if (!(f2 > 1e-30f && f2 < 1e30f)) return -1;
+    const float q = c.K / fminf(sqrtf(f2) * c.field_au, c.fmax);
+    const float t1 = c.expo * log2f(q), t2 = -0.480898347f * q;   // log2(e) / 3
+    const float x = t1 + t2 + c.lead, m = 4e-6f * (fabsf(t1) + fabsf(t2) + fabsf(c.lead) + fabsf(c.expo) + 1.0f);
+    const float u = (float)(uint32_t)(r >> 29) * 0x1.0p-24f;      // u <= the number < u + 2^-24
+    const float hi = -expm1f(-exp2f(x + m)), lo = -expm1f(-exp2f(x - m));
+    if (u > hi * 1.00001f + 1e-30f) return 0;
+    if (u + 0x1.0p-24f < lo * 0.99999f) return 1;
+    return -1;
+}
+
 // One thread per slot: the decision of the particle in that slot.  prefix[seg]
-// is the index of the segment's first particle in the species' order.
+// is the index of the segment's first particle in the species' order.  |E|^2 is
+// gathered in FP64; the rate's power and exponentials run in FP64 only for the
+// particles that FP32 bounds leave undecided (a few in 10,000), which with every
+// lane in FP64 took most of the pass: 0.8M particles 245 -> 38 us.
 template <typename R>
 __global__ void k_ion_mark(GridArgs<R> g, int64_t nslot, const int32_t *__restrict__ prefix,
                            const int32_t *__restrict__ cell, const R *__restrict__ ox, const R *__restrict__ oy,
-                           const V4<R> *__restrict__ E, IonChain c, int64_t step, uint64_t seed,
+                           const V4<R> *__restrict__ E, const IonChain c, const IonChain32 c32, int64_t step, uint64_t seed,
                            int32_t *__restrict__ flag_by_index, int32_t *__restrict__ slot_by_index,
                            int32_t *__restrict__ removed) {
     const int64_t slot = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -61,17 +99,12 @@ __global__ void k_ion_mark(GridArgs<R> g, int64_t nslot, const int32_t *__restri
     const double Ex = w00 * (double)a.x + w10 * (double)b.x + w01 * (double)d.x + w11 * (double)e.x;
     const double Ey = w00 * (double)a.y + w10 * (double)b.y + w01 * (double)d.y + w11 * (double)e.y;
     const double Ez = w00 * (double)a.z + w10 * (double)b.z + w01 * (double)d.z + w11 * (double)e.z;
-    const double F = sqrt(Ex * Ex + Ey * Ey + Ez * Ez) * c.field_au;
-    double prob = 0.0;
-    if (F > 0.0) {
-        const double Fp = F < c.fmax ? F : c.fmax;
-        const double w = c.c2ip * pow(c.K / Fp, c.expo) * exp(-c.K / (3.0 * Fp));
-        prob = -expm1(-w * c.dt_au);
-    }
+    const double F2 = Ex * Ex + Ey * Ey + Ez * Ez;
     uint64_t x[4] = {(uint64_t)idx, (uint64_t)c.species, (uint64_t)step, 0ull};
     philox4x64_10(x, seed, 0ull);
-    const double u = (double)(x[0] >> 11) * 0x1.0p-53;
-    const int32_t f = (u < prob) ? 1 : 0;
+    const uint64_t r = x[0] >> 11;
+    int32_t f = ion_bounds(F2, c32, r);
+    if (f < 0) f = ion_decide(F2, c, r) ? 1 : 0;
     flag_by_index[idx] = f;
     slot_by_index[idx] = (int32_t)slot;
     removed[slot] = f;
@@ -155,8 +188,9 @@ static int ion_chain_t(pic_t *h, const IonChain &c, uint64_t seed, int32_t *scel
     if (n == 0) return 0;
     GridArgs<R> g = grid_args<R>(h);
     const int b = S.bins;
+    const IonChain32 c32{(float)log2(c.c2ip * c.dt_au), (float)c.expo, (float)c.K, (float)c.fmax, (float)c.field_au};
     k_ion_mark<R><<<(unsigned)((S.cap + 255) / 256), 256, 0, h->st>>>(
-        g, S.cap, prefix, S.cell[b], (const R *)S.ox[b], (const R *)S.oy[b], (const V4<R> *)h->E[h->ecur], c, h->step,
+        g, S.cap, prefix, S.cell[b], (const R *)S.ox[b], (const R *)S.oy[b], (const V4<R> *)h->E[h->ecur], c, c32, h->step,
         seed, flag, slot_by_index, removed);
     count_launch(h);
     if (int rc = ion_chain_t_launch_check("k_ion_mark")) return rc;
