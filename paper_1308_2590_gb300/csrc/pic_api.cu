@@ -7,6 +7,7 @@
 #include <stdlib.h>
 #include <string.h>
 
+#include <algorithm>
 #include <mutex>
 #include <vector>
 
@@ -152,6 +153,12 @@ static int dalloc(void **p, size_t bytes, const char *what) {
     return 0;
 }
 
+int Slab::commit(void **base, const char *what) {
+    if (int rc = dalloc(base, bytes, what)) return rc;
+    for (const Part &q : parts) *q.p = (char *)*base + q.at;
+    return 0;
+}
+
 int ensure_stage_doubles(pic_t *h, int64_t ndoubles) {
     if (ndoubles <= h->stage_cap) return 0;
     cudaStreamSynchronize(h->st);
@@ -173,26 +180,15 @@ static int64_t init_stage_doubles(const pic_t *h) {
 }
 
 static void free_particle_buffers(SpeciesBuf &S) {
+    cudaFree(S.mem);
+    S.mem = nullptr;
     for (int b = 0; b < 3; ++b) {
-        cudaFree(S.cell[b]); cudaFree(S.ox[b]); cudaFree(S.oy[b]);
-        cudaFree(S.ux[b]); cudaFree(S.uy[b]); cudaFree(S.uz[b]); cudaFree(S.w[b]); cudaFree(S.carry[b]);
         S.cell[b] = nullptr; S.ox[b] = S.oy[b] = S.ux[b] = S.uy[b] = S.uz[b] = S.w[b] = nullptr;
         S.carry[b] = nullptr;
     }
-    cudaFree(S.segd);
-    cudaFree(S.segn[0]);
-    cudaFree(S.segn[1]);
-    cudaFree(S.segml);
     S.segd = nullptr;
     S.segn[0] = S.segn[1] = S.segml = nullptr;
     S.cap = 0;
-}
-
-static void free_species(SpeciesBuf &S) {
-    free_particle_buffers(S);
-    cudaFree(S.bstart); cudaFree(S.useg[0]); cudaFree(S.useg[1]); cudaFree(S.tcount); cudaFree(S.cstart);
-    cudaFree(S.cend);
-    S.bstart = S.useg[0] = S.useg[1] = S.tcount = S.cstart = S.cend = nullptr;
 }
 
 // Grow a species' three buffer sets to at least `slots` slots, keeping the
@@ -206,26 +202,16 @@ static int ensure_species_capacity(pic_t *h, int s, int64_t slots) {
     }
     int64_t cap = slots;
     SpeciesBuf N;
-    size_t rb = h->rs * cap;
-    int rc = 0;
-    for (int b = 0; b < 3 && !rc; ++b) {
-        rc = dalloc((void **)&N.cell[b], cap * sizeof(int32_t), "particles");
-        if (!rc) rc = dalloc(&N.ox[b], rb, "particles");
-        if (!rc) rc = dalloc(&N.oy[b], rb, "particles");
-        if (!rc) rc = dalloc(&N.ux[b], rb, "particles");
-        if (!rc) rc = dalloc(&N.uy[b], rb, "particles");
-        if (!rc) rc = dalloc(&N.uz[b], rb, "particles");
-        if (!rc) rc = dalloc(&N.w[b], rb, "particles");
-        if (!rc && !h->fp32) rc = dalloc((void **)&N.carry[b], (size_t)NCARRY * cap * sizeof(double), "particles");
+    const size_t rb = h->rs * cap, sb = (cap / SEG) * sizeof(int32_t);
+    Slab slab;
+    for (int b = 0; b < 3; ++b) {
+        slab.add(&N.cell[b], cap * sizeof(int32_t));
+        for (void **q : {&N.ox[b], &N.oy[b], &N.ux[b], &N.uy[b], &N.uz[b], &N.w[b]}) slab.add(q, rb);
+        if (!h->fp32) slab.add(&N.carry[b], (size_t)NCARRY * cap * sizeof(double));
     }
-    if (!rc) rc = dalloc((void **)&N.segd, (cap / SEG) * sizeof(unsigned long long), "segment counts");
-    if (!rc) rc = dalloc((void **)&N.segn[0], (cap / SEG) * sizeof(int32_t), "segment counts");
-    if (!rc) rc = dalloc((void **)&N.segn[1], (cap / SEG) * sizeof(int32_t), "segment counts");
-    if (!rc) rc = dalloc((void **)&N.segml, (cap / SEG) * sizeof(int32_t), "segment counts");
-    if (rc) {
-        free_particle_buffers(N);
-        return rc;
-    }
+    slab.add(&N.segd, (cap / SEG) * sizeof(unsigned long long));
+    for (int32_t **q : {&N.segn[0], &N.segn[1], &N.segml}) slab.add(q, sb);
+    if (int rc = slab.commit(&N.mem, "particles")) return rc;
     if (S.cap > 0) {
         int c = S.bins;
         int64_t keep = S.cap;
@@ -241,6 +227,7 @@ static int ensure_species_capacity(pic_t *h, int s, int64_t slots) {
         cudaStreamSynchronize(h->st);
     }
     free_particle_buffers(S);
+    S.mem = N.mem;
     for (int b = 0; b < 3; ++b) {
         S.cell[b] = N.cell[b]; S.ox[b] = N.ox[b]; S.oy[b] = N.oy[b];
         S.ux[b] = N.ux[b]; S.uy[b] = N.uy[b]; S.uz[b] = N.uz[b]; S.w[b] = N.w[b];
@@ -360,15 +347,10 @@ static int destroy_impl(pic_t *h) {
         if (f.freed) cudaEventDestroy(f.freed);
     }
     if (h->pf_st) cudaStreamDestroy(h->pf_st);
-    for (int s = 0; s < PIC_MAX_SPECIES; ++s) free_species(h->sp[s]);
-    void *bufs[] = {h->E[0], h->E[1], h->H[0], h->H[1], h->Ehalf, h->B[0], h->B[1], h->M, h->Mlo, h->Mfix, h->Mc, h->cn,
-                    h->cn_red, h->cn_out, h->d_removed, h->d_flags, h->d_step_flags, h->keys[0], h->keys[1],
-                    h->vals[0], h->vals[1], h->hist, h->stage, h->d_diag, h->chunk_prefix, h->ticket,
-                    h->d_bad, h->scan_sums, h->occ, h->touched, h->touch_list, h->rg_list, h->list_n,
-                    h->ion_cell, h->ion_val, h->ion_dcell, h->ion_dval};
+    for (int s = 0; s < PIC_MAX_SPECIES; ++s) free_particle_buffers(h->sp[s]);
+    void *bufs[] = {h->mem, h->sort_mem, h->stage, h->ion_cell, h->ion_val, h->ion_dcell, h->ion_dval};
     for (void *p : bufs) cudaFree(p);
     if (h->h_step_flags) cudaFreeHost(h->h_step_flags);
-    if (h->h_diag) cudaFreeHost(h->h_diag);
     for (cudaEvent_t ev : h->ev_flags)
         if (ev) cudaEventDestroy(ev);
     if (h->ev_batch) cudaEventDestroy(h->ev_batch);
@@ -549,58 +531,56 @@ extern "C" PIC_API int pic_init(const pic_config *cfg, pic_t **out) {
     if (int rc = validate_config(c)) return rc;
     pic_t *h = new pic_t();
     setup_geometry(h, c);
-    size_t v4 = 4 * h->rs;
-    int rc = 0;
-    for (int k = 0; k < 2 && !rc; ++k) rc = dalloc(&h->E[k], h->nnode * v4, "E");
-    for (int k = 0; k < 2 && !rc; ++k) rc = dalloc(&h->H[k], h->ncell * v4, "H");
-    for (int k = 0; k < 2 && !rc; ++k) rc = dalloc(&h->B[k], h->npad * v4, "B");
-    if (!rc) rc = dalloc(&h->Ehalf, h->npad * v4, "Ehalf");
-    if (!rc) rc = dalloc(&h->M, (size_t)NMOM * h->nnode * h->rs, "moments");
-    if (!rc && h->fp32) rc = dalloc(&h->Mlo, (size_t)NMOM * h->nnode * h->rs, "moment compensation");
-    if (!rc && h->det) rc = dalloc((void **)&h->Mfix, (size_t)NMOM * h->nnode * 8, "fixed-point moments");
-    if (!rc && uses_cell_sums(h)) {
-        rc = dalloc((void **)&h->Mc, cell_sum_bytes(h), "cell moment sums");
-        if (!rc && cudaMemset(h->Mc, 0, cell_sum_bytes(h)) != cudaSuccess) rc = check_launch("cell moment sums");
-    }
-    if (!rc) rc = dalloc((void **)&h->d_removed, PIC_MAX_SPECIES * sizeof(int64_t), "counters");
-    if (!rc) rc = dalloc((void **)&h->d_flags, sizeof(int32_t), "flags");
-    if (!rc) rc = dalloc((void **)&h->d_bad, PIC_MAX_SPECIES * sizeof(unsigned long long), "load check");
-    if (!rc) rc = dalloc((void **)&h->scan_sums, (size_t)scan_sums_entries() * sizeof(uint32_t), "scan scratch");
-    if (!rc) rc = dalloc((void **)&h->d_step_flags, 2 * sizeof(int32_t), "flags");
-    if (!rc) rc = dalloc((void **)&h->occ, (size_t)h->ntiles, "tile occupancy");
-    if (!rc) rc = dalloc((void **)&h->touched, (size_t)h->ntiles, "touched tiles");
-    if (!rc) rc = dalloc((void **)&h->touch_list, (size_t)h->ntiles * sizeof(int32_t), "touched tiles");
-    if (!rc) rc = dalloc((void **)&h->rg_list, (size_t)h->ntiles * sizeof(int32_t), "regroup tiles");
-    if (!rc) rc = dalloc((void **)&h->list_n, (2 + PIC_MAX_SPECIES) * sizeof(int32_t), "tile lists");
-    size_t tb = (size_t)(h->ntiles + 1) * sizeof(int32_t);
-    for (int s = 0; s < h->nsp && !rc; ++s) {
+    const size_t v4 = 4 * h->rs, mb = (size_t)NMOM * h->nnode, nt = (size_t)h->ntiles, tb = (nt + 1) * sizeof(int32_t);
+    Slab slab;
+    for (int k = 0; k < 2; ++k) slab.add(&h->E[k], h->nnode * v4);
+    for (int k = 0; k < 2; ++k) slab.add(&h->H[k], h->ncell * v4);
+    for (int k = 0; k < 2; ++k) slab.add(&h->B[k], h->npad * v4);
+    slab.add(&h->Ehalf, h->npad * v4);
+    slab.add(&h->M, mb * h->rs);
+    if (h->fp32) slab.add(&h->Mlo, mb * h->rs);
+    if (h->det) slab.add(&h->Mfix, mb * 8);
+    if (uses_cell_sums(h)) slab.add(&h->Mc, cell_sum_bytes(h));
+    slab.add(&h->d_removed, PIC_MAX_SPECIES * sizeof(int64_t));
+    slab.add(&h->d_flags, sizeof(int32_t));
+    slab.add(&h->d_step_flags, 2 * sizeof(int32_t));
+    slab.add(&h->list_n, (2 + PIC_MAX_SPECIES) * sizeof(int32_t));
+    for (int s = 0; s < h->nsp; ++s) {
         SpeciesBuf &S = h->sp[s];
-        rc = dalloc((void **)&S.bstart, tb, "bins");
-        if (!rc) rc = dalloc((void **)&S.useg[0], tb, "bins");
-        if (!rc) rc = dalloc((void **)&S.useg[1], tb, "bins");
-        if (!rc) rc = dalloc((void **)&S.tcount, tb, "bins");
-        if (!rc) rc = dalloc((void **)&S.cstart, tb, "bins");
-        if (!rc) rc = dalloc((void **)&S.cend, tb, "bins");
+        for (int32_t **q : {&S.bstart, &S.useg[0], &S.useg[1], &S.tcount}) slab.add(q, tb);
     }
-    if (!rc) rc = dalloc((void **)&h->chunk_prefix, ((size_t)h->nsp * h->ntiles + 1) * sizeof(int32_t), "work list");
-    if (!rc) rc = dalloc((void **)&h->ticket, PIC_MAX_SPECIES * sizeof(int32_t), "work queue");
+    if (c.field_mode == PIC_FIELD_CN) slab.add(&h->cn_out, 3 * sizeof(double));
+    const size_t zeroed = slab.bytes;   // all of the above starts at zero
+    for (int s = 0; s < h->nsp; ++s) {
+        slab.add(&h->sp[s].cstart, tb);
+        slab.add(&h->sp[s].cend, tb);
+    }
+    slab.add(&h->d_bad, PIC_MAX_SPECIES * sizeof(unsigned long long));
+    slab.add(&h->scan_sums, (size_t)scan_sums_entries() * sizeof(uint32_t));
+    slab.add(&h->occ, nt);
+    slab.add(&h->touched, nt);
+    slab.add(&h->touch_list, nt * sizeof(int32_t));
+    slab.add(&h->rg_list, nt * sizeof(int32_t));
+    slab.add(&h->nbr, 9 * nt * sizeof(int32_t));
+    slab.add(&h->chunk_prefix, ((size_t)h->nsp * nt + 1) * sizeof(int32_t));
+    slab.add(&h->ticket, PIC_MAX_SPECIES * sizeof(int32_t));
     h->diag_cap = diag_scratch_doubles(h->nsp, h->ntiles);
-    if (!rc) rc = dalloc((void **)&h->d_diag, h->diag_cap * sizeof(double), "diagnostics");
-    if (!rc && c.field_mode == PIC_FIELD_CN) {
-        rc = dalloc(&h->cn, cn_bytes(h), "CN solver vectors");
+    slab.add(&h->d_diag, h->diag_cap * sizeof(double));
+    if (c.field_mode == PIC_FIELD_CN) {
         int dev = 0, nsm = 0;
         cudaGetDevice(&dev);
         cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
         h->cn_red_cap = nsm * 8;
-        if (!rc) rc = dalloc((void **)&h->cn_red, 6 * (size_t)h->cn_red_cap * sizeof(double), "CN reductions");
-        if (!rc) rc = dalloc((void **)&h->cn_out, 3 * sizeof(double), "CN status");
+        slab.add(&h->cn, cn_bytes(h));
+        slab.add(&h->cn_red, 6 * (size_t)h->cn_red_cap * sizeof(double));
     }
-    if (!rc && (cudaHostAlloc((void **)&h->h_step_flags, 8 * sizeof(int32_t), cudaHostAllocDefault) != cudaSuccess ||
-                cudaHostAlloc(&h->h_diag, diag_record_bytes(), cudaHostAllocDefault) != cudaSuccess)) {
+    int rc = slab.commit(&h->mem, "fields, moments and bins");
+    if (!rc && cudaHostAlloc((void **)&h->h_step_flags, 64 + diag_record_bytes(), cudaHostAllocDefault) != cudaSuccess) {
         cudaGetLastError();
         set_error("pinned host allocation failed");
         rc = PIC_ERR_OOM;
     }
+    if (!rc) h->h_diag = (char *)h->h_step_flags + 64;
     if (!rc && (cudaEventCreateWithFlags(&h->ev_flags[0], cudaEventDisableTiming) != cudaSuccess ||
                 cudaEventCreateWithFlags(&h->ev_flags[1], cudaEventDisableTiming) != cudaSuccess ||
                 !create_events(&h->ev_batch, 1) || !create_events(&h->ev_load, 1) ||
@@ -618,17 +598,9 @@ extern "C" PIC_API int pic_init(const pic_config *cfg, pic_t **out) {
         destroy_impl(h);
         return rc;
     }
-    void *zero[] = {h->E[0], h->E[1], h->H[0], h->H[1], h->B[0], h->B[1], h->Ehalf};
-    size_t zb[] = {h->nnode * v4, h->nnode * v4, h->ncell * v4, h->ncell * v4, h->npad * v4, h->npad * v4, h->npad * v4};
-    for (int k = 0; k < 7; ++k) cudaMemsetAsync(zero[k], 0, zb[k], h->st);
-    clear_moments(h);
-    cudaMemsetAsync(h->d_removed, 0, PIC_MAX_SPECIES * sizeof(int64_t), h->st);
-    cudaMemsetAsync(h->d_flags, 0, sizeof(int32_t), h->st);
-    cudaMemsetAsync(h->d_step_flags, 0, 2 * sizeof(int32_t), h->st);
-    for (int s = 0; s < h->nsp; ++s) init_empty_bins(h, s);
-    if (h->cn_out) cudaMemsetAsync(h->cn_out, 0, 3 * sizeof(double), h->st);
-    if (cudaStreamSynchronize(h->st) != cudaSuccess) {
-        rc = check_launch("pic_init");
+    if (cudaMemsetAsync(h->mem, 0, zeroed, h->st) != cudaSuccess) rc = check_launch("pic_init");
+    if (rc || cudaStreamSynchronize(h->st) != cudaSuccess) {
+        if (!rc) rc = check_launch("pic_init");
         destroy_impl(h);
         return rc ? rc : PIC_ERR_CUDA;
     }
@@ -636,6 +608,13 @@ extern "C" PIC_API int pic_init(const pic_config *cfg, pic_t **out) {
         destroy_impl(h);
         return rc;
     }
+    int64_t most = 0;
+    for (int s = 0; s < h->nsp; ++s) most = std::max<int64_t>(most, c.capacity[s]);
+    if (most > 0 && slots_needed(h, most) <= (1ll << 30))   // the sort scratch of the largest species, once
+        if (int r = ensure_sort_capacity(h, 2 * slots_needed(h, most))) {
+            destroy_impl(h);
+            return r;
+        }
     for (int s = 0; s < h->nsp; ++s)
         if (c.capacity[s] > 0) {
             if (int r = ensure_species_capacity(h, s, slots_needed(h, c.capacity[s]))) {

@@ -470,27 +470,17 @@ int ensure_sort_capacity(pic_t *h, int64_t n) {
     if (n <= h->sort_cap) return 0;
     int64_t cap = n + n / 8 + 4096;
     cudaStreamSynchronize(h->st);
+    cudaFree(h->sort_mem);
+    h->sort_mem = nullptr;
+    h->sort_cap = 0;
+    const int64_t hist_entries = RADIX * sort_blocks(cap) + 2 * SCAN_IPB;
+    Slab slab;
     for (int k = 0; k < 2; ++k) {
-        cudaFree(h->keys[k]);
-        cudaFree(h->vals[k]);
-        h->keys[k] = h->vals[k] = nullptr;
+        slab.add(&h->keys[k], cap * sizeof(uint32_t));
+        slab.add(&h->vals[k], cap * sizeof(uint32_t));
     }
-    cudaFree(h->hist);
-    h->hist = nullptr;
-    int64_t hist_entries = RADIX * sort_blocks(cap) + 2 * SCAN_IPB;
-    for (int k = 0; k < 2; ++k) {
-        if (cudaMalloc(&h->keys[k], cap * sizeof(uint32_t)) != cudaSuccess ||
-            cudaMalloc(&h->vals[k], cap * sizeof(uint32_t)) != cudaSuccess) {
-            set_error("sort scratch allocation of %lld items failed", (long long)cap);
-            cudaGetLastError();
-            return PIC_ERR_OOM;
-        }
-    }
-    if (cudaMalloc(&h->hist, hist_entries * sizeof(uint32_t)) != cudaSuccess) {
-        set_error("sort histogram allocation failed");
-        cudaGetLastError();
-        return PIC_ERR_OOM;
-    }
+    slab.add(&h->hist, hist_entries * sizeof(uint32_t));
+    if (int rc = slab.commit(&h->sort_mem, "sort scratch")) return rc;
     h->sort_cap = cap;
     h->hist_cap = hist_entries;
     return 0;

@@ -1676,11 +1676,6 @@ static int neighbour_table(pic_t *h) {
         tab[(size_t)t * 9] = n;
         for (int q = 0; q < n; ++q) tab[(size_t)t * 9 + 1 + q] = nb[q];
     }
-    if (cudaMalloc(&h->nbr, tab.size() * sizeof(int32_t)) != cudaSuccess) {
-        cudaGetLastError();
-        set_error("neighbour table allocation failed");
-        return PIC_ERR_OOM;
-    }
     if (cudaMemcpy(h->nbr, tab.data(), tab.size() * sizeof(int32_t), cudaMemcpyHostToDevice) != cudaSuccess) {
         cudaGetLastError();
         set_error("neighbour table upload failed");
@@ -1776,8 +1771,6 @@ void tile_free(pic_t *h) {
     if (h->items) cudaFree(h->items);
     h->items = nullptr;
     h->items_cap = 0;
-    if (h->nbr) cudaFree(h->nbr);
-    h->nbr = nullptr;
 }
 
 template <typename R>
