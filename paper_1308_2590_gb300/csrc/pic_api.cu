@@ -285,8 +285,8 @@ static int pending_flags(pic_t *h, int32_t *f) {
         set_error("step flags: %s", cudaGetErrorString(e));
         return PIC_ERR_CUDA;
     }
-    *f = h->h_step_flags[4 * p];
-    return flag_error(h->h_step_flags[4 * p + 1]);
+    *f = h->h_step_flags[4 * p + p];
+    return flag_error(h->h_step_flags[4 * p + 2]);
 }
 
 // Regroup every species with the full sort from the pending step's push-time
@@ -489,9 +489,9 @@ static uint64_t estimate_bytes(const pic_t *h, const int64_t *n) {
     uint64_t b = 2 * nn * v4 + 2 * nc * v4 + 3 * np * v4;
     b += (uint64_t)NMOM * nn * h->rs * (h->fp32 ? 2 : 1) + (h->det ? (uint64_t)NMOM * nn * 8 : 0);
     if (uses_cell_sums(h)) b += cell_sum_bytes(h);
-    b += (uint64_t)h->nsp * 6 * (h->ntiles + 1) * 4 + ((uint64_t)h->nsp * h->ntiles + 1) * 4 + 256;
+    b += (uint64_t)h->nsp * 6 * (h->ntiles + 1) * 4 + 256;
     b += (uint64_t)h->ntiles * 9 * 4 + 8 + (uint64_t)scan_sums_entries() * 4;   // neighbour table, load check, scan
-    b += 10ull * (uint64_t)h->ntiles + 8;                                         // occupancy, touched and regroup tiles
+    b += 19ull * (uint64_t)h->ntiles;                                             // touched and regroup tiles
     b += (uint64_t)diag_scratch_doubles(h->nsp, h->ntiles) * 8;
     if (h->cfg.field_mode == PIC_FIELD_CN) b += cn_bytes(h) + 6ull * 8 * 1024 * 8 + 24;
     int64_t stage = init_stage_doubles(h), maxcap = 0;
@@ -542,9 +542,8 @@ extern "C" PIC_API int pic_init(const pic_config *cfg, pic_t **out) {
     if (h->det) slab.add(&h->Mfix, mb * 8);
     if (uses_cell_sums(h)) slab.add(&h->Mc, cell_sum_bytes(h));
     slab.add(&h->d_removed, PIC_MAX_SPECIES * sizeof(int64_t));
-    slab.add(&h->d_flags, sizeof(int32_t));
-    slab.add(&h->d_step_flags, 2 * sizeof(int32_t));
-    slab.add(&h->list_n, (2 + PIC_MAX_SPECIES) * sizeof(int32_t));
+    slab.add(&h->d_step_flags, 3 * sizeof(int32_t));
+    slab.add(&h->counters, 3 * LC_SIZE * sizeof(int32_t));
     for (int s = 0; s < h->nsp; ++s) {
         SpeciesBuf &S = h->sp[s];
         for (int32_t **q : {&S.bstart, &S.useg[0], &S.useg[1], &S.tcount}) slab.add(q, tb);
@@ -557,12 +556,10 @@ extern "C" PIC_API int pic_init(const pic_config *cfg, pic_t **out) {
     }
     slab.add(&h->d_bad, PIC_MAX_SPECIES * sizeof(unsigned long long));
     slab.add(&h->scan_sums, (size_t)scan_sums_entries() * sizeof(uint32_t));
-    slab.add(&h->occ, nt);
-    slab.add(&h->touched, nt);
-    slab.add(&h->touch_list, nt * sizeof(int32_t));
+    slab.add(&h->touched, 3 * nt);
+    slab.add(&h->touch_list, 3 * nt * sizeof(int32_t));
     slab.add(&h->rg_list, nt * sizeof(int32_t));
     slab.add(&h->nbr, 9 * nt * sizeof(int32_t));
-    slab.add(&h->chunk_prefix, ((size_t)h->nsp * nt + 1) * sizeof(int32_t));
     slab.add(&h->ticket, PIC_MAX_SPECIES * sizeof(int32_t));
     h->diag_cap = diag_scratch_doubles(h->nsp, h->ntiles);
     slab.add(&h->d_diag, h->diag_cap * sizeof(double));
@@ -580,7 +577,10 @@ extern "C" PIC_API int pic_init(const pic_config *cfg, pic_t **out) {
         set_error("pinned host allocation failed");
         rc = PIC_ERR_OOM;
     }
-    if (!rc) h->h_diag = (char *)h->h_step_flags + 64;
+    if (!rc) {
+        h->h_diag = (char *)h->h_step_flags + 64;
+        h->d_flags = h->d_step_flags + 2;
+    }
     if (!rc && (cudaEventCreateWithFlags(&h->ev_flags[0], cudaEventDisableTiming) != cudaSuccess ||
                 cudaEventCreateWithFlags(&h->ev_flags[1], cudaEventDisableTiming) != cudaSuccess ||
                 !create_events(&h->ev_batch, 1) || !create_events(&h->ev_load, 1) ||
@@ -860,7 +860,7 @@ static int load_impl(pic_t *h, int nload, const int *species, const pic_species_
     unsigned long long *bad = (unsigned long long *)h->h_diag;   // page-locked; diagnostics use it only inside their call
     if (!rc && (cudaMemcpyAsync(bad, h->d_bad, h->nsp * sizeof(unsigned long long), cudaMemcpyDeviceToHost,
                                 main_st) != cudaSuccess ||
-                (fresh && cudaMemcpyAsync(h->h_step_flags + 2, h->d_flags, sizeof(int32_t), cudaMemcpyDeviceToHost,
+                (fresh && cudaMemcpyAsync(h->h_step_flags + 3, h->d_flags, sizeof(int32_t), cudaMemcpyDeviceToHost,
                                           main_st) != cudaSuccess) ||
                 cudaStreamSynchronize(main_st) != cudaSuccess))
         rc = check_launch("particle load check");
@@ -906,11 +906,11 @@ static int load_impl(pic_t *h, int nload, const int *species, const pic_species_
             if (d[e].n > 0)
                 if (int r = rebuild_species(h, species[e], REBUILD_FROM_LOAD, d[e].n)) return r;
     h->moments_stale = !eager;   // else deposited at the next step or readout
-    if (!fresh && (cudaMemcpyAsync(h->h_step_flags + 2, h->d_flags, sizeof(int32_t), cudaMemcpyDeviceToHost,
+    if (!fresh && (cudaMemcpyAsync(h->h_step_flags + 3, h->d_flags, sizeof(int32_t), cudaMemcpyDeviceToHost,
                                    main_st) != cudaSuccess ||
                    cudaStreamSynchronize(main_st) != cudaSuccess))
         return check_launch(fn);
-    if (int r = flag_error(h->h_step_flags[2])) return r;
+    if (int r = flag_error(h->h_step_flags[3])) return r;
     for (int e = 0; e < nload; ++e) {
         if (d[e].n == 0) continue;
         SpeciesBuf &S = h->sp[species[e]];
@@ -1229,16 +1229,22 @@ extern "C" PIC_API int pic_clear_particles(pic_t *h) {
     return cudaStreamSynchronize(h->st) == cudaSuccess ? PIC_OK : check_launch("pic_clear_particles");
 }
 
-// A step's flags word (parity p) zeroed, the tile lists reset and, if asked,
-// the push's work items built from the current layout.
-static int step_reset(pic_t *h, int p, bool prep) {
-    cudaMemsetAsync(h->d_step_flags + p, 0, sizeof(int32_t), h->st);
-    if (int rc = reset_lists(h)) return rc;
-    return prep ? push_prep(h, false) : 0;
+// The tile lists of the push just queued (parity p) describe the moments from here
+// on: the next field solve reads them, and the clear before the next push.
+static void lists_used(pic_t *h, int p) {
+    h->touch_cur = h->lists;
+    h->touch_far = h->d_step_flags + p;
+    h->touch_all = false;
+}
+
+// A step's flags (parity p) and the sticky ones to the host, and their event.
+static void copy_flags(pic_t *h, int p) {
+    cudaMemcpyAsync(h->h_step_flags + 4 * p, h->d_step_flags, 3 * sizeof(int32_t), cudaMemcpyDeviceToHost, h->st);
+    cudaEventRecord(h->ev_flags[p], h->st);
 }
 
 // The particle part of a step (parity p): push (+ the exact deposit's
-// conversion), touch map, the FP64 cell sums into node moments (on the field
+// conversion), the FP64 cell sums into node moments (on the field
 // stream when it overlaps), regroup, and the flags copied to the host.  guard:
 // the previous step's flags word; the kernels do nothing if it holds a failure.
 static int particle_step(pic_t *h, int p, const int32_t *guard, cudaStream_t main_st, bool overlap) {
@@ -1249,13 +1255,11 @@ static int particle_step(pic_t *h, int p, const int32_t *guard, cudaStream_t mai
     } reset{h};
     timing_begin(h);
     int64_t l0 = h->timing.launches[4];
-    if (int rc = particle_tiles(h, true)) return rc;
+    if (int rc = particle_tiles(h)) return rc;
     if (h->det)
         if (int rc = fix_to_moments(h)) return rc;
     timing_end(h, 0, (int)(h->timing.launches[4] - l0));
-    // node tiles this deposit may have written: read by the next field solve and cleared before the next push
-    if (int rc = touch_map(h)) return rc;
-    h->touch_all = false;
+    lists_used(h, p);
     if (overlap) cudaEventRecord(h->ev_push, main_st);
     // the FP64 push's cell sums into the node moments (beside the regroup; before the next field solve)
     if (h->Mc) {
@@ -1274,9 +1278,7 @@ static int particle_step(pic_t *h, int p, const int32_t *guard, cudaStream_t mai
     timing_begin(h);
     if (int rc = regroup_tiles(h)) return rc;
     timing_end(h, 1, 1);
-    cudaMemcpyAsync(h->h_step_flags + 4 * p, h->d_step_flags + p, sizeof(int32_t), cudaMemcpyDeviceToHost, h->st);
-    cudaMemcpyAsync(h->h_step_flags + 4 * p + 1, h->d_flags, sizeof(int32_t), cudaMemcpyDeviceToHost, h->st);
-    cudaEventRecord(h->ev_flags[p], h->st);
+    copy_flags(h, p);
     if (overlap && h->Mc) cudaStreamWaitEvent(main_st, h->ev_cellm, 0);   // later work reads the node moments
     return 0;
 }
@@ -1287,7 +1289,8 @@ static int particle_step(pic_t *h, int p, const int32_t *guard, cudaStream_t mai
 static int step_deposit(pic_t *h, int p, const int32_t *guard) {
     timing_begin(h);
     const int64_t l0 = h->timing.launches[4];
-    if (int rc = push_prep(h, false)) return rc;
+    // (a step whose guard is set left its own flags word zero; its lists are made again with the step)
+    if (int rc = push_prep(h, h->d_step_flags + p, nullptr)) return rc;
     if (int rc = deposit_step(h, h->d_step_flags + p, guard)) return rc;
     timing_end(h, 0, (int)(h->timing.launches[4] - l0));
     return 0;
@@ -1328,19 +1331,23 @@ extern "C" PIC_API int pic_step(pic_t *h, int nsteps) {
         }
         if (rc) return rc;
         // 2. the moments the field solve has read cleared (the literal solve zeroes them itself), this
-        //    step's flags and the tile lists reset, and the push's work items (unless the previous step
-        //    queued them behind its regroup)
+        //    step's flags zeroed, and the push's work items and tile lists (unless the previous step queued
+        //    both behind its regroup)
         const int p = (int)(h->step & 1);
+        const bool prev = h->flags_pending;
+        const int32_t *guard = prev ? h->d_step_flags + (1 - p) : nullptr;
         timing_begin(h);
         l0 = h->timing.launches[4];
         if ((rc = clear_step_moments(h))) return rc;
-        if ((rc = step_reset(h, p, !prepped))) return rc;
+        if (!prepped) {
+            if ((rc = push_prep(h, guard, h->d_step_flags + p))) return rc;
+        } else if (h->post) {
+            cudaMemsetAsync(h->d_step_flags + p, 0, sizeof(int32_t), h->st);
+        }
         prepped = false;
         timing_end(h, 3, (int)(h->timing.launches[4] - l0));
         // 3. push, deposit, regroup -- queued at once: they do nothing if the previous step's regroup
         //    (still in flight) fails, and the host redoes them after the full sort below
-        const bool prev = h->flags_pending;
-        const int32_t *guard = prev ? h->d_step_flags + (1 - p) : nullptr;
         if ((rc = particle_step(h, p, guard, main_st, overlap))) return rc;
         commit_regroup(h);
         if (h->post) {
@@ -1362,7 +1369,7 @@ extern "C" PIC_API int pic_step(pic_t *h, int nsteps) {
                     if ((rc = field_cn(h))) return rc;
                     if ((rc = clear_step_moments(h))) return rc;
                 }
-                if ((rc = step_reset(h, p, true))) return rc;
+                if ((rc = push_prep(h, nullptr, h->d_step_flags + p))) return rc;
                 if ((rc = particle_step(h, p, nullptr, main_st, overlap))) return rc;
                 commit_regroup(h);
                 if (h->post)
@@ -1381,7 +1388,7 @@ extern "C" PIC_API int pic_step(pic_t *h, int nsteps) {
         if (k + 1 < nsteps && !h->post) {
             timing_begin(h);
             l0 = h->timing.launches[4];
-            if ((rc = push_prep(h, false))) return rc;
+            if ((rc = push_prep(h, h->d_step_flags + p, h->d_step_flags + (1 - p)))) return rc;
             timing_end(h, 3, (int)(h->timing.launches[4] - l0));
             prepped = true;
         }
@@ -1487,9 +1494,7 @@ extern "C" PIC_API int pic_batch_step(pic_batch *p, pic_t **hs, int n, int nstep
             prev[r] = h->flags_pending ? 1 : 0;
             h->guard = prev[r] ? h->d_step_flags + (1 - ph) : nullptr;
             if (int rc = clear_step_moments(h)) return rc;
-            cudaMemsetAsync(h->d_step_flags + ph, 0, sizeof(int32_t), h->st);
-            if (int rc = push_work_list(h)) return rc;
-            if (int rc = reset_lists(h)) return rc;
+            if (int rc = push_prep(h, h->guard, h->d_step_flags + ph)) return rc;
             cudaEventRecord(h->ev_batch, h->st);
             cudaStreamWaitEvent(b.st, h->ev_batch, 0);
         }
@@ -1506,15 +1511,10 @@ extern "C" PIC_API int pic_batch_step(pic_batch *p, pic_t **hs, int n, int nstep
         for (int r = 0; r < n; ++r) {
             pic_t *h = hs[r];
             cudaStreamWaitEvent(h->st, b.ev_done, 0);
-            // the run's touched tiles, as after its own push (the batched regroup visited every tile)
-            if (int rc = touch_map(h)) return rc;
-            h->touch_all = false;
             h->guard = nullptr;
             const int ph = (int)(h->step & 1);
-            cudaMemcpyAsync(h->h_step_flags + 4 * ph, h->d_step_flags + ph, sizeof(int32_t), cudaMemcpyDeviceToHost,
-                            h->st);
-            cudaMemcpyAsync(h->h_step_flags + 4 * ph + 1, h->d_flags, sizeof(int32_t), cudaMemcpyDeviceToHost, h->st);
-            cudaEventRecord(h->ev_flags[ph], h->st);
+            lists_used(h, ph);
+            copy_flags(h, ph);
             commit_regroup(h);
         }
         // the previous step's regroup decisions (the host waits for their flags while the GPU works)
@@ -1529,7 +1529,7 @@ extern "C" PIC_API int pic_batch_step(pic_batch *p, pic_t **hs, int n, int nstep
                 // the one the previous push left; the full sort, then the step alone on the run's stream
                 cudaMemsetAsync(h->d_step_flags + (1 - ph), 0, sizeof(int32_t), h->st);
                 if (int rc = rebuild_from_step(h)) return rc;
-                if (int rc = step_reset(h, ph, true)) return rc;
+                if (int rc = push_prep(h, nullptr, h->d_step_flags + ph)) return rc;
                 if (int rc = particle_step(h, ph, nullptr, h->st, false)) return rc;
                 commit_regroup(h);
                 if (h->post)

@@ -63,6 +63,7 @@ __device__ inline void curl_h_parts(const GridArgs<R> &g, const V4<R> *__restric
 template <typename R>
 struct TouchArgs {
     const uint8_t *touched;
+    const int32_t *far;    // (or nullptr) the push's flags: bit 0, a far move, and every tile may hold moments
     int tnx, tny, ntx;
     R *clr, *clr_lo;
 };
@@ -118,7 +119,7 @@ __global__ void __launch_bounds__(128, 6) k_field_E_literal(GridArgs<R> g, const
     const int i = (int)(blockIdx.x * blockDim.x + threadIdx.x) + (g.periodic_x ? 0 : 1), j = blockIdx.y;
     if (i >= g.nx) return;
     const int64_t node = (int64_t)j * g.nxn + i;
-    const uint8_t *map = tm.touched ? tm.touched + (j / tm.tny) * tm.ntx : nullptr;
+    const uint8_t *map = tm.touched && !(tm.far && (*tm.far & 1)) ? tm.touched + (j / tm.tny) * tm.ntx : nullptr;
     const bool touched = !map || map[min(i / tm.tnx, tm.ntx - 1)];
     R u, v, sy, sx;
     curl_h_parts(g, H, i, j, u, v, sy, sx);   // curl_h H = (u/(2 dy), v/(2 dx), sy/(2 dx) - sx/(2 dy))
@@ -1638,7 +1639,7 @@ static int field_literal_t(pic_t *h) {
     int en = 1 - h->ecur;
     // the exact deposit rewrites every moment from its fixed-point sums; the others deposit into the
     // moments this solve has read and zeroed
-    TouchArgs<R> tm{h->touch_all ? nullptr : h->touched, h->tnx, h->tny, h->ntx, h->det ? nullptr : (R *)h->M,
+    TouchArgs<R> tm{h->touch_all ? nullptr : h->touched + (size_t)h->touch_cur * h->ntiles, h->touch_far, h->tnx, h->tny, h->ntx, h->det ? nullptr : (R *)h->M,
                     h->det ? nullptr : (R *)h->Mlo};
     const pic_config &c = h->cfg;
     const int cols = h->periodic_x ? h->nx : h->nx - 1;   // (the walls' columns by their neighbours' threads)

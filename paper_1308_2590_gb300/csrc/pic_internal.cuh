@@ -101,6 +101,10 @@ struct Slab {
     int commit(void **base, const char *what);   // the allocation (freed by its base alone) and every pointer
 };
 
+// Counters of a set of tile lists.
+enum { LC_TOUCH = 0, LC_REGROUP = 1, LC_QUEUE = 2, LC_ITEMS = LC_QUEUE + PIC_MAX_SPECIES, LC_TICKET, LC_DEPOSIT, LC_SIZE = 16 };
+static_assert(LC_DEPOSIT < LC_SIZE, "counters of a set");
+
 struct Timing {
     bool enabled = false;
     double ms[4] = {0, 0, 0, 0};
@@ -158,16 +162,19 @@ struct pic_t {
     double *Mc = nullptr;               // FP64 L2-reduction push (linear shape): cell sums [ncell][13][4]
     double wabs[PIC_MAX_SPECIES] = {0, 0, 0, 0, 0, 0, 0, 0};  // sum of |w| loaded per species
     void *tmaps = nullptr;              // host storage of the TMA descriptors
-    int32_t *chunk_prefix = nullptr;    // [nsp*ntiles + 1] work items of the push, exclusive scan
     int2 *items = nullptr;              // work item k of the push -> (species-tile index, run within it)
     int64_t items_cap = 0;
-    int32_t *ticket = nullptr;          // work-queue counter of the persistent push
+    int32_t *ticket = nullptr;          // work-queue counters of a deposit at rest
     int32_t *nbr = nullptr;             // [ntiles][9] neighbour count, then the neighbour tiles ascending
-    uint8_t *occ = nullptr;             // [ntiles] tiles holding particles when the last push started
-    uint8_t *touched = nullptr;         // [ntiles] node tiles whose moments the last push may have written
-    int32_t *touch_list = nullptr;      // [ntiles] the touched tiles, in no particular order
+    // Tile lists, three sets in turn (push_prep): the field solve and the clear of a step read the set of the
+    // last push (touch_cur) while the next push's set (lists) is made, which zeroes the third one's counters.
+    int32_t *counters = nullptr;        // [3][pic::LC_SIZE]
+    uint8_t *touched = nullptr;         // [3][ntiles] node tiles whose moments the push may write
+    int32_t *touch_list = nullptr;      // [3][ntiles] the touched tiles, in no particular order
     int32_t *rg_list = nullptr;         // [ntiles] tiles the regroup must visit (an occupied tile or neighbour)
-    int32_t *list_n = nullptr;          // [2 + PIC_MAX_SPECIES] entries of touch_list, rg_list; regroup queues
+    int lists = 0, touch_cur = 0;
+    bool lists_zero[3] = {true, true, true};   // the set's counters are (or will be, in stream order) zero
+    const int32_t *touch_far = nullptr; // flags word of the last push: bit 0 (a far move), every tile is touched
     int regroup_blocks = 0;             // blocks per species of the list-driven regroup
     bool touch_all = true;              // no touched-tile map: moments may be non-zero anywhere (after init)
     bool moments_cleared = false;       // the last literal field solve zeroed the moments it read
@@ -1000,19 +1007,17 @@ struct BatchScratch {
 size_t batch_args_bytes();              // one argument block (the larger of the two forms)
 int batch_push(BatchScratch &b, pic_t **hs, int n);
 int batch_regroup(BatchScratch &b, pic_t **hs, int n);
-int push_work_list(pic_t *h);           // k_chunk_counts + scan on the run's stream
 
 // tiled step (pic_tile.cu)
 int tile_setup(pic_t *h);
-int particle_tiles(pic_t *h, bool prepared = false);
-int push_prep(pic_t *h, bool next);
+int particle_tiles(pic_t *h);
+int push_prep(pic_t *h, const int32_t *guard, int32_t *word);   // the next push's work items and tile lists
+int32_t *list_counters(const pic_t *h, int set);
 int cell_moments(pic_t *h);      // FP64 cell sums -> node moments (the listed touched tiles)
 int rest_touch(pic_t *h);        // touched[] and its list after a deposit at rest into cleared moments
-int reset_lists(pic_t *h);       // the tile lists and regroup queues, emptied before a push
 int regroup_tiles(pic_t *h);     // per-tile stable cell sort of stayers + arrivals into the spare set
 int scan_tiles(pic_t *h, const int32_t *in, int32_t *out);
 int tile_counts(pic_t *h, int s);   // tcount[t] = particles of tile t (device)
-int touch_map(pic_t *h);            // touched[] of the push just queued (occupancy dilated, far movers: all)
 
 // sort and rebuild (pic_sort.cu)
 enum RebuildSource { REBUILD_FROM_STEP = 0, REBUILD_FROM_LOAD = 1 };

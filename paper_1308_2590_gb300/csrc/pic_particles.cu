@@ -676,11 +676,10 @@ int deposit_step(pic_t *h, const int32_t *guard0, const int32_t *guard1) {
     a.B = (const V4<float> *)h->B[1 - h->bcur];   // the new node B (the step's flip follows)
     for (int s = 0; s < h->nsp; ++s) a.sp[s] = cell_dep_species(h, s);
     a.ch = push_item_segs(h);
-    a.nitems = h->chunk_prefix + (int64_t)h->nsp * h->ntiles;
-    a.ticket = h->ticket + 2;
+    a.nitems = list_counters(h, h->lists) + LC_ITEMS;
+    a.ticket = list_counters(h, h->lists) + LC_DEPOSIT;
     a.guard0 = guard0;
     a.guard1 = guard1;
-    cudaMemsetAsync(a.ticket, 0, sizeof(int32_t), h->st);
     return cell_dep_launch(h, a);
 }
 
@@ -714,13 +713,13 @@ static int deposit_only_t(pic_t *h, int s) {
     a.tnx = h->tnx;
     a.tny = h->tny;
     a.ntx = h->ntx;
-    // the work items (the queue's counters: words 1 and 2 beside the push's)
+    // the work items (words 0 and 1 of the queue's counters)
     if (int rc = ensure_items(h)) return rc;
     a.items = h->items;
-    a.nitems = h->ticket + 1;
-    a.ticket = h->ticket + 2;
-    cudaMemsetAsync(h->ticket + 1, 0, 2 * sizeof(int32_t), h->st);
-    k_rest_items<<<(h->ntiles + 255) / 256, 256, 0, h->st>>>(a.useg, h->ntiles, h->items, h->ticket + 1);
+    a.nitems = h->ticket;
+    a.ticket = h->ticket + 1;
+    cudaMemsetAsync(h->ticket, 0, 2 * sizeof(int32_t), h->st);
+    k_rest_items<<<(h->ntiles + 255) / 256, 256, 0, h->st>>>(a.useg, h->ntiles, h->items, h->ticket);
     count_launch(h);
     const size_t tab = h->fp32 ? 0 : (size_t)h->tnx * h->tny * sizeof(CellC<double>);   // B in cell form
     if (h->fp32 && !h->det && h->shape == 1) {
@@ -753,15 +752,17 @@ int deposit_only(pic_t *h, int s) {
 
 // Zero the 13 moment planes (and the FP32 compensation) on the nodes of the
 // touched tiles only: a fixed grid takes the tiles of the touched list in
-// turn.  Node column i belongs to tile min(i / tnx, ntx - 1), so a wall's last
+// turn (every tile after a far move).  Node column i belongs to tile min(i / tnx, ntx - 1), so a wall's last
 // column joins the last tile.
 template <typename R>
 __global__ void __launch_bounds__(128) k_clear_touched(const int32_t *__restrict__ list, const int32_t *__restrict__ list_n,
-                                                       int tnx, int tny, int ntx, int nx, int ny, int nxn, int64_t nnode,
-                                                       R *__restrict__ M, R *__restrict__ Mlo) {
-    const int n = list_n[0];
+                                                       const int32_t *__restrict__ far, int ntiles, int tnx, int tny,
+                                                       int ntx, int nx, int ny, int nxn, int64_t nnode, R *__restrict__ M,
+                                                       R *__restrict__ Mlo) {
+    const bool all = far && (*far & 1);
+    const int n = all ? ntiles : *list_n;
     for (int li = blockIdx.x; li < n; li += gridDim.x) {
-        const int T = list[li];
+        const int T = all ? li : list[li];
         const int tx = T % ntx, ty = T / ntx;
         const int i0 = tx * tnx, j0 = ty * tny;
         const int i1 = (tx == ntx - 1) ? nxn : min(i0 + tnx, nx);
@@ -803,12 +804,15 @@ int clear_step_moments(pic_t *h) {
         cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
         unsigned grid = (unsigned)(nsm > 0 ? 8 * nsm : 1024);
         if (grid > (unsigned)h->ntiles) grid = (unsigned)h->ntiles;
+        const int32_t *list = h->touch_list + (size_t)h->touch_cur * h->ntiles;
+        const int32_t *n = list_counters(h, h->touch_cur) + LC_TOUCH;
         if (h->fp32)
-            k_clear_touched<float><<<grid, 128, 0, h->st>>>(h->touch_list, h->list_n, h->tnx, h->tny, h->ntx, h->nx,
-                                                            h->ny, h->nxn, h->nnode, (float *)h->M, (float *)h->Mlo);
+            k_clear_touched<float><<<grid, 128, 0, h->st>>>(list, n, h->touch_far, h->ntiles, h->tnx, h->tny, h->ntx,
+                                                            h->nx, h->ny, h->nxn, h->nnode, (float *)h->M,
+                                                            (float *)h->Mlo);
         else
-            k_clear_touched<double><<<grid, 128, 0, h->st>>>(h->touch_list, h->list_n, h->tnx, h->tny, h->ntx, h->nx,
-                                                             h->ny, h->nxn, h->nnode, (double *)h->M, nullptr);
+            k_clear_touched<double><<<grid, 128, 0, h->st>>>(list, n, h->touch_far, h->ntiles, h->tnx, h->tny, h->ntx,
+                                                             h->nx, h->ny, h->nxn, h->nnode, (double *)h->M, nullptr);
         count_launch(h);
         return check_launch("k_clear_touched");
     }

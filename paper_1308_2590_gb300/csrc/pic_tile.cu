@@ -133,8 +133,8 @@ struct TileArgs {
     const V4<R> *Eh, *Bo;           // padded E^{n+1/2} and push B (the batched push loads its tiles from them)
     int32_t *step_flags, *flags;
     const int32_t *guard;           // the previous step's flags (set: this step's kernels do nothing for the run)
-    const int32_t *chunk_prefix;    // [nsp*ntiles + 1]
-    const int2 *items;              // item -> (species-tile index, run within it); single-run launches
+    const int32_t *nitems;          // work items of the push
+    const int2 *items;              // item -> (species-tile index, run within it)
     const int32_t *nbr;             // [ntiles][9]: neighbour count, then the neighbour tiles ascending
     int32_t *ticket;
     int ch;                         // segments per work item
@@ -380,9 +380,9 @@ __global__ void __launch_bounds__(TILE_BS, kDep ? push_min_blocks<R>() : 3)
     uint64_t *bar = (uint64_t *)smem;
     int *scr = (int *)(smem + 16);
     V4<R> *sE = (V4<R> *)(smem + SMEM_HEADER);
-    // work items: chunk_prefix over (species, tile), species-major, of one run or, batched, of every run
+    // work items of one run or, batched, of every run
     if (!kBatch && a0.guard && (*a0.guard & 3)) return;   // the previous regroup failed: the host redoes the step
-    const int nitems = kBatch ? run_items[nrun] : a0.chunk_prefix[a0.nsp * a0.ntiles];
+    const int nitems = kBatch ? run_items[nrun] : *a0.nitems;
     const unsigned lt = (1u << lane) - 1u;
     if (!kBatch && tid == 0) {
         mbar_init(bar, 1);
@@ -392,22 +392,12 @@ __global__ void __launch_bounds__(TILE_BS, kDep ? push_min_blocks<R>() : 3)
     }
     __syncthreads();
     for (int iter = 0;; ++iter) {
-        if (!kBatch && tid == 0) {
-            const int item = atomicAdd(a0.ticket, 1);
-            scr[0] = item;
-            if (item < nitems) {
-                const int2 it = a0.items[item];   // one load instead of a search over the prefix
-                scr[1] = it.x;
-                scr[2] = it.y;
-            }
-            scr[4] = 0;
-        }
-        if (kBatch && tid == 0) {
+        if (tid == 0) {
             int item = atomicAdd(a0.ticket, 1);
             scr[0] = item;
+            scr[4] = 0;
             if (item < nitems) {
-                int r = 0;
-                const TileArgs<R> *ar = &a0;
+                const int2 *items = a0.items;
                 if (kBatch) {
                     int lo = 0, hi = nrun;   // largest r with run_items[r] <= item
                     while (hi - lo > 1) {
@@ -415,19 +405,13 @@ __global__ void __launch_bounds__(TILE_BS, kDep ? push_min_blocks<R>() : 3)
                         if (run_items[mid] <= item) lo = mid;
                         else hi = mid;
                     }
-                    r = lo;
-                    item -= run_items[r];
-                    ar = runs + r;
+                    item -= run_items[lo];
+                    items = runs[lo].items;
+                    scr[4] = lo;
                 }
-                int lo = 0, hi = ar->nsp * ar->ntiles;   // largest idx with chunk_prefix[idx] <= item
-                while (hi - lo > 1) {
-                    int mid = (lo + hi) >> 1;
-                    if (ar->chunk_prefix[mid] <= item) lo = mid;
-                    else hi = mid;
-                }
-                scr[1] = lo;
-                scr[2] = item - ar->chunk_prefix[lo];
-                scr[4] = r;
+                const int2 it = items[item];
+                scr[1] = it.x;
+                scr[2] = it.y;
             }
         }
         __syncthreads();
@@ -798,7 +782,7 @@ __global__ void __launch_bounds__(TILE_BS, push_s_min_blocks<R>()) k_push_s(cons
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
     __shared__ int scr[3];
     const GridArgs<R> &g = a.g;
-    const int nitems = a.chunk_prefix[a.nsp * a.ntiles];
+    const int nitems = *a.nitems;
     const unsigned lt = (1u << lane) - 1u;
     SplineDep<R, N> dep;
     if (!kFix) dep.init(ssm + wid * SplineDep<R, N>::kWarpBytes, lane);
@@ -966,82 +950,132 @@ __global__ void __launch_bounds__(TILE_BS, push_s_min_blocks<R>()) k_push_s(cons
     if constexpr (!kFix) dep.flush(GlobalSink<R>{g, a.M}, lane);
 }
 
-// Work items of the push: ch-segment runs of every (species, tile), in
-// species-major, tile order; the counts are scanned afterwards (the entry
-// after the last holds the total).  Also resets the work queue (the tile
-// lists are reset separately, just before the push: reset_lists).
 struct UsegPtrs {
     const int32_t *p[PIC_MAX_SPECIES];
 };
-
-__global__ void k_chunk_counts(UsegPtrs u, int nsp, int ntiles, int ch, int32_t *__restrict__ out,
-                               int32_t *__restrict__ ticket, uint8_t *__restrict__ occ) {
-    const int n = nsp * ntiles;
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n) {
-        const int s = i / ntiles, t = i - s * ntiles;
-        out[i] = (u.p[s][t] + ch - 1) / ch;
-        if (s == 0) {   // occupancy of the tile by any species at the start of the push
-            int any = 0;
-            for (int q = 0; q < nsp; ++q) any |= u.p[q][t];
-            occ[t] = any != 0;
-        }
-    } else if (i == n) {
-        out[n] = 0;
-        *ticket = 0;
-    }
-}
-
-// Node tiles a push may have deposited into.  A particle of occupied tile a
-// ends in tile a-1, a or a+1 on each axis (a farther move sets bit 0 of the
-// step flags), and its corner nodes lie in its new cell's tile or the next one
-// (node column i is in tile min(i / tnx, ntx - 1)); the FP32 flush region is
-// the tile plus a halo of fewer than a tile's cells.  So node tile T is touched
-// if a tile of T-2 .. T+1 on both axes (wrapping where the box is periodic) was
-// occupied (spline shapes reach further: touch_map), and every tile is touched
-// after a far move.  The same pass lists
-// the tiles the regroup must visit -- those with an occupied tile among T-1 ..
-// T+1 on both axes (stayers or arrivals; after a far move the regroup's output
-// is replaced by the full sort) -- and empties the next bins of the others.
 struct UsegOut {
     int32_t *p[PIC_MAX_SPECIES];
 };
 
-__global__ void k_touch_map(const uint8_t *__restrict__ occ, const int32_t *__restrict__ step_flags,
-                            const int32_t *__restrict__ guard, int ntx, int nty,
-                            int periodic_x, uint8_t *__restrict__ touched, int32_t *__restrict__ touch_list,
-                            int32_t *__restrict__ rg_list, int32_t *__restrict__ list_n, UsegOut useg2, int nsp,
-                            int dlx, int dly, int dhx, int dhy) {
-    const int T = blockIdx.x * blockDim.x + threadIdx.x;
-    if (T >= ntx * nty) return;
-    if (guard && (*guard & 3)) return;
-    const bool far = (*step_flags & 1) != 0;
-    const int tx = T % ntx, ty = T / ntx;
-    bool touch = far, near = false;
-    for (int dy = -dly; dy <= dhy; ++dy) {
-        int y = ty + dy;
-        y = y < 0 ? y + nty : (y >= nty ? y - nty : y);
-        if (y < 0 || y >= nty) continue;   // fewer than 3 tile rows: a wrap may still leave the range
-        for (int dx = -dlx; dx <= dhx; ++dx) {
-            int x = tx + dx;
+// Everything the next push and its regroup need to know of the tiles, in one
+// pass over them, a thread per tile:
+// - the push's work items, runs of ch segments of every (species, tile);
+// - the node tiles the push may deposit into.  A particle of occupied tile a
+//   ends in tile a-1, a or a+1 on each axis (a farther move sets bit 0 of the
+//   step's flags, and every tile is touched), and its corner nodes lie in its new
+//   cell's tile or the next one (node column i is in tile min(i / tnx, ntx - 1));
+//   the FP32 flush region is the tile plus a halo of fewer than a tile's cells.
+//   So node tile T is touched if a tile of T-2 .. T+1 on both axes (wrapping where
+//   the box is periodic) is occupied (spline shapes reach further: push_prep);
+// - the tiles the regroup must visit, those with an occupied tile among T-1 ..
+//   T+1 on both axes (stayers or arrivals; after a far move the regroup's output
+//   is replaced by the full sort); the next bins of the others are emptied.
+// The lists' order is the order of the warps' reservations, which nothing
+// depends on.  Also zeroed: the counters of the set after this one, and the step's
+// flags word.  Nothing is written for a run whose previous regroup failed: the
+// host makes the lists again from the restored layout.
+// It stands between a regroup and the next push, so its length counts in full: a
+// single block's counts, scan and item table, a touch map of its own after the
+// push and two memsets took 24 + 6.5 + 2 x 2 us for the 8192 tiles of a foil and
+// 6 + 5.3 + 2 x 2 us for the 960 of a small run; now 7 us for either.
+// kNear: the linear shape's 4 x 4 tiles, every load of a species in flight at once.
+template <bool kNear>
+__global__ void __launch_bounds__(128) k_step_lists(UsegPtrs u, UsegOut u2, int nsp, int ntx, int nty, int periodic_x,
+                                                    int ch, int dlx, int dly, int dhx, int dhy,
+                                                    const int32_t *__restrict__ guard, int32_t *__restrict__ word,
+                                                    int32_t *__restrict__ cnt, int32_t *__restrict__ cnt_next,
+                                                    uint8_t *__restrict__ touched, int32_t *__restrict__ touch_list,
+                                                    int32_t *__restrict__ rg_list, int2 *__restrict__ items) {
+    const int T = blockIdx.x * blockDim.x + threadIdx.x, lane = threadIdx.x & 31, ntiles = ntx * nty;
+    if (blockIdx.x == 0) {
+        if (threadIdx.x < LC_SIZE) cnt_next[threadIdx.x] = 0;
+        if (threadIdx.x == 32 && word) *word = 0;
+    }
+    const bool on = T < ntiles, skip = guard && (*guard & 3);
+    int c = 0;
+    bool touch = false, near = false;
+    if (on) {
+        const int tx = T % ntx, ty = T / ntx;
+        // the tile dx, dy away, or -1 (a wrap wider than the box may still leave the range)
+        auto tile_at = [&](int dx, int dy) {
+            int x = tx + dx, y = ty + dy;
+            y = y < 0 ? y + nty : (y >= nty ? y - nty : y);
             if (periodic_x) x = x < 0 ? x + ntx : (x >= ntx ? x - ntx : x);
-            if (x < 0 || x >= ntx) continue;
-            if (occ[y * ntx + x]) {
-                touch = true;
-                if (dx >= -1 && dy >= -1) near = true;
+            return x < 0 || x >= ntx || y < 0 || y >= nty ? -1 : y * ntx + x;
+        };
+        for (int s = 0; s < nsp; ++s) {
+            const int32_t *p = u.p[s];
+            c += (p[T] + ch - 1) / ch;
+            if constexpr (kNear) {
+                int v[16];
+#pragma unroll
+                for (int k = 0; k < 16; ++k) {
+                    const int q = tile_at(k % 4 - 2, k / 4 - 2);
+                    v[k] = p[q < 0 ? T : q];
+                    v[k] = q < 0 ? 0 : v[k];
+                }
+#pragma unroll
+                for (int k = 0; k < 16; ++k) {
+                    touch |= v[k] > 0;
+                    near |= v[k] > 0 && k % 4 > 0 && k / 4 > 0;
+                }
+            } else {
+                for (int dy = -dly; dy <= dhy; ++dy)
+                    for (int dx = -dlx; dx <= dhx; ++dx) {
+                        const int q = tile_at(dx, dy);
+                        if (q < 0 || p[q] == 0) continue;
+                        touch = true;
+                        near |= dx >= -1 && dy >= -1 && dx <= 1 && dy <= 1;
+                    }
             }
         }
     }
-    touched[T] = touch ? 1 : 0;
-    if (touch) touch_list[atomicAdd(&list_n[0], 1)] = T;
-    if (near) rg_list[atomicAdd(&list_n[1], 1)] = T;
-    else
-        for (int s = 0; s < nsp; ++s) useg2.p[s][T] = 0;
+    if (skip) return;
+    if (on) {
+        touched[T] = touch ? 1 : 0;
+        if (!near)
+            for (int s = 0; s < nsp; ++s) u2.p[s][T] = 0;
+    }
+    // a reservation per warp and list
+    const unsigned lt = (1u << lane) - 1u, mt = __ballot_sync(FULL, touch), mr = __ballot_sync(FULL, near);
+    int incl = c;
+    for (int o = 1; o < 32; o <<= 1) {
+        const int y = __shfl_up_sync(FULL, incl, o);
+        if (lane >= o) incl += y;
+    }
+    int b = 0;
+    if (lane == 31 && incl) b = atomicAdd(&cnt[LC_ITEMS], incl);
+    if (lane == 0 && mt) b = atomicAdd(&cnt[LC_TOUCH], __popc(mt));
+    if (lane == 1 && mr) b = atomicAdd(&cnt[LC_REGROUP], __popc(mr));
+    const int bi = __shfl_sync(FULL, b, 31), bt = __shfl_sync(FULL, b, 0), br = __shfl_sync(FULL, b, 1);
+    if (touch) touch_list[bt + __popc(mt & lt)] = T;
+    if (near) rg_list[br + __popc(mr & lt)] = T;
+    int at = bi + incl - c;
+    if (c)
+        for (int s = 0; s < nsp; ++s) {
+            const int n = (u.p[s][T] + ch - 1) / ch;
+            for (int k = 0; k < n; ++k) items[at++] = make_int2(s * ntiles + T, k);
+        }
 }
 
-int touch_map(pic_t *h) {
+int32_t *list_counters(const pic_t *h, int set) { return h->counters + set * LC_SIZE; }
+
+// The next push's work items and tile lists from the current layout of the bins
+// (of the regroup just queued: guard is its flags word, with which nothing is
+// done if it failed).  word (or nullptr): the step's flags word, zeroed.
+int push_prep(pic_t *h, const int32_t *guard, int32_t *word) {
+    if (int rc = ensure_items(h)) return rc;   // grown before any launch that would use it
+    UsegPtrs u;
     UsegOut u2;
-    for (int s = 0; s < PIC_MAX_SPECIES; ++s) u2.p[s] = (s < h->nsp) ? h->sp[s].useg[1 - h->sp[s].scur] : nullptr;
+    for (int s = 0; s < PIC_MAX_SPECIES; ++s) {
+        u.p[s] = (s < h->nsp) ? h->sp[s].useg[h->sp[s].scur] : nullptr;
+        u2.p[s] = (s < h->nsp) ? h->sp[s].useg[1 - h->sp[s].scur] : nullptr;
+    }
+    h->items_ch = item_segs(h);
+    const int set = (h->touch_cur + 1) % 3, after = (set + 1) % 3;
+    int32_t *cnt = list_counters(h, set);
+    if (!h->lists_zero[set] && cudaMemsetAsync(cnt, 0, LC_SIZE * sizeof(int32_t), h->st) != cudaSuccess)
+        return check_launch("tile lists");
     // occupied tiles T - dl .. T + dh can deposit into node tile T: the nodes of a particle in cell c
     // are c + lo .. c + hi (order 1: 0 .. 1; 2: -1 .. 2; 3: -1 .. 2; 4: -2 .. 3), in node tiles
     // b - ceil(-lo / tile) .. b + ceil(hi / tile) of the new cell's tile b, itself within one tile
@@ -1049,21 +1083,16 @@ int touch_map(pic_t *h) {
     const int lo = -(h->shape / 2), hi = (h->shape + 2) / 2;
     const int dlx = 1 + (hi + h->tnx - 1) / h->tnx, dly = 1 + (hi + h->tny - 1) / h->tny;
     const int dhx = 1 + (-lo + h->tnx - 1) / h->tnx, dhy = 1 + (-lo + h->tny - 1) / h->tny;
-    k_touch_map<<<(h->ntiles + 255) / 256, 256, 0, h->st>>>(h->occ, h->d_step_flags + (h->step & 1), h->guard,
-                                                            h->ntx, h->nty,
-                                                            h->periodic_x ? 1 : 0, h->touched, h->touch_list,
-                                                            h->rg_list, h->list_n, u2, h->nsp, dlx, dly, dhx, dhy);
+    const auto kernel = dlx == 2 && dly == 2 && dhx == 1 && dhy == 1 ? k_step_lists<true> : k_step_lists<false>;
+    kernel<<<(h->ntiles + 127) / 128, 128, 0, h->st>>>(
+        u, u2, h->nsp, h->ntx, h->nty, h->periodic_x ? 1 : 0, h->items_ch, dlx, dly, dhx, dhy, guard, word, cnt,
+        list_counters(h, after), h->touched + (size_t)set * h->ntiles, h->touch_list + (size_t)set * h->ntiles, h->rg_list,
+        h->items);
     count_launch(h);
-    return check_launch("k_touch_map");
-}
-
-// The push's item table from the scanned item counts: item c of species-tile
-// index i (c0 = prefix[i] <= c < prefix[i + 1]) -> (i, c - c0).
-__global__ void k_item_table(const int32_t *__restrict__ prefix, int n, int2 *__restrict__ items) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    const int c0 = prefix[i], c1 = prefix[i + 1];
-    for (int c = c0; c < c1; ++c) items[c] = make_int2(i, c - c0);
+    h->lists_zero[set] = false;
+    h->lists_zero[after] = true;
+    h->lists = set;
+    return check_launch("k_step_lists");
 }
 
 // Exclusive block scan of one int per thread; *total = block sum.
@@ -1828,36 +1857,17 @@ static TileArgs<R> tile_args(pic_t *h) {
     a.step_flags = h->d_step_flags + (h->step & 1);
     a.guard = h->guard;
     a.flags = h->d_flags;
-    a.chunk_prefix = h->chunk_prefix;
+    a.nitems = list_counters(h, h->lists) + LC_ITEMS;
     a.items = h->items;
     a.nbr = h->nbr;
-    a.ticket = h->ticket;
+    a.ticket = list_counters(h, h->lists) + LC_TICKET;
     a.ch = h->items_ch > 0 ? h->items_ch : item_segs(h);
     a.rg_list = h->rg_list;
-    a.list_n = h->list_n;
+    a.list_n = list_counters(h, h->lists);
     return a;
 }
 
-int push_work_list(pic_t *h) {
-    UsegPtrs u;
-    for (int s = 0; s < PIC_MAX_SPECIES; ++s) u.p[s] = (s < h->nsp) ? h->sp[s].useg[h->sp[s].scur] : nullptr;
-    const int nitems = h->nsp * h->ntiles;
-    h->items_ch = item_segs(h);
-    k_chunk_counts<<<(nitems + 256) / 256, 256, 0, h->st>>>(u, h->nsp, h->ntiles, h->items_ch, h->chunk_prefix,
-                                                            h->ticket, h->occ);
-    count_launch(h);
-    return scan_i32_inplace(h, h->chunk_prefix, nitems + 1);
-}
-
 int push_item_segs(const pic_t *h) { return h->items_ch; }
-
-// The touch and regroup lists and the regroup queues, emptied for the next
-// push (after whatever read the previous push's lists: the clear of its tiles).
-int reset_lists(pic_t *h) {
-    if (cudaMemsetAsync(h->list_n, 0, (2 + PIC_MAX_SPECIES) * sizeof(int32_t), h->st) != cudaSuccess)
-        return check_launch("tile lists");
-    return 0;
-}
 
 // ---------------------------------------------------------------------------- batched runs
 
@@ -1875,7 +1885,7 @@ __global__ void k_batch_items(const TileArgs<R> *__restrict__ runs, int n, int32
     for (int r = 0; r < n; ++r) {
         items[r] = acc;
         const TileArgs<R> &a = runs[r];
-        if (!(a.guard && (*a.guard & 3))) acc += a.chunk_prefix[a.nsp * a.ntiles];
+        if (!(a.guard && (*a.guard & 3))) acc += *a.nitems;
     }
     items[n] = acc;
     *ticket = 0;
@@ -1961,15 +1971,17 @@ int batch_regroup(BatchScratch &b, pic_t **hs, int n) {
 // once (a thread per cell, its 13 moments in turn: 87 us for the 98,000 cells of a
 // thin foil; now 24 us).
 __global__ void __launch_bounds__(256) k_cell_moments(const int32_t *__restrict__ list,
-                                                      const int32_t *__restrict__ list_n, int tnx, int tny, int ntx,
-                                                      GridArgs<double> g, double *__restrict__ Mc,
+                                                      const int32_t *__restrict__ list_n,
+                                                      const int32_t *__restrict__ far, int tnx, int tny, int ntx,
+                                                      int ntiles, GridArgs<double> g, double *__restrict__ Mc,
                                                       double *__restrict__ M, const int32_t *__restrict__ guard) {
     if (guard && (*guard & 3)) return;
     const int tc = tnx * tny, tm = tc * NMOM;
-    const int64_t total = (int64_t)list_n[0] * tm;
+    const bool all = far && (*far & 1);   // every tile, whatever the list holds
+    const int64_t total = (int64_t)(all ? ntiles : *list_n) * tm;
     for (int64_t w = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; w < total; w += (int64_t)gridDim.x * blockDim.x) {
         const int li = (int)(w / tm), r = (int)(w - (int64_t)li * tm), c = r / NMOM, k = r - c * NMOM;
-        const int T = list[li], tx = T % ntx, ty = T / ntx;
+        const int T = all ? li : list[li], tx = T % ntx, ty = T / ntx;
         const int ly = c / tnx;
         const int cx = tx * tnx + (c - ly * tnx), cy = ty * tny + ly;
         if (cx >= g.nx || cy >= g.ny) continue;
@@ -1993,7 +2005,8 @@ int cell_moments(pic_t *h) {
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
     k_cell_moments<<<(unsigned)(nsm > 0 ? 8 * nsm : 1024), 256, 0, h->st>>>(
-        h->touch_list, h->list_n, h->tnx, h->tny, h->ntx, grid_args<double>(h), h->Mc, (double *)h->M, h->guard);
+        h->touch_list + (size_t)h->touch_cur * h->ntiles, list_counters(h, h->touch_cur) + LC_TOUCH, h->touch_far, h->tnx,
+        h->tny, h->ntx, h->ntiles, grid_args<double>(h), h->Mc, (double *)h->M, h->guard);
     count_launch(h);
     return check_launch("k_cell_moments");
 }
@@ -2022,89 +2035,21 @@ __global__ void k_rest_touch(UsegPtrs u, int nsp, int ntx, int nty, int periodic
 int rest_touch(pic_t *h) {
     UsegPtrs u;
     for (int s = 0; s < PIC_MAX_SPECIES; ++s) u.p[s] = (s < h->nsp) ? h->sp[s].useg[h->sp[s].scur] : nullptr;
-    // nodes c + lo .. c + hi of a particle in cell c (as in touch_map; the splines' may cross a ragged last
+    // nodes c + lo .. c + hi of a particle in cell c (as in push_prep; the splines' may cross a ragged last
     // tile into the one after it)
     const int lo = -(h->shape / 2), hi = (h->shape + 2) / 2, one = h->shape > 1 ? 1 : 0;
-    if (cudaMemsetAsync(h->list_n, 0, sizeof(int32_t), h->st) != cudaSuccess) return check_launch("tile lists");
+    int32_t *cnt = list_counters(h, h->touch_cur) + LC_TOUCH;
+    if (cudaMemsetAsync(cnt, 0, sizeof(int32_t), h->st) != cudaSuccess) return check_launch("tile lists");
+    h->lists_zero[h->touch_cur] = false;
+    h->touch_far = nullptr;
     k_rest_touch<<<(h->ntiles + 255) / 256, 256, 0, h->st>>>(
-        u, h->nsp, h->ntx, h->nty, h->periodic_x ? 1 : 0, h->touched, h->touch_list, h->list_n,
+        u, h->nsp, h->ntx, h->nty, h->periodic_x ? 1 : 0, h->touched + (size_t)h->touch_cur * h->ntiles,
+        h->touch_list + (size_t)h->touch_cur * h->ntiles, cnt,
         one + (hi + h->tnx - 1) / h->tnx, one + (hi + h->tny - 1) / h->tny, one + (-lo + h->tnx - 1) / h->tnx,
         one + (-lo + h->tny - 1) / h->tny);
     count_launch(h);
     h->touch_all = false;
     return check_launch("k_rest_touch");
-}
-
-// The push's work items in one block, for up to PREP_ONE_BLOCK (species, tile)
-// entries: the same counts, occupancy bytes, exclusive prefix (total at the
-// end) and item table as k_chunk_counts + scan + k_item_table, without the
-// launches between them (they sit between the regroup and the next push).
-// The segment counts are read once, coalesced, into shared memory.
-constexpr int PREP_BS = 1024;
-constexpr int PREP_ONE_BLOCK = 16 * 1024;
-__global__ void __launch_bounds__(PREP_BS) k_prep_one_block(UsegPtrs u, int nsp, int ntiles, int ch,
-                                                            int32_t *__restrict__ prefix, int32_t *__restrict__ ticket,
-                                                            uint8_t *__restrict__ occ, int2 *__restrict__ items) {
-    extern __shared__ int cnt[];   // [nsp * ntiles] segment counts, then chunk counts
-    __shared__ int wsum[PREP_BS / 32];
-    const int n = nsp * ntiles, tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
-    {
-        // every load in flight before the first store (n <= PREP_ONE_BLOCK)
-        constexpr int PER = PREP_ONE_BLOCK / PREP_BS;
-        int v[PER];
-#pragma unroll
-        for (int k = 0; k < PER; ++k) {
-            const int i = tid + k * PREP_BS;
-            const int ic = (i < n) ? i : 0;   // an in-range index even where the load is not taken
-            const int s = ic / ntiles;
-            v[k] = (i < n) ? u.p[s][ic - s * ntiles] : 0;
-        }
-#pragma unroll
-        for (int k = 0; k < PER; ++k)
-            if (tid + k * PREP_BS < n) cnt[tid + k * PREP_BS] = v[k];
-    }
-    __syncthreads();
-    for (int t = tid; t < ntiles; t += PREP_BS) {   // occupancy of the tile by any species at the start of the push
-        int any = 0;
-        for (int q = 0; q < nsp; ++q) any |= cnt[q * ntiles + t];
-        occ[t] = any != 0;
-    }
-    __syncthreads();
-    for (int i = tid; i < n; i += PREP_BS) cnt[i] = (cnt[i] + ch - 1) / ch;
-    __syncthreads();
-    const int per = (n + PREP_BS - 1) / PREP_BS;
-    const int i0 = min(tid * per, n), i1 = min(i0 + per, n);
-    int local = 0;
-    for (int i = i0; i < i1; ++i) local += cnt[i];
-    // exclusive block scan of the per-thread sums (entries are contiguous per thread)
-    int incl = local;
-    for (int o = 1; o < 32; o <<= 1) {
-        const int y = __shfl_up_sync(FULL, incl, o);
-        if (lane >= o) incl += y;
-    }
-    if (lane == 31) wsum[wid] = incl;
-    __syncthreads();
-    if (wid == 0) {
-        const int x = wsum[lane];
-        int xi = x;
-        for (int o = 1; o < 32; o <<= 1) {
-            const int y = __shfl_up_sync(FULL, xi, o);
-            if (lane >= o) xi += y;
-        }
-        wsum[lane] = xi - x;
-    }
-    __syncthreads();
-    int run = wsum[wid] + incl - local;
-    for (int i = i0; i < i1; ++i) {
-        const int c = cnt[i];
-        prefix[i] = run;
-        for (int k = 0; k < c; ++k) items[run + k] = make_int2(i, k);
-        run += c;
-    }
-    if (tid == PREP_BS - 1) {
-        prefix[n] = run;   // the last thread's running sum is the total
-        *ticket = 0;
-    }
 }
 
 // The item table: at most one item per segment slot.
@@ -2124,45 +2069,13 @@ int ensure_items(pic_t *h) {
     return 0;
 }
 
-// The push's work items: the chunk counts of every (species, tile), their scan
-// and the item table, from the bins' layout in slot next ? scur ^ 1 : scur of
-// each species (next: the slot the pending per-tile regroup writes, so that a
-// step can prepare its push before the host has seen that regroup's flags).
-int push_prep(pic_t *h, bool next) {
-    UsegPtrs u;
-    for (int s = 0; s < PIC_MAX_SPECIES; ++s)
-        u.p[s] = (s < h->nsp) ? h->sp[s].useg[next ? h->sp[s].scur ^ 1 : h->sp[s].scur] : nullptr;
-    const int nitems = h->nsp * h->ntiles;
-    if (int rc = ensure_items(h)) return rc;   // grown before any launch that would use it
-    h->items_ch = item_segs(h);
-    if (nitems <= PREP_ONE_BLOCK) {
-        const int sm = nitems * (int)sizeof(int);
-        if (sm > 48 * 1024 && cudaFuncSetAttribute(k_prep_one_block, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                   PREP_ONE_BLOCK * (int)sizeof(int)) != cudaSuccess)
-            return check_launch("push work items set-up");
-        k_prep_one_block<<<1, PREP_BS, sm, h->st>>>(u, h->nsp, h->ntiles, h->items_ch, h->chunk_prefix, h->ticket,
-                                                    h->occ, h->items);
-        count_launch(h);
-        return check_launch("push work items");
-    }
-    k_chunk_counts<<<(nitems + 256) / 256, 256, 0, h->st>>>(u, h->nsp, h->ntiles, h->items_ch, h->chunk_prefix,
-                                                            h->ticket, h->occ);
-    count_launch(h);
-    if (int rc = scan_i32_inplace(h, h->chunk_prefix, nitems + 1)) return rc;
-    k_item_table<<<(nitems + 255) / 256, 256, 0, h->st>>>(h->chunk_prefix, nitems, h->items);
-    count_launch(h);
-    return check_launch("push work items");
-}
-
 template <typename R>
-static int particle_tiles_t(pic_t *h, bool prepared) {
+static int particle_tiles_t(pic_t *h) {
     struct Both {
         TMaps *a;
         CUtensorMap *b;
     };
     Both *both = (Both *)h->tmaps;
-    if (!prepared)
-        if (int rc = push_prep(h, false)) return rc;
     TileArgs<R> a = tile_args<R>(h);
     if (h->det)
         if (int rc = fix_scale(h, &a.fs)) return rc;
@@ -2196,9 +2109,7 @@ static int particle_tiles_t(pic_t *h, bool prepared) {
     return check_launch("k_push");
 }
 
-int particle_tiles(pic_t *h, bool prepared) {
-    return h->fp32 ? particle_tiles_t<float>(h, prepared) : particle_tiles_t<double>(h, prepared);
-}
+int particle_tiles(pic_t *h) { return h->fp32 ? particle_tiles_t<float>(h) : particle_tiles_t<double>(h); }
 
 template <typename R>
 static int regroup_t(pic_t *h) {
