@@ -177,7 +177,7 @@ struct pic_t {
     const int32_t *touch_far = nullptr; // flags word of the last push: bit 0 (a far move), every tile is touched
     int regroup_blocks = 0;             // blocks per species of the list-driven regroup
     bool touch_all = true;              // no touched-tile map: moments may be non-zero anywhere (after init)
-    bool moments_cleared = false;       // the last literal field solve zeroed the moments it read
+    bool moments_cleared = false;       // the last field solve zeroed the moments it read
     unsigned long long *d_bad = nullptr;  // per species: first invalid particle index of a load
     uint32_t *scan_sums = nullptr;      // per-block totals of the multi-block scans
     bool moments_stale = false;         // particles or B changed since the last deposit at rest
@@ -274,6 +274,38 @@ __host__ __device__ inline int64_t pidx(const GridArgs<R> &g, int i, int j) {
 }
 
 // --------------------------------------------------------------------------- device helpers
+
+// The FP32 value nearest to v (ties to even) and the FP64 value of f, from
+// their bits: a conversion instruction issues on the FP64 pipe.  In 32-bit halves,
+// since a mask that takes the sign off the whole word is compiled to an FP64
+// operation as well (the load conversion issued 18 of them per particle, 8 of
+// which are arithmetic).
+__device__ inline float narrow(double v) {
+    const unsigned hi = (unsigned)__double2hiint(v), lo = (unsigned)__double2loint(v), h = hi & 0x7fffffffu, e = h >> 20;
+    unsigned r;
+    if (e >= 897) {
+        r = __funnelshift_l(lo, hi, 3) - (896u << 23);
+        r += (lo & 0x1fffffffu) > 0x10000000u - (r & 1u) ? 1u : 0u;
+        if (e > 1150) r = h > 0x7ff00000u || (h == 0x7ff00000u && lo) ? 0x7fffffffu : 0x7f800000u;
+    } else {   // FP32 denormals and zero
+        const unsigned sh = 926 - e;
+        const unsigned long long q = ((unsigned long long)((h & 0xfffffu) | 0x100000u) << 32) | lo;
+        r = sh > 54 ? 0u : (unsigned)((q + ((1ull << (sh - 1)) - 1) + ((q >> sh) & 1)) >> sh);
+    }
+    return __uint_as_float(r | (hi & 0x80000000u));
+}
+__device__ inline double widen(float f) {
+    const unsigned u = __float_as_uint(f), m = u & 0x7fffffffu;
+    unsigned long long d = 0;
+    if (m >= 0x00800000u) {
+        d = ((unsigned long long)m << 29) + ((m >= 0x7f800000u ? 1792ull : 896ull) << 52);
+    } else if (m) {
+        const int z = __clz(m);
+        d = ((unsigned long long)((m << (z - 8)) & 0x7fffffu) << 29) | ((unsigned long long)(905 - z) << 52);
+    }
+    return __longlong_as_double((long long)(d | (unsigned long long)(u & 0x80000000u) << 32));
+}
+__device__ inline double widen(double v) { return v; }
 
 // 1/sqrt(x) and 1/x: in FP32 the hardware approximations (2 ulp, far below the
 // FP32 form's tolerances); in FP64 the library's correctly rounded forms.

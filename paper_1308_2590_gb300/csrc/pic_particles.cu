@@ -431,15 +431,6 @@ __device__ inline double div_by(double x, double d, double rd) {
     return fma(fma(-q, d, x), rd, q);
 }
 
-// The FP32 value nearest to v (ties to even) from its bits: a conversion
-// instruction issues on the FP64 pipe.
-__device__ inline float narrow(double v) {
-    const unsigned long long u = (unsigned long long)__double_as_longlong(v), m = u & 0x7fffffffffffffffull;
-    const unsigned e = (unsigned)(m >> 52);
-    if (e < 897 || e > 1150) return (float)v;   // zero, FP32 denormals, overflow
-    const unsigned long long t = m - (896ull << 52) + 0x0fffffffull + ((m >> 29) & 1);
-    return __uint_as_float((unsigned)(t >> 29) | ((unsigned)(u >> 32) & 0x80000000u));
-}
 template <typename R>
 __device__ inline R stored(double v) {
     if constexpr (sizeof(R) == 4) return narrow(v);
@@ -466,7 +457,7 @@ __device__ inline bool in_box(double x, double L) {
     return (b >= 0 && b < __double_as_longlong(L)) || b == (long long)0x8000000000000000ull;
 }
 __device__ inline bool finite_bits(double x) {
-    return (__double_as_longlong(x) & 0x7FF0000000000000ll) != 0x7FF0000000000000ll;
+    return (__double2hiint(x) & 0x7FF00000) != 0x7FF00000;   // (the 64-bit form compiles to an FP64 compare)
 }
 
 template <typename R>
@@ -794,7 +785,7 @@ int clear_moments(pic_t *h) {
 // rest, which keeps no touched-tile map).
 int clear_step_moments(pic_t *h) {
     if (!h->det) {
-        if (h->moments_cleared) {   // zeroed by the literal field solve that read them
+        if (h->moments_cleared) {   // zeroed by the field solve that read them
             h->moments_cleared = false;
             return 0;
         }
