@@ -680,11 +680,7 @@ struct SplineN {
 // without branches); returns the first node relative to the cell.
 template <typename R, int N>
 __device__ inline int spline_axis(R f, R (&w)[N + 1]) {
-    if constexpr (N == 1) {
-        w[0] = R(1) - f;
-        w[1] = f;
-        return 0;
-    } else if constexpr (N == 3) {
+    if constexpr (N == 3) {
         const R g = R(1) - f, f2 = f * f, g2 = g * g;
         w[0] = g2 * (g * R(1.0 / 6.0));
         w[1] = fma_r(f2, fma_r(R(0.5), f, R(-1)), R(2.0 / 3.0));
@@ -825,14 +821,6 @@ struct GlobalSink {
         atomicAdd(&M[(int64_t)k * g.nnode + (int64_t)spline_row(g, j) * g.nxn + spline_col(g, i)], v);
     }
 };
-// TileSink: a block's accumulator of W nodes per row, RN per moment, in shared memory.
-template <typename R>
-struct TileSink {
-    R *acc;
-    int W, RN;
-    __device__ inline void operator()(int i, int j, int k, R v) const { atomicAdd(&acc[k * RN + j * W + i], v); }
-};
-
 template <typename R, int N>
 struct SplineDep {
     static constexpr int NP = N + 1, NN = NP * NP, NS = NN * NMOM;
@@ -840,9 +828,9 @@ struct SplineDep {
     // a particle's row: 13 values (padded to VS), then the NN weights; FP32 row strides of 4 mod 8
     // words keep the 16-byte stores of 8 lanes on different banks
     static constexpr int VS = kFlat ? 14 : 16;
-    static constexpr int RS = kFlat ? (VS + NN + (NN & 1)) : (N == 1 ? 20 : N == 2 ? 28 : N == 3 ? 36 : 44);
-    static constexpr int HG = N == 1 ? 8 : N == 2 ? 3 : N == 3 ? 2 : 1;     // FP32: lanes per node
-    static constexpr int KW = N == 1 ? 2 : N == 2 ? 4 : N == 3 ? 8 : 13;    // and moments per lane
+    static constexpr int RS = kFlat ? (VS + NN + (NN & 1)) : (N == 2 ? 28 : N == 3 ? 36 : 44);
+    static constexpr int HG = N == 2 ? 3 : N == 3 ? 2 : 1;     // FP32: lanes per node
+    static constexpr int KW = N == 2 ? 4 : N == 3 ? 8 : 13;    // and moments per lane
     static constexpr int J = kFlat ? (NS + 31) / 32 : (N == 2 ? 5 : KW);    // sums per lane
     static constexpr int kWarpBytes = 32 * RS * (int)sizeof(R);
 
@@ -911,21 +899,15 @@ struct SplineDep {
             for (int p = p0; p < p1; ++p) {
                 const float *r = (const float *)rows + p * RS;
                 const float w = r[VS + node];
-                if constexpr (N == 1) {
-                    const float2 v = *(const float2 *)(r + m0);
-                    acc[0] = fmaf(w, v.x, acc[0]);
-                    acc[1] = fmaf(w, v.y, acc[1]);
-                } else {
 #pragma unroll
-                    for (int q = 0; q < (N == 4 ? 3 : KW / 4); ++q) {
-                        const float4 v = *(const float4 *)(r + m0 + 4 * q);
-                        acc[4 * q] = fmaf(w, v.x, acc[4 * q]);
-                        acc[4 * q + 1] = fmaf(w, v.y, acc[4 * q + 1]);
-                        acc[4 * q + 2] = fmaf(w, v.z, acc[4 * q + 2]);
-                        acc[4 * q + 3] = fmaf(w, v.w, acc[4 * q + 3]);
-                    }
-                    if constexpr (N != 3) acc[J - 1] = fmaf(w, r[12], acc[J - 1]);   // moment 12
+                for (int q = 0; q < (N == 4 ? 3 : KW / 4); ++q) {
+                    const float4 v = *(const float4 *)(r + m0 + 4 * q);
+                    acc[4 * q] = fmaf(w, v.x, acc[4 * q]);
+                    acc[4 * q + 1] = fmaf(w, v.y, acc[4 * q + 1]);
+                    acc[4 * q + 2] = fmaf(w, v.z, acc[4 * q + 2]);
+                    acc[4 * q + 3] = fmaf(w, v.w, acc[4 * q + 3]);
                 }
+                if constexpr (N != 3) acc[J - 1] = fmaf(w, r[12], acc[J - 1]);   // moment 12
             }
         }
     }

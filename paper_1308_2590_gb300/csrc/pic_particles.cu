@@ -5,6 +5,8 @@
 // (pic_internal.cuh).
 #include <math.h>
 
+#include <algorithm>
+
 #include "pic_internal.cuh"
 
 namespace pic {
@@ -33,15 +35,15 @@ struct DepArgs {
     int32_t *ticket;
 };
 
-// Work items of a deposit at rest: the runs of REST_SEGS segments of every
-// occupied bin, in any order; resident blocks take them from a queue.  (A grid
+// Work items of a deposit at rest: the runs of ch segments (REST_SEGS, the FP32
+// cell deposit more: rest_segs) of every occupied bin, in any order; resident blocks take them from a queue.  (A grid
 // of four blocks per tile started mostly empty blocks: 0.72 ms per species for
 // 0.16M particles in 131,072 tiles, whatever they held.)
 constexpr int REST_SEGS = 32;
-__global__ void k_rest_items(const int32_t *__restrict__ useg, int ntiles, int2 *__restrict__ items,
+__global__ void k_rest_items(const int32_t *__restrict__ useg, int ntiles, int ch, int2 *__restrict__ items,
                              int32_t *__restrict__ nitems) {
     const int t = blockIdx.x * blockDim.x + threadIdx.x;
-    const int n = t < ntiles ? (useg[t] + REST_SEGS - 1) / REST_SEGS : 0;
+    const int n = t < ntiles ? (useg[t] + ch - 1) / ch : 0;
     // one queue reservation per warp
     const int lane = threadIdx.x & 31;
     int incl = n;
@@ -206,16 +208,110 @@ __global__ void k_deposit_bins(DepArgs<R> a) {
     }
 }
 
+// FP32 sums of a cell's particles times its corner weights, in a warp's registers:
+// the particles' 13 values and 4 weights go to rows in shared memory, and 8 lanes,
+// (4 moments) x (2 corners), add every fourth row, the four groups of 8 rows of
+// their own: 10 instructions a lane and 4 rows, where lanes that each took 2
+// moments of a corner and every row spent 16, and half the shared memory
+// wavefronts that bound it.  The groups meet when the warp goes on to another cell.
+struct CellDep {
+    static constexpr int RS = 20;   // a row: 13 values, 3 of padding, weights (0,0), (1,0), (0,1), (1,1)
+    static constexpr int kWarpBytes = 32 * RS * (int)sizeof(float);
+    float *rows, *acc;              // acc: the block's tile, RN nodes of W per row and moment
+    int W, RN;
+    int node;                       // first node of the warp's cell, or -1
+    float s[8];                     // moments 4 (lane % 4) + .. of corner 2 (lane / 4 % 2), then of the next
+
+    __device__ inline void init(void *mem, float *tile, int w, int rn) {
+        rows = (float *)mem;
+        acc = tile;
+        W = w;
+        RN = rn;
+        node = -1;
+#pragma unroll
+        for (int k = 0; k < 8; ++k) s[k] = 0.f;
+    }
+
+    __device__ inline void flush(int lane) {
+        if (node < 0) return;
+        const bool h16 = lane & 16, h8 = lane & 8;
+        float r[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const float send = h16 ? s[k] : s[4 + k], own = h16 ? s[4 + k] : s[k];
+            r[k] = own + __shfl_xor_sync(0xffffffffu, send, 16);
+        }
+        const int m = 4 * (lane & 3) + (h8 ? 2 : 0);
+        float *a = acc + m * RN + node + (lane & 4 ? W : 0) + (h16 ? 1 : 0);
+#pragma unroll
+        for (int k = 0; k < 2; ++k) {
+            const float send = h8 ? r[k] : r[2 + k], own = h8 ? r[2 + k] : r[k];
+            const float t = own + __shfl_xor_sync(0xffffffffu, send, 8);
+            if (m + k < NMOM && t != 0.f) atomicAdd(a + k * RN, t);
+        }
+        node = -1;
+#pragma unroll
+        for (int k = 0; k < 8; ++k) s[k] = 0.f;
+    }
+
+    // All lanes: the particle of every valid lane, in the cell with first node n0.  Neighbouring lanes of
+    // a cell form a run (the bins are in cell order).
+    __device__ inline void add(bool valid, int n0, float fx, float fy, const float *val, int lane) {
+        const unsigned full = 0xffffffffu;
+        const int key = valid ? n0 : -1, prev = __shfl_up_sync(full, key, 1);
+        const bool head = valid && (lane == 0 || prev != key);
+        unsigned heads = __ballot_sync(full, head);
+        const unsigned ends = heads | __ballot_sync(full, !valid);
+        __syncwarp();   // the previous segment's rows have been read
+        if (valid) {
+            float4 *d = (float4 *)(rows + lane * RS);
+            d[0] = make_float4(val[0], val[1], val[2], val[3]);
+            d[1] = make_float4(val[4], val[5], val[6], val[7]);
+            d[2] = make_float4(val[8], val[9], val[10], val[11]);
+            d[3] = make_float4(val[12], 0.f, 0.f, 0.f);
+            d[4] = make_float4((1.f - fx) * (1.f - fy), fx * (1.f - fy), (1.f - fx) * fy, fx * fy);
+        }
+        __syncwarp();
+        const float *mine = rows + (lane >> 3) * RS;
+        const int ov = 4 * (lane & 3), ow = 16 + ((lane >> 1) & 2);
+        while (heads) {
+            const int p0 = __ffs(heads) - 1;
+            heads &= heads - 1;
+            const unsigned after = ends & ~((2u << p0) - 1u);
+            const int n = (after ? __ffs(after) - 1 : 32) - p0 - (lane >> 3);
+            const int k = __shfl_sync(full, key, p0);
+            if (k != node) {
+                flush(lane);
+                node = k;
+            }
+#pragma unroll 2
+            for (int p = 0; p < n; p += 4) {
+                const float *r = mine + (p0 + p) * RS;
+                const float4 v = *(const float4 *)(r + ov);
+                const float2 w = *(const float2 *)(r + ow);
+                s[0] = fmaf(w.x, v.x, s[0]);
+                s[1] = fmaf(w.x, v.y, s[1]);
+                s[2] = fmaf(w.x, v.z, s[2]);
+                s[3] = fmaf(w.x, v.w, s[3]);
+                s[4] = fmaf(w.y, v.x, s[4]);
+                s[5] = fmaf(w.y, v.y, s[5]);
+                s[6] = fmaf(w.y, v.z, s[6]);
+                s[7] = fmaf(w.y, v.w, s[7]);
+            }
+        }
+    }
+};
+
 // FP32 deposit with area weights from cell-ordered bins (at rest, and in the
 // steps that deposit after the regroup): a block takes an item (species, tile,
 // run of ch segments); its warps take contiguous segments and add them up cell
-// by cell (SplineDep, N = 1: the cell's 52 sums over the lanes, in registers)
-// into an accumulator over the tile's nodes in shared memory, which goes to the
-// global moments once per item with a TwoSum compensation term.  Every particle
-// lies in its bin's tile, so nothing leaves the accumulator's nodes.  Issue
-// bound (the row loop: two shared loads and two FMAs per particle and lane).
-// Per species at rest, 33.5M particles, 32 per cell: 0.87 ms with a butterfly
-// per segment and cell -> 0.67 ms.
+// by cell (CellDep) into an accumulator over the tile's nodes in shared memory,
+// which goes to the global moments once per item with a TwoSum compensation term.
+// Every particle lies in its bin's tile, so nothing leaves the accumulator's nodes.
+// 33.5M particles, 32 per cell: per species at rest 0.87 ms with a butterfly per
+// segment and cell; a step's two species 1.34 ms with a stencil's sums dealt over the
+// lanes, 1.35 with CellDep, 1.11 with the next segment's loads in flight as well
+// (issue 56 % and loads waited for before).
 struct CellDepSp {
     const int32_t *cell, *bstart, *useg, *segn;
     const float *ox, *oy, *ux, *uy, *uz, *w;
@@ -237,7 +333,7 @@ struct CellDepArgs {
 
 __host__ __device__ inline int cell_dep_nodes(int tnx, int tny) { return (tnx + 1) * (tny + 1); }
 __host__ __device__ inline int cell_dep_smem(int tnx, int tny) {
-    return cell_dep_nodes(tnx, tny) * (int)(sizeof(V4<float>) + NMOM * sizeof(float)) + 8 * SplineDep<float, 1>::kWarpBytes;
+    return cell_dep_nodes(tnx, tny) * (int)(sizeof(V4<float>) + NMOM * sizeof(float)) + 8 * CellDep::kWarpBytes;
 }
 
 __global__ void __launch_bounds__(256, 3) k_deposit_cells(const __grid_constant__ CellDepArgs a) {
@@ -248,10 +344,9 @@ __global__ void __launch_bounds__(256, 3) k_deposit_cells(const __grid_constant_
     const GridArgs<float> &g = a.g;
     const int W = a.tnx + 1, RN = W * (a.tny + 1);
     V4<float> *sB = (V4<float> *)dsm;
-    SplineDep<float, 1> dep;
-    dep.init((unsigned char *)(sB + RN) + wid * SplineDep<float, 1>::kWarpBytes, lane);
-    float *acc = (float *)((unsigned char *)(sB + RN) + 8 * SplineDep<float, 1>::kWarpBytes);
-    const TileSink<float> sink{acc, W, RN};
+    float *acc = (float *)((unsigned char *)(sB + RN) + 8 * CellDep::kWarpBytes);
+    CellDep dep;
+    dep.init((unsigned char *)(sB + RN) + wid * CellDep::kWarpBytes, acc, W, RN);
     const int nitems = *a.nitems;
     int2 it;
     while (next_item(a.items, nitems, a.ticket, &s_item, it)) {
@@ -268,20 +363,30 @@ __global__ void __launch_bounds__(256, 3) k_deposit_cells(const __grid_constant_
         const int64_t b0 = P.bstart[t];
         const int j0 = it.y * a.ch, j1 = min(j0 + a.ch, P.useg[t]);
         const int per = (j1 - j0 + 7) / 8, m0 = j0 + wid * per, m1 = min(m0 + per, j1);
-        for (int j = m0; j < m1; ++j) {
+        // the next segment's particles are in flight while this one's are added up (slots past a segment's
+        // count are allocated, their values unused)
+        struct {
+            int n;
+            int32_t c;
+            float fx, fy, ux, uy, uz, w;
+        } next = {0, 0, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+        auto fetch = [&](int j) {
             const int64_t p = b0 + (int64_t)j * SEG + lane;
-            bool valid = lane < P.segn[b0 / SEG + j];
-            int32_t c = 0;
-            float fx = 0.f, fy = 0.f, ux = 0.f, uy = 0.f, uz = 0.f, w = 0.f;
-            if (valid) {
-                c = P.cell[p];
-                fx = P.ox[p];
-                fy = P.oy[p];
-                ux = P.ux[p];
-                uy = P.uy[p];
-                uz = P.uz[p];
-                w = P.w[p];
-            }
+            next.n = P.segn[b0 / SEG + j];
+            next.c = P.cell[p];
+            next.fx = P.ox[p];
+            next.fy = P.oy[p];
+            next.ux = P.ux[p];
+            next.uy = P.uy[p];
+            next.uz = P.uz[p];
+            next.w = P.w[p];
+        };
+        if (m0 < m1) fetch(m0);
+        for (int j = m0; j < m1; ++j) {
+            bool valid = lane < next.n;
+            const int32_t c = valid ? next.c : 0;
+            const float fx = next.fx, fy = next.fy, ux = next.ux, uy = next.uy, uz = next.uz, w = next.w;
+            if (j + 1 < m1) fetch(j + 1);
             int cx, cy;
             cell_split(c, g.nx, a.magic_nx, cx, cy);
             const int lx = cx - X0, ly = cy - Y0;
@@ -291,9 +396,7 @@ __global__ void __launch_bounds__(256, 3) k_deposit_cells(const __grid_constant_
                 valid = false;
             }
             float val[NMOM];
-            SplineN<float, 1> sp;
             if (valid) {
-                sp = spline_n<float, 1>(lx, ly, fx, fy);
                 const V4<float> *r0 = sB + ly * W + lx, *r1 = r0 + W;
                 const V4<float> n00 = r0[0], n10 = r0[1], n01 = r1[0], n11 = r1[1];
                 const float w00 = (1.f - fx) * (1.f - fy), w10 = fx * (1.f - fy), w01 = (1.f - fx) * fy, w11 = fx * fy;
@@ -303,10 +406,9 @@ __global__ void __launch_bounds__(256, 3) k_deposit_cells(const __grid_constant_
                 float ig, bx, by, bz, inv;
                 particle_moments_c(P.q, P.kb, P.hq, w, ux, uy, uz, Bx, By, Bz, val, ig, bx, by, bz, inv);
             }
-            dep.add(sink, a.tnx, a.tny, valid, sp, val, lane);
+            dep.add(valid, ly * W + lx, fx, fy, val, lane);
         }
-        dep.flush(sink, lane);
-        dep.some = false;   // the next item's tile has other nodes
+        dep.flush(lane);   // (the next item's tile has other nodes)
         __syncthreads();
         for (int r = threadIdx.x; r < RN; r += 256) {
             const int ly = r / W, lx = r - ly * W;
@@ -674,6 +776,19 @@ int deposit_step(pic_t *h, const int32_t *guard0, const int32_t *guard1) {
     return cell_dep_launch(h, a);
 }
 
+// Segments per item of the FP32 cell deposit at rest: an item ends with the tile's
+// nodes going to the global moments (13 pairs of reductions each), so an item is
+// as long as leaves every resident block about four of them (the capacity is
+// about twice the particles).  With that and the loads ahead, 33.5M particles:
+// 0.88 ms in items of 32 -> 0.47 ms in items of 256; 3.3M: 85 -> 66 us.
+static int rest_segs(const SpeciesBuf &S) {
+    int dev = 0, nsm = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
+    const int64_t ch = S.cap / SEG / 2 / (12 * (nsm > 0 ? nsm : 1));
+    return (int)std::min<int64_t>(std::max<int64_t>(ch, REST_SEGS), 256);
+}
+
 template <typename R>
 static int deposit_only_t(pic_t *h, int s) {
     SpeciesBuf &S = h->sp[s];
@@ -710,13 +825,15 @@ static int deposit_only_t(pic_t *h, int s) {
     a.nitems = h->ticket;
     a.ticket = h->ticket + 1;
     cudaMemsetAsync(h->ticket, 0, 2 * sizeof(int32_t), h->st);
-    k_rest_items<<<(h->ntiles + 255) / 256, 256, 0, h->st>>>(a.useg, h->ntiles, h->items, h->ticket);
+    const bool cells = h->fp32 && !h->det && h->shape == 1;
+    const int ch = cells ? rest_segs(S) : REST_SEGS;
+    k_rest_items<<<(h->ntiles + 255) / 256, 256, 0, h->st>>>(a.useg, h->ntiles, ch, h->items, h->ticket);
     count_launch(h);
     const size_t tab = h->fp32 ? 0 : (size_t)h->tnx * h->tny * sizeof(CellC<double>);   // B in cell form
-    if (h->fp32 && !h->det && h->shape == 1) {
+    if (cells) {
         CellDepArgs c = cell_dep_args(h);
         c.sp[0] = cell_dep_species(h, s);
-        c.ch = REST_SEGS;
+        c.ch = ch;
         c.nitems = a.nitems;
         c.ticket = a.ticket;
         return cell_dep_launch(h, c);
