@@ -696,8 +696,12 @@ static const int32_t *device_view(const int32_t *p) {
 // before any regroup.
 // cells: checkpoint form (restore): per entry the cell indices, with x, y of d
 // holding the in-cell offsets; nullptr for global positions.
+// added (or nullptr): where the moments are current and kept as FP64 cell sums, the
+// new particles' are added to them (*added set; the caller brings the sums to the
+// nodes), instead of every particle's being deposited anew before they are next read.
+// The new particles must lie in tiles of the current tile lists.
 static int load_impl(pic_t *h, int nload, const int *species, const pic_species_data *d, const char *fn,
-                     const int32_t *const *cells = nullptr) {
+                     const int32_t *const *cells = nullptr, bool *added = nullptr) {
     bool seen[PIC_MAX_SPECIES] = {false};
     for (int e = 0; e < nload; ++e) {
         const int s = species[e];
@@ -901,11 +905,16 @@ static int load_impl(pic_t *h, int nload, const int *species, const pic_species_
         }
         return PIC_ERR_ARG;
     }
+    const bool add = added && !fresh && !h->moments_stale && h->Mc;
     if (!fresh)
         for (int e = 0; e < nload; ++e)
-            if (d[e].n > 0)
+            if (d[e].n > 0) {
+                if (add)
+                    if (int r = deposit_spare(h, species[e], d[e].n)) return r;
                 if (int r = rebuild_species(h, species[e], REBUILD_FROM_LOAD, d[e].n)) return r;
-    h->moments_stale = !eager;   // else deposited at the next step or readout
+            }
+    if (add) *added = true;
+    else h->moments_stale = !eager;   // else deposited at the next step or readout
     if (!fresh && (cudaMemcpyAsync(h->h_step_flags + 3, h->d_flags, sizeof(int32_t), cudaMemcpyDeviceToHost,
                                    main_st) != cudaSuccess ||
                    cudaStreamSynchronize(main_st) != cudaSuccess))
@@ -1065,7 +1074,14 @@ extern "C" PIC_API int pic_ionize(pic_t *h, const pic_ionization *p, int64_t *n_
         moff = pos;
     }
     if (int rc = check_launch("ionisation staging copies")) return rc;
-    if (int rc = load_impl(h, ndest, dest, data, "pic_ionize", cells)) return rc;
+    bool added = false;
+    if (int rc = load_impl(h, ndest, dest, data, "pic_ionize", cells, &added)) return rc;
+    if (added) {
+        // (the ionised particles lie in tiles that the last deposit's lists name: they have not moved since)
+        for (int c = 0; c < p->n_chains; ++c)
+            if (int rc = deposit_leavers(h, p->ion[c], nc[c], h->ion_cell + off[c], h->ion_val + off[c], h->ion_cap)) return rc;
+        if (int rc = cell_moments(h)) return rc;
+    }
     if (n_ionized) *n_ionized = done;
     return PIC_OK;
 }

@@ -992,6 +992,8 @@ int download_fields(pic_t *h, double *E3, double *H3);
 
 // particles (pic_particles.cu): conversion, deposit at rest, state export
 int deposit_only(pic_t *h, int s);
+int deposit_spare(pic_t *h, int s, int64_t n);   // FP64 cell sums: new particles still in the spare set
+int deposit_leavers(pic_t *h, int s, int64_t n, const int32_t *cell, const double *v, int64_t plane);   // and those gone
 bool post_deposit(const pic_t *h);      // the form whose steps deposit after the regroup
 int deposit_step(pic_t *h, const int32_t *guard0, const int32_t *guard1);   // that deposit, over the push's next work items
 int push_item_segs(const pic_t *h);     // segments per work item of the push

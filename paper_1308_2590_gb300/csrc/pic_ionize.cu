@@ -137,7 +137,7 @@ __global__ void k_ion_stage(int64_t n, const int32_t *__restrict__ pos, const in
 template <typename R>
 __global__ void k_ion_compact(const int32_t *__restrict__ bstart, const int32_t *__restrict__ useg,
                               int32_t *__restrict__ segn, const int32_t *__restrict__ removed, int32_t *cell, R *ox,
-                              R *oy, R *ux, R *uy, R *uz, R *w) {
+                              R *oy, R *ux, R *uy, R *uz, R *w, double *cr, int64_t ccap) {
     const int t = blockIdx.x;
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
     const int64_t b0 = bstart[t];
@@ -146,18 +146,26 @@ __global__ void k_ion_compact(const int32_t *__restrict__ bstart, const int32_t 
         const int64_t sg = b0 / SEG + j, slot = b0 + (int64_t)j * SEG + lane;
         const int n = segn[sg];
         const bool keep = lane < n && !removed[slot];
+        if (__all_sync(0xffffffffu, keep || lane >= n)) continue;
         int32_t c = 0;
         R a = R(0), b = R(0), d = R(0), e = R(0), f = R(0), h = R(0);
         if (keep) {
             c = cell[slot];
             a = ox[slot]; b = oy[slot]; d = ux[slot]; e = uy[slot]; f = uz[slot]; h = w[slot];
         }
+        double q[NCARRY];
+        if (cr && keep)
+#pragma unroll
+            for (int k = 0; k < NCARRY; ++k) q[k] = cr[k * ccap + slot];
         const unsigned m = __ballot_sync(0xffffffffu, keep);
         __syncwarp();
         if (keep) {
             const int64_t dst = b0 + (int64_t)j * SEG + __popc(m & ((1u << lane) - 1u));
             cell[dst] = c;
             ox[dst] = a; oy[dst] = b; ux[dst] = d; uy[dst] = e; uz[dst] = f; w[dst] = h;
+            if (cr)
+#pragma unroll
+                for (int k = 0; k < NCARRY; ++k) cr[k * ccap + dst] = q[k];
         }
         if (lane == 0) segn[sg] = __popc(m);
     }
@@ -212,7 +220,7 @@ static int ion_chain_t(pic_t *h, const IonChain &c, uint64_t seed, int32_t *scel
     if (int rc = ion_chain_t_launch_check("k_ion_stage")) return rc;
     k_ion_compact<R><<<h->ntiles, 256, 0, h->st>>>(S.bstart, S.useg[S.scur], S.segn[S.scur], removed, S.cell[b],
                                                    (R *)S.ox[b], (R *)S.oy[b], (R *)S.ux[b], (R *)S.uy[b],
-                                                   (R *)S.uz[b], (R *)S.w[b]);
+                                                   (R *)S.uz[b], (R *)S.w[b], S.carry[b], S.cap);
     count_launch(h);
     if (int rc = ion_chain_t_launch_check("k_ion_compact")) return rc;
     *n_out = k;

@@ -137,7 +137,7 @@ __global__ void k_radix_scatter(const uint32_t *__restrict__ kin, const uint32_t
 constexpr uint32_t DEAD = 0xFFFFFFFFu;
 
 // Keys of the particle order: tile * cpt + (ly * tile_nx + lx), the cell
-// inside the tile in row-major order (cpt = tile_nx * tile_ny).
+// inside the tile in row-major order (cpt = tile_nx * tile_ny, or more).
 struct KeyGeom {
     int nx, tnx, tny, ntx;
     uint32_t cpt;
@@ -344,8 +344,9 @@ __global__ void k_rebuild_gather(const uint32_t *__restrict__ keys, const uint32
 }
 
 // Load into a species that already holds particles: its bins are grouped by tile
-// as they are, so only the new particles are sorted globally, and each tile then
-// orders its bin's particles and its run of new ones by cell.
+// as they are, so only the new particles are grouped by tile (the key's bits above
+// the cell's), and each tile then orders its bin's particles and its run of new ones
+// by cell.
 //
 // ends[t] = cstart[t] + the tile's particles after the load (a warp per tile).
 __global__ void __launch_bounds__(256) k_merge_counts(const int32_t *__restrict__ bstart, const int32_t *__restrict__ useg,
@@ -367,7 +368,7 @@ __global__ void __launch_bounds__(256) k_merge_counts(const int32_t *__restrict_
 // counts before the scan over (cell, warp) are its places after it and the second
 // pass needs no block barrier.  Bound by the scattered 8-byte stores of the
 // twelve arrays (they stay inside the tile's few 100 KB: L2).  A carbon foil of
-// 0.8M ions FP64: 73 us, and 170 us a load less than the radix sort of
+// 0.8M ions FP64: 80 us, and 200 us a load less than the radix sort of
 // 2 x capacity keys and the gather that every load ran.
 constexpr int MERGE_WARPS = RADIX / 32;
 template <typename R>
@@ -438,9 +439,9 @@ __global__ void __launch_bounds__(RADIX) k_merge_tiles(
         d.cell[di] = (old ? s0.cell : s1.cell)[si];
 #pragma unroll
         for (int q = 0; q < 6; ++q) d.a[q][di] = (old ? s0.a[q] : s1.a[q])[si];
-        if (d.cr && old)   // (new particles carry nothing yet: their deposit at rest fills the planes)
+        if (d.cr)   // (a load's new particles carry nothing yet: their deposit at rest fills the planes)
 #pragma unroll
-            for (int q = 0; q < NCARRY; ++q) d.cr[q * d.ccap + di] = s0.cr[q * s0.ccap + si];
+            for (int q = 0; q < NCARRY; ++q) d.cr[q * d.ccap + di] = (old ? s0.cr : s1.cr)[q * d.ccap + si];
     }
 }
 
@@ -487,15 +488,15 @@ int ensure_sort_capacity(pic_t *h, int64_t n) {
 }
 
 // Stable radix sort of keys[0][0..n) (values = index); returns the index of
-// the key/value buffers that hold the result.
-static int radix_sort(pic_t *h, int64_t n, int bits, int *cur_out) {
-    int passes = (bits + 7) / 8;
+// the key/value buffers that hold the result.  By the bits from low on.
+static int radix_sort(pic_t *h, int64_t n, int bits, int *cur_out, int low = 0) {
+    int passes = (bits - low + 7) / 8;
     int64_t nb = sort_blocks(n);
     k_iota<<<(unsigned)((n + 255) / 256), 256, 0, h->st>>>(h->vals[0], n);
     count_launch(h);
     int cur = 0;
     for (int p = 0; p < passes; ++p) {
-        int shift = 8 * p;
+        int shift = low + 8 * p;
         k_radix_hist<<<(unsigned)nb, SORT_BS, 0, h->st>>>(h->keys[cur], n, shift, h->hist, nb);
         count_launch(h);
         if (int rc = check_launch("k_radix_hist")) return rc;
@@ -582,7 +583,7 @@ int init_empty_bins(pic_t *h, int s) {
 template <typename R>
 static int merge_load(pic_t *h, SpeciesBuf &S, const KeyGeom &kg, int64_t n_second, int bits) {
     int cur = 0;
-    if (int rc = radix_sort(h, n_second, bits, &cur)) return rc;
+    if (int rc = radix_sort(h, n_second, bits, &cur, 8)) return rc;   // (kg.cpt = 2^8)
     const size_t tb = (size_t)(h->ntiles + 1) * sizeof(int32_t);
     cudaMemsetAsync(S.cstart, 0, tb, h->st);
     cudaMemsetAsync(S.cend, 0, tb, h->st);
@@ -611,13 +612,14 @@ int rebuild_species(pic_t *h, int s, int source, int64_t n_second) {
     if (cap == 0) return 0;
     // a load into an empty species sorts only the new particles
     const bool fresh = (source == REBUILD_FROM_LOAD && S.n == 0);
-    const bool merge = source == REBUILD_FROM_LOAD && !fresh && h->tnx * h->tny <= RADIX;
+    const bool merge = source == REBUILD_FROM_LOAD && !fresh && h->tnx * h->tny <= RADIX &&
+                       (int64_t)h->ntiles * RADIX < 0xFFFFFFFell;
     const int64_t n = (fresh || merge) ? n_second : 2 * cap;
     if (n == 0) return 0;
     if (int rc = ensure_sort_capacity(h, n)) return rc;
     cudaMemsetAsync(h->keys[0], 0xFF, n * sizeof(uint32_t), h->st);
     int32_t *useg = S.useg[S.scur], *segn = S.segn[S.scur];
-    KeyGeom kg{h->nx, h->tnx, h->tny, h->ntx, (uint32_t)(h->tnx * h->tny)};
+    KeyGeom kg{h->nx, h->tnx, h->tny, h->ntx, merge ? (uint32_t)RADIX : (uint32_t)(h->tnx * h->tny)};
     const uint32_t div = kg.cpt;
     const int64_t maxkey = (int64_t)h->ntiles * kg.cpt;
     int second, out;
