@@ -182,6 +182,7 @@ struct pic_t {
     uint32_t *scan_sums = nullptr;      // per-block totals of the multi-block scans
     bool moments_stale = false;         // particles or B changed since the last deposit at rest
     bool post = false;                  // steps deposit after the regroup (post_deposit)
+    bool shared_gpu = false;            // steps beside other runs': no second stream (set_shared)
     cudaEvent_t ev_batch = nullptr;     // a batched step: this run's prologue is queued
     cudaStream_t st2 = nullptr;         // loads: regroups of converted species, beside the next conversion
     cudaEvent_t ev_load = nullptr;      // loads: st2's work joined back to st

@@ -24,6 +24,10 @@
 
 #include "pic.h"
 
+namespace pic {
+void set_shared(pic_t *h, bool on);   // pic_api.cu
+}
+
 namespace {
 
 struct Request {
@@ -184,6 +188,7 @@ void worker_loop(pic_server *srv) {
             if ((int)grp.size() < min_batch || kv.first >= 4) {
                 // a lone run (or a run of a spline shape: no batched form) steps on its own stream
                 for (Request *r : grp) {
+                    pic::set_shared(r->h, srv->running.size() > 1);
                     const int rc = pic_step(r->h, (int)k);
                     std::lock_guard<std::mutex> lk(srv->mu);
                     if (rc) r->st.error = rc;
