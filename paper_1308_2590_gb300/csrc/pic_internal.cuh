@@ -1003,6 +1003,8 @@ int clear_moments(pic_t *h);
 int clear_step_moments(pic_t *h);       // what a step's deposit adds into (the touched node tiles only)
 int fix_to_moments(pic_t *h);           // deterministic deposit: Mfix -> M (+ Mlo)
 int fix_scale(const pic_t *h, FixScale *out);
+constexpr int ABS_SUM_BLOCKS = 256;
+int abs_sum(pic_t *h, const double *w, int64_t n, double *part);   // part[ABS_SUM_BLOCKS]: shares of the sum of |w|
 int load_convert(pic_t *h, int s, int buf, int64_t n, const double *const src[6], unsigned long long *bad,
                  bool over_link, const int32_t *csrc = nullptr);
 // over_link: the arrays are page-locked host memory read in place; csrc: checkpoint form (src[0], src[1]

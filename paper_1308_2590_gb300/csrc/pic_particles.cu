@@ -988,6 +988,26 @@ int clear_step_moments(pic_t *h) {
     return 0;
 }
 
+// Shares of a sum of |w|: thread and block totals in a fixed order.
+__global__ void __launch_bounds__(256) k_abs_sum(const double *__restrict__ w, int64_t n, double *__restrict__ part) {
+    __shared__ double sh[256];
+    double a = 0.0;
+    for (int64_t p = (int64_t)blockIdx.x * 256 + threadIdx.x; p < n; p += (int64_t)gridDim.x * 256) a += fabs(w[p]);
+    sh[threadIdx.x] = a;
+    __syncthreads();
+    for (int o = 128; o > 0; o >>= 1) {
+        if (threadIdx.x < o) sh[threadIdx.x] += sh[threadIdx.x + o];
+        __syncthreads();
+    }
+    if (threadIdx.x == 0) part[blockIdx.x] = sh[0];
+}
+
+int abs_sum(pic_t *h, const double *w, int64_t n, double *part) {
+    k_abs_sum<<<ABS_SUM_BLOCKS, 256, 0, h->st>>>(w, n, part);
+    count_launch(h);
+    return check_launch("k_abs_sum");
+}
+
 // Class bounds from the weights loaded so far (see FixScale).
 int fix_scale(const pic_t *h, FixScale *out) {
     double B[3] = {0, 0, 0};
@@ -1002,7 +1022,9 @@ int fix_scale(const pic_t *h, FixScale *out) {
         int e = 0;
         if (B[c] > 0) {
             int x = 0;
-            frexp(B[c], &x);   // B <= 2^x
+            // B <= 2^x; a bound that is a power of two but for the order its sum was taken in (on the host or
+            // the device) is taken as one
+            frexp(B[c] * (1.0 + 0x1p-30), &x);
             e = 62 - x;
         }
         if (e < -120) {
