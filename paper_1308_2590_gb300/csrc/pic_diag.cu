@@ -318,7 +318,7 @@ __global__ void k_moments_out(const R *__restrict__ M, const R *__restrict__ Mlo
 #pragma unroll
         for (int k = 0; k < NMOM; ++k) {
             const int64_t t = (int64_t)k * nnode + n;
-            const double v = Mlo ? (double)M[t] + (double)Mlo[t] : (double)M[t];
+            const double v = Mlo ? widen(M[t]) + widen(Mlo[t]) : widen(M[t]);
             out[t] = v * f;
         }
     }

@@ -245,8 +245,16 @@ __global__ void __launch_bounds__(32 * FIELD_WARPS) k_field_HB(GridArgs<R> g, co
         const RowPair<RE> p = row_pair(ea, eb), q = shfl_down(p);   // columns i and i + 1
         eb = ea;
         // 2 dy dEz/dy = dz + dz', 2 dx dEz/dx = sz' - sz, 2 dx dEy/dx = sy' - sy, 2 dy dEx/dy = dx + dx'
-        const V4<R> w{(R)fma(-ky, p.dz + q.dz, (RE)h.x), (R)fma(kx, q.sz - p.sz, (RE)h.y),
-                      (R)fma(ky, p.dx + q.dx, fma(-kx, q.sy - p.sy, (RE)h.z)), R(0)};
+        auto in = [](R x) -> RE {
+            if constexpr (sizeof(RE) == 8) return widen(x);
+            else return x;
+        };
+        auto out = [](RE x) -> R {
+            if constexpr (sizeof(RE) == 8) return stored<R>(x);
+            else return x;
+        };
+        const V4<R> w{out(fma(-ky, p.dz + q.dz, in(h.x))), out(fma(kx, q.sz - p.sz, in(h.y))),
+                      out(fma(ky, p.dx + q.dx, fma(-kx, q.sy - p.sy, in(h.z)))), R(0)};
         if (j >= y0) {
             if (cell) Hout[(int64_t)j * g.nx + i] = w;
             const V4<R> s{below.x + w.x, below.y + w.y, below.z + w.z, R(0)};   // cells (i, j - 1) and (i, j)
@@ -1355,7 +1363,7 @@ __global__ void __launch_bounds__(BS, kCluster ? 1 : 3) k_cn_solve(GridArgs<doub
             V4<double> ax = apply_A_from_cells(g, v.x, v.cc, Md + N, ia, c2 * hx, c2 * hy, i, j, wr.cw, wr.cv);
             V4<double> b = v.b[n];
             V4<double> r{b.x - ax.x, b.y - ax.y, b.z - ax.z, 0.0};
-            V4<float> rf{(float)r.x, (float)r.y, (float)r.z, 0.f};
+            V4<float> rf{narrow(r.x), narrow(r.y), narrow(r.z), 0.f};
             v.r[n] = rf;
             if (!(v.fft && sc.sweep)) v.r0[n] = rf;
             s_rr += dot(r, r);
@@ -1396,7 +1404,7 @@ __global__ void __launch_bounds__(BS, kCluster ? 1 : 3) k_cn_solve(GridArgs<doub
                     V4<float> d{0.f, 0.f, 0.f, 0.f};
                     if (!first) d = v.d[n];
                     const V4<double> x = v.x[n];
-                    v.x[n] = V4<double>{x.x + (double)(d.x + z.x), x.y + (double)(d.y + z.y), x.z + (double)(d.z + z.z), 0.0};
+                    v.x[n] = V4<double>{x.x + widen(d.x + z.x), x.y + widen(d.y + z.y), x.z + widen(d.z + z.z), 0.0};
                 };
                 auto load_r = [&](int64_t n) { return v.r[n]; };
                 ++total;
@@ -1435,7 +1443,7 @@ __global__ void __launch_bounds__(BS, kCluster ? 1 : 3) k_cn_solve(GridArgs<doub
                     for (int n = tid; n < N; n += stride) {
                         const V4<double> x = v.x[n];
                         const V4<float> d = v.d[n];
-                        v.x[n] = V4<double>{x.x + (double)d.x, x.y + (double)d.y, x.z + (double)d.z, 0.0};
+                        v.x[n] = V4<double>{x.x + widen(d.x), x.y + widen(d.y), x.z + widen(d.z), 0.0};
                     }
                     break;
                 }
@@ -1574,7 +1582,7 @@ __global__ void __launch_bounds__(BS, kCluster ? 1 : 3) k_cn_solve(GridArgs<doub
             for (int n = tid; n < N; n += stride) {
                 V4<double> x = v.x[n];
                 V4<float> d = v.d[n];
-                v.x[n] = V4<double>{x.x + (double)d.x, x.y + (double)d.y, x.z + (double)d.z, 0.0};
+                v.x[n] = V4<double>{x.x + widen(d.x), x.y + widen(d.y), x.z + widen(d.z), 0.0};
             }
         grid.sync();
     }
@@ -1595,8 +1603,10 @@ __global__ void k_cn_finish(GridArgs<R> g, const V4<double> *__restrict__ X, con
     int64_t node = (int64_t)j * g.nxn + i;
     V4<double> x = X[node];
     V4<R> e = E[node];
-    Enew[node] = V4<R>{(R)(2.0 * x.x - (double)e.x), (R)(2.0 * x.y - (double)e.y), (R)(2.0 * x.z - (double)e.z), R(0)};
-    store_padded(Esum, g, i, j, V4<R>{(R)(2.0 * x.x), (R)(2.0 * x.y), (R)(2.0 * x.z), R(0)});
+    // (widths changed by their bits: 1024 x 1024 FP32 32 -> 16 us, and k_field_HB 52 -> 37)
+    Enew[node] = V4<R>{stored<R>(2.0 * x.x - widen(e.x)), stored<R>(2.0 * x.y - widen(e.y)),
+                       stored<R>(2.0 * x.z - widen(e.z)), R(0)};
+    store_padded(Esum, g, i, j, V4<R>{stored<R>(2.0 * x.x), stored<R>(2.0 * x.y), stored<R>(2.0 * x.z), R(0)});
 }
 
 // --------------------------------------------------------------------------- host side

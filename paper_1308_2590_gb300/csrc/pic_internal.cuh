@@ -307,6 +307,12 @@ __device__ inline double widen(float f) {
     return __longlong_as_double((long long)(d | (unsigned long long)(u & 0x80000000u) << 32));
 }
 __device__ inline double widen(double v) { return v; }
+// v in the storage type (FP64 or FP32).
+template <typename R>
+__device__ inline R stored(double v) {
+    if constexpr (sizeof(R) == 4) return narrow(v);
+    else return v;
+}
 
 // 1/sqrt(x) and 1/x: in FP32 the hardware approximations (2 ulp, far below the
 // FP32 form's tolerances); in FP64 the library's correctly rounded forms.

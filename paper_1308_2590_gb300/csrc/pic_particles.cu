@@ -592,12 +592,6 @@ __device__ inline double div_by(double x, double d, double rd) {
     return fma(fma(-q, d, x), rd, q);
 }
 
-template <typename R>
-__device__ inline R stored(double v) {
-    if constexpr (sizeof(R) == 4) return narrow(v);
-    else return v;
-}
-
 // floor(x) of 0 <= x < 2^31 as a double and an integer, from the bits.
 __device__ inline double floor_cell(double x, int &c) {
     const long long b = __double_as_longlong(x);
