@@ -7,6 +7,8 @@
 // tile keeps first the particles that stayed, in their previous order, then
 // the arrivals in their previous order; removed particles carry the largest
 // key and end up past the live count.
+#include <cooperative_groups.h>
+
 #include <utility>
 
 #include "pic_internal.cuh"
@@ -225,25 +227,30 @@ __device__ inline long long block_excl_scan(long long c, long long *wsum, long l
     return ex;
 }
 
-// One block; each thread takes LAYOUT_IPT tiles of a round, so that a grid of
-// 131,072 tiles takes 16 rounds of scans instead of 128 (298 -> 240 us).
-constexpr int LAYOUT_IPT = 8;
-__global__ void __launch_bounds__(1024) k_layout(const int32_t *__restrict__ cstart, const int32_t *__restrict__ cend,
-                                                 int ntiles, int64_t cap, int32_t *__restrict__ bstart,
-                                                 int32_t *__restrict__ tcount, int32_t *__restrict__ useg,
-                                                 int32_t *__restrict__ flags) {
-    __shared__ long long wsum[33];
+// A cluster of LAYOUT_BLOCKS blocks, each with a contiguous part of the tiles (one
+// block took 240 us for 131,072 tiles and 18 us for 8192; now 38 and 10 us); each
+// thread takes LAYOUT_IPT tiles of a round.
+constexpr int LAYOUT_IPT = 8, LAYOUT_BLOCKS = 8;
+__global__ void __cluster_dims__(LAYOUT_BLOCKS, 1, 1) __launch_bounds__(1024)
+    k_layout(const int32_t *__restrict__ cstart, const int32_t *__restrict__ cend, int ntiles, int64_t cap,
+             int32_t *__restrict__ bstart, int32_t *__restrict__ tcount, int32_t *__restrict__ useg,
+             int32_t *__restrict__ flags) {
+    __shared__ long long wsum[33], mine[2];   // mine: this block's shares of the two totals
+    const auto cluster = cooperative_groups::this_cluster();
+    const int rank = (int)cluster.block_rank();
+    const int part = (ntiles + LAYOUT_BLOCKS * LAYOUT_IPT - 1) / (LAYOUT_BLOCKS * LAYOUT_IPT) * LAYOUT_IPT;
+    const int lo = min(rank * part, ntiles), hi = min(lo + part, ntiles);
     long long tot_slack = 0, tot_tight = 0;
     auto rnd = [](long long v) { return (v + SEG - 1) / SEG * SEG; };
     const int per = blockDim.x * LAYOUT_IPT;
     {
         long long a = 0, b = 0;   // this thread's shares of the two totals
-        for (int base = 0; base < ntiles; base += per) {
+        for (int base = lo; base < hi; base += per) {
             int n[LAYOUT_IPT];   // all in flight at once
 #pragma unroll
             for (int k = 0; k < LAYOUT_IPT; ++k) {
                 const int t = base + k * (int)blockDim.x + (int)threadIdx.x;
-                n[k] = t < ntiles ? cend[t] - cstart[t] : -1;
+                n[k] = t < hi ? cend[t] - cstart[t] : -1;
             }
 #pragma unroll
             for (int k = 0; k < LAYOUT_IPT; ++k) {
@@ -254,15 +261,31 @@ __global__ void __launch_bounds__(1024) k_layout(const int32_t *__restrict__ cst
                 }
             }
         }
-        block_excl_scan(a, wsum, tot_slack);
-        block_excl_scan(b, wsum, tot_tight);
+        long long ta, tb;
+        block_excl_scan(a, wsum, ta);
+        block_excl_scan(b, wsum, tb);
+        if (threadIdx.x == 0) {
+            mine[0] = ta;
+            mine[1] = tb;
+        }
     }
+    cluster.sync();
+    long long before[2] = {0, 0};   // the shares of the blocks before this one
+    for (int r = 0; r < LAYOUT_BLOCKS; ++r) {
+        const long long *m = cluster.map_shared_rank(mine, r);
+        const long long ta = m[0], tb = m[1];
+        tot_slack += ta;
+        tot_tight += tb;
+        before[0] += r < rank ? ta : 0;
+        before[1] += r < rank ? tb : 0;
+    }
+    cluster.sync();   // (every block has read the others' shares before one leaves)
     const int mode = (tot_slack <= cap) ? 0 : (tot_tight <= cap ? 1 : 2);
-    long long carry = 0;
-    for (int base = 0; base < ntiles; base += per) {
+    long long carry = mode == 2 ? 0 : before[mode];
+    for (int base = lo; base < hi; base += per) {
         const int t0 = base + (int)threadIdx.x * LAYOUT_IPT;
         alignas(16) int n[LAYOUT_IPT], s[LAYOUT_IPT];
-        if (t0 + LAYOUT_IPT <= ntiles) {   // (the arrays are 256-byte aligned, t0 a multiple of 8)
+        if (t0 + LAYOUT_IPT <= hi) {   // (the arrays are 256-byte aligned, t0 a multiple of 8)
             *(int4 *)n = *(const int4 *)(cend + t0);
             *(int4 *)(n + 4) = *(const int4 *)(cend + t0 + 4);
             *(int4 *)s = *(const int4 *)(cstart + t0);
@@ -270,16 +293,16 @@ __global__ void __launch_bounds__(1024) k_layout(const int32_t *__restrict__ cst
         } else {
 #pragma unroll
             for (int k = 0; k < LAYOUT_IPT; ++k) {
-                n[k] = t0 + k < ntiles ? cend[t0 + k] : 0;
-                s[k] = t0 + k < ntiles ? cstart[t0 + k] : 0;
+                n[k] = t0 + k < hi ? cend[t0 + k] : 0;
+                s[k] = t0 + k < hi ? cstart[t0 + k] : 0;
             }
         }
         long long cnt[LAYOUT_IPT], c[LAYOUT_IPT], sum = 0;
 #pragma unroll
         for (int k = 0; k < LAYOUT_IPT; ++k) {
             const int t = t0 + k;
-            cnt[k] = (t < ntiles && mode != 2) ? (long long)(n[k] - s[k]) : 0;
-            c[k] = (t < ntiles && mode != 2) ? (mode == 0 ? rnd(cnt[k] + cnt[k] / 4 + 2 * SEG) : rnd(cnt[k])) : 0;
+            cnt[k] = (t < hi && mode != 2) ? (long long)(n[k] - s[k]) : 0;
+            c[k] = (t < hi && mode != 2) ? (mode == 0 ? rnd(cnt[k] + cnt[k] / 4 + 2 * SEG) : rnd(cnt[k])) : 0;
             sum += c[k];
         }
         long long tot;
@@ -287,7 +310,7 @@ __global__ void __launch_bounds__(1024) k_layout(const int32_t *__restrict__ cst
 #pragma unroll
         for (int k = 0; k < LAYOUT_IPT; ++k) {
             const int t = t0 + k;
-            if (t < ntiles) {
+            if (t < hi) {
                 bstart[t] = (int32_t)at;
                 tcount[t] = (int32_t)cnt[k];
                 useg[t] = (int32_t)((cnt[k] + SEG - 1) / SEG);
@@ -296,7 +319,7 @@ __global__ void __launch_bounds__(1024) k_layout(const int32_t *__restrict__ cst
         }
         carry += tot;
     }
-    if (threadIdx.x == 0) {
+    if (threadIdx.x == 0 && rank == LAYOUT_BLOCKS - 1) {
         bstart[ntiles] = (int32_t)carry;
         if (mode == 2) atomicOr(flags, 4);
     }
@@ -594,7 +617,7 @@ static int merge_load(pic_t *h, SpeciesBuf &S, const KeyGeom &kg, int64_t n_seco
     cudaMemcpyAsync(old, S.bstart, tb, cudaMemcpyDeviceToDevice, h->st);
     const unsigned nbt = (unsigned)((h->ntiles + 7) / 8);
     k_merge_counts<<<nbt, 256, 0, h->st>>>(old, S.useg[o], S.segn[o], h->ntiles, S.cend, ends);
-    k_layout<<<1, 1024, 0, h->st>>>(S.cstart, ends, h->ntiles, S.cap, S.bstart, S.tcount, S.useg[nw], h->d_flags);
+    k_layout<<<LAYOUT_BLOCKS, 1024, 0, h->st>>>(S.cstart, ends, h->ntiles, S.cap, S.bstart, S.tcount, S.useg[nw], h->d_flags);
     k_layout_segs<<<nbt, 256, 0, h->st>>>(S.bstart, S.tcount, h->ntiles, S.segn[nw]);
     k_merge_tiles<R><<<h->ntiles, RADIX, 0, h->st>>>(old, S.useg[o], S.segn[o], h->keys[cur], h->vals[cur], S.cstart,
                                                      S.cend, S.bstart, S.tcount, kg, buf7<R>(S, S.bins),
@@ -656,7 +679,7 @@ int rebuild_species(pic_t *h, int s, int source, int64_t n_second) {
     cudaMemsetAsync(S.cend, 0, tb, h->st);
     k_run_bounds<<<(unsigned)((n + 255) / 256), 256, 0, h->st>>>(h->keys[cur], n, div, S.cstart, S.cend);
     count_launch(h);
-    k_layout<<<1, 1024, 0, h->st>>>(S.cstart, S.cend, h->ntiles, cap, S.bstart, S.tcount, useg, h->d_flags);
+    k_layout<<<LAYOUT_BLOCKS, 1024, 0, h->st>>>(S.cstart, S.cend, h->ntiles, cap, S.bstart, S.tcount, useg, h->d_flags);
     count_launch(h);
     k_layout_segs<<<(h->ntiles + 7) / 8, 256, 0, h->st>>>(S.bstart, S.tcount, h->ntiles, segn);
     count_launch(h);
