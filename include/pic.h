@@ -533,7 +533,7 @@ PIC_API double pic_server_now(pic_server *srv);
 
 /* Batched stepping of several runs (what the server uses).  A batch owns the
  * scratch of the batched launches: up to max_runs argument blocks in device
- * and page-locked host memory and the work-list prefixes.  pic_batch_step
+ * and page-locked host memory and their work-item prefixes.  pic_batch_step
  * advances n runs by nsteps: each run's field solve, regroup decision and
  * clears stay on its own stream, then ONE persistent push launch over the
  * (run, species, tile, segment run) work items of all n runs and ONE regroup

@@ -1084,16 +1084,28 @@ int load_convert(pic_t *h, int s, int buf, int64_t n, const double *const src[6]
                    : load_convert_t<double>(h, s, buf, n, src, bad, over_link, csrc);
 }
 
-int count_species(pic_t *h, int s, int64_t *n_out) {
-    SpeciesBuf &S = h->sp[s];
-    if (S.cap == 0) {
-        *n_out = 0;
-        return 0;
+// *total += the particles of the tiles, a warp per tile.
+__global__ void __launch_bounds__(256) k_count(const int32_t *__restrict__ bstart, const int32_t *__restrict__ useg,
+                                               const int32_t *__restrict__ segn, int ntiles, int32_t *__restrict__ total) {
+    __shared__ int sum;
+    if (threadIdx.x == 0) sum = 0;
+    __syncthreads();
+    const int lane = threadIdx.x & 31;
+    int c = 0;
+    for (int t = blockIdx.x * 8 + (threadIdx.x >> 5); t < ntiles; t += gridDim.x * 8) {
+        const int64_t sb = bstart[t] / SEG;
+        const int u = useg[t];
+        for (int j = lane; j < u; j += 32) c += segn[sb + j];
     }
-    if (int rc = tile_counts(h, s)) return rc;
-    if (int rc = scan_tiles(h, S.tcount, S.cstart)) return rc;
+    for (int o = 16; o > 0; o >>= 1) c += __shfl_down_sync(0xffffffffu, c, o);
+    if (lane == 0 && c) atomicAdd(&sum, c);
+    __syncthreads();
+    if (threadIdx.x == 0 && sum) atomicAdd(total, sum);
+}
+
+static int read_count(pic_t *h, SpeciesBuf &S, const int32_t *src, int64_t *n_out) {
     int32_t tot = 0;
-    cudaError_t e = cudaMemcpyAsync(&tot, S.cstart + h->ntiles, sizeof(int32_t), cudaMemcpyDeviceToHost, h->st);
+    cudaError_t e = cudaMemcpyAsync(&tot, src, sizeof(int32_t), cudaMemcpyDeviceToHost, h->st);
     if (e == cudaSuccess) e = cudaStreamSynchronize(h->st);
     if (e != cudaSuccess) {
         set_error("count readback: %s", cudaGetErrorString(e));
@@ -1103,6 +1115,37 @@ int count_species(pic_t *h, int s, int64_t *n_out) {
     S.n = tot;
     S.n_exact = true;
     return 0;
+}
+
+// Live particles of a species (known on the host unless a step ran since): one sum over the segment
+// counts (counts per tile and their scan, which only the export needs, took five launches: 23 us
+// against 4 us on 8192 tiles, five times in an ionisation pass).
+int count_species(pic_t *h, int s, int64_t *n_out) {
+    SpeciesBuf &S = h->sp[s];
+    if (S.cap == 0 || S.n_exact) {
+        *n_out = S.cap == 0 ? 0 : S.n;
+        return 0;
+    }
+    int dev = 0, nsm = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
+    int32_t *total = h->ticket + 2;   // (words 0 and 1: a deposit at rest)
+    cudaMemsetAsync(total, 0, sizeof(int32_t), h->st);
+    const int blocks = std::min((h->ntiles + 7) / 8, 8 * (nsm > 0 ? nsm : 1));
+    k_count<<<blocks, 256, 0, h->st>>>(S.bstart, S.useg[S.scur], S.segn[S.scur], h->ntiles, total);
+    count_launch(h);
+    if (int rc = check_launch("k_count")) return rc;
+    return read_count(h, S, total, n_out);
+}
+
+// The same with the tiles' compact starts in cstart.
+static int count_starts(pic_t *h, int s, int64_t *n_out) {
+    SpeciesBuf &S = h->sp[s];
+    *n_out = 0;
+    if (S.cap == 0) return 0;
+    if (int rc = tile_counts(h, s)) return rc;
+    if (int rc = scan_tiles(h, S.tcount, S.cstart)) return rc;
+    return read_count(h, S, S.cstart + h->ntiles, n_out);
 }
 
 int ensure_stage_doubles(pic_t *h, int64_t ndoubles);
@@ -1124,7 +1167,7 @@ static int to_stage_t(pic_t *h, int s, int64_t n, bool raw) {
 // raw: the stored in-cell offsets instead of global positions.
 int particles_to_stage(pic_t *h, int s, int64_t *n_out, bool raw) {
     int64_t n = 0;
-    if (int rc = count_species(h, s, &n)) return rc;  // also leaves the compact starts in cstart
+    if (int rc = count_starts(h, s, &n)) return rc;
     *n_out = n;
     if (n == 0) return 0;
     if (int rc = ensure_stage_doubles(h, 7 * n)) return rc;
