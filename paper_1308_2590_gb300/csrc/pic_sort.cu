@@ -25,9 +25,20 @@ constexpr int SCAN_IPB = SCAN_BS * SCAN_IPT;
 
 static int64_t sort_blocks(int64_t n) { return (n + SORT_IPB - 1) / SORT_IPB; }
 
+// The passes over a load's items: 256 threads a block, EACH items a thread.  With an
+// item a thread, 131,072 blocks for 33.5M items, the start of the blocks and one
+// load in flight bound them: keys 121 us, runs of the tiles 124 us, gather of the
+// FP32 state 572 us; now 100, 75 and 378 us.
+constexpr int EACH = 4;
+static unsigned each_blocks(int64_t n) { return (unsigned)((n + 256 * EACH - 1) / (256 * EACH)); }
+__device__ inline int64_t each_item(int k) { return (int64_t)blockIdx.x * (256 * EACH) + k * 256 + threadIdx.x; }
+
 __global__ void k_iota(uint32_t *v, int64_t n) {
-    int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (t < n) v[t] = (uint32_t)t;
+#pragma unroll
+    for (int k = 0; k < EACH; ++k) {
+        const int64_t t = each_item(k);
+        if (t < n) v[t] = (uint32_t)t;
+    }
 }
 
 // Per-block digit histogram, stored digit-major: hist[d * nblocks + b].
@@ -180,21 +191,33 @@ __global__ void k_keys_mirror(const int32_t *__restrict__ bstart, const int32_t 
 // keys of freshly loaded particles (compact, in load order), from key index off
 __global__ void k_keys_stage(const int32_t *__restrict__ cell, int64_t n, KeyGeom kg, int64_t off,
                              uint32_t *__restrict__ keys) {
-    int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (p >= n) return;
-    keys[off + p] = order_key(kg, cell[p]);
+    int32_t c[EACH];
+#pragma unroll
+    for (int k = 0; k < EACH; ++k) c[k] = each_item(k) < n ? cell[each_item(k)] : 0;
+#pragma unroll
+    for (int k = 0; k < EACH; ++k)
+        if (each_item(k) < n) keys[off + each_item(k)] = order_key(kg, c[k]);
 }
 
 // start / end of each tile's run in the sorted keys (tile = key / div)
 __global__ void k_run_bounds(const uint32_t *__restrict__ keys, int64_t n, uint32_t div, int32_t *__restrict__ cstart,
                              int32_t *__restrict__ cend) {
-    int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (p >= n) return;
-    uint32_t k = keys[p];
-    if (k == DEAD) return;
-    uint32_t t = k / div;
-    if (p == 0 || keys[p - 1] / div != t) cstart[t] = (int32_t)p;
-    if (p + 1 == n || keys[p + 1] == DEAD || keys[p + 1] / div != t) cend[t] = (int32_t)(p + 1);
+    uint32_t key[EACH], before[EACH], after[EACH];
+#pragma unroll
+    for (int k = 0; k < EACH; ++k) {
+        const int64_t p = each_item(k);
+        key[k] = p < n ? keys[p] : DEAD;
+        before[k] = p > 0 && p < n ? keys[p - 1] : DEAD;
+        after[k] = p + 1 < n ? keys[p + 1] : DEAD;
+    }
+#pragma unroll
+    for (int k = 0; k < EACH; ++k) {
+        if (key[k] == DEAD) continue;
+        const int64_t p = each_item(k);
+        const uint32_t t = key[k] / div;
+        if (before[k] == DEAD || before[k] / div != t) cstart[t] = (int32_t)p;   // (sorted: none dead before)
+        if (after[k] == DEAD || after[k] / div != t) cend[t] = (int32_t)(p + 1);
+    }
 }
 
 // New bins from the run lengths: capacity count + count/4 + 32 per tile while
@@ -349,21 +372,34 @@ __global__ void k_rebuild_gather(const uint32_t *__restrict__ keys, const uint32
                                  uint32_t div, int64_t cap, const int32_t *__restrict__ cstart,
                                  const int32_t *__restrict__ bstart, const int32_t *__restrict__ flags, Buf7<R> s0,
                                  Buf7<R> s1, Buf7<R> d) {
-    int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (p >= n) return;
-    uint32_t k = keys[p];
-    if (k == DEAD || (*flags & 4)) return;
-    uint32_t t = k / div;
-    uint32_t v = vals[p];
-    const Buf7<R> &src = (v < cap) ? s0 : s1;
-    int64_t si = (v < cap) ? (int64_t)v : (int64_t)v - cap;
-    int64_t di = (int64_t)bstart[t] + (p - cstart[t]);
-    d.cell[di] = src.cell[si];
+    if (*flags & 4) return;
+    int64_t si[EACH], di[EACH];   // (di -1: none)
+    bool first[EACH];
 #pragma unroll
-    for (int q = 0; q < 6; ++q) d.a[q][di] = src.a[q][si];
+    for (int k = 0; k < EACH; ++k) {
+        const int64_t p = each_item(k);
+        const uint32_t key = p < n ? keys[p] : DEAD, v = p < n ? vals[p] : 0u;
+        first[k] = (int64_t)v < cap;
+        si[k] = first[k] ? (int64_t)v : (int64_t)v - cap;
+        di[k] = -1;
+        if (key == DEAD) continue;
+        const uint32_t t = key / div;
+        di[k] = (int64_t)bstart[t] + (p - cstart[t]);
+    }
+    auto move = [&](const auto *a, const auto *b, auto *out) {
+        decltype(a[0] + a[0]) v[EACH];   // every load before a store
+#pragma unroll
+        for (int k = 0; k < EACH; ++k) v[k] = di[k] >= 0 ? (first[k] ? a : b)[si[k]] : 0;
+#pragma unroll
+        for (int k = 0; k < EACH; ++k)
+            if (di[k] >= 0) out[di[k]] = v[k];
+    };
+    move(s0.cell, s1.cell, d.cell);
+#pragma unroll
+    for (int q = 0; q < 6; ++q) move(s0.a[q], s1.a[q], d.a[q]);
     if (d.cr)   // (a load's new particles carry nothing yet: their deposit at rest fills the planes)
 #pragma unroll
-        for (int q = 0; q < NCARRY; ++q) d.cr[q * d.ccap + di] = src.cr[q * src.ccap + si];
+        for (int q = 0; q < NCARRY; ++q) move(s0.cr + q * s0.ccap, s1.cr + q * s1.ccap, d.cr + q * d.ccap);
 }
 
 // Load into a species that already holds particles: its bins are grouped by tile
@@ -515,7 +551,7 @@ int ensure_sort_capacity(pic_t *h, int64_t n) {
 static int radix_sort(pic_t *h, int64_t n, int bits, int *cur_out, int low = 0) {
     int passes = (bits - low + 7) / 8;
     int64_t nb = sort_blocks(n);
-    k_iota<<<(unsigned)((n + 255) / 256), 256, 0, h->st>>>(h->vals[0], n);
+    k_iota<<<each_blocks(n), 256, 0, h->st>>>(h->vals[0], n);
     count_launch(h);
     int cur = 0;
     for (int p = 0; p < passes; ++p) {
@@ -610,7 +646,7 @@ static int merge_load(pic_t *h, SpeciesBuf &S, const KeyGeom &kg, int64_t n_seco
     const size_t tb = (size_t)(h->ntiles + 1) * sizeof(int32_t);
     cudaMemsetAsync(S.cstart, 0, tb, h->st);
     cudaMemsetAsync(S.cend, 0, tb, h->st);
-    k_run_bounds<<<(unsigned)((n_second + 255) / 256), 256, 0, h->st>>>(h->keys[cur], n_second, kg.cpt, S.cstart, S.cend);
+    k_run_bounds<<<each_blocks(n_second), 256, 0, h->st>>>(h->keys[cur], n_second, kg.cpt, S.cstart, S.cend);
     // the sort's other buffers hold at least 2 x capacity words, more than the tiles
     int32_t *old = (int32_t *)h->vals[1 - cur], *ends = (int32_t *)h->keys[1 - cur];
     const int o = S.scur, nw = 1 - o;
@@ -657,7 +693,7 @@ int rebuild_species(pic_t *h, int s, int source, int64_t n_second) {
         out = S.spare;
     } else {
         if (n_second > 0) {
-            k_keys_stage<<<(unsigned)((n_second + 255) / 256), 256, 0, h->st>>>(S.cell[S.spare], n_second, kg,
+            k_keys_stage<<<each_blocks(n_second), 256, 0, h->st>>>(S.cell[S.spare], n_second, kg,
                                                                               fresh || merge ? 0 : cap, h->keys[0]);
             count_launch(h);
         }
@@ -677,14 +713,14 @@ int rebuild_species(pic_t *h, int s, int source, int64_t n_second) {
     size_t tb = (size_t)(h->ntiles + 1) * sizeof(int32_t);
     cudaMemsetAsync(S.cstart, 0, tb, h->st);
     cudaMemsetAsync(S.cend, 0, tb, h->st);
-    k_run_bounds<<<(unsigned)((n + 255) / 256), 256, 0, h->st>>>(h->keys[cur], n, div, S.cstart, S.cend);
+    k_run_bounds<<<each_blocks(n), 256, 0, h->st>>>(h->keys[cur], n, div, S.cstart, S.cend);
     count_launch(h);
     k_layout<<<LAYOUT_BLOCKS, 1024, 0, h->st>>>(S.cstart, S.cend, h->ntiles, cap, S.bstart, S.tcount, useg, h->d_flags);
     count_launch(h);
     k_layout_segs<<<(h->ntiles + 7) / 8, 256, 0, h->st>>>(S.bstart, S.tcount, h->ntiles, segn);
     count_launch(h);
     if (int rc = check_launch("rebuild layout")) return rc;
-    unsigned nbk = (unsigned)((n + 255) / 256);
+    const unsigned nbk = each_blocks(n);
     // item v < cap comes from the first buffer (the bins, or the new particles when fresh), else the second
     const int first = fresh ? second : S.bins;
     if (h->fp32)
@@ -800,7 +836,7 @@ extern "C" PIC_API int pic_sort_keys_noalloc(const uint32_t *keys, int64_t n, ui
     int64_t nb = (n + SORT_IPB - 1) / SORT_IPB;
     // every pass overwrites the histogram and the buffers it reads, so nothing
     // in the scratch has to start at zero
-    k_iota<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(vbuf[0], n);
+    k_iota<<<each_blocks(n), 256, 0, st>>>(vbuf[0], n);
     if (int rc = check_launch("pic_sort_keys_noalloc iota")) return rc;
     const uint32_t *kin = keys;
     const uint32_t *vin = vbuf[0];
