@@ -427,8 +427,9 @@ __global__ void __launch_bounds__(256) k_merge_counts(const int32_t *__restrict_
 // counts before the scan over (cell, warp) are its places after it and the second
 // pass needs no block barrier.  Bound by the scattered 8-byte stores of the
 // twelve arrays (they stay inside the tile's few 100 KB: L2).  A carbon foil of
-// 0.8M ions FP64: 80 us, and 200 us a load less than the radix sort of
-// 2 x capacity keys and the gather that every load ran.
+// 0.8M ions FP64: 58 us with two segments a warp in flight (80 with one), and 220 us
+// a load less than the radix sort of 2 x capacity keys and the gather that every
+// load ran.
 constexpr int MERGE_WARPS = RADIX / 32;
 template <typename R>
 __global__ void __launch_bounds__(RADIX) k_merge_tiles(
@@ -483,24 +484,44 @@ __global__ void __launch_bounds__(RADIX) k_merge_tiles(
     for (int w = 0; w < MERGE_WARPS; ++w) cnt[w][threadIdx.x] += base;
     __syncthreads();
     const int64_t n0 = newstart[t];
-    for (int j = j0; j < j1; ++j) {
-        const uint32_t k = cell_of(j);
-        const unsigned mask = __match_any_sync(0xffffffffu, k);
-        const bool on = k < RADIX;
-        const uint32_t at = on ? cnt[wid][k] : 0u;
-        __syncwarp();
-        if (on && __ffs(mask) - 1 == lane) cnt[wid][k] = at + __popc(mask);
-        __syncwarp();
-        if (!on) continue;
-        const int64_t di = n0 + at + __popc(mask & lt);
-        const bool old = j < u;
-        const int64_t si = old ? b0 + (int64_t)j * SEG + lane : (int64_t)vals[c0 + (j - u) * SEG + lane];
-        d.cell[di] = (old ? s0.cell : s1.cell)[si];
+    constexpr int D = 2;   // segments whose particles are in flight at once
+    constexpr int NC = sizeof(R) == 8 ? NCARRY : 1;
+    for (int jj = j0; jj < j1; jj += D) {
+        uint32_t k[D];
+        int32_t c[D];
+        R v[D][6];
+        double w[D][NC];
 #pragma unroll
-        for (int q = 0; q < 6; ++q) d.a[q][di] = (old ? s0.a[q] : s1.a[q])[si];
-        if (d.cr)   // (a load's new particles carry nothing yet: their deposit at rest fills the planes)
+        for (int u2 = 0; u2 < D; ++u2) {
+            const int j = jj + u2;
+            k[u2] = j < j1 ? cell_of(j) : RADIX + lane;
+            if (k[u2] >= RADIX) continue;
+            const bool old = j < u;
+            const int64_t si = old ? b0 + (int64_t)j * SEG + lane : (int64_t)vals[c0 + (j - u) * SEG + lane];
+            c[u2] = (old ? s0.cell : s1.cell)[si];
 #pragma unroll
-            for (int q = 0; q < NCARRY; ++q) d.cr[q * d.ccap + di] = (old ? s0.cr : s1.cr)[q * d.ccap + si];
+            for (int q = 0; q < 6; ++q) v[u2][q] = (old ? s0.a[q] : s1.a[q])[si];
+            if (sizeof(R) == 8 && d.cr)   // (a load's new particles carry nothing yet: their deposit at rest fills the planes)
+#pragma unroll
+                for (int q = 0; q < NC; ++q) w[u2][q] = (old ? s0.cr : s1.cr)[q * d.ccap + si];
+        }
+#pragma unroll
+        for (int u2 = 0; u2 < D; ++u2) {
+            const unsigned mask = __match_any_sync(0xffffffffu, k[u2]);
+            const bool on = k[u2] < RADIX;
+            const uint32_t at = on ? cnt[wid][k[u2]] : 0u;
+            __syncwarp();
+            if (on && __ffs(mask) - 1 == lane) cnt[wid][k[u2]] = at + __popc(mask);
+            __syncwarp();
+            if (!on) continue;
+            const int64_t di = n0 + at + __popc(mask & lt);
+            d.cell[di] = c[u2];
+#pragma unroll
+            for (int q = 0; q < 6; ++q) d.a[q][di] = v[u2][q];
+            if (sizeof(R) == 8 && d.cr)
+#pragma unroll
+                for (int q = 0; q < NC; ++q) d.cr[q * d.ccap + di] = w[u2][q];
+        }
     }
 }
 
