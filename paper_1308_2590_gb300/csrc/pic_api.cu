@@ -313,7 +313,7 @@ static int resolve_pending(pic_t *h, bool *rebuilt = nullptr) {
     if (f & 3) {
         commit_regroup(h);   // back to the layout the push left
         if (int rc = rebuild_from_step(h)) return rc;
-        if (h->post) h->moments_stale = true;   // that step's deposit, after its regroup, did nothing
+        if (h->pending_post) h->moments_stale = true;   // that step's deposit, after its regroup, did nothing
         if (rebuilt) *rebuilt = true;
     }
     return 0;
@@ -1320,6 +1320,25 @@ static int step_deposit(pic_t *h, int p, const int32_t *guard) {
     return 0;
 }
 
+// A step (parity p) whose particle kernels did nothing because the previous step's
+// regroup had failed: its commit undid the previous one, so the layout is the one
+// the previous push left.  The full sort, and the step again.  Where the previous
+// step's deposit comes after its regroup it did nothing either, and this step's field
+// solve ran without those moments: the deposit, and the field solve again.
+static int redo_step(pic_t *h, int p, cudaStream_t main_st, bool overlap) {
+    cudaMemsetAsync(h->d_step_flags + (1 - p), 0, sizeof(int32_t), h->st);
+    if (int rc = rebuild_from_step(h)) return rc;
+    if (h->pending_post) {
+        if (int rc = redeposit(h)) return rc;
+        if (int rc = field_cn(h)) return rc;
+        if (int rc = clear_step_moments(h)) return rc;
+    }
+    if (int rc = push_prep(h, nullptr, h->d_step_flags + p)) return rc;
+    if (int rc = particle_step(h, p, nullptr, main_st, overlap)) return rc;
+    commit_regroup(h);
+    return h->post ? step_deposit(h, p, nullptr) : 0;
+}
+
 namespace pic {
 // Whether the handle's steps run beside those of other runs on the same GPU.  The
 // others then fill what a regroup leaves idle, and the second stream of the field
@@ -1392,25 +1411,12 @@ extern "C" PIC_API int pic_step(pic_t *h, int nsteps) {
             int32_t f = 0;
             if ((rc = pending_flags(h, &f))) return rc;
             if (f & 3) {
-                // this step's particle kernels did nothing and its commit undid the previous one: the
-                // layout is the one the previous push left
-                cudaMemsetAsync(h->d_step_flags + (1 - p), 0, sizeof(int32_t), h->st);
-                if ((rc = rebuild_from_step(h))) return rc;
-                if (h->post) {
-                    // nor were that step's moments deposited: this step's field solve again from them
-                    if ((rc = redeposit(h))) return rc;
-                    if ((rc = field_cn(h))) return rc;
-                    if ((rc = clear_step_moments(h))) return rc;
-                }
-                if ((rc = push_prep(h, nullptr, h->d_step_flags + p))) return rc;
-                if ((rc = particle_step(h, p, nullptr, main_st, overlap))) return rc;
-                commit_regroup(h);
-                if (h->post)
-                    if ((rc = step_deposit(h, p, nullptr))) return rc;
+                if ((rc = redo_step(h, p, main_st, overlap))) return rc;
             }
         }
         h->flags_pending = true;
         h->pending_p = p;
+        h->pending_post = h->post;
         h->ecur = 1 - h->ecur;
         h->hcur = 1 - h->hcur;
         h->bcur = 1 - h->bcur;
@@ -1507,7 +1513,7 @@ extern "C" PIC_API int pic_batch_step(pic_batch *p, pic_t **hs, int n, int nstep
     for (int r = 0; r < n; ++r)
         if (hs[r]->moments_stale || hs[r]->post)   // (post: a pending step's moments exist once its regroup succeeded)
             if (int rc = settle(hs[r])) return rc;
-    std::vector<char> prev(n);
+    std::vector<char> prev(n), redone(n);
     struct Reset {
         pic_t **hs;
         int n;
@@ -1525,6 +1531,7 @@ extern "C" PIC_API int pic_batch_step(pic_batch *p, pic_t **hs, int n, int nstep
             pic_t *h = hs[r];
             const int ph = (int)(h->step & 1);
             prev[r] = h->flags_pending ? 1 : 0;
+            redone[r] = 0;
             h->guard = prev[r] ? h->d_step_flags + (1 - ph) : nullptr;
             if (int rc = clear_step_moments(h)) return rc;
             if (int rc = push_prep(h, h->guard, h->d_step_flags + ph)) return rc;
@@ -1558,21 +1565,16 @@ extern "C" PIC_API int pic_batch_step(pic_batch *p, pic_t **hs, int n, int nstep
             int32_t f = 0;
             if (int rc = pending_flags(h, &f)) return rc;
             if (f & 3) {
-                // this step did nothing for the run and its commit undid the previous one: the layout is
-                // the one the previous push left; the full sort, then the step alone on the run's stream
-                cudaMemsetAsync(h->d_step_flags + (1 - ph), 0, sizeof(int32_t), h->st);
-                if (int rc = rebuild_from_step(h)) return rc;
-                if (int rc = push_prep(h, nullptr, h->d_step_flags + ph)) return rc;
-                if (int rc = particle_step(h, ph, nullptr, h->st, false)) return rc;
-                commit_regroup(h);
-                if (h->post)
-                    if (int rc = step_deposit(h, ph, nullptr)) return rc;
+                // the step alone on the run's stream
+                if (int rc = redo_step(h, ph, h->st, false)) return rc;
+                redone[r] = 1;
             }
         }
         for (int r = 0; r < n; ++r) {
             pic_t *h = hs[r];
             h->flags_pending = true;
             h->pending_p = (int)(h->step & 1);
+            h->pending_post = h->post && redone[r];   // (the batched push deposits itself)
             h->ecur = 1 - h->ecur;
             h->hcur = 1 - h->hcur;
             h->bcur = 1 - h->bcur;

@@ -155,6 +155,7 @@ struct pic_t {
     cudaEvent_t ev_flags[2] = {nullptr, nullptr};   // per step parity: that step's flags are on the host
     bool flags_pending = false;         // a step's regroup flags are in flight (its regroup already committed)
     int pending_p = 0;                  // that step's parity
+    bool pending_post = false;          // that step deposits after its regroup (nothing if the regroup failed)
     int halo = 1;                       // deposit halo of a tile, in cells
     void *Mlo = nullptr;                // FP32 form: compensation of the moment sums
     bool det = false;                   // deterministic deposit: exact fixed-point sums in Mfix
