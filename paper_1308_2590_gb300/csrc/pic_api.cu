@@ -1511,7 +1511,7 @@ extern "C" PIC_API int pic_batch_step(pic_batch *p, pic_t **hs, int n, int nstep
     }
     BatchScratch &b = p->b;
     for (int r = 0; r < n; ++r)
-        if (hs[r]->moments_stale || hs[r]->post)   // (post: a pending step's moments exist once its regroup succeeded)
+        if (hs[r]->moments_stale)   // (a pending step without moments, its regroup failed, is met in the loop)
             if (int rc = settle(hs[r])) return rc;
     std::vector<char> prev(n), redone(n);
     struct Reset {
