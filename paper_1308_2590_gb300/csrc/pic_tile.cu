@@ -966,7 +966,7 @@ struct UsegOut {
 //   cell's tile or the next one (node column i is in tile min(i / tnx, ntx - 1));
 //   the FP32 flush region is the tile plus a halo of fewer than a tile's cells.
 //   So node tile T is touched if a tile of T-2 .. T+1 on both axes (wrapping where
-//   the box is periodic) is occupied (spline shapes reach further: push_prep);
+//   the box is periodic) is occupied (spline shapes reach further: node_reach);
 // - the tiles the regroup must visit, those with an occupied tile among T-1 ..
 //   T+1 on both axes (stayers or arrivals; after a far move the regroup's output
 //   is replaced by the full sort); the next bins of the others are emptied.
@@ -1058,6 +1058,23 @@ __global__ void __launch_bounds__(128) k_step_lists(UsegPtrs u, UsegOut u2, int 
         }
 }
 
+// Tiles that the nodes of a particle in cell c, c - dn .. c + up (order 1: 0, 1; 2 and 3: 1, 2; 4: 2, 3), reach
+// from the cell's tile, on each axis.  Where the axis wraps and its last tile is narrower than that, the nodes lie
+// on its far side as well (1 cell of 8, order 3: a particle in the last row of the tile before it has nodes in that
+// tile, in the narrow one and in tile 0).
+struct NodeReach {
+    int upx, upy, dnx, dny;
+};
+static NodeReach node_reach(const pic_t *h) {
+    const int dn = h->shape / 2, up = (h->shape + 2) / 2;
+    auto tiles = [](int cells, int tile, int n, bool wraps) {
+        const int last = n % tile, t = (cells + tile - 1) / tile;
+        return wraps && last > 0 && last < cells ? std::max(t, 1 + (cells - last + tile - 1) / tile) : t;
+    };
+    return NodeReach{tiles(up, h->tnx, h->nx, h->periodic_x), tiles(up, h->tny, h->ny, true),
+                     tiles(dn, h->tnx, h->nx, h->periodic_x), tiles(dn, h->tny, h->ny, true)};
+}
+
 int32_t *list_counters(const pic_t *h, int set) { return h->counters + set * LC_SIZE; }
 
 // The next push's work items and tile lists from the current layout of the bins
@@ -1076,13 +1093,10 @@ int push_prep(pic_t *h, const int32_t *guard, int32_t *word) {
     int32_t *cnt = list_counters(h, set);
     if (!h->lists_zero[set] && cudaMemsetAsync(cnt, 0, LC_SIZE * sizeof(int32_t), h->st) != cudaSuccess)
         return check_launch("tile lists");
-    // occupied tiles T - dl .. T + dh can deposit into node tile T: the nodes of a particle in cell c
-    // are c + lo .. c + hi (order 1: 0 .. 1; 2: -1 .. 2; 3: -1 .. 2; 4: -2 .. 3), in node tiles
-    // b - ceil(-lo / tile) .. b + ceil(hi / tile) of the new cell's tile b, itself within one tile
-    // of the occupied one
-    const int lo = -(h->shape / 2), hi = (h->shape + 2) / 2;
-    const int dlx = 1 + (hi + h->tnx - 1) / h->tnx, dly = 1 + (hi + h->tny - 1) / h->tny;
-    const int dhx = 1 + (-lo + h->tnx - 1) / h->tnx, dhy = 1 + (-lo + h->tny - 1) / h->tny;
+    // occupied tiles T - dl .. T + dh can deposit into node tile T: the nodes of a particle (node_reach) from its
+    // new cell's tile, itself within one tile of the occupied one
+    const NodeReach r = node_reach(h);
+    const int dlx = 1 + r.upx, dly = 1 + r.upy, dhx = 1 + r.dnx, dhy = 1 + r.dny;
     const auto kernel = dlx == 2 && dly == 2 && dhx == 1 && dhy == 1 ? k_step_lists<true> : k_step_lists<false>;
     kernel<<<(h->ntiles + 127) / 128, 128, 0, h->st>>>(
         u, u2, h->nsp, h->ntx, h->nty, h->periodic_x ? 1 : 0, h->items_ch, dlx, dly, dhx, dhy, guard, word, cnt,
@@ -2035,9 +2049,7 @@ __global__ void k_rest_touch(UsegPtrs u, int nsp, int ntx, int nty, int periodic
 int rest_touch(pic_t *h) {
     UsegPtrs u;
     for (int s = 0; s < PIC_MAX_SPECIES; ++s) u.p[s] = (s < h->nsp) ? h->sp[s].useg[h->sp[s].scur] : nullptr;
-    // nodes c + lo .. c + hi of a particle in cell c (as in push_prep; the splines' may cross a ragged last
-    // tile into the one after it)
-    const int lo = -(h->shape / 2), hi = (h->shape + 2) / 2, one = h->shape > 1 ? 1 : 0;
+    const NodeReach r = node_reach(h);
     int32_t *cnt = list_counters(h, h->touch_cur) + LC_TOUCH;
     if (cudaMemsetAsync(cnt, 0, sizeof(int32_t), h->st) != cudaSuccess) return check_launch("tile lists");
     h->lists_zero[h->touch_cur] = false;
@@ -2045,8 +2057,7 @@ int rest_touch(pic_t *h) {
     k_rest_touch<<<(h->ntiles + 255) / 256, 256, 0, h->st>>>(
         u, h->nsp, h->ntx, h->nty, h->periodic_x ? 1 : 0, h->touched + (size_t)h->touch_cur * h->ntiles,
         h->touch_list + (size_t)h->touch_cur * h->ntiles, cnt,
-        one + (hi + h->tnx - 1) / h->tnx, one + (hi + h->tny - 1) / h->tny, one + (-lo + h->tnx - 1) / h->tnx,
-        one + (-lo + h->tny - 1) / h->tny);
+        r.upx, r.upy, r.dnx, r.dny);
     count_launch(h);
     h->touch_all = false;
     return check_launch("k_rest_touch");
