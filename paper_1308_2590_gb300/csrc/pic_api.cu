@@ -24,6 +24,15 @@ void set_error(const char *fmt, ...) {
     va_end(ap);
 }
 
+cudaError_t allow_smem(const void *kernel, size_t bytes) {
+    static std::mutex mu;   // between reading the limit and raising it
+    std::lock_guard<std::mutex> lk(mu);
+    cudaFuncAttributes a;
+    const cudaError_t e = cudaFuncGetAttributes(&a, kernel);
+    if (e != cudaSuccess || (size_t)a.maxDynamicSharedSizeBytes >= bytes) return e;
+    return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+}
+
 int check_launch(const char *what) {
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) {

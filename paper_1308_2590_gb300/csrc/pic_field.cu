@@ -1811,7 +1811,7 @@ static bool cn_single_cluster(const pic_t *h, size_t smem) {
     cn_cluster_config(lc, at, smem, h->st);
     int n = 0;   // (clusters of more than 8 blocks are opt-in, and may not fit a partitioned GPU)
     if (cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess ||
-        cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess ||
+        allow_smem(k, smem) != cudaSuccess ||
         cudaOccupancyMaxActiveClusters(&n, k, &lc) != cudaSuccess) {
         cudaGetLastError();
         return false;
@@ -1854,7 +1854,7 @@ static int field_cn_t(pic_t *h) {
     } else {
         const void *k = (const void *)k_cn_solve<false, CN_BS>;
         // the whole grid must be resident: fix the shared-memory split before asking how many blocks fit
-        cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        allow_smem(k, smem);
         cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, CN_BS, smem);
         int nb = per_sm * nsm;

@@ -987,6 +987,9 @@ struct SplineDep {
 // --------------------------------------------------------------------------- host entry points
 
 int check_launch(const char *what);
+// Lets a kernel be launched with `bytes` of dynamic shared memory: the limit is the kernel's, whichever run launches
+// it, and is only ever raised.
+cudaError_t allow_smem(const void *kernel, size_t bytes);
 void timing_begin(pic_t *h);
 void timing_end(pic_t *h, int cls, int nlaunch);
 inline void count_launch(pic_t *h, int n = 1) { h->timing.launches[4] += n; }

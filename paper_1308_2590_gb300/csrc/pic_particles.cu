@@ -752,7 +752,7 @@ static int rest_launch(pic_t *h, void (*kernel)(DepArgs<R>), const DepArgs<R> &a
     int dev = 0, nsm = 0, per = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-    if (smem > 32 * 1024) cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (smem > 32 * 1024) allow_smem((const void *)kernel, smem);
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kernel, 256, smem) != cudaSuccess || per < 1) {
         cudaGetLastError();
         per = 1;
@@ -794,7 +794,7 @@ static int cell_dep_launch(pic_t *h, const CellDepArgs &a) {
     int dev = 0, nsm = 0, per = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-    if (smem > 32 * 1024) cudaFuncSetAttribute(k_deposit_cells, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    if (smem > 32 * 1024) allow_smem((const void *)k_deposit_cells, smem);
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_deposit_cells, 256, smem) != cudaSuccess || per < 1) {
         cudaGetLastError();
         per = 1;

@@ -1656,7 +1656,7 @@ static Carve carve(const pic_t *h) {
 
 template <typename R, bool kFix, bool kBatch = false, bool kDep = true>
 static int push_occupancy(pic_t *h, int bytes, int *blocks_per_sm) {
-    cudaError_t e = cudaFuncSetAttribute(k_push<R, kFix, kBatch, kDep>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+    cudaError_t e = allow_smem((const void *)k_push<R, kFix, kBatch, kDep>, bytes);
     if (e == cudaSuccess)
         e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, k_push<R, kFix, kBatch, kDep>, TILE_BS, bytes);
     if (e != cudaSuccess) {
@@ -1672,7 +1672,7 @@ static constexpr int push_s_smem() { return TILE_WARPS * SplineDep<R, N>::kWarpB
 template <typename R, bool kFix, int N>
 static int push_s_occupancy_n(int *blocks_per_sm) {
     const int bytes = kFix ? 0 : push_s_smem<R, N>();
-    cudaError_t e = cudaFuncSetAttribute(k_push_s<R, kFix, N>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+    cudaError_t e = allow_smem((const void *)k_push_s<R, kFix, N>, bytes);
     if (e == cudaSuccess)
         e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, k_push_s<R, kFix, N>, TILE_BS, bytes);
     if (e != cudaSuccess) {
@@ -1783,7 +1783,7 @@ int tile_setup(pic_t *h) {
     }
     const int rb = regroup_smem_bytes(h);
     const void *rk = regroup_kernel(h);
-    cudaError_t e = cudaFuncSetAttribute(rk, cudaFuncAttributeMaxDynamicSharedMemorySize, rb);
+    cudaError_t e = allow_smem(rk, rb);
     if (e != cudaSuccess) {
         set_error("regroup kernel set-up: %s", cudaGetErrorString(e));
         return PIC_ERR_CUDA;
@@ -1961,7 +1961,7 @@ static int batch_regroup_t(BatchScratch &b, pic_t **hs, int n) {
         if (bytes > smem) smem = bytes;
         if (hs[r]->nsp > nsp) nsp = hs[r]->nsp;
     }
-    if (cudaFuncSetAttribute(k_regroup<R, true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess)
+    if (allow_smem((const void *)k_regroup<R, true, false>, smem) != cudaSuccess)
         return check_launch("regroup (batched) set-up");
     const TileArgs<R> *dargs = (const TileArgs<R> *)b.args_dev;
     const int32_t *tiles_dev = b.idx + (b.cap + 1);
