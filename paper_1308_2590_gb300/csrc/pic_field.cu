@@ -104,7 +104,9 @@ struct Inc {
 // and solve, running alone: 540 us).  The FP64 pipe bounds the FP64 form, so the
 // factors dt/(2 dx), dt/(2 dy) go into the update's FMAs and the sum E^n + E^{n+1}
 // that the push gathers is stored without its half (the push's factor has it):
-// 17 operations per vacuum node instead of 23.  4096 x 2048 nodes FP64, vacuum but
+// 17 operations per vacuum node instead of 23.  The FP32 form is bound by memory and
+// forms the change first, so that E rounds once (chained FMAs round at its size
+// two to three times).  4096 x 2048 nodes FP64, vacuum but
 // for a thin foil: 472 -> 300 us (the two passes of H and B: 425 -> 339 us).
 //
 // Walls (reading of the missing boundary and source equations): the wall node is
@@ -130,9 +132,15 @@ __global__ void __launch_bounds__(128, 6) k_field_E_literal(GridArgs<R> g, const
         // with no moment read and no 3x3 solve.  The same operations as the solve below on such a node
         // (where the 3x3 solve returns its right-hand side exactly), so a node's bits do not depend on
         // whether its tile was marked.
-        z.x = fma_r(g.khy, u, e.x);
-        z.y = fma_r(g.khx, v, e.y);
-        z.z = fma_r(g.khx, sy, fma_r(-g.khy, sx, e.z));
+        if constexpr (sizeof(R) == 8) {
+            z.x = fma_r(g.khy, u, e.x);
+            z.y = fma_r(g.khx, v, e.y);
+            z.z = fma_r(g.khx, sy, fma_r(-g.khy, sx, e.z));
+        } else {
+            z.x = fma_r(g.dt, u * g.hy, e.x);
+            z.y = fma_r(g.dt, v * g.hx, e.y);
+            z.z = fma_r(g.dt, fma_r(sy, g.hx, -(sx * g.hy)), e.z);
+        }
     } else {
         const R ia = g.inv_dx * g.inv_dy;
         const R ev[3] = {e.x, e.y, e.z};
@@ -148,11 +156,19 @@ __global__ void __launch_bounds__(128, 6) k_field_E_literal(GridArgs<R> g, const
                 s_e += ((row == col ? R(1) : R(0)) - S) * ev[col];
             }
             const int64_t ji = (int64_t)(10 + row) * g.nnode + node;
-            r[row] = fma_r(-g.dt, (Mlo ? M[ji] + Mlo[ji] : M[ji]) * ia, s_e);
+            const R m = Mlo ? M[ji] + Mlo[ji] : M[ji];
+            if constexpr (sizeof(R) == 8) {
+                r[row] = fma_r(-g.dt, m * ia, s_e);
+            } else {
+                const R c = row == 0 ? u * g.hy : row == 1 ? v * g.hx : fma_r(sy, g.hx, -(sx * g.hy));
+                r[row] = fma_r(g.dt, fma_r(-m, ia, c), s_e);
+            }
         }
-        r[0] = fma_r(g.khy, u, r[0]);
-        r[1] = fma_r(g.khx, v, r[1]);
-        r[2] = fma_r(g.khx, sy, fma_r(-g.khy, sx, r[2]));
+        if constexpr (sizeof(R) == 8) {
+            r[0] = fma_r(g.khy, u, r[0]);
+            r[1] = fma_r(g.khx, v, r[1]);
+            r[2] = fma_r(g.khx, sy, fma_r(-g.khy, sx, r[2]));
+        }
         if (tm.clr) clear_node_moments(g, tm, node);   // read above by this thread only
         solve3(a, r, w);
         z.x = w[0];
