@@ -201,20 +201,14 @@ __global__ void __launch_bounds__(128, 6) k_field_E_literal(GridArgs<R> g, const
     }
 }
 
-// Vertical halves of curl_e over two rows of V4 values a (upper), b (lower).
+// Differences of a row's y and z to the next column's (the next lane's).
 template <typename R>
-struct RowPair {
-    R sy, sz, dx, dz;   // sums of y and z, differences (upper - lower) of x and z
+struct RowDiff {
+    R y, z;
 };
 template <typename R>
-__device__ inline RowPair<R> row_pair(const V4<R> &a, const V4<R> &b) {
-    return RowPair<R>{a.y + b.y, a.z + b.z, a.x - b.x, a.z - b.z};
-}
-template <typename R>
-__device__ inline RowPair<R> shfl_down(const RowPair<R> &p) {
-    const unsigned f = 0xffffffffu;
-    return RowPair<R>{__shfl_down_sync(f, p.sy, 1), __shfl_down_sync(f, p.sz, 1), __shfl_down_sync(f, p.dx, 1),
-                      __shfl_down_sync(f, p.dz, 1)};
+__device__ inline RowDiff<R> row_diff(const V4<R> &e) {
+    return RowDiff<R>{__shfl_down_sync(0xffffffffu, e.y, 1) - e.y, __shfl_down_sync(0xffffffffu, e.z, 1) - e.z};
 }
 
 constexpr int FIELD_WARPS = 4;   // warps of a block of k_field_HB, each with rows of its own
@@ -222,8 +216,11 @@ constexpr int HB_COLS = 30;      // columns a warp produces: the outer two lanes
 
 // Eq. 5 and the node B of the new H in one pass: a warp walks down rows of
 // HB_COLS columns, lane l holding E column c0 + l.  H_out = H_in - dt curl_e(Ec)
-// at the cells (kx = dt/(2 dx), ky = dt/(2 dy), vertical halves of curl_e and
-// the right neighbour's by a shuffle: 12 FP64 operations per cell); B = the sum
+// at the cells (kx = dt/(2 dx), ky = dt/(2 dy), the right neighbour's values by
+// shuffles: 12 FP64 operations per cell).  Differences of neighbours come before
+// any sum, as they are exact where the field is smooth: sums of two rows first
+// would round at twice the size of E (FP32, fields of 1.5: H off by 1.5 half ulps
+// instead of 1).  B = the sum
 // of the four cells sharing the node, without its quarter (the deposits' factor
 // has it; on a wall column twice the two inside cells): 6 operations per node
 // instead of 12, and H is not read again.  A row of H above the strip is formed
@@ -250,6 +247,7 @@ __global__ void __launch_bounds__(32 * FIELD_WARPS) k_field_HB(GridArgs<R> g, co
     const int jb = y0 == 0 ? g.ny - 1 : y0 - 1;
     V4<RE> eb = Ec[(int64_t)jb * g.nxn + n], en = Ec[(int64_t)y0 * g.nxn + n];
     V4<R> hn = Hin[(int64_t)jb * g.nx + c];
+    RowDiff<RE> db = row_diff(eb);
     V4<R> below{R(0), R(0), R(0), R(0)};   // the new H of the row above the strip, then of the previous row
     for (int j = y0 - 1; j < y1; ++j) {
         const V4<RE> ea = en;               // E rows j + 1 (ea) and j (eb), H row j
@@ -258,9 +256,13 @@ __global__ void __launch_bounds__(32 * FIELD_WARPS) k_field_HB(GridArgs<R> g, co
             en = Ec[(int64_t)(j + 2 >= g.ny ? j + 2 - g.ny : j + 2) * g.nxn + n];
             hn = Hin[(int64_t)(j + 1) * g.nx + c];
         }
-        const RowPair<RE> p = row_pair(ea, eb), q = shfl_down(p);   // columns i and i + 1
+        // 2 dy dEz/dy and 2 dy dEx/dy over columns i and i + 1, 2 dx dEz/dx and 2 dx dEy/dx over rows j and j + 1
+        const RowDiff<RE> da = row_diff(ea);
+        const RE vz = ea.z - eb.z, vx = ea.x - eb.x;
+        const RE zy = vz + __shfl_down_sync(0xffffffffu, vz, 1), xy = vx + __shfl_down_sync(0xffffffffu, vx, 1);
+        const RE zx = da.z + db.z, yx = da.y + db.y;
         eb = ea;
-        // 2 dy dEz/dy = dz + dz', 2 dx dEz/dx = sz' - sz, 2 dx dEy/dx = sy' - sy, 2 dy dEx/dy = dx + dx'
+        db = da;
         auto in = [](R x) -> RE {
             if constexpr (sizeof(RE) == 8) return widen(x);
             else return x;
@@ -269,8 +271,7 @@ __global__ void __launch_bounds__(32 * FIELD_WARPS) k_field_HB(GridArgs<R> g, co
             if constexpr (sizeof(RE) == 8) return stored<R>(x);
             else return x;
         };
-        const V4<R> w{out(fma(-ky, p.dz + q.dz, in(h.x))), out(fma(kx, q.sz - p.sz, in(h.y))),
-                      out(fma(ky, p.dx + q.dx, fma(-kx, q.sy - p.sy, in(h.z)))), R(0)};
+        const V4<R> w{out(fma(-ky, zy, in(h.x))), out(fma(kx, zx, in(h.y))), out(fma(ky, xy, fma(-kx, yx, in(h.z)))), R(0)};
         if (j >= y0) {
             if (cell) Hout[(int64_t)j * g.nx + i] = w;
             const V4<R> s{below.x + w.x, below.y + w.y, below.z + w.z, R(0)};   // cells (i, j - 1) and (i, j)

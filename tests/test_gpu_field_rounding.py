@@ -1,8 +1,11 @@
-"""FP32 literal field step: E^{n+1} is E^n plus a small change, so it rounds at its own size once.  Against FP64 arithmetic
-on the same FP32 values, with powers of two for dx, dy and dt, so that every factor is exact, and fields of 1.5 +- 2^-9,
-so that differences of neighbours are exact: one rounding in [1, 2), 2^-24, and that of the change, sums of at most
-2^-6 (2^-30 each, twice two of them times hx = 2) and of the curl, at most 2^-4 (2^-29), times dt = 2^-3: below 2^-30.
-Vacuum, and tiles marked by a particle too light to change a bit, whose nodes take the full solve and must round alike."""
+"""FP32 literal field step: E^{n+1} is E^n plus a small change and H^{n+3/2} is H^{n+1/2} plus one, so each rounds at its own
+size and not at the size of intermediate sums.  Against FP64 arithmetic on the same FP32 values, with powers of two
+for dx, dy and dt, so that every factor is exact, and fields of 1.5 +- 2^-9, so that differences of neighbours are
+exact.  E: one rounding in [1, 2), 2^-24, and that of the change: sums of at most 2^-6 (2^-30 each, twice two of them
+times hx = 2) and of the curl, at most 2^-4 (2^-29), times dt = 2^-3: below 2^-30.  H, from the E that the step made
+(1.5 +- 2^-6): sums of at most 2^-4 (2^-29) times dt/(2 dx) = 2^-2, two of them: 2^-30; one rounding in [1, 2) for x
+and y, two (an FMA for each derivative) for z.  Vacuum, and tiles marked by a particle too light to change a bit,
+whose nodes take the full solve and must round alike."""
 import numpy as np
 import pytest
 
@@ -51,3 +54,12 @@ def test_fp32_e_rounds_once(light):
     want = E + cfg.dt * _curl(cfg, H, 1)
     assert _in_range(want, E)
     assert np.max(np.abs(Eg - want)) <= 2.0 ** -24 + 2.0 ** -30
+
+
+@pytest.mark.parametrize("light", [False, True])
+def test_fp32_h_rounds_at_its_own_size(light):
+    cfg, _, H, Eg, Hg = _step(light)
+    want = H - cfg.dt * _curl(cfg, Eg, -1)
+    assert _in_range(want, H)
+    assert np.max(np.abs(Hg[:2] - want[:2])) <= 2.0 ** -24 + 2.0 ** -30
+    assert np.max(np.abs(Hg[2] - want[2])) <= 2.0 ** -23 + 2.0 ** -30
