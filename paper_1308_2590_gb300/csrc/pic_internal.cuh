@@ -157,7 +157,7 @@ struct pic_t {
     int pending_p = 0;                  // that step's parity
     bool pending_post = false;          // that step deposits after its regroup (nothing if the regroup failed)
     int halo = 1;                       // deposit halo of a tile, in cells
-    void *Mlo = nullptr;                // FP32 form: compensation of the moment sums
+    void *Mlo = nullptr;                // FP32 form: second part of the moment sums (compensation, stragglers)
     bool det = false;                   // deterministic deposit: exact fixed-point sums in Mfix
     unsigned long long *Mfix = nullptr; // [13][nnode] two's-complement fixed-point moment sums
     double *Mc = nullptr;               // FP64 L2-reduction push (linear shape): cell sums [ncell][13][4]
