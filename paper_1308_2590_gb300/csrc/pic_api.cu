@@ -33,7 +33,25 @@ cudaError_t allow_smem(const void *kernel, size_t bytes) {
     return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
 }
 
+#ifdef PIC_CHECKS
+// Checks build: what a failed call leaves behind can be tested without a failing GPU.  The nth check or allocation
+// of this name from now on reports a failure that did not happen.
+static thread_local char g_fail[64] = "";
+static thread_local int g_fail_nth = 0;
+extern "C" PIC_API void pic_checks_fail(const char *what, int nth) {
+    snprintf(g_fail, sizeof(g_fail), "%s", what);
+    g_fail_nth = nth;
+}
+static bool fails(const char *what) { return g_fail_nth > 0 && !strcmp(what, g_fail) && --g_fail_nth == 0; }
+#else
+static bool fails(const char *) { return false; }
+#endif
+
 int check_launch(const char *what) {
+    if (fails(what)) {
+        set_error("%s: reported as failed", what);
+        return PIC_ERR_CUDA;
+    }
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) {
         set_error("%s: %s", what, cudaGetErrorString(e));
@@ -153,7 +171,7 @@ static int harvest(pic_t *h) {
 static int dalloc(void **p, size_t bytes, const char *what) {
     *p = nullptr;
     if (bytes == 0) return 0;
-    if (cudaMalloc(p, bytes) != cudaSuccess) {
+    if (fails(what) || cudaMalloc(p, bytes) != cudaSuccess) {
         cudaGetLastError();
         set_error("cudaMalloc of %zu bytes for %s failed", bytes, what);
         *p = nullptr;
@@ -727,7 +745,8 @@ static int weight_sums(pic_t *h, int nload, const pic_species_data *d, double *s
 // added (or nullptr): where the moments are current and kept as FP64 cell sums, the
 // new particles' are added to them (*added set; the caller brings the sums to the
 // nodes), instead of every particle's being deposited anew before they are next read.
-// The new particles must lie in tiles of the current tile lists.
+// The new particles must lie in tiles of the current tile lists, and after an error the
+// caller empties the sums.
 static int load_impl(pic_t *h, int nload, const int *species, const pic_species_data *d, const char *fn,
                      const int32_t *const *cells = nullptr, bool *added = nullptr) {
     bool seen[PIC_MAX_SPECIES] = {false};
@@ -924,6 +943,7 @@ static int load_impl(pic_t *h, int nload, const int *species, const pic_species_
         return PIC_ERR_ARG;
     }
     const bool add = added && !fresh && !h->moments_stale && h->Mc;
+    if (!add) h->moments_stale = !eager;   // deposited at the next step or readout, whatever fails below
     if (!fresh)
         for (int e = 0; e < nload; ++e)
             if (d[e].n > 0) {
@@ -932,7 +952,6 @@ static int load_impl(pic_t *h, int nload, const int *species, const pic_species_
                 if (int r = rebuild_species(h, species[e], REBUILD_FROM_LOAD, d[e].n)) return r;
             }
     if (add) *added = true;
-    else h->moments_stale = !eager;   // else deposited at the next step or readout
     if (!fresh && (cudaMemcpyAsync(h->h_step_flags + 3, h->d_flags, sizeof(int32_t), cudaMemcpyDeviceToHost,
                                    main_st) != cudaSuccess ||
                    cudaStreamSynchronize(main_st) != cudaSuccess))
@@ -1014,6 +1033,16 @@ extern "C" PIC_API int pic_ionize(pic_t *h, const pic_ionization *p, int64_t *n_
     }
     const double HARTREE_EV = 27.211386245988;
     int64_t off[PIC_MAX_SPECIES] = {0}, nc[PIC_MAX_SPECIES] = {0}, done = 0;
+    // from here to the end the moments are not those of the particles: an error leaves them to a deposit of every
+    // particle, and the cell sums empty
+    struct Unsettled {
+        pic_t *h;
+        ~Unsettled() {
+            if (!h) return;
+            if (h->Mc) cudaMemsetAsync(h->Mc, 0, cell_sum_bytes(h), h->st);
+            h->moments_stale = true;
+        }
+    } unsettled{h};
     for (int c = 0; c < p->n_chains; ++c) {
         const double ip = p->ip_ev[c] / HARTREE_EV, Z = h->sp[p->target[c]].q;
         const double n = Z / sqrt(2.0 * ip), K = 2.0 * pow(2.0 * ip, 1.5);
@@ -1031,7 +1060,10 @@ extern "C" PIC_API int pic_ionize(pic_t *h, const pic_ionization *p, int64_t *n_
         h->sp[p->ion[c]].n = counts[c] - nc[c];
         h->sp[p->ion[c]].n_exact = true;
     }
-    if (done == 0) return PIC_OK;
+    if (done == 0) {
+        unsettled.h = nullptr;
+        return PIC_OK;
+    }
     // destinations: each target and electron species, its sources in chain order
     int dest[PIC_MAX_SPECIES], ndest = 0;
     int64_t dn[PIC_MAX_SPECIES] = {0}, dsrc_count[PIC_MAX_SPECIES] = {0};
@@ -1100,6 +1132,7 @@ extern "C" PIC_API int pic_ionize(pic_t *h, const pic_ionization *p, int64_t *n_
             if (int rc = deposit_leavers(h, p->ion[c], nc[c], h->ion_cell + off[c], h->ion_val + off[c], h->ion_cap)) return rc;
         if (int rc = cell_moments(h)) return rc;
     }
+    unsettled.h = nullptr;
     if (n_ionized) *n_ionized = done;
     return PIC_OK;
 }
