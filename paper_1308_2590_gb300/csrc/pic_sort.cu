@@ -9,6 +9,7 @@
 // key and end up past the live count.
 #include <cooperative_groups.h>
 
+#include <algorithm>
 #include <utility>
 
 #include "pic_internal.cuh"
@@ -668,7 +669,7 @@ static int merge_load(pic_t *h, SpeciesBuf &S, const KeyGeom &kg, int64_t n_seco
     cudaMemsetAsync(S.cstart, 0, tb, h->st);
     cudaMemsetAsync(S.cend, 0, tb, h->st);
     k_run_bounds<<<each_blocks(n_second), 256, 0, h->st>>>(h->keys[cur], n_second, kg.cpt, S.cstart, S.cend);
-    // the sort's other buffers hold at least 2 x capacity words, more than the tiles
+    // the sort's other buffers hold an entry per tile (rebuild_species)
     int32_t *old = (int32_t *)h->vals[1 - cur], *ends = (int32_t *)h->keys[1 - cur];
     const int o = S.scur, nw = 1 - o;
     cudaMemcpyAsync(old, S.bstart, tb, cudaMemcpyDeviceToDevice, h->st);
@@ -696,7 +697,9 @@ int rebuild_species(pic_t *h, int s, int source, int64_t n_second) {
                        (int64_t)h->ntiles * RADIX < 0xFFFFFFFell;
     const int64_t n = (fresh || merge) ? n_second : 2 * cap;
     if (n == 0) return 0;
-    if (int rc = ensure_sort_capacity(h, n)) return rc;
+    // (a merge keeps two arrays over the tiles in the scratch, which is smaller than 2 x capacity words where an
+    // allocation of that size has failed before)
+    if (int rc = ensure_sort_capacity(h, merge ? std::max<int64_t>(n, h->ntiles + 1) : n)) return rc;
     cudaMemsetAsync(h->keys[0], 0xFF, n * sizeof(uint32_t), h->st);
     int32_t *useg = S.useg[S.scur], *segn = S.segn[S.scur];
     KeyGeom kg{h->nx, h->tnx, h->tny, h->ntx, merge ? (uint32_t)RADIX : (uint32_t)(h->tnx * h->tny)};

@@ -1,5 +1,5 @@
 """What a call that fails half way leaves behind, with failures that the checks build only reports (a launch check or an
-allocation named by the test): the moments are those of the particles that are there."""
+allocation named by the test): the moments are those of the particles that are there, and later calls stay in bounds."""
 import ctypes
 import json
 import os
@@ -57,6 +57,34 @@ def ionisation(what, nth):
     return out
 
 
+def scratch(what, nth):
+    """Particles in a species, a larger load whose sort scratch cannot be allocated, then a small load."""
+    from tests.test_gpu_parity import small_uniform
+    cfg = small_uniform(n=256, ppc=1, tile=2)
+    rng = np.random.default_rng(9)
+
+    def some(n):
+        return dict(x=cfg.nx * cfg.dx * rng.random(n), y=cfg.ny * cfg.dy * rng.random(n),
+                    **{k: 0.1 * rng.standard_normal(n) for k in ("ux", "uy", "uz")}, w=np.arange(1.0, n + 1))
+
+    first, large, small = some(100), some(200000), some(20)
+    out, states = {}, []
+    for fail in (True, False):
+        with pic.Pic(cfg, stream=stream()) as g:
+            g.load(0, first)
+            if fail:
+                pic.lib().pic_checks_fail(what.encode(), nth)
+                try:
+                    g.load(0, large)
+                except pic.PicError as e:
+                    out["error"] = str(e)
+            g.load(0, small)
+            out["count"] = g.pic_particle_count(0)
+            states.append(g.pic_save_particles(0))
+    out["same"] = all(np.array_equal(states[0][k], states[1][k]) for k in states[0])
+    return out
+
+
 def _child(*args):
     r = subprocess.run([sys.executable, os.path.abspath(__file__), B.build(checks=True), *map(str, args)],
                        capture_output=True, text=True, timeout=600, cwd=ROOT)
@@ -74,6 +102,13 @@ def test_moments_after_a_failed_ionisation_pass(what, nth):
     assert out["now"] < 1e-13 and out["step"] < 1e-13, out
 
 
+
+def test_small_load_after_a_failed_allocation_of_the_sort_scratch():
+    """More tiles (128 x 126) than the scratch of a sort of 20 particles has entries."""
+    out = _child("scratch", "sort scratch", 1)
+    assert "sort scratch" in out["error"] and out["count"] == 120 and out["same"], out
+
+
 if __name__ == "__main__":
     pic.lib(sys.argv[1]).pic_checks_fail.argtypes = [ctypes.c_char_p, ctypes.c_int]
-    print(json.dumps({"ionisation": ionisation}[sys.argv[2]](sys.argv[3], int(sys.argv[4]))))
+    print(json.dumps({"ionisation": ionisation, "scratch": scratch}[sys.argv[2]](sys.argv[3], int(sys.argv[4]))))
