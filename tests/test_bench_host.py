@@ -34,6 +34,14 @@ def test_source_hash_is_stable_and_covers_the_header_sections():
     assert "int push_work_list(pic_t *h);" not in kept               # nor the host entry points
 
 
+def test_source_hash_leaves_out_the_host_entry_points_of_the_header():
+    with open(os.path.join(ROOT, "paper_1308_2590_gb300/csrc/pic_internal.cuh")) as f:
+        text = f.read()
+    kept = bench.kernel_source_text(text)
+    for host in ("struct pic_t {", "int regroup_tiles(pic_t *h);", "int rebuild_species(pic_t *h, int s, int source"):
+        assert host in text and host not in kept
+
+
 def _r(push_ms_per_step, steps, n):
     return {"kernel_ms": [push_ms_per_step * steps, 0.0, 0.0, 0.0], "n_local": n}
 
