@@ -1286,7 +1286,11 @@ struct SolveScalars {
 // r -= A P^{-1} r, where S varies little: the error is multiplied by at most
 // rho = max |S - mean| / (1 + mean).  Below CN_SWEEP_RHO the solve takes them
 // instead of BiCGSTAB: no dot products, half the vectors, four barriers per
-// application instead of four and a half.
+// application instead of four and a half.  The field solve of uniform plasmas of
+// growing density, corrections / BiCGSTAB (us, FP64; FP32 alike): 64 x 64 rho 0.05
+// 157 / 203, 0.13 216 / 246, 0.20 250 / 277; 256 x 256 0.10 317 / 419, 0.17 416 /
+// 420, 0.25 490 / 471; 512 x 512 0.08 676 / 768, 0.13 722 / 873, 0.19 1053 / 926,
+// 0.26 1205 / 1030.  They meet between 0.16 (large grids) and above 0.2 (small).
 constexpr float CN_SWEEP_RHO = 0.2f;
 
 // The whole solve in one launch (grid-wide barriers between the dependent

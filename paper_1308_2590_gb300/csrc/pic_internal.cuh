@@ -147,9 +147,10 @@ struct pic_t {
     pic::SpeciesBuf sp[PIC_MAX_SPECIES];
     int64_t *d_removed = nullptr;       // [nsp] cumulative wall removals
     int32_t *d_flags = nullptr;         // sticky: bit 0 far mover seen, bit 2 capacity, bit 3 TMA wait timeout
-    int32_t *d_step_flags = nullptr;    // [2], one per step parity: bit 0 far mover, bit 1 bin overflow -> full rebuild
-    int32_t *h_step_flags = nullptr;    // pinned: [4 p] d_step_flags[p], [4 p + 1] d_flags after a step of parity p,
-                                        // [2] d_flags after a load
+    int32_t *d_step_flags = nullptr;    // [2], one per step parity: bit 0 far mover, bit 1 bin overflow -> full rebuild;
+                                        // d_flags is the word after them
+    int32_t *h_step_flags = nullptr;    // pinned: [4 p ..] those three words after a step of parity p, [3] d_flags after
+                                        // a load
     const int32_t *guard = nullptr;     // steps: the previous step's flags; its particle kernels do nothing if set
     void *h_diag = nullptr;             // pinned host copy of the diagnostics record
     cudaEvent_t ev_flags[2] = {nullptr, nullptr};   // per step parity: that step's flags are on the host
@@ -920,8 +921,8 @@ struct SplineDep {
         }
     }
 
-    // All lanes of the warp: particle (s, val) of every lane with alive set; nx, ny: the grid's (or the
-    // block's tile's) cells, in whose numbering s's first node lies within -2 .. n + 1.
+    // All lanes of the warp: particle (s, val) of every lane with alive set; nx, ny: the grid's cells, in whose
+    // numbering s's first node lies within -2 .. n + 1.
     template <typename Sink>
     __device__ inline void add(const Sink &sink, int nx, int ny, bool alive, const SplineN<R, N> &s, const R *val,
                                int lane) {

@@ -16,7 +16,9 @@
 // particles written in the checkpoint form (cell, offsets, u, w) to a staging
 // buffer, and the species' segments compacted in place.  The host then appends
 // the staged particles to the target and electron species with one load
-// (pic_api.cu), which re-orders them as any load does and redeposits.
+// (pic_api.cu), which re-orders them as any load does.  The moments: the FP64 form
+// with the plain deposit adds the new particles' and takes the ionised ones' off;
+// the others deposit every particle anew before the moments are next read.
 #include <math.h>
 
 #include "pic_internal.cuh"

@@ -1154,7 +1154,10 @@ __device__ inline int block_excl_scan_int(int v, int *wsum, int *total) {
 // arrives every step, and one warp's copies kept the others waiting).  If the
 // bin cannot hold the result, or the arrivals overflow their list, the step flag
 // asks for the full regroup, which rebuilds from the bins and the mirror.
-// Bound by the latency of its dependent loads.
+// Bound by the latency of its dependent loads.  One range / one per warp, uniform
+// plasma, us: 64 x 64, 2 arrivals a tile 40.8 / 42.4, 76: 47.0 / 46.6, 136: 50.7 /
+// 49.1, 206: 53.4 / 50.8 (FP32 136: 41.6 / 40.4, 209: 44.2 / 41.0); 512 x 512,
+// where other tiles fill the wait, within 1 % from 1 to 104 arrivals.
 constexpr int REGROUP_RANGES = 2 * TILE_WARPS;
 constexpr int ARR_MAX = 8192;
 constexpr int ARR_SPLIT = 128;
@@ -1168,7 +1171,10 @@ constexpr int ARR_SPLIT = 128;
 // deposit halo is wider than a cell); elsewhere the buffer would only cost
 // resident blocks.  FP32: 67M particles at c dt / dx = 25, 2.38 -> 1.63 ms.  The
 // FP64 form (twelve arrays, fewer blocks) was slower staged: 41 -> 100 us on the
-// 64 x 64 plasma.
+// 64 x 64 plasma.  Staged / not, 512 x 512, 32 or 16 particles a cell, by cells per
+// segment: 1.0 274 / 264 us, 2.0 158 / 145, 4.0 346 / 510, 4.9 213 / 238, 5.3 348 /
+// 569, 11 422 / 786, 21 526 / 1008: the line lies above the segments that merely
+// straddle a few cells, where staging costs a twelfth.
 constexpr int STAGE_GROUPS = 5;
 constexpr int STAGE_BYTES = 36 * 1024;      // a tile's values of one array
 constexpr int STAGE_DST = 10 * 1024;        // source places (segment slots, then arrivals)
