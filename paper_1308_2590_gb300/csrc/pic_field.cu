@@ -1297,9 +1297,9 @@ constexpr float CN_SWEEP_RHO = 0.2f;
 // phases).  Thread partial sums of the FP32 phases are FP32 (a few nodes per
 // thread), block and grid sums FP64 in a fixed order.
 // out = [FP32 iterations, relative FP64 residual, refinements].
-// 64 x 64 periodic: 322 us (BiCGSTAB throughout, grid barriers, transposes, FP64
-// scalars in every thread) -> 142 us; 1024 x 1024: 2.56 -> 1.45 ms; 1024 x 512
-// with walls (block-Jacobi): 1.07 -> 0.85 ms.
+// Launch times, against BiCGSTAB throughout with grid barriers, transposes and FP64
+// scalars in every thread: 64 x 64 periodic 303 -> 150 us; 1024 x 1024, FP32, 2.56 ->
+// 1.58 ms; 1024 x 512 with walls (block-Jacobi) 1.04 -> 0.80 ms.
 template <bool kCluster, int BS>
 __global__ void __launch_bounds__(BS, kCluster ? 1 : 3) k_cn_solve(GridArgs<double> g, const double *__restrict__ Md, CNVec v, double c2, double tol,
                            int max_iter, double *part, double *out, WallRows wr) {
